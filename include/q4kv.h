@@ -112,8 +112,8 @@ enum { Q4KV_OUT_F32 = 0, Q4KV_OUT_BF16 = 1 };
 /* Accuracy of the attention entry points (float32 output, against the attention over the exactly
  * dequantized values evaluated in float64).  Let M be the largest |code*scale + bias| among the
  * attended keys and values.
- *   - Kernels that multiply the 4-bit codes (decode with d_qk = d_v in {128, 256} or d_qk 192 / d_v 128
- *     and at most four query heads per KV head; decode on the MLA-latent cache when the tile kernel
+ *   - Kernels that multiply the 4-bit codes (decode with d_qk = d_v in {128, 256} or d_qk 192 / d_v 128;
+ *     decode on the MLA-latent cache when the tile kernel
  *     below is not allowed; prefill with d in {128, 256} when it is not; the shape-agnostic kernels
  *     every other case falls back to): the products are exact, sums are float32, the
  *     probabilities enter the value product as a two-term binary16 pair or as float32.  Error

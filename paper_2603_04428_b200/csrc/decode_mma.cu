@@ -1,27 +1,24 @@
-// q4kv_decode_attention, tensor-core path for GQA shapes (d_qk = d_v in {128, 256}, at most four
-// query heads per KV head): one query token per agent over its whole Q4 cache, read in place
-// (Section 3.4 "Batched Quantized Inference": fused attention on the Q4 tensors; Section 3.6:
-// GQA head mapping and sliding-window layers).
+// q4kv_decode_attention, tensor-core path for GQA shapes (d_qk = d_v in {128, 256}, or d_qk 192 with d_v 128): one
+// query token per agent over its whole Q4 cache, read in place (Section 3.4 "Batched Quantized Inference": fused
+// attention on the Q4 tensors; Section 3.6: GQA head mapping and sliding-window layers).
 //
-// The kernel is bound by HBM bandwidth, so it is organised around the byte stream:
-//   * Work = the flattened list of 32-token chunks of all (agent, KV head) pairs inside their key
-//     range [lo, kv_len).  The list is cut into equal contiguous ranges, one per persistent CTA
-//     (one CTA per SM), so ragged lengths balance by construction.  A CTA's range may cover
-//     parts of several pairs ("segments").  A pair that lies inside one CTA is finished there;
-//     otherwise every CTA that holds a piece writes a partial (m, l, acc) record and takes a
-//     ticket, and the CTA that draws the last ticket combines the records -- one launch, no
-//     waiting on other CTAs.
-//   * The CTA's chunks stream through a shared-memory ring with one bulk asynchronous copy per
-//     chunk (a chunk is one contiguous byte range of the pool) completing on an mbarrier.  A
-//     planner warp walks the CTA's range ahead of the copies, 32 chunks per step in lockstep, and
-//     leaves each chunk's pool offset in a small shared-memory table; between steps it polls the
-//     ring, one lane per slot but all lanes on one path, and issues the copy of the next chunk of
-//     every slot whose previous chunk has been consumed.  The
-//     consumer warps run independently of one another: each claims the next chunk from a shared
-//     counter, keeps its own online-softmax state, and on leaving a segment deposits that state in
-//     shared memory; the warp that makes the deposit count complete combines the deposits and does
-//     the segment's epilogue (output, or record + ticket) while the others are already working on
-//     the next segment.  No CTA-wide barrier after start-up.
+// The floor is HBM bandwidth; what a launch of a few MB per SM actually spends is latency (the first bytes, the merge of
+// the partial results at its end) and instruction issue (about 450 warp instructions per 32-token chunk at d = 128).  So:
+//   * Work = the list of 32-token chunks of all (agent, KV head) pairs inside their key range [lo, kv_len), cut into
+//     contiguous ranges, one per CTA.  Where that costs few chunks (kWholeSlack) every pair is cut into equal parts of its
+//     own and a CTA holds one part; otherwise the list is cut into equal ranges, so that ragged lengths balance by
+//     construction, and a CTA may hold parts of several pairs ("segments").  A pair that lies inside one CTA is finished
+//     there; otherwise every CTA that holds a piece writes a partial (acc, m, l) record and takes a ticket, and the CTA
+//     that draws the pair's last ticket combines the records -- one launch, no waiting on other CTAs.
+//   * Eight warps per CTA, two CTAs per SM, 128 registers: four warps per scheduler.  One warp's chunk is one dependent
+//     chain (wait, products, maximum, exponentials, transposes, products), so the schedulers need that many to keep
+//     busy; the earlier form with two (seven consumer warps of 255 registers and a planner warp) issued 0.45
+//     instructions per scheduler and clock.  A second CTA also works through the first one's barriers and merges.
+//   * The chunks of a CTA's range are dealt to its warps in turn, and every warp streams its own through its own slots
+//     with one bulk asynchronous copy per chunk (a chunk is one contiguous byte range of the pool; two copies at
+//     d = 256, keys and values, so that the key half is refilled while the values are in work).  Pool offsets are
+//     looked up 32 chunks at a time, one per lane, before the warp needs them.  No two warps share a slot, so there
+//     is nothing to hand over; warps meet only at the end of a segment.
 //   * Arithmetic runs on the 4-bit codes, not on dequantized values.  With x^ = c*s + b and one
 //     (s, b) per token and 64-element group,
 //         q.k_t   = sum_g [ s_tg * (sum_{d in g} q_d c_td) + b_tg * (sum_{d in g} q_d) ]
@@ -33,13 +30,20 @@
 //     query is scaled per row by a power of two into binary16, so nothing is rounded before the
 //     products, which are exact.  (The 8-bit float forms of mma.sync are not used: on this part
 //     each costs two f16 tensor instructions plus conversions and adds.)
-//   * In the score product the key codes are the A operand (16 tokens x 16 head-dim elements) and the
-//     query the B operand (eight columns: the query heads 0..3 and their repeats), so a KV head's
-//     codes are unpacked once for all its query heads.  The probabilities times the token's value
-//     scale are transposed across the warp (movmatrix) into the B operand of the value product,
-//     whose A operand is the token-packed value words.  Columns 4..7 carry the low half of a
-//     two-term binary16 split of p*s, which makes the value product accurate to ~2^-22 at no
-//     extra MMA.
+//   * In the score product the key codes are the A operand (16 tokens x 16 head-dim elements) and the query the B
+//     operand, so a KV head's codes are unpacked once for all its query heads.  The probabilities times the token's
+//     value scale enter the value product as a two-term binary16 split (accurate to ~2^-22), transposed across the warp
+//     (movmatrix) into its B operand; the A operand is the token-packed value words.  Two forms by the eight columns of
+//     the B operands: up to four query heads per KV head -- columns 4..7 repeat the heads in the score product and
+//     carry the low halves of the split in the value product -- and, at d = 128, up to eight, the low halves in
+//     products of their own.  More query heads per KV head are cut into equal sets (at most four heads wide, eight at
+//     d = 128) that are attended like KV heads of their own and read the chunks again, from L2 for the most part.
+// Measured per launch in a replayed step (before: the form with seven consumer warps and a planner): d = 128, 4 heads per
+// KV head, 8 KV heads, agents x 4096 tokens: 1 agent 14.1 -> 8.9 us, 5 agents 17.5 -> 11.8 us (2.0 TB/s), 40 agents 72.9
+// -> 49.8 us (3.8 TB/s); d = 256, 16 agents x 8192 tokens, 81.4 -> 72.1 us (4.2 TB/s); 8 query heads per KV head, 12 agents
+// x 4096 tokens: 26 us with the append, 1.5 ms on the shape-agnostic kernel.
+//   * The reference of a warp's online softmax is taken over the warp, and the accumulators are rescaled, only when one
+//     vote says that some score outgrew it; it is then set kMargin above the maximum, so that it moves less often.
 #include <climits>
 
 #include "q4kv_layout.cuh"
@@ -49,7 +53,13 @@ namespace q4kv {
 
 namespace {
 
-constexpr int kMaxGrid = 512;                          // upper bound on the persistent grid (one CTA per SM)
+constexpr int kMaxGrid = 512;                          // upper bound on the grid (records are sized for it)
+constexpr int kCtasPerSm = 2;
+// warps per CTA: eight of 128 registers, or at d = 256, where the accumulators alone are 64, six of 168
+__host__ __device__ constexpr int warps_of(int G) { return G == 4 ? 6 : 8; }
+constexpr int kWholeSlack = 12;                        // see find_range
+constexpr float kMargin = 0.35f;                       // see chunk_values
+constexpr int kMaxRecords = 32;                        // a pair is cut over about this many CTAs at most (the merge reads them all)
 constexpr uint32_t kSpinLimit = 1u << 22;              // bounded mbarrier waits (each try blocks a while in hardware)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kMaskLo = 0x000F000Fu, kMaskHi = 0x00F000F0u;
@@ -79,7 +89,6 @@ __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: gives up after kSpinLimit tries or as soon as another warp has given up.
 __device__ inline bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -89,8 +98,8 @@ __device__ inline bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_test_wait(bar, parity)) return true;        // the usual case: the chunk landed long ago (a blocking try costs more)
+// Bounded wait: gives up after kSpinLimit tries or as soon as another warp has given up.
+__device__ __noinline__ bool mbar_wait_long(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   for (uint32_t i = 0; i < kSpinLimit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((i & 63u) == 63u && *abort_flag) return false;
@@ -98,18 +107,12 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* a
   *abort_flag = 1;
   return false;
 }
-// Bounded spin on a shared-memory word until it reaches `want`.
-__device__ inline bool spin_until_ge(volatile int* word, int want, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < (kSpinLimit << 4); ++i) {
-    if (*word >= want) return true;
-#ifdef Q4KV_SPIN_SLEEP
-    __nanosleep(Q4KV_SPIN_SLEEP);
-#endif
-    if ((i & 255u) == 255u && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
+// Whole warp.  The usual case is that the bytes landed long ago (a blocking try costs more).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_long(bar, parity, abort_flag));
 }
+__device__ inline void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ inline void prefetch_l2_bulk(const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
@@ -157,6 +160,7 @@ struct DecodeParams {
   const int32_t* kv_lens;
   const uint16_t* q;          // bf16 [layer_count][A][Hq][D]
   float scale_log2;           // softmax_scale * log2(e)
+  int Hkv, n_rep, sets;       // pairs are over sets of query heads: Hkv = y.Hkv * sets, n_rep = y.n_rep / sets
   int32_t* tickets;           // [A*Hkv], zero between calls
   float* partials;            // [A*Hkv + grid][n_rep][Dv + 4]
   void* out;
@@ -200,21 +204,58 @@ struct Partition {
 
 // Warp-cooperative: total number of units U, this CTA's range and the agent that contains its
 // first unit.  One pass over the agents when there are at most 32 of them.
-struct RangeStart { uint32_t U, u_begin, u_end, agent_start; int n_ctas, agent; bool any_bad; Partition part; };
+struct RangeStart {
+  uint32_t U, u_begin, u_end, agent_start;
+  int n_ctas, agent;
+  bool any_bad;
+  Partition part;
+  int split, splits, pair;  // splits > 0: this CTA holds part `split` of the `splits` parts of head set `pair` of the agent,
+  AgentRange r;             // whose range this is
+};
 
-__device__ inline RangeStart find_range(const DecodeParams& P, int cta, int grid) {
+// The agent that contains the CTA's first unit, among more than 32 of them (out of line: instruction fetches are what a
+// launch starts with).
+__device__ __noinline__ void find_agent(const DecodeParams& P, RangeStart& rs) {
   const int lane = threadIdx.x & 31;
-  const int n_agents = P.n_agents, Hkv = P.y.Hkv;
+  uint32_t cum = 0;
+#pragma unroll 1
+  for (int base = 0; base < P.n_agents; base += 32) {
+    const int a = base + lane;
+    uint32_t cnt = 0;
+    bool bad = false;
+    if (a < P.n_agents) cnt = (uint32_t)(agent_range(P, a, bad).nc * P.Hkv);
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+    if (rs.u_begin < cum + tot) {
+      const int l = __ffs(__ballot_sync(0xffffffffu, cum + inc > rs.u_begin)) - 1;
+      rs.agent = base + l;
+      rs.agent_start = cum + __shfl_sync(0xffffffffu, inc, l) - __shfl_sync(0xffffffffu, cnt, l);
+      return;
+    }
+    cum += tot;
+  }
+}
+
+__device__ inline RangeStart find_range(const DecodeParams& P, int cta, int grid, uint32_t nw) {
+  const int lane = threadIdx.x & 31;
+  const int n_agents = P.n_agents, Hkv = P.Hkv;
   RangeStart rs;
   rs.any_bad = false;
   rs.agent = -1;
   rs.agent_start = 0;
   uint32_t cum = 0, inc0 = 0, cnt0 = 0;
+  rs.r.n = 0; rs.r.lo = 0; rs.r.cf = 0; rs.r.nc = 0;
+#pragma unroll 1
   for (int base = 0; base < n_agents; base += 32) {
     const int a = base + lane;
     uint32_t cnt = 0;
     bool bad = false;
-    if (a < n_agents) cnt = (uint32_t)(agent_range(P, a, bad).nc * Hkv);
+    if (a < n_agents) { rs.r = agent_range(P, a, bad); cnt = (uint32_t)(rs.r.nc * Hkv); }
     rs.any_bad |= __any_sync(0xffffffffu, bad);
     uint32_t inc = cnt;
 #pragma unroll
@@ -226,10 +267,61 @@ __device__ inline RangeStart find_range(const DecodeParams& P, int cta, int grid
     cum += __shfl_sync(0xffffffffu, inc, 31);
   }
   rs.U = cum;
-  rs.n_ctas = (uint32_t)grid < cum ? grid : (int)cum;
+  // at least a chunk for every warp of a CTA, and not more CTAs on a pair than the merge takes quickly
+  const uint32_t most = min((uint32_t)grid, (uint32_t)(n_agents * Hkv) * (uint32_t)kMaxRecords);
+  rs.n_ctas = (int)min(most, (cum + nw - 1) / nw);
   rs.u_begin = rs.u_end = 0;
   rs.part.U = 0; rs.part.n = 1; rs.part.q = 0; rs.part.r = 0;
-  if (cum == 0 || cta >= rs.n_ctas) return rs;
+  rs.splits = 0; rs.split = 0; rs.pair = 0;
+  if (cum == 0) return rs;
+  if (n_agents <= 32) {
+    // Cut every pair into equal parts of at most `size` chunks if that takes at most kWholeSlack chunks per CTA more than
+    // an equal division of the list: a CTA then holds one segment, and the end of a segment (barriers, combination, the
+    // next query: about two rounds of chunks) comes once.  Lane l tries size + l.
+    const int nc = lane < n_agents ? rs.r.nc : 0;
+    int nc_max = nc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nc_max = max(nc_max, __shfl_xor_sync(0xffffffffu, nc_max, o));
+    const int size0 = max(max((int)nw, (int)((cum + most - 1) / most)), (nc_max + kMaxRecords - 1) / kMaxRecords);
+    const int size = size0 + lane;
+    const float inv = 1.f / (float)size;
+    auto parts_of = [](int n, int sz, float rcp) {       // ceil(n / sz)
+      int q = (int)((float)n * rcp);
+      q += q * sz < n;
+      q -= (q - 1) * sz >= n;
+      return q;
+    };
+    int total = 0;
+#pragma unroll 1
+    for (int a = 0; a < n_agents; ++a) total += parts_of(__shfl_sync(0xffffffffu, nc, a), size, inv);
+    const unsigned fits = __ballot_sync(0xffffffffu, total * Hkv <= (int)most && lane <= kWholeSlack);
+    if (fits) {
+      const int l = __ffs(fits) - 1;
+      const int best = size0 + l;
+      rs.n_ctas = __shfl_sync(0xffffffffu, total, l) * Hkv;
+      if (cta >= rs.n_ctas) return rs;
+      const int m = parts_of(nc, best, __shfl_sync(0xffffffffu, inv, l));
+      int inc = m * Hkv;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      const int a = __ffs(__ballot_sync(0xffffffffu, inc > cta)) - 1;
+      rs.agent = a;
+      rs.splits = __shfl_sync(0xffffffffu, m, a);
+      const int at = cta - (__shfl_sync(0xffffffffu, inc, a) - rs.splits * Hkv), n = __shfl_sync(0xffffffffu, nc, a);
+      rs.pair = at / rs.splits;
+      rs.split = at - rs.pair * rs.splits;
+      rs.agent_start = 0;                                // units count from the pair's first chunk here
+      rs.r.n = __shfl_sync(0xffffffffu, rs.r.n, a); rs.r.lo = __shfl_sync(0xffffffffu, rs.r.lo, a);
+      rs.r.cf = __shfl_sync(0xffffffffu, rs.r.cf, a); rs.r.nc = n;
+      rs.u_begin = (uint32_t)n * (uint32_t)rs.split / (uint32_t)rs.splits;
+      rs.u_end = (uint32_t)n * (uint32_t)(rs.split + 1) / (uint32_t)rs.splits;
+      return rs;
+    }
+  }
+  if (cta >= rs.n_ctas) return rs;
   rs.part.init(cum, (uint32_t)rs.n_ctas);
   rs.u_begin = rs.part.begin(cta);
   rs.u_end = rs.part.begin(cta + 1);
@@ -241,84 +333,64 @@ __device__ inline RangeStart find_range(const DecodeParams& P, int cta, int grid
     rs.agent_start = __shfl_sync(0xffffffffu, inc0, l) - __shfl_sync(0xffffffffu, cnt0, l);
     return rs;
   }
-  cum = 0;
-  for (int base = 0; base < n_agents; base += 32) {
-    const int a = base + lane;
-    uint32_t cnt = 0;
-    bool bad = false;
-    if (a < n_agents) cnt = (uint32_t)(agent_range(P, a, bad).nc * Hkv);
-    uint32_t inc = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += v;
-    }
-    const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
-    if (want < cum + tot) {
-      const unsigned bal = __ballot_sync(0xffffffffu, cum + inc > want);
-      const int l = __ffs(bal) - 1;
-      rs.agent = base + l;
-      rs.agent_start = cum + __shfl_sync(0xffffffffu, inc, l) - __shfl_sync(0xffffffffu, cnt, l);
-      return rs;
-    }
-    cum += tot;
-  }
+  find_agent(P, rs);
   return rs;
 }
 
-// One segment: the part of pair (agent a, KV head hk) inside this CTA's unit range.  A segment is walked from its last
-// chunk to its first (the order does not matter to the online softmax).  With the fused append, the chunk of the agent's
-// newest position -- the pair's last chunk -- is patched by the planner warp after it has landed; it is moved a few
-// places back in the walk (to place tail_pos), so that the consumers have other chunks to work on meanwhile.
-constexpr int kTailPos = 14;
+// One segment: the part of pair (agent a, head set hk) inside this CTA's unit range.
 struct Segment {
-  int a, hk, c0, c1;      // (virtual) agent, KV head, logical chunk indices [c0, c1) of the agent
+  int a, hk, c0, c1;      // (virtual) agent, head set, logical chunk indices [c0, c1) of the agent
   int ar, li;             // real agent (lengths, block table) and layer of the call (pool layer)
   int n, lo;              // key range of the agent
   int cf, nc;             // the pair's whole chunk range
   int k0;                 // running chunk counter of the CTA at c0
-  uint32_t u0;            // global unit index at c0
-  int tail_pos;           // place in the walk of the chunk that receives the new token; -1: none in this segment
-  __device__ void set_tail(bool fused) {
-    const int cnt = c1 - c0;
-    tail_pos = (fused && c1 == cf + nc) ? (cnt - 1 < kTailPos ? cnt - 1 : kTailPos) : -1;
-  }
-  __device__ int chunk_at(int j) const {    // logical chunk at place j of the walk, 0 <= j < c1 - c0
-    if (tail_pos < 0 || j > tail_pos) return c1 - 1 - j;
-    return j == tail_pos ? c1 - 1 : c1 - 2 - j;
-  }
+  int first, last;        // CTAs that hold the pair's first and last chunk
 };
 
+// The one segment of a CTA that holds a part of one pair.
+__device__ inline void whole_segment(const DecodeParams& P, const RangeStart& rs, Segment& s) {
+  s.li = P.layer_count > 1 ? rs.agent / P.n_real : 0; s.ar = rs.agent - s.li * P.n_real;
+  s.a = rs.agent; s.hk = rs.pair; s.c0 = rs.r.cf + (int)rs.u_begin; s.c1 = rs.r.cf + (int)rs.u_end;
+  s.n = rs.r.n; s.lo = rs.r.lo; s.cf = rs.r.cf; s.nc = rs.r.nc; s.k0 = 0;
+  s.first = (int)blockIdx.x - rs.split;
+  s.last = s.first + rs.splits - 1;
+}
+
 struct Walker {
-  const DecodeParams* P;
   int n_agents, Hkv;
   uint32_t u, u_end;
   int k, a, hk, c;
-  bool fused;               // the launch appends one token per agent
   AgentRange r;
 
-  __device__ void init(const DecodeParams& P_, const RangeStart& rs) {
-    P = &P_; n_agents = P_.n_agents; Hkv = P_.y.Hkv; fused = P_.k_new != nullptr;
+  __device__ __forceinline__ void init(const DecodeParams& P_, const RangeStart& rs) {
+    n_agents = P_.n_agents; Hkv = P_.Hkv;
     u = rs.u_begin; u_end = rs.u_end; k = 0;
     a = rs.agent; hk = 0; c = 0;
     r.n = 0; r.lo = 0; r.cf = 0; r.nc = 0;
     if (u < u_end && a >= 0) {
       bool bad;
-      r = agent_range(*P, a, bad);
-      const uint32_t rem = u - rs.agent_start;
-      hk = (int)(rem / (uint32_t)r.nc);
-      c = r.cf + (int)(rem - (uint32_t)hk * (uint32_t)r.nc);
+      r = agent_range(P_, a, bad);
+      {
+        const uint32_t rem = u - rs.agent_start;
+        hk = (int)(rem / (uint32_t)r.nc);
+        c = r.cf + (int)(rem - (uint32_t)hk * (uint32_t)r.nc);
+      }
     }
   }
-  __device__ bool next(Segment& s) {
-    if (u >= u_end || a < 0) return false;
+  __device__ __forceinline__ bool next(const DecodeParams& P, const RangeStart& rs, Segment& s) {
+    if (u >= u_end || a < 0) { s.a = -1; return false; }
     const int pair_end = r.cf + r.nc;
     const uint32_t left = u_end - u;
     const int c1 = (uint32_t)(pair_end - c) <= left ? pair_end : c + (int)left;
-    s.li = P->layer_count > 1 ? a / P->n_real : 0; s.ar = a - s.li * P->n_real;
-    s.a = a; s.hk = hk; s.c0 = c; s.c1 = c1; s.n = r.n; s.lo = r.lo; s.cf = r.cf; s.nc = r.nc; s.k0 = k; s.u0 = u;
-    s.set_tail(fused);
+    s.li = P.layer_count > 1 ? a / P.n_real : 0; s.ar = a - s.li * P.n_real;
+    s.a = a; s.hk = hk; s.c0 = c; s.c1 = c1; s.n = r.n; s.lo = r.lo; s.cf = r.cf; s.nc = r.nc; s.k0 = k;
     const int cnt = c1 - c;
+    s.first = s.last = 0;
+    if (cnt != r.nc) {
+      const uint32_t pair_u0 = u - (uint32_t)(c - r.cf);
+      s.first = rs.part.cta_of(pair_u0);
+      s.last = rs.part.cta_of(pair_u0 + (uint32_t)r.nc - 1u);
+    }
     u += (uint32_t)cnt; k += cnt;
     if (c1 == pair_end) {
       ++hk;
@@ -328,7 +400,7 @@ struct Walker {
         do {
           ++a;
           if (a >= n_agents) { a = -1; break; }
-          r = agent_range(*P, a, bad);
+          r = agent_range(P, a, bad);
         } while (r.nc == 0);
       }
       if (a >= 0) c = r.cf;
@@ -342,198 +414,159 @@ struct Walker {
 // ---------------------------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------------------------
-
-__host__ __device__ constexpr int kRecStride(int Dv) { return Dv + 4; }
 // The kernel is instantiated by the number of key groups G: 2 and 4 are the symmetric shapes (d_qk = d_v = 64 G), 3 is
-// the asymmetric per-head MLA cache of Section 3.6 (d_qk 192, d_v 128).
-__host__ __device__ constexpr int value_groups(int G) { return G == 3 ? 2 : G; }   // acc[Dv], m, l, pad: 16-byte multiples
-constexpr int kQBufs = 4;      // query-fragment buffers (segments s, s+4, ... share one)
-constexpr int kOffCap = 256;   // entries of the planner's offset table (a ring over the CTA's chunk indices)
-constexpr int kTailQ = 8;      // chunks waiting for the planner's patch (planning stops while the queue is full)
-constexpr uint32_t kOffBad = 0xFFFFFFFFu;   // table entry of a chunk whose block id is outside the pool
-constexpr int kSmemBudget = 232448 - 2048;   // 227 KB per CTA, less the small arrays of the structure below
+// the asymmetric per-head MLA cache of Section 3.6 (d_qk 192, d_v 128); by the head columns H (4 or 8); and by the type
+// of the scales and biases.
+__host__ __device__ constexpr int kRecStride(int Dv) { return Dv + 4; }      // acc[Dv], m, l, pad: 16-byte multiples
+__host__ __device__ constexpr int value_groups(int G) { return G == 3 ? 2 : G; }
+constexpr uint32_t kOffBad = 0xFFFFFFFFu;   // pool offset of a chunk whose block id is outside the pool
 
-// consumer warps per CTA.  Two warps per scheduler: the hot loop wants ~180 registers per thread at d = 128 and ~245 at
-// d = 256, and with three warps per scheduler (168 registers) what the compiler moves to local memory costs more than
-// the third warp brings, since almost no L1 is left beside the ring (measured: 78 against 71 us on 40 agents x 4096)
-#ifndef Q4KV_DECODE_WARPS_D128
-#define Q4KV_DECODE_WARPS_D128 7
-#endif
-#ifndef Q4KV_DECODE_WARPS_D256
-#define Q4KV_DECODE_WARPS_D256 7
-#endif
-
-template <int G, int NW>
+template <int G, int H>
 struct Smem {
   static constexpr int D = 64 * G, Gv = value_groups(G), Dv = 64 * Gv;
-  static constexpr int kChunkBytes = 32 * (D / 2 + 4 * G + Dv / 2 + 4 * Gv);
-  static constexpr int kMergeStride = Dv + 8;           // acc[Dv], m, l, bias[Gv], pad
-  // deposit buffers (consecutive segments alternate).  One at d = 256: its 30 KB are worth more as four ring slots (20
-  // instead of 16: the global layer of the ragged benchmark runs 1.2 % faster, bytes in flight being what limits it)
-  static constexpr int kMBufs = G == 4 ? 1 : 2;
-  static constexpr int kRingBudget = kSmemBudget - kMBufs * NW * 4 * kMergeStride * 4 - kQBufs * 2 * G * 32 * 16;
-  static constexpr int kSlots = kRingBudget / kChunkBytes < 32 ? kRingBudget / kChunkBytes : 32;   // one producer lane per slot
-  alignas(128) uint8_t ring[kSlots * kChunkBytes];
-  alignas(16) float merge[kMBufs][NW][4][kMergeStride];
-  alignas(16) uint4 qfrag[kQBufs][2 * G][32];           // [buffer][key word of a lane][lane = row * 4 + tid] = A registers
-  float qsum[kQBufs][4][G];                             // scale_log2 * sum of the true q over each group
-  float kappa[kQBufs][4];                               // scale_log2 * 2^(ex + 13)
-  alignas(8) uint64_t full[kSlots];
-  uint32_t src_off[kOffCap];    // pool offset (16-byte units inside the layer) of chunk k at k % kOffCap; kOffBad: bad block id
-  int released[kSlots];         // number of times each slot has been consumed (monotonic: no parity aliasing)
-  int patched[kSlots];          // round + 1 of the last chunk the planner has patched in each slot (fused append)
-  int4 tail_q[kTailQ];          // planner's queue of chunks to patch: (chunk index in the CTA, agent, KV head, token in chunk)
-  int bad[kSlots];
-  int q_tag[kQBufs];            // s + 1 once the query of segment s is staged in buffer s % kQBufs
-  int deposits[kMBufs];         // running count of deposits into each buffer
-  int epilogues[kMBufs];        // number of completed epilogues of each buffer
-  int next_chunk;               // claim counter
-  int epi_claim[kMBufs];        // uses of each deposit buffer whose epilogue has been taken (by a consumer or the planner)
-  int all_issued;               // set by the planner once every chunk of the CTA has been issued
-  int fin_arrived;              // last segment: head warps whose record is written
-  int fin_ticket;               // last segment: 0 until the ticket is drawn, then 1 (not the last) or 2 (combine the records)
+  static constexpr int kKeyBytes = 32 * (D / 2 + 4 * G), kValBytes = 32 * (Dv / 2 + 4 * Gv);
+  static constexpr int kChunkBytes = kKeyBytes + kValBytes;
+  static constexpr int NW = warps_of(G);
+  // Slots of a warp.  Two whole chunks (147 KB per SM in flight: twice what HBM latency asks for); at d = 256 two key
+  // halves and one value half, each with a barrier of its own (166 KB per SM).
+  static constexpr bool kHalves = G == 4;
+  static constexpr int kSlots = 2, kValSlots = kHalves ? 1 : 2;
+  static constexpr int kWarpRing = kHalves ? kSlots * kKeyBytes + kValSlots * kValBytes : kSlots * kChunkBytes;
+  static constexpr int kDepUnits = H * Dv / 128;
+  alignas(128) uint8_t ring[NW][kWarpRing];
+  alignas(16) float4 dep[NW][kDepUnits][32];            // accumulators of every warp, bias sums added (see deposit)
+  float dep_m[NW][H], dep_l[NW][H];
+  alignas(16) uint4 qfrag[2 * G][32];                   // [key word of a lane][lane = column * 4 + tid] = B registers
+  float qsum[H][G];                                     // sum of the query over each group, in units of the score products
+  float kappa[H];                                       // score products -> log2 units
+  alignas(8) uint64_t full[NW][kSlots], full_v[NW][kValSlots];   // full_v: only where halves are copied
+  RangeStart range;                                     // the CTA's range, for walks that start over
+  Walker walker;                                        // runs two segments ahead
+  uint32_t new_words[8 * (G + Gv)], new_sb[G + Gv];     // the quantized new row of the segment: K groups, then V groups
+  Segment seg[3];                                       // segments s, s + 1, s + 2 at s % 3; a < 0: none
+  int fin[2][4];                                        // the CTA's first and last segment: pair, first CTA, last CTA, row
+  int fin_last[2];                                      // this CTA drew the pair's last ticket
   int abort_flag;
 };
 
-// Online-softmax state of one warp for one segment.  A lane owns two score columns (2 * tid, 2 * tid + 1 of eight:
-// columns 0..3 are the query heads, 4..7 repeat them) and, of every 32-token chunk, the four tokens 4 * g .. 4 * g + 3;
-// m, l and the bias sums are per column, partial over the lane's tokens.
+// Online-softmax state of one warp for one segment.  A lane owns two score columns (2 tid, 2 tid + 1 of eight) and, of
+// every 32-token chunk, the four tokens 4 g .. 4 g + 3; l and the bias sums are per column, partial over the lane's
+// tokens; the reference maximum m is common to the lanes of a column.
 template <int G>
 struct WarpState {
   static constexpr int Gv = value_groups(G);
-  float m[2], l_e[2], l_o[2], bias_e[2][Gv], bias_o[2][Gv];
+  float m[2], l[2], bias[2][Gv];
   float o[4 * Gv][4];
+  int head_room;                                         // H = 8: see chunk_values
+  uint32_t vlimit;
   __device__ void reset() {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      m[c] = -INFINITY; l_e[c] = 0.f; l_o[c] = 0.f;
+      m[c] = -INFINITY; l[c] = 0.f;
 #pragma unroll
-      for (int i = 0; i < Gv; ++i) { bias_e[c][i] = 0.f; bias_o[c][i] = 0.f; }
+      for (int i = 0; i < Gv; ++i) bias[c][i] = 0.f;
     }
 #pragma unroll
     for (int i = 0; i < 4 * Gv; ++i) { o[i][0] = 0.f; o[i][1] = 0.f; o[i][2] = 0.f; o[i][3] = 0.f; }
+    head_room = 40;
+    vlimit = 0u;
   }
 };
 
-// Warp-level: stage the query rows of one pair as binary16 in A-fragment order (each row scaled by a
-// power of two, so nothing is rounded), plus the per-group sums of the true query and the per-head
-// factor that undoes the scaling.  Key word w = 8*gi + 4*i2 + t of a token holds elements 8w..8w+7
-// and feeds two 16x8x16 products: (0,4 | 1,5) and (2,6 | 3,7), where the second pair of each meets
-// codes in nibble 1 of their 16-bit lanes (a factor 16, divided out of the query here).  The uint4
-// of word p = 2*gi + i2 is {a0, a2} of the first product and {a0, a2} of the second, for the lane
-// (row h, t); rows h + 4 repeat rows h, so that lanes g and g + 4 see the same scores.
-template <int G>
-__device__ __noinline__ void stage_query(uint4 (*qfrag)[32], float (*qsum)[G], float* kappa,
-                                         const uint16_t* __restrict__ q, int Hq, int n_rep, float scale_log2, int a,
-                                         int hk, int lane) {
+// One warp stages one query row (column h) as binary16 in B-fragment order, scaled by a power of two so that nothing is
+// rounded, plus the per-group sums of the query and the factor that undoes the scaling.  Key word w = 8*gi + 4*i2 + t of
+// a token holds elements 8w..8w+7 and feeds two 16x8x16 products: (0,4 | 1,5) and (2,6 | 3,7), where the second pair of
+// each meets codes in nibble 1 of their 16-bit lanes (a factor 16, divided out of the query here).  The uint4 of word
+// p = 2*gi + i2 is {b0, b1} of the first product and {b0, b1} of the second, for the lane (column h, t).  The sign of
+// the softmax scale goes into the query, so that the factor is positive.
+template <int G, int H>
+__device__ __forceinline__ void stage_query_row(uint4 (*qfrag)[32], float (*qsum)[G], float* kappa, const uint4 v, float scale_log2,
+                                                int h, int lane) {
   constexpr int D = 64 * G;
-  // a row's D / 8 words sit in kRowLanes consecutive lanes (a power of two, so that the row maximum is a butterfly)
-  constexpr int kRowLanes = D / 8 <= 16 ? 16 : 32;
-  for (int base = 0; base < n_rep * kRowLanes; base += 32) {
-    const int idx = base + lane;
-    const int h_raw = idx / kRowLanes, w = idx % kRowLanes;
-    const bool valid = h_raw < n_rep && w < D / 8;
-    const int h = valid ? h_raw : 0;
-    const uint16_t* qrow = q + ((size_t)a * Hq + (size_t)hk * n_rep + h) * D;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (valid) v = *reinterpret_cast<const uint4*>(qrow + 8 * w);
-    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-    float x[8];
+  const int w = lane;
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};          // lanes at or beyond D / 8 hold zeros
+  float x[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { x[2 * i] = __uint_as_float(u[i] << 16); x[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
-    // row maximum and group sums: the D/8 lanes of a row are consecutive (16 or 32)
-    float mx = 0.f, sum = 0.f;
+  for (int i = 0; i < 4; ++i) { x[2 * i] = __uint_as_float(u[i] << 16); x[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
+  float mx = 0.f, sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { mx = fmaxf(mx, fabsf(x[i])); sum += x[i]; }
+  for (int i = 0; i < 8; ++i) { mx = fmaxf(mx, fabsf(x[i])); sum += x[i]; }
 #pragma unroll
-    for (int o = kRowLanes / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);   // 8 words per group
-    if (!valid) continue;
-    int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
-    if (mx == 0.f) ex = 0;
-    ex = min(max(ex, -100), 100);
-    const float sf = __uint_as_float((uint32_t)(127 + 11 - ex) << 23);         // 2048 <= max |q| * sf < 4096
-    const float sl = sf * 0.0625f;
+  for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);   // 8 words per group
+  int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
+  if (mx == 0.f) ex = 0;
+  ex = min(max(ex, -100), 100);
+  float sf = __uint_as_float((uint32_t)(127 + 11 - ex) << 23);                 // 2048 <= max |q| * sf < 4096
+  const float kap = fabsf(scale_log2) * __uint_as_float((uint32_t)(127 + 13 + ex) << 23);   // 2^24 / sf
+  if (scale_log2 < 0.f) sf = -sf;
+  if (scale_log2 == 0.f) sf = 0.f;
+  const float sl = sf * 0.0625f;
+  if (w < D / 8) {
     const uint4 f = make_uint4(f32x2_to_h2_rn(x[0] * sf, x[4] * sf), f32x2_to_h2_rn(x[1] * sl, x[5] * sl),
                                f32x2_to_h2_rn(x[2] * sf, x[6] * sf), f32x2_to_h2_rn(x[3] * sl, x[7] * sl));
     const int gi = w >> 3, i2 = (w >> 2) & 1, t = w & 3;
     qfrag[2 * gi + i2][h * 4 + t] = f;
-    qfrag[2 * gi + i2][(h + 4) * 4 + t] = f;
-    if ((w & 7) == 0) qsum[h][gi] = sum * scale_log2;
-    if (w == 0) kappa[h] = scale_log2 * __uint_as_float((uint32_t)(127 + 13 + ex) << 23);  // 2^24 / sf
+    if (H == 4) qfrag[2 * gi + i2][(h + 4) * 4 + t] = f;                       // columns 4..7 repeat the heads
+    if ((w & 7) == 0) qsum[h][gi] = sum * sf * 5.9604644775390625e-8f;         // 2^-24: the codes enter as c * 2^-24
+    if (w == 0) kappa[h] = kap > 0.f ? kap : 1.f;
   }
 }
 
-// Fused append (one new token per agent): the planner warp of the CTA that holds the chunk of an agent's newest position
-// quantizes that token's K and V rows (Section 3.2 quantizer, the same device function the append kernel uses) and
-// writes them into the chunk once it has landed -- in shared memory for this launch, in the pool for the following
-// ones -- and then lets the chunk's consumer go on.  Every chunk is held by exactly one CTA of the grid, so nobody else
-// reads or writes these words during the launch.
-// Eight consecutive lanes own one 64-element group; the 8-lane shuffles never straddle K and V (D / 8 is a multiple
-// of 8).  The value codes are token-packed: one nibble of each of the row's d_v words is replaced.
-template <int G>
-__device__ __noinline__ void append_new_token(uint8_t* chunk, uint8_t* gchunk, const Layout& y,
-                                              const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
-                                              int a, int hk, int tau, int lane) {
-  constexpr int D = 64 * G, Gv = value_groups(G), Dv = 64 * Gv, W = D / 8, Wv = Dv / 8;   // words per K row, per V row
-  const size_t head = (size_t)a * y.Hkv + hk;
-#pragma unroll
-  for (int base = 0; base < W + Wv; base += 32) {
-    const int idx = base + lane;
-    const bool live = idx < W + Wv;                      // W + Wv need not be a multiple of 32: idle lanes quantize zeros
-    const bool is_v = idx >= W;
-    const int w = is_v ? (idx - W) % Wv : idx;
-    float x[8];
-    {
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (live) v = *reinterpret_cast<const uint4*>(is_v ? v_new + head * Dv + 8 * w : k_new + head * D + 8 * w);
-      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { x[2 * i] = __uint_as_float(u[i] << 16); x[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u); }
-    }
-    const QuantOut qo = quantize_eight(x, y.sb_bf16 != 0);
-    const uint32_t sb = qo.sb;
-    if (!live) continue;
-    if (!is_v) {
-      const uint32_t at = y.off_kc + 4u * k_word_offset(tau, w, G);
-      *reinterpret_cast<uint32_t*>(chunk + at) = qo.word;
-      *reinterpret_cast<uint32_t*>(gchunk + at) = qo.word;
-      if ((w & 7) == 0) {
-        const uint32_t sat = y.off_ksb + 4u * sb_offset(tau, w >> 3, G);
-        *reinterpret_cast<uint32_t*>(chunk + sat) = sb;
-        *reinterpret_cast<uint32_t*>(gchunk + sat) = sb;
-      }
-    } else {
-      const int shift = 4 * (tau & 7);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const uint32_t at = y.off_vc + 4u * v_word_offset(tau >> 3, 8 * w + e);
-        const uint32_t old = *reinterpret_cast<const uint32_t*>(chunk + at);
-        const uint32_t nw = (old & ~(0xFu << shift)) | (((qo.word >> (4 * e)) & 0xFu) << shift);
-        *reinterpret_cast<uint32_t*>(chunk + at) = nw;
-        *reinterpret_cast<uint32_t*>(gchunk + at) = nw;
-      }
-      if ((w & 7) == 0) {
-        const uint32_t sat = y.off_vsb + 4u * sb_offset(tau, w >> 3, Gv);
-        *reinterpret_cast<uint32_t*>(chunk + sat) = sb;
-        *reinterpret_cast<uint32_t*>(gchunk + sat) = sb;
-      }
-    }
+// The fused append (one new token per agent).  The CTA that holds the chunk of an agent's newest position quantizes that
+// token's K and V rows (Section 3.2 quantizer, the arithmetic of the append kernel) when it stages the segment's query: a
+// warp per 64-element group, two elements per lane, by the warps that have no query row to stage, so that neither waits
+// for the other.  The warp that holds the chunk writes the words into it once it has landed -- in shared memory for this
+// launch, in the pool for the following ones.  Every chunk is held by exactly one warp of the grid, so nobody else reads
+// or writes these words during the launch.  (One warp doing all of it, eight elements per lane, was 3.5 us on the
+// critical path of every launch: 500 instructions that run once per launch and come from far away.)
+template <int G, int H>
+__device__ __forceinline__ void quantize_new_group(Smem<G, H>& sm, uint32_t two, int grp, bool bf16, int lane) {
+  const float x0 = __uint_as_float(two << 16), x1 = __uint_as_float(two & 0xffff0000u);
+  float mn = fminf(x0, x1), mx = fmaxf(x0, x1);
+  asm("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(mn));
+  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(mx));
+  const GroupScale gs = group_scale(mn, mx, bf16);
+  uint32_t w = 0u;
+  if (gs.sf != 0.f) {
+    const float inv = __frcp_rn(gs.sf);
+    w = (quantize_code(x0, gs, inv) | (quantize_code(x1, gs, inv) << 4)) << (8 * (lane & 3));
   }
-  __syncwarp();                                          // the patched chunk is read by the same warp
+  w |= __shfl_xor_sync(0xffffffffu, w, 1);
+  w |= __shfl_xor_sync(0xffffffffu, w, 2);
+  if ((lane & 3) == 0) sm.new_words[8 * grp + (lane >> 2)] = w;
+  if (lane == 0) sm.new_sb[grp] = gs.hs | (gs.hb << 16);
 }
-
-// Ask for the new token's rows early (when the segment's query is staged), so that the warp that later owns the
-// chunk finds them in L2.
-template <int G>
-__device__ inline void prefetch_new_token(const uint16_t* k_new, const uint16_t* v_new, int Hkv, int a, int hk, int lane) {
-  constexpr int D = 64 * G, Dv = 64 * value_groups(G), kLines = D * 2 / 128, kLinesV = Dv * 2 / 128;   // 128-byte lines per row
-  if (lane < kLines + kLinesV) {
-    const size_t head = (size_t)a * Hkv + hk;
-    const uint16_t* p = lane < kLines ? k_new + head * D + lane * 64 : v_new + head * Dv + (lane - kLines) * 64;
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+// The value codes are token-packed: one nibble of each of the row's d_v words is replaced.
+template <int G, int H>
+__device__ __noinline__ void patch_new_row(const Smem<G, H>& sm, uint8_t* keys, uint8_t* values, uint8_t* gchunk, int tau, int lane) {
+  constexpr int D = 64 * G, Gv = value_groups(G), Dv = 64 * Gv;
+  constexpr uint32_t off_ksb = 32 * (D / 2), key_bytes = off_ksb + 128 * G, off_vsb = 32 * (Dv / 2);
+  auto put = [&](uint8_t* half, uint32_t base, uint32_t at, uint32_t v) {
+    *reinterpret_cast<uint32_t*>(half + at) = v;
+    *reinterpret_cast<uint32_t*>(gchunk + base + at) = v;
+  };
+  if (lane < 8 * G) put(keys, 0u, 4u * k_word_offset(tau, lane, G), sm.new_words[lane]);
+  if (lane < G) put(keys, 0u, off_ksb + 4u * sb_offset(tau, lane, G), sm.new_sb[lane]);
+  if (lane < Gv) put(values, key_bytes, off_vsb + 4u * sb_offset(tau, lane, Gv), sm.new_sb[G + lane]);
+  const int shift = 4 * (tau & 7);
+#pragma unroll 1
+  for (int d = lane; d < Dv; d += 32) {
+    const uint32_t code = (sm.new_words[8 * G + (d >> 3)] >> (4 * (d & 7))) & 15u;
+    const uint32_t at = 4u * v_word_offset(tau >> 3, d);
+    put(values, key_bytes, at, (*reinterpret_cast<const uint32_t*>(values + at) & ~(15u << shift)) | (code << shift));
   }
+}
+// A chunk that sticks out of the key range: the slots outside may hold anything, their value scales and biases become
+// zero in shared memory (their scores are masked), so that the common path need not look.
+template <int G>
+__device__ __noinline__ void clear_outside(uint8_t* vsb, int pos0, int key_lo, int key_n, int lane) {
+  constexpr int Gv = value_groups(G);
+  const int pos = pos0 + lane;
+  if (pos >= key_lo && pos < key_n) return;
+#pragma unroll
+  for (int gi = 0; gi < Gv; ++gi) reinterpret_cast<uint32_t*>(vsb)[sb_offset(lane, gi, Gv)] = 0u;
 }
 
 // Transpose of an 8 x 8 matrix of 16-bit elements held one row per lane group (lane l: row l / 4, columns 2 * (l % 4)
@@ -544,98 +577,87 @@ __device__ inline uint32_t transpose_8x8_b16(uint32_t a) {
   return d;
 }
 
-// One 32-token chunk against this warp's query fragments.
-//   Scores: the key codes are the A operand (16 tokens x 16 head-dim elements per product: lane (g, tid) holds the words
-//   of the tokens 4g + i, i = 0..3, so products pair the token rows (0, 1) and (2, 3)), the query the B operand (eight
-//   columns: heads 0..3 and their repeats).  A lane ends up with the scores of its four tokens for columns 2 tid and
-//   2 tid + 1.  The probabilities, multiplied by the token's value scale, are packed two columns to a register and
-//   transposed across the warp (movmatrix) into the B operand of the value product, whose A operand is the token-packed
-//   value words; columns 4..7 carry the low half of the two-term split of p * s.
+// Scores of one 32-token chunk: sc[i][c] of token 4g + i for column 2 tid + c, times kappa in log2 units.
+// The key codes are the A operand (16 tokens x 16 head-dim elements per product: lane (g, tid) holds the words of the
+// tokens 4g + i, i = 0..3, so products pair the token rows (0, 1) and (2, 3)), the query the B operand.  A group's
+// integer dot products meet the token's scale, and its bias the group's query sum, as soon as the group is done.
 template <int G, bool kBf>
-__device__ __forceinline__ void process_chunk(const uint8_t* chunk, int pos0, int key_lo, int key_n, int g, int tid,
-                                              const uint4* qb, const float (&qs)[2][G], const float (&kap)[2],
-                                              uint32_t split_mask, WarpState<G>& st) {
-  constexpr int D = 64 * G, Gv = value_groups(G), Dv = 64 * Gv;
+__device__ __forceinline__ void chunk_scores(const uint8_t* chunk, int g, int tid, const uint4* qb, const float* qs0,
+                                             const float* qs1, float (&sc)[4][2]) {
+  constexpr int D = 64 * G;
+  constexpr int kPairs = 2;                 // token-row pairs in work together (registers)
   const uint4* kc4 = reinterpret_cast<const uint4*>(chunk);
   const uint8_t* ksb = chunk + 32 * (D / 2);
-  const uint4* vc4 = reinterpret_cast<const uint4*>(chunk + 32 * (D / 2) + 128 * G);
-  const uint8_t* vsb = chunk + 32 * (D / 2) + 128 * G + 32 * (Dv / 2);
-  const bool edge = pos0 < key_lo || pos0 + 32 > key_n;
-
-  // ---- scores sc[i][c] of token 4g + i for column 2 tid + c, in log2 units ----
-  float sc[4][2];
-  {
-    float acc[2][G][4];                                  // [token-row pair][group]
 #pragma unroll
-    for (int pr = 0; pr < 2; ++pr)
+  for (int half = 0; half < (G + 1) / 2; ++half) {       // groups 2*half, 2*half+1: a 16-byte piece per token row
+    const bool odd = (G & 1) && half == G / 2;           // the last group of an odd count: an 8-byte piece per token row
 #pragma unroll
-      for (int gi = 0; gi < G; ++gi) { acc[pr][gi][0] = 0.f; acc[pr][gi][1] = 0.f; acc[pr][gi][2] = 0.f; acc[pr][gi][3] = 0.f; }
+    for (int pr0 = 0; pr0 < 2; pr0 += kPairs) {
+      float acc[kPairs][2][4];                           // [token-row pair][group]
 #pragma unroll
-    for (int half = 0; half < G / 2; ++half) {           // groups 2*half, 2*half+1: a 16-byte piece per token row
-      uint4 kw[4];
+      for (int pr = 0; pr < kPairs; ++pr)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) kw[i] = kc4[i * 16 * G + half * 32 + g * 4 + tid];
+        for (int gi = 0; gi < 2; ++gi) { acc[pr][gi][0] = 0.f; acc[pr][gi][1] = 0.f; acc[pr][gi][2] = 0.f; acc[pr][gi][3] = 0.f; }
+      uint4 kw[2 * kPairs];
+#pragma unroll
+      for (int i = 0; i < 2 * kPairs; ++i) {
+        if (odd) {
+          const uint2 t = reinterpret_cast<const uint2*>(chunk)[((2 * pr0 + i) * 64 * G + (G / 2) * 128) / 2 + g * 4 + tid];
+          kw[i] = make_uint4(t.x, t.y, 0u, 0u);
+        } else {
+          kw[i] = kc4[(2 * pr0 + i) * 16 * G + half * 32 + g * 4 + tid];
+        }
+      }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {                      // word p = 4*half + j: group 2*half + j/2
+        if (odd && j >= 2) break;
         const uint4 b = qb[(4 * half + j) * 32];
 #pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
+        for (int pr = 0; pr < kPairs; ++pr) {
           const uint4 &k0 = kw[2 * pr], &k1 = kw[2 * pr + 1];
           const uint32_t w0 = j == 0 ? k0.x : j == 1 ? k0.y : j == 2 ? k0.z : k0.w;
           const uint32_t w1 = j == 0 ? k1.x : j == 1 ? k1.y : j == 2 ? k1.z : k1.w;
           const uint32_t h0 = w0 >> 8, h1 = w1 >> 8;
-          float (&a)[4] = acc[pr][2 * half + (j >> 1)];
+          float (&a)[4] = acc[pr][j >> 1];
           mma_f16(a, w0 & kMaskLo, w1 & kMaskLo, w0 & kMaskHi, w1 & kMaskHi, b.x, b.y);
           mma_f16(a, h0 & kMaskLo, h1 & kMaskLo, h0 & kMaskHi, h1 & kMaskHi, b.z, b.w);
         }
       }
-    }
-    if (G & 1) {                                         // the last group of an odd count: an 8-byte piece per token row
-      uint2 kw[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        kw[i] = reinterpret_cast<const uint2*>(chunk)[(i * 64 * G + (G / 2) * 128) / 2 + g * 4 + tid];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const uint4 b = qb[(4 * (G / 2) + j) * 32];
-#pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-          const uint32_t w0 = j == 0 ? kw[2 * pr].x : kw[2 * pr].y;
-          const uint32_t w1 = j == 0 ? kw[2 * pr + 1].x : kw[2 * pr + 1].y;
-          const uint32_t h0 = w0 >> 8, h1 = w1 >> 8;
-          float (&a)[4] = acc[pr][G - 1];
-          mma_f16(a, w0 & kMaskLo, w1 & kMaskLo, w0 & kMaskHi, w1 & kMaskHi, b.x, b.y);
-          mma_f16(a, h0 & kMaskLo, h1 & kMaskLo, h0 & kMaskHi, h1 & kMaskHi, b.z, b.w);
-        }
-      }
-    }
-    // the token's scale meets the integer dot products, its bias the per-group query sums
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float ks[G], kb[G];
-      if (G == 3) {
-        const uint32_t* v = reinterpret_cast<const uint32_t*>(ksb + (i * 8 + g) * 12);
-#pragma unroll
-        for (int gi = 0; gi < 3; ++gi) { const float2 f = sb_to_f2<kBf>(v[gi]); ks[gi] = f.x; kb[gi] = f.y; }
-      } else if (G == 2) {
-        const uint2 v = *reinterpret_cast<const uint2*>(ksb + (i * 8 + g) * 8);
+      for (int i = 2 * pr0; i < 2 * (pr0 + kPairs); ++i) {
+        const uint8_t* at = ksb + (i * 8 + g) * 4 * G + 8 * half;
+        uint2 v;
+        if (odd) v = make_uint2(*reinterpret_cast<const uint32_t*>(at), 0u);
+        else if (G & 1) v = make_uint2(*reinterpret_cast<const uint32_t*>(at), *reinterpret_cast<const uint32_t*>(at + 4));
+        else v = *reinterpret_cast<const uint2*>(at);
         const float2 f0 = sb_to_f2<kBf>(v.x), f1 = sb_to_f2<kBf>(v.y);
-        ks[0] = f0.x; kb[0] = f0.y; ks[1] = f1.x; kb[1] = f1.y;
-      } else {
-        const uint4 v = *reinterpret_cast<const uint4*>(ksb + (i * 8 + g) * 16);
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        const float (&a)[2][4] = acc[(i >> 1) - pr0];
 #pragma unroll
-        for (int gi = 0; gi < 4; ++gi) { const float2 f = sb_to_f2<kBf>(u[gi]); ks[gi] = f.x; kb[gi] = f.y; }
-      }
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float t = acc[i >> 1][0][2 * (i & 1) + c] * ks[0], u = qs[c][0] * kb[0];
-#pragma unroll
-        for (int gi = 1; gi < G; ++gi) { t = fmaf(acc[i >> 1][gi][2 * (i & 1) + c], ks[gi], t); u = fmaf(qs[c][gi], kb[gi], u); }
-        sc[i][c] = fmaf(kap[c], t, u);
+        for (int c = 0; c < 2; ++c) {
+          float t = a[0][2 * (i & 1) + c] * f0.x;
+          if (half > 0) t += sc[i][c];
+          t = fmaf((c == 0 ? qs0 : qs1)[2 * half], f0.y, t);
+          if (!odd) {
+            t = fmaf(a[1][2 * (i & 1) + c], f1.x, t);
+            t = fmaf((c == 0 ? qs0 : qs1)[2 * half + 1], f1.y, t);
+          }
+          sc[i][c] = t;
+        }
       }
     }
   }
+}
+
+// Softmax step and value product of the chunk.  vc: its value half (codes, then scale/bias pairs).
+//   The probabilities, multiplied by the token's value scale, are packed two columns to a register and transposed across
+//   the warp into the B operand of the value product, whose A operand is the token-packed value words.
+template <int G, int H, bool kBf>
+__device__ __forceinline__ void chunk_values(const uint8_t* vhalf, bool edge, int pos0, int key_lo, int key_n, int g, int tid,
+                                             const float (&kap)[2], uint32_t split_mask, float margin, float (&sc)[4][2],
+                                             WarpState<G>& st) {
+  constexpr int Gv = value_groups(G), Dv = 64 * Gv;
+  const uint4* vc4 = reinterpret_cast<const uint4*>(vhalf);
+  const uint8_t* vsb = vhalf + 32 * (Dv / 2);
   if (edge) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -643,87 +665,115 @@ __device__ __forceinline__ void process_chunk(const uint8_t* chunk, int pos0, in
       if (pos < key_lo || pos >= key_n) { sc[i][0] = -INFINITY; sc[i][1] = -INFINITY; }
     }
   }
-  // ---- online softmax over the chunk ----
-  float p[4][2], corr[2];
+  // H = 4: probabilities stay at most 1, so p*s stays inside binary16 for every scale.  H = 8: the reference leaves the
+  // probabilities as many binary orders above 1 as the value scales seen so far allow (p*s below 2^15), because the low
+  // half of the split loses what falls below 2^-24 and the odd token rows (p/16 against 16c) lose sixteen times as much.
+  float cm[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) cm[c] = fmaxf(fmaxf(sc[0][c], sc[1][c]), fmaxf(sc[2][c], sc[3][c])) * kap[c];
+  bool grow;
+  uint32_t vmax = 0u;                                    // H = 8: the largest value scale of the lane's tokens (bit pattern)
+  if (H == 8) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int gp = 0; gp < Gv / 2; ++gp) {
+        const uint2 v = *reinterpret_cast<const uint2*>(vsb + (i * 8 + g) * 4 * Gv + 8 * gp);
+        vmax = __vmaxu2(vmax, __vmaxu2(v.x, v.y));
+      }
+    vmax &= 0xFFFFu;
+    const float top = (float)st.head_room + 1.f;
+    grow = cm[0] > st.m[0] + top || cm[1] > st.m[1] + top || vmax > st.vlimit;
+  } else {
+    grow = cm[0] > st.m[0] || cm[1] > st.m[1];
+  }
+  if (__any_sync(0xffffffffu, grow)) {
+    int room = 0, old_room = 0;
+    if (H == 8) {
+      // scales below 2^e leave 14 - e binary orders for the probabilities
+      vmax = __reduce_max_sync(0xffffffffu, vmax);
+      if (vmax > 0x7FFFu) vmax = 0x7FFFu;                // a negative scale: no room
+      const int e = kBf ? (int)(vmax >> 7) - 126 : (int)(vmax >> 10) - 14;
+      old_room = st.head_room;
+      room = min(st.head_room, 14 - max(e, -26));
+      st.head_room = room;
+      st.vlimit = max(st.vlimit, vmax | (kBf ? 0x7Fu : 0x3FFu));
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float x = cm[c];
+      x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 4));
+      x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 8));
+      x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 16));
+      if (H == 8) x = fmaxf(st.m[c] + (float)old_room, x) - (float)room;
+      else x = x > st.m[c] ? x + margin : st.m[c];
+      const float f = fast_exp2(st.m[c] - x);            // m = -inf: 0
+      st.m[c] = x;
+      st.l[c] *= f;
+#pragma unroll
+      for (int gi = 0; gi < Gv; ++gi) st.bias[c][gi] *= f;
+#pragma unroll
+      for (int mt = 0; mt < Dv / 16; ++mt) { st.o[mt][c] *= f; st.o[mt][2 + c] *= f; }
+    }
+  }
+  float p[4][2];
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    float cm = fmaxf(fmaxf(sc[0][c], sc[1][c]), fmaxf(sc[2][c], sc[3][c]));
-    cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 4));
-    cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 8));
-    cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
-    float m_new = fmaxf(st.m[c], cm);
-    if (m_new == -INFINITY) m_new = 0.f;
-    corr[c] = fast_exp2(st.m[c] - m_new);
-    st.m[c] = m_new;
-    p[0][c] = fast_exp2(sc[0][c] - m_new);
-    p[1][c] = fast_exp2(sc[1][c] - (m_new + 4.f));       // odd token rows: p / 16 (their value codes carry a factor 16)
-    p[2][c] = fast_exp2(sc[2][c] - m_new);
-    p[3][c] = fast_exp2(sc[3][c] - (m_new + 4.f));
-    st.l_e[c] = fmaf(st.l_e[c], corr[c], p[0][c] + p[2][c]);
-    st.l_o[c] = fmaf(st.l_o[c], corr[c], p[1][c] + p[3][c]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i][c] = fast_exp2(fmaf(sc[i][c], kap[c], -st.m[c]));
+    st.l[c] += (p[0][c] + p[1][c]) + (p[2][c] + p[3][c]);
   }
-  // rescale the accumulators when any head's running maximum moved (the lane owns the same two columns there)
-  if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
+  for (int gp = 0; gp < Gv / 2; ++gp) {
+    uint2 sbw[4];
 #pragma unroll
-      for (int gi = 0; gi < Gv; ++gi) { st.bias_e[c][gi] *= corr[c]; st.bias_o[c][gi] *= corr[c]; }
+    for (int i = 0; i < 4; ++i) sbw[i] = *reinterpret_cast<const uint2*>(vsb + (i * 8 + g) * 4 * Gv + 8 * gp);
 #pragma unroll
-    for (int mt = 0; mt < Dv / 16; ++mt) { st.o[mt][0] *= corr[0]; st.o[mt][1] *= corr[1]; st.o[mt][2] *= corr[0]; st.o[mt][3] *= corr[1]; }
-  }
-  // ---- p * s_v per group as two-term binary16 (columns 0..3: high part, columns 4..7: low part), transposed into
-  // the B operand of the value product: bfr[group][token row] = half2(tokens 8 tid + i, 8 tid + 4 + i) of column g ----
-  uint32_t bfr[Gv][4];
+    for (int e = 0; e < 2; ++e) {
+      const int gi = 2 * gp + e;
+      // p * s_v as a two-term binary16 pair, transposed: bh[i] = half2(tokens 8 tid + i, 8 tid + 4 + i) of column g
+      uint32_t bh[4], bl[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float vs[Gv], vb[Gv];
-    if (Gv == 2) {
-      const uint2 v = *reinterpret_cast<const uint2*>(vsb + (i * 8 + g) * 8);
-      const float2 f0 = sb_to_f2<kBf>(v.x), f1 = sb_to_f2<kBf>(v.y);
-      vs[0] = f0.x; vb[0] = f0.y; vs[1] = f1.x; vb[1] = f1.y;
-    } else {
-      const uint4 v = *reinterpret_cast<const uint4*>(vsb + (i * 8 + g) * 16);
-      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int gi = 0; gi < 4; ++gi) { const float2 f = sb_to_f2<kBf>(u[gi]); vs[gi] = f.x; vb[gi] = f.y; }
-    }
-    if (edge) {
-      const int pos = pos0 + 4 * g + i;
-      if (pos < key_lo || pos >= key_n) {
-#pragma unroll
-        for (int gi = 0; gi < Gv; ++gi) { vs[gi] = 0.f; vb[gi] = 0.f; }
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = sb_to_f2<kBf>(e == 0 ? sbw[i].x : sbw[i].y);
+        const float vs = (i & 1) ? f.x * 0.0625f : f.x;  // odd token rows: their value codes carry a factor 16
+        const float x0 = p[i][0] * vs, x1 = p[i][1] * vs;
+        st.bias[0][gi] = fmaf(p[i][0], f.y, st.bias[0][gi]);
+        st.bias[1][gi] = fmaf(p[i][1], f.y, st.bias[1][gi]);
+        if (H == 4) {
+          // columns 0..3: trunc16(x); columns 4..7: trunc16(x - trunc11bits(x)) -- the binary16 conversion truncates
+          const float r0 = x0 - __uint_as_float(__float_as_uint(x0) & split_mask);
+          const float r1 = x1 - __uint_as_float(__float_as_uint(x1) & split_mask);
+          bh[i] = transpose_8x8_b16(f32x2_to_h2_rz(r0, r1));
+        } else {
+          const float r0 = x0 - __uint_as_float(__float_as_uint(x0) & 0xFFFFE000u);
+          const float r1 = x1 - __uint_as_float(__float_as_uint(x1) & 0xFFFFE000u);
+          bh[i] = transpose_8x8_b16(f32x2_to_h2_rz(x0, x1));
+          bl[i] = transpose_8x8_b16(f32x2_to_h2_rz(r0, r1));
+        }
       }
-    }
+      // P.V on the codes: 16 value rows x 8 columns x 32 tokens per accumulator tile
 #pragma unroll
-    for (int gi = 0; gi < Gv; ++gi) {
-      const float x0 = p[i][0] * vs[gi], x1 = p[i][1] * vs[gi];
-      // columns 0..3: trunc16(x); columns 4..7: trunc16(x - trunc11bits(x)) -- the binary16 conversion truncates
-      const float r0 = x0 - __uint_as_float(__float_as_uint(x0) & split_mask);
-      const float r1 = x1 - __uint_as_float(__float_as_uint(x1) & split_mask);
-      bfr[gi][i] = transpose_8x8_b16(f32x2_to_h2_rz(r0, r1));
-      if (i & 1) {
-        st.bias_o[0][gi] = fmaf(p[i][0], vb[gi], st.bias_o[0][gi]);
-        st.bias_o[1][gi] = fmaf(p[i][1], vb[gi], st.bias_o[1][gi]);
-      } else {
-        st.bias_e[0][gi] = fmaf(p[i][0], vb[gi], st.bias_e[0][gi]);
-        st.bias_e[1][gi] = fmaf(p[i][1], vb[gi], st.bias_e[1][gi]);
+      for (int q4 = 2 * gi; q4 < 2 * gi + 2; ++q4) {
+        const uint4 w4 = vc4[(q4 * 8 + g) * 4 + tid];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const uint32_t x = t == 0 ? w4.x : w4.z, y = t == 0 ? w4.y : w4.w, xh = x >> 8, yh = y >> 8;
+          float (&o)[4] = st.o[2 * q4 + t];
+          if (H == 4) {
+            mma_f16(o, x & kMaskLo, y & kMaskLo, x & kMaskHi, y & kMaskHi, bh[0], bh[1]);
+            mma_f16(o, xh & kMaskLo, yh & kMaskLo, xh & kMaskHi, yh & kMaskHi, bh[2], bh[3]);
+          } else {
+            // the small terms first, and the chunk's sum joins the running one outside: the tensor cores truncate
+            float a[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_f16(a, x & kMaskLo, y & kMaskLo, x & kMaskHi, y & kMaskHi, bl[0], bl[1]);
+            mma_f16(a, xh & kMaskLo, yh & kMaskLo, xh & kMaskHi, yh & kMaskHi, bl[2], bl[3]);
+            mma_f16(a, x & kMaskLo, y & kMaskLo, x & kMaskHi, y & kMaskHi, bh[0], bh[1]);
+            mma_f16(a, xh & kMaskLo, yh & kMaskLo, xh & kMaskHi, yh & kMaskHi, bh[2], bh[3]);
+            o[0] += a[0]; o[1] += a[1]; o[2] += a[2]; o[3] += a[3];
+          }
+        }
       }
-    }
-  }
-  // ---- P.V on the codes: 16 value rows x 8 columns (heads hi|lo) x 32 tokens per tile pair ----
-#pragma unroll
-  for (int q4 = 0; q4 < Dv / 32; ++q4) {
-    const uint4 w4 = vc4[(q4 * 8 + g) * 4 + tid];
-    const int gi = q4 >> 1;
-    {
-      const uint32_t xh = w4.x >> 8, yh = w4.y >> 8;
-      mma_f16(st.o[2 * q4], w4.x & kMaskLo, w4.y & kMaskLo, w4.x & kMaskHi, w4.y & kMaskHi, bfr[gi][0], bfr[gi][1]);
-      mma_f16(st.o[2 * q4], xh & kMaskLo, yh & kMaskLo, xh & kMaskHi, yh & kMaskHi, bfr[gi][2], bfr[gi][3]);
-    }
-    {
-      const uint32_t xh = w4.z >> 8, yh = w4.w >> 8;
-      mma_f16(st.o[2 * q4 + 1], w4.z & kMaskLo, w4.w & kMaskLo, w4.z & kMaskHi, w4.w & kMaskHi, bfr[gi][0], bfr[gi][1]);
-      mma_f16(st.o[2 * q4 + 1], xh & kMaskLo, yh & kMaskLo, xh & kMaskHi, yh & kMaskHi, bfr[gi][2], bfr[gi][3]);
     }
   }
 }
@@ -732,754 +782,539 @@ __device__ inline void store_out(const DecodeParams& P, size_t index, float v) {
   if (P.out_dtype == Q4KV_OUT_BF16) reinterpret_cast<__nv_bfloat16*>(P.out)[index] = __float2bfloat16_rn(v);
   else reinterpret_cast<float*>(P.out)[index] = v;
 }
+__device__ __forceinline__ void store_four(const DecodeParams& P, size_t index, const float (&x)[4], float mul) {
+  if (P.out_dtype == Q4KV_OUT_BF16) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(x[0] * mul, x[1] * mul), hi = __floats2bfloat162_rn(x[2] * mul, x[3] * mul);
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(P.out) + index) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  } else {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(P.out) + index) = make_float4(x[0] * mul, x[1] * mul, x[2] * mul, x[3] * mul);
+  }
+}
 
-// Epilogue of one segment, run by the single warp that made the deposit count complete: combine
-// the NW deposits; a pair that lies wholly inside this CTA is normalised and written out, otherwise
-// the combination becomes this CTA's partial record and the warp takes a ticket -- the CTA whose
-// ticket is the pair's last combines all records of the pair.  Each lane owns 4 consecutive output
-// elements (per 128), so every access is a 16-byte one.  Deposits and records are walked in loops with a
-// few loads in flight and running sums in registers: the register need does not grow with the number of
-// warps or records.
-template <int G, int NW>
-__device__ __forceinline__ void segment_epilogue(const float* merge_buf, int* epilogues_word, int use, const DecodeParams& P,
-                                              const Segment& seg, int cta, const Partition& part, int lane) {
-  constexpr int Dv = 64 * value_groups(G), V = Dv / 128;
-  constexpr int kStride = Dv + 8;
-  static_assert(NW <= 32, "one lane per deposit in the weight pass");
-  const Layout& y = P.y;
-  const int n_rep = y.n_rep;
-  const int pair = seg.a * y.Hkv + seg.hk;
-  const bool whole = seg.c0 == seg.cf && seg.c1 == seg.cf + seg.nc;
-  const size_t row0 = (size_t)seg.a * y.Hq + (size_t)seg.hk * n_rep;
-  const size_t rstride = (size_t)n_rep * kRecStride(Dv);
-  float* rec = P.partials + (size_t)(pair + cta) * rstride;
-  auto store4 = [&](int h, int d, float4 v) {
-    if (P.out_dtype == Q4KV_OUT_BF16) {
-      __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-      uint2 u = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-      *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(P.out) + (row0 + h) * Dv + d) = u;
+// Leave this warp's state of a segment in its deposit, in fragment order (16 bytes per lane and unit): the accumulators
+// with the bias sums added, and m, l per head.
+//   H = 4: columns 4..7 (lanes tid 2, 3) hold the low-part products of heads 0..3; a pair of lanes exchanges the halves it
+//   does not keep.  Unit u of lane (g, tid) is value rows 32 u + g + 8 * (tid / 2) (+ 16) of heads 2 * (tid % 2) (+ 1):
+//   {row, head} {row, head + 1} {row + 16, head} {row + 16, head + 1}.
+//   H = 8: unit u is value rows 16 u + g (+ 8) of heads 2 tid (+ 1): {row, head} {row, head + 1} {row + 8, ..} {row + 8, ..}.
+template <int G, int H>
+__device__ __forceinline__ void deposit(Smem<G, H>& sm, int warp, int lane, WarpState<G>& st, bool bad) {
+  constexpr int Gv = value_groups(G);
+  const int g = lane >> 2, tid = lane & 3;
+  float bias[2][Gv];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    float l = st.l[c];                                   // over the lane's tokens -> over the chunk's (lanes of equal tid)
+    l += __shfl_xor_sync(0xffffffffu, l, 4);
+    l += __shfl_xor_sync(0xffffffffu, l, 8);
+    l += __shfl_xor_sync(0xffffffffu, l, 16);
+#pragma unroll
+    for (int gi = 0; gi < Gv; ++gi) {
+      float bb = st.bias[c][gi];
+      bb += __shfl_xor_sync(0xffffffffu, bb, 4);
+      bb += __shfl_xor_sync(0xffffffffu, bb, 8);
+      bb += __shfl_xor_sync(0xffffffffu, bb, 16);
+      bias[c][gi] = bb;
+    }
+    if (g == 0 && (H == 8 || tid < 2)) {
+      sm.dep_m[warp][2 * tid + c] = st.m[c];
+      sm.dep_l[warp][2 * tid + c] = bad ? -1.f : l;
+    }
+  }
+  constexpr float k24 = 16777216.f;
+#pragma unroll
+  for (int u = 0; u < Smem<G, H>::kDepUnits; ++u) {
+    float4 v;
+    if (H == 4) {
+      const bool up = tid >= 2;
+      float x[2][2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float (&o)[4] = st.o[(2 * u + e) & (4 * Gv - 1)];
+        x[e][0] = (up ? o[2] : o[0]) + __shfl_xor_sync(0xffffffffu, up ? o[0] : o[2], 2);
+        x[e][1] = (up ? o[3] : o[1]) + __shfl_xor_sync(0xffffffffu, up ? o[1] : o[3], 2);
+      }
+      const float b0 = bias[0][u >> 1], b1 = bias[1][u >> 1];
+      v = make_float4(fmaf(x[0][0], k24, b0), fmaf(x[0][1], k24, b1), fmaf(x[1][0], k24, b0), fmaf(x[1][1], k24, b1));
     } else {
-      *reinterpret_cast<float4*>(reinterpret_cast<float*>(P.out) + (row0 + h) * Dv + d) = v;
+      const float (&o)[4] = st.o[u & (4 * Gv - 1)];
+      const float b0 = bias[0][(u >> 2) & (Gv - 1)], b1 = bias[1][(u >> 2) & (Gv - 1)];
+      v = make_float4(fmaf(o[0], k24, b0), fmaf(o[1], k24, b1), fmaf(o[2], k24, b0), fmaf(o[3], k24, b1));
     }
-  };
-  // weights of the deposits, all heads side by side: lane w looks at deposit w
-  float wgt[4], Mh[4], Lh[4];
-  bool badh[4];
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    const float* mine = merge_buf + ((size_t)(lane < NW ? lane : 0) * 4 + h) * kStride;
-    const float2 ml = *reinterpret_cast<const float2*>(mine + Dv);
-    const float mw = (lane < NW && h < n_rep) ? ml.x : -INFINITY, lw = (lane < NW && h < n_rep) ? ml.y : 0.f;
-    float M = mw;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    wgt[h] = mw == -INFINITY ? 0.f : fast_exp2(mw - M);
-    float L = wgt[h] * lw;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-    badh[h] = __any_sync(0xffffffffu, lw < 0.f);
-    Mh[h] = M;
-    Lh[h] = badh[h] ? 0.f : L;
+    sm.dep[warp][u][lane] = v;
   }
-  float4 acc[4][V];
-#pragma unroll
-  for (int h = 0; h < 4; ++h)
-#pragma unroll
-    for (int v = 0; v < V; ++v) acc[h][v] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-  for (int w = 0; w < NW; ++w) {
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const float ww = __shfl_sync(0xffffffffu, wgt[h], w);
-      const bool on = ww != 0.f;                         // an empty deposit holds stale bytes
-      const float* dep = merge_buf + ((size_t)w * 4 + h) * kStride;
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const float4 x = *reinterpret_cast<const float4*>(dep + 128 * v + 4 * lane);
-        const float bs = dep[Dv + 2 + ((128 * v + 4 * lane) >> 6)];
-        acc[h][v].x = fmaf(ww, on ? x.x + bs : 0.f, acc[h][v].x); acc[h][v].y = fmaf(ww, on ? x.y + bs : 0.f, acc[h][v].y);
-        acc[h][v].z = fmaf(ww, on ? x.z + bs : 0.f, acc[h][v].z); acc[h][v].w = fmaf(ww, on ? x.w + bs : 0.f, acc[h][v].w);
-      }
-    }
-  }
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    if (h >= n_rep) continue;
-    const float inv = whole ? (Lh[h] > 0.f ? 1.f / Lh[h] : 0.f) : 1.f;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float4 o = acc[h][v];
-      o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
-      const int d = 128 * v + 4 * lane;
-      if (whole) store4(h, d, o);
-      else *reinterpret_cast<float4*>(rec + (size_t)h * kRecStride(Dv) + d) = o;
-    }
-    if (lane == 0) {
-      if (whole) { if (P.lse) P.lse[row0 + h] = Lh[h] > 0.f ? (Mh[h] + log2f(Lh[h])) / kLog2e : -INFINITY; }
-      else *reinterpret_cast<float2*>(rec + (size_t)h * kRecStride(Dv) + Dv) = make_float2(Mh[h], badh[h] ? -1.f : Lh[h]);
-    }
-  }
-  // the deposit buffer can be reused from here on
-  __threadfence_block();
-  __syncwarp();
-  if (lane == 0) *(volatile int*)epilogues_word = use + 1;
-  if (whole) return;
+}
 
-  // ticket: the CTA whose record arrives last combines all records of the pair
-  const uint32_t pair_u0 = seg.u0 - (uint32_t)(seg.c0 - seg.cf);
-  const int c_first = part.cta_of(pair_u0), c_last = part.cta_of(pair_u0 + (uint32_t)seg.nc - 1u);
-  // The warp's record stores are ordered before lane 0's release by the warp barrier, and the other lanes' record loads
-  // after its acquire by the second one: one acquire-release atomic takes the place of a fence on either side.
-  __syncwarp();
-  int final_merge = 0;
-  if (lane == 0) {
-    int old;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(&P.tickets[pair]) : "memory");
-    final_merge = old == c_last - c_first;
-    if (final_merge) P.tickets[pair] = 0;            // ready for the next call
+// Combine the eight warps' deposits of a segment: unit `unit` (one warp each).  A pair that lies wholly inside this CTA is
+// normalised and written out, otherwise the combination becomes this CTA's partial record.
+template <int G, int H>
+__device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const DecodeParams& P, const Segment& seg, int cta, int unit,
+                                                 int lane) {
+  constexpr int Dv = Smem<G, H>::Dv, NW = Smem<G, H>::NW;
+  const int g = lane >> 2, tid = lane & 3, n_rep = P.n_rep;
+  const bool whole = seg.c1 - seg.c0 == seg.nc;
+  // (m, l) of (warp, head): H = 4: lane 4 * warp + head; H = 8: two per lane, warps lane / 8 and lane / 8 + 4
+  constexpr int kPer = (NW * H + 31) / 32;
+  float e[kPer], M, L = 0.f;
+  bool bad = false;
+  {
+    float m[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) m[k] = 32 * k + lane < NW * H ? (&sm.dep_m[0][0])[32 * k + lane] : -INFINITY;
+    M = m[0];
+#pragma unroll
+    for (int k = 1; k < kPer; ++k) M = fmaxf(M, m[k]);
+#pragma unroll
+    for (int o = H; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const float l = 32 * k + lane < NW * H ? (&sm.dep_l[0][0])[32 * k + lane] : 0.f;
+      e[k] = m[k] == -INFINITY ? 0.f : fast_exp2(m[k] - M);
+      L = fmaf(e[k], l, L);
+      bad |= l < 0.f;
+    }
+#pragma unroll
+    for (int o = H; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    bad = __any_sync(0xffffffffu, bad);
+    if (bad) L = 0.f;
   }
-  final_merge = __shfl_sync(0xffffffffu, final_merge, 0);
-  if (!final_merge) return;
-  __syncwarp();
-  const int R = c_last - c_first + 1;
-  const float* base = P.partials + (size_t)(pair + c_first) * rstride;
-  // The records sit in L2, a microsecond away: all heads travel together, and the first batch of record loads is issued
-  // before the (m, l) pass, so that a pair with few records costs two round trips in all.
-  constexpr int RB = V == 1 ? 5 : 2;
-  float mr[RB][4];
-  float4 xv[RB][4][V];
-  auto load_batch = [&](int rb) {
+  const int h0 = 2 * (tid & (H / 2 - 1));                // this lane's heads h0, h0 + 1
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < RB; ++i) {
-      const int r = rb + i < R ? rb + i : R - 1;
+  for (int w = 0; w < NW; ++w) {
+    const float e0 = __shfl_sync(0xffffffffu, e[w * H / 32], (w * H & 31) + h0);
+    const float e1 = __shfl_sync(0xffffffffu, e[w * H / 32], (w * H & 31) + h0 + 1);
+    if (e0 != 0.f || e1 != 0.f) {                        // an empty deposit holds stale bytes
+      const float4 x = sm.dep[w][unit][lane];
+      a[0] = fmaf(e0, x.x, a[0]); a[1] = fmaf(e1, x.y, a[1]);
+      a[2] = fmaf(e0, x.z, a[2]); a[3] = fmaf(e1, x.w, a[3]);
+    }
+  }
+  const float L0 = __shfl_sync(0xffffffffu, L, h0), L1 = __shfl_sync(0xffffffffu, L, h0 + 1);
+  const int d = H == 4 ? 32 * unit + g + 8 * (tid >> 1) : 16 * unit + g, step = H == 4 ? 16 : 8;
+  const size_t row0 = (size_t)seg.a * P.y.Hq + (size_t)seg.hk * n_rep;
+  if (whole) {
+    const float i0 = L0 > 0.f ? 1.f / L0 : 0.f, i1 = L1 > 0.f ? 1.f / L1 : 0.f;
+    if (h0 < n_rep) { store_out(P, (row0 + h0) * Dv + d, a[0] * i0); store_out(P, (row0 + h0) * Dv + d + step, a[2] * i0); }
+    if (h0 + 1 < n_rep) { store_out(P, (row0 + h0 + 1) * Dv + d, a[1] * i1); store_out(P, (row0 + h0 + 1) * Dv + d + step, a[3] * i1); }
+    if (unit == 0 && lane < n_rep && P.lse) P.lse[row0 + lane] = L > 0.f ? (M + log2f(L)) / kLog2e : -INFINITY;
+  } else {
+    float* rec = P.partials + (size_t)(seg.a * P.Hkv + seg.hk + cta) * n_rep * kRecStride(Dv);
+    float* r0 = rec + h0 * kRecStride(Dv) + d;
+    if (h0 < n_rep) { r0[0] = a[0]; r0[step] = a[2]; }
+    if (h0 + 1 < n_rep) { r0[kRecStride(Dv)] = a[1]; r0[kRecStride(Dv) + step] = a[3]; }
+    if (unit == 0 && lane < n_rep)
+      *reinterpret_cast<float2*>(rec + lane * kRecStride(Dv) + Dv) = make_float2(M, bad ? -1.f : L);
+  }
+}
+
+// Combination of the records of one pair for one head and 128 output elements, by one warp (lane: four elements).  The
+// records sit in L2, a microsecond away: a batch of loads is in flight together with the (m, l) pairs.
+__device__ __forceinline__ void combine_records(const DecodeParams& P, const float* base, size_t rstride, int R, int Dv, int d,
+                                                size_t row, int lane) {
+  constexpr int RB = 8;
+  float M = -INFINITY, L = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+  bool bad = false;
+#pragma unroll 1
+  for (int r0 = 0; r0 < R; r0 += 32) {
+    const int n = min(32, R - r0);
+    const float2 ml = lane < n ? __ldcg(reinterpret_cast<const float2*>(base + (size_t)(r0 + lane) * rstride + Dv))
+                               : make_float2(-INFINITY, 0.f);
+    float e = 0.f;
+#pragma unroll 1
+    for (int b = 0; b < n; b += RB) {
+      float4 x[RB];
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const float* rh = base + r * rstride + (size_t)(h < n_rep ? h : 0) * kRecStride(Dv);
-        mr[i][h] = __ldcg(rh + Dv);
+      for (int i = 0; i < RB; ++i)
+        x[i] = __ldcg(reinterpret_cast<const float4*>(base + (size_t)(r0 + min(b + i, n - 1)) * rstride + d));
+      if (b == 0) {
+        float Mn = ml.x;
 #pragma unroll
-        for (int v = 0; v < V; ++v) xv[i][h][v] = __ldcg(reinterpret_cast<const float4*>(rh + 128 * v + 4 * lane));
+        for (int o = 16; o > 0; o >>= 1) Mn = fmaxf(Mn, __shfl_xor_sync(0xffffffffu, Mn, o));
+        Mn = fmaxf(M, Mn);
+        const float f = Mn == -INFINITY ? 0.f : fast_exp2(M - Mn);       // M = -inf: 0
+        e = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - Mn);
+        bad |= __any_sync(0xffffffffu, ml.y < 0.f);
+        float s = e * ml.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        L = L * f + s;
+        M = Mn;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] *= f;
       }
-    }
-  };
-  load_batch(0);
-  // pass 1: maximum and sum per head.  Lane l looks at (record, head) pairs l, l + 32, ...; its head is l % 4.
-  const int hl = lane & 3;
-  float Ml = -INFINITY, Ll = 0.f;
-  int badl = 0;
-  if (hl < n_rep) {
-    for (int r = lane >> 2; r < R; r += 8) {
-      const float2 t = __ldcg(reinterpret_cast<const float2*>(base + r * rstride + (size_t)hl * kRecStride(Dv) + Dv));
-      if (t.y < 0.f) badl = 1;
-      const float Mn = fmaxf(Ml, t.x);
-      if (Mn != -INFINITY) Ll = Ll * fast_exp2(Ml - Mn) + t.y * fast_exp2(t.x - Mn);
-      Ml = Mn;
-    }
-  }
 #pragma unroll
-  for (int o = 4; o < 32; o <<= 1) {
-    const float Mo = __shfl_xor_sync(0xffffffffu, Ml, o), Lo = __shfl_xor_sync(0xffffffffu, Ll, o);
-    const float Mn = fmaxf(Ml, Mo);
-    if (Mn != -INFINITY) Ll = Ll * fast_exp2(Ml - Mn) + Lo * fast_exp2(Mo - Mn);
-    Ml = Mn;
-  }
-  const bool any_bad = __any_sync(0xffffffffu, badl);
-  // pass 2: weighted sum of the records, RB at a time, all heads together (nothing is stored before the end)
-  float Mr[4], Lr[4];
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    Mr[h] = __shfl_sync(0xffffffffu, Ml, h);
-    Lr[h] = any_bad ? 0.f : __shfl_sync(0xffffffffu, Ll, h);
-  }
-  float4 racc[4][V];
-#pragma unroll
-  for (int h = 0; h < 4; ++h)
-#pragma unroll
-    for (int v = 0; v < V; ++v) racc[h][v] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int rb = 0; rb < R; rb += RB) {
-    if (rb > 0) load_batch(rb);
-#pragma unroll
-    for (int i = 0; i < RB; ++i)
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const float e = (rb + i >= R || mr[i][h] == -INFINITY) ? 0.f : fast_exp2(mr[i][h] - Mr[h]);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          racc[h][v].x = fmaf(e, xv[i][h][v].x, racc[h][v].x); racc[h][v].y = fmaf(e, xv[i][h][v].y, racc[h][v].y);
-          racc[h][v].z = fmaf(e, xv[i][h][v].z, racc[h][v].z); racc[h][v].w = fmaf(e, xv[i][h][v].w, racc[h][v].w);
+      for (int i = 0; i < RB; ++i) {
+        const float w = __shfl_sync(0xffffffffu, e, (b + i) & 31);       // past the last record: 0, or not added
+        if (b + i < n) {
+          acc[0] = fmaf(w, x[i].x, acc[0]); acc[1] = fmaf(w, x[i].y, acc[1]);
+          acc[2] = fmaf(w, x[i].z, acc[2]); acc[3] = fmaf(w, x[i].w, acc[3]);
         }
       }
-  }
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    if (h >= n_rep) continue;
-    const float inv = Lr[h] > 0.f ? 1.f / Lr[h] : 0.f;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float4 o = racc[h][v];
-      o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
-      store4(h, 128 * v + 4 * lane, o);
     }
-    if (lane == 0 && P.lse) P.lse[row0 + h] = Lr[h] > 0.f ? (Mr[h] + log2f(Lr[h])) / kLog2e : -INFINITY;
   }
-}
-
-// Epilogue of a CTA's last segment, one warp per query head (warp h < n_rep handles head h; the caller has waited for
-// all NW deposits).  Same arithmetic as segment_epilogue; the heads run side by side instead of one after the other,
-// which shortens the tail every launch ends with: combine, record, ticket, final combination.  The head warps meet
-// twice through shared memory: once so that a single thread draws the pair's ticket after all heads' records are
-// written and fenced, once to learn whether this CTA combines the pair's records.
-template <int G, int NW>
-__device__ __forceinline__ void last_segment_by_heads(const float* merge_buf, int* fin_arrived, int* fin_ticket,
-                                                      volatile int* abort_flag, const DecodeParams& P, const Segment& seg,
-                                                      int cta, const Partition& part, int h, int lane) {
-  constexpr int Dv = 64 * value_groups(G), V = Dv / 128;
-  constexpr int kStride = Dv + 8;
-  const Layout& y = P.y;
-  const int n_rep = y.n_rep;
-  const int pair = seg.a * y.Hkv + seg.hk;
-  const bool whole = seg.c0 == seg.cf && seg.c1 == seg.cf + seg.nc;
-  const size_t row = (size_t)seg.a * y.Hq + (size_t)seg.hk * n_rep + h;
-  const size_t rstride = (size_t)n_rep * kRecStride(Dv);
-  float* rec = P.partials + (size_t)(pair + cta) * rstride + (size_t)h * kRecStride(Dv);
-  auto store4 = [&](int d, float4 v) {
-    if (P.out_dtype == Q4KV_OUT_BF16) {
-      __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-      uint2 u = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-      *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(P.out) + row * Dv + d) = u;
-    } else {
-      *reinterpret_cast<float4*>(reinterpret_cast<float*>(P.out) + row * Dv + d) = v;
-    }
-  };
-  // weights of the deposits: lane w looks at deposit w
-  const float* mine = merge_buf + ((size_t)(lane < NW ? lane : 0) * 4 + h) * kStride;
-  const float2 ml = *reinterpret_cast<const float2*>(mine + Dv);
-  const float mw = lane < NW ? ml.x : -INFINITY, lw = lane < NW ? ml.y : 0.f;
-  float M = mw;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  const float wgt = mw == -INFINITY ? 0.f : fast_exp2(mw - M);
-  float L = wgt * lw;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-  const bool bad = __any_sync(0xffffffffu, lw < 0.f);
   if (bad) L = 0.f;
-  float4 acc[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-  for (int w = 0; w < NW; ++w) {
-    const float ww = __shfl_sync(0xffffffffu, wgt, w);
-    const bool on = ww != 0.f;                           // an empty deposit holds stale bytes
-    const float* dep = merge_buf + ((size_t)w * 4 + h) * kStride;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float4 x = *reinterpret_cast<const float4*>(dep + 128 * v + 4 * lane);
-      const float bs = dep[Dv + 2 + ((128 * v + 4 * lane) >> 6)];
-      acc[v].x = fmaf(ww, on ? x.x + bs : 0.f, acc[v].x); acc[v].y = fmaf(ww, on ? x.y + bs : 0.f, acc[v].y);
-      acc[v].z = fmaf(ww, on ? x.z + bs : 0.f, acc[v].z); acc[v].w = fmaf(ww, on ? x.w + bs : 0.f, acc[v].w);
-    }
-  }
-  if (whole) {
-    const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-    for (int v = 0; v < V; ++v) store4(128 * v + 4 * lane, make_float4(acc[v].x * inv, acc[v].y * inv, acc[v].z * inv, acc[v].w * inv));
-    if (lane == 0 && P.lse) P.lse[row] = L > 0.f ? (M + log2f(L)) / kLog2e : -INFINITY;
-    return;
-  }
-#pragma unroll
-  for (int v = 0; v < V; ++v) *reinterpret_cast<float4*>(rec + 128 * v + 4 * lane) = acc[v];
-  if (lane == 0) *reinterpret_cast<float2*>(rec + Dv) = make_float2(M, bad ? -1.f : L);
-  // every head's record is written and fenced before one thread draws the ticket
-  const uint32_t pair_u0 = seg.u0 - (uint32_t)(seg.c0 - seg.cf);
-  const int c_first = part.cta_of(pair_u0), c_last = part.cta_of(pair_u0 + (uint32_t)seg.nc - 1u);
-  // Ordering: each head warp's record stores come before its lane 0's arrival (warp barrier, then a CTA-scope
-  // fence); the last arrival draws the ticket with one acquire-release atomic at GPU scope, which publishes all the
-  // head warps' records and, if the ticket is the pair's last, makes the other CTAs' records readable; the answer
-  // reaches the other head warps through shared memory and a CTA-scope fence.
-  __syncwarp();
-  int state = 0;
-  if (lane == 0) {
-    __threadfence_block();
-    if (atomicAdd(fin_arrived, 1) == n_rep - 1) {
-      __threadfence_block();
-      int old;
-      asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(&P.tickets[pair]) : "memory");
-      const int final_merge = old == c_last - c_first;
-      if (final_merge) P.tickets[pair] = 0;          // ready for the next call
-      __threadfence_block();
-      *(volatile int*)fin_ticket = 1 + final_merge;
-    }
-    for (uint32_t i = 0; i < (kSpinLimit << 4) && (state = *(volatile int*)fin_ticket) == 0; ++i)
-      if ((i & 255u) == 255u && *abort_flag) break;
-    __threadfence_block();
-  }
-  state = __shfl_sync(0xffffffffu, state, 0);
-  if (state != 2) return;
-  __syncwarp();
-  // this CTA drew the pair's last ticket: head h of all records, the loads of up to RB records in flight together
-  const int R = c_last - c_first + 1;
-  const float* base = P.partials + (size_t)(pair + c_first) * rstride + (size_t)h * kRecStride(Dv);
-  constexpr int RB = V == 1 ? 8 : 4;
-  float Mr = -INFINITY, Lr = 0.f;
-  bool any_bad = false;
-  float4 racc[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) racc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int rb = 0; rb < R; rb += RB) {
-    float2 mlr[RB];
-    float4 xv[RB][V];
-#pragma unroll
-    for (int i = 0; i < RB; ++i) {
-      const float* rh = base + (size_t)(rb + i < R ? rb + i : R - 1) * rstride;
-      mlr[i] = __ldcg(reinterpret_cast<const float2*>(rh + Dv));
-#pragma unroll
-      for (int v = 0; v < V; ++v) xv[i][v] = __ldcg(reinterpret_cast<const float4*>(rh + 128 * v + 4 * lane));
-    }
-    float Mn = Mr;
-#pragma unroll
-    for (int i = 0; i < RB; ++i) if (rb + i < R) Mn = fmaxf(Mn, mlr[i].x);
-    const float c0 = Mn == -INFINITY ? 0.f : fast_exp2(Mr - Mn);      // Mr = -inf gives 0
-    Lr *= c0;
-#pragma unroll
-    for (int v = 0; v < V; ++v) { racc[v].x *= c0; racc[v].y *= c0; racc[v].z *= c0; racc[v].w *= c0; }
-#pragma unroll
-    for (int i = 0; i < RB; ++i) {
-      if (rb + i >= R) continue;
-      if (mlr[i].y < 0.f) any_bad = true;
-      const float e = mlr[i].x == -INFINITY ? 0.f : fast_exp2(mlr[i].x - Mn);
-      Lr = fmaf(e, mlr[i].y, Lr);
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        racc[v].x = fmaf(e, xv[i][v].x, racc[v].x); racc[v].y = fmaf(e, xv[i][v].y, racc[v].y);
-        racc[v].z = fmaf(e, xv[i][v].z, racc[v].z); racc[v].w = fmaf(e, xv[i][v].w, racc[v].w);
-      }
-    }
-    Mr = Mn;
-  }
-  if (any_bad) Lr = 0.f;
-  const float inv = Lr > 0.f ? 1.f / Lr : 0.f;
-#pragma unroll
-  for (int v = 0; v < V; ++v) store4(128 * v + 4 * lane, make_float4(racc[v].x * inv, racc[v].y * inv, racc[v].z * inv, racc[v].w * inv));
-  if (lane == 0 && P.lse) P.lse[row] = Lr > 0.f ? (Mr + log2f(Lr)) / kLog2e : -INFINITY;
+  store_four(P, row * Dv + d, acc, L > 0.f ? 1.f / L : 0.f);
+  if (d == 0 && P.lse) P.lse[row] = L > 0.f ? (M + log2f(L)) / kLog2e : -INFINITY;
 }
 
-template <int G, int NW, bool kBf>
-__global__ void __launch_bounds__((NW + 1) * 32, 1) decode_mma_kernel(const __grid_constant__ DecodeParams P) {
-  constexpr int Gv = value_groups(G), Dv = 64 * Gv;
-  using S = Smem<G, NW>;
-  constexpr int kSlots = S::kSlots, kChunkBytes = S::kChunkBytes, kMBufs = S::kMBufs;
-  static_assert(kSlots >= NW + 4, "the ring must hold the chunks in work and a few in flight");
+// Agents first, first + step, ... without any key (kv_len == 0 or a rejected length): zeros, lse = -inf.
+__device__ __forceinline__ void clear_empty_agents(const DecodeParams& P, int first, int step, int Dv, int lane) {
+#pragma unroll 1
+  for (int a = first; a < P.n_agents; a += step) {
+    bool bad_len;
+    if (agent_range(P, a, bad_len).nc > 0) continue;
+#pragma unroll 1
+    for (int i = lane; i < P.y.Hq * Dv; i += 32) store_out(P, (size_t)a * P.y.Hq * Dv + i, 0.f);
+#pragma unroll 1
+    for (int i = lane; i < P.y.Hq && P.lse; i += 32) P.lse[(size_t)a * P.y.Hq + i] = -INFINITY;
+  }
+}
+
+// Pool offsets (16-byte units inside the layers of the call) of the warp's chunks 32 b .. 32 b + 31, one per lane: a walk
+// of the CTA's segments from the start, out of line (a warp needs it once per 32 chunks).
+__device__ __forceinline__ uint32_t chunk_offset(const DecodeParams& P, const Segment& s, int c, uint32_t chunk_bytes) {
+  const int blk = P.tables[(size_t)s.ar * P.max_blocks + (c >> 3)];
+  if (blk < 0 || blk >= P.n_blocks) { raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK); return kOffBad; }
+  return (uint32_t)(((uint64_t)s.li * P.y.layer_bytes + (uint64_t)blk * P.y.block_bytes +
+                     (uint64_t)(s.hk / P.sets) * P.y.head_block_bytes + (uint64_t)(c & 7) * chunk_bytes) >> 4);
+}
+__device__ __noinline__ uint32_t batch_offsets(const DecodeParams& P, const RangeStart& rs, int nw, int warp, int b, uint32_t chunk_bytes) {
+  Segment s;
+  uint32_t off = kOffBad;
+  const int my_k = warp + nw * (32 * b + (int)(threadIdx.x & 31)), end = min((int)(rs.u_end - rs.u_begin), nw * 32 * (b + 1));
+  if (rs.splits > 0) {
+    whole_segment(P, rs, s);
+    if (my_k < s.c1 - s.c0) off = chunk_offset(P, s, s.c0 + my_k, chunk_bytes);
+    return off;
+  }
+  Walker wk;
+  wk.init(P, rs);
+  while (wk.next(P, rs, s)) {
+    const int k1 = s.k0 + (s.c1 - s.c0);
+    if (my_k >= s.k0 && my_k < k1) off = chunk_offset(P, s, s.c0 + (my_k - s.k0), chunk_bytes);
+    if (k1 >= end) break;
+  }
+  return off;
+}
+
+template <int G, int H, bool kBf>
+__global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kernel(const __grid_constant__ DecodeParams P) {
+  using S = Smem<G, H>;
+  constexpr int NW = S::NW, D = S::D, Gv = S::Gv, Dv = S::Dv, kSlots = S::kSlots, kValSlots = S::kValSlots;
+  constexpr bool kHalves = S::kHalves;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   S& sm = *reinterpret_cast<S*>(smem_raw);
 
   const Layout& y = P.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int cta = blockIdx.x;
-  const int n_rep = y.n_rep;
+  const int n_rep = P.n_rep;
 
   grid_launch_dependents();
-  // rows of query heads that do not exist (n_rep < 4) are never staged: they stay zero
-  for (int i = threadIdx.x; i < kQBufs * 2 * G * 32; i += blockDim.x) (&sm.qfrag[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kSlots; ++s) { mbar_init(&sm.full[s], 1); sm.released[s] = 0; sm.bad[s] = 0; sm.patched[s] = 0; }
-    for (int i = 0; i < kQBufs; ++i) sm.q_tag[i] = 0;
-    for (int i = 0; i < kMBufs; ++i) { sm.deposits[i] = 0; sm.epilogues[i] = 0; sm.epi_claim[i] = 0; }
-    sm.all_issued = 0;
-    sm.next_chunk = 0;
-    sm.fin_arrived = 0; sm.fin_ticket = 0;
-    sm.abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  // ---- this CTA's unit range and its first two segments: one warp, the others set up shared memory (lengths and block
+  // tables are inputs that no kernel writes) ----
+  if (warp == 0) {
+    const RangeStart rs = find_range(P, cta, gridDim.x, NW);
+    if (lane == 0) {
+      if (rs.any_bad && cta == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
+      sm.range = rs;
+      if (rs.splits > 0) {
+        whole_segment(P, rs, sm.seg[0]);
+        sm.seg[1].a = -1; sm.seg[1].c0 = 0; sm.seg[1].c1 = 0; sm.seg[1].k0 = 0;
+      } else {
+        sm.walker.init(P, rs);
+        sm.walker.next(P, rs, sm.seg[0]);
+        sm.walker.next(P, rs, sm.seg[1]);
+      }
+    }
+  } else {
+    // columns of query heads that do not exist are never staged: they stay zero (factor 1)
+    for (int i = threadIdx.x - 32; i < 2 * G * 32; i += (NW - 1) * 32) (&sm.qfrag[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == NW - 1) {
+      for (int i = lane; i < H * G; i += 32) (&sm.qsum[0][0])[i] = 0.f;
+      if (lane < H) sm.kappa[lane] = 1.f;
+    }
+    if (warp == NW - 2) {
+      for (int i = lane; i < NW * kSlots; i += 32) mbar_init(&sm.full[0][0] + i, 1);
+      for (int i = lane; i < NW * kValSlots; i += 32) mbar_init(&sm.full_v[0][0] + i, 1);
+      if (lane == 0) { sm.abort_flag = 0; sm.fin[0][0] = -1; sm.fin[1][0] = -1; }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
   }
   __syncthreads();
-
-  // ---- this CTA's unit range (every warp computes it for itself; these inputs are not written by any kernel) ----
-  const RangeStart rs = find_range(P, cta, gridDim.x);
-  if (rs.any_bad && cta == 0 && threadIdx.x == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
-  const int n_chunks = (int)(rs.u_end - rs.u_begin);
-  Walker wk;
-  wk.init(P, rs);
-  Segment seg;
-
+  const int n_chunks = (int)(sm.range.u_end - sm.range.u_begin);
   const uint8_t* layer_base = P.pool + (uint64_t)P.layer * y.layer_bytes;
-  // hand ring slot `slot` to the chunk whose table entry is `off`
-  auto issue_copy = [&](int slot, uint32_t off) {
-    if (off == kOffBad) {
-      sm.bad[slot] = 1;
-      mbar_arrive(&sm.full[slot]);
-    } else {
-      sm.bad[slot] = 0;
-      mbar_arrive_expect_tx(&sm.full[slot], kChunkBytes);
-      bulk_load(sm.ring + (size_t)slot * kChunkBytes, layer_base + (uint64_t)off * 16u, kChunkBytes, &sm.full[slot]);
+  uint32_t off = kOffBad;                                // pool offset of the warp's chunk number `lane` (of 32 at a time)
+  {
+    const int k = warp + NW * lane;
+    const Segment &s0 = sm.seg[0], &s1 = sm.seg[1];
+    if (k < n_chunks) {
+      const int n0 = s0.c1 - s0.c0;
+      if (k < n0) off = chunk_offset(P, s0, s0.c0 + k, S::kChunkBytes);
+      else if (k < n0 + (s1.c1 - s1.c0)) off = chunk_offset(P, s1, s1.c0 + k - n0, S::kChunkBytes);
     }
+    if (sm.range.splits == 0 && n_chunks > s0.c1 - s0.c0 && n_chunks > s1.k0 + (s1.c1 - s1.c0)) off = batch_offsets(P, sm.range, NW, warp, 0, S::kChunkBytes);
+  }
+  uint8_t* const ring = sm.ring[warp];
+  auto issue_keys = [&](int slot, uint32_t off) {        // the whole chunk unless it is copied in halves
+    uint64_t* bar = &sm.full[warp][slot];
+    constexpr uint32_t bytes = kHalves ? S::kKeyBytes : S::kChunkBytes;
+    if (off == kOffBad) { mbar_arrive(bar); return; }
+    mbar_arrive_expect_tx(bar, bytes);
+    bulk_load(ring + slot * bytes, layer_base + (uint64_t)off * 16u, bytes, bar);
+  };
+  auto issue_values = [&](int slot, uint32_t off) {
+    uint64_t* bar = &sm.full_v[warp][slot];
+    if (off == kOffBad) { mbar_arrive(bar); return; }
+    mbar_arrive_expect_tx(bar, S::kValBytes);
+    bulk_load(ring + kSlots * S::kKeyBytes + slot * S::kValBytes, layer_base + (uint64_t)off * 16u + S::kKeyBytes, S::kValBytes, bar);
   };
 
-  // =============================== planner warp ================================================
-  if (warp == NW) {
-    // Planning step: 32 chunks, one per lane: block-table entry -> pool offset -> table entry k % kOffCap.  Issue
-    // step: lane s owns ring slot s and the chunks s, s + kSlots, ...; it copies its next chunk once the slot's
-    // previous chunk has been consumed and the chunk has its table entry.  All lanes follow one path.  Lengths and
-    // block tables are inputs that no kernel writes, so the first planning steps run while the preceding kernel drains;
-    // the pool is read only after it.
-    static_assert(kSlots <= 32 && kOffCap >= 2 * 32 + kSlots, "table ring: a step of entries ahead of every reader");
-    // Once every chunk has been issued this warp has time to spare, and it takes the epilogues of the segments that
-    // complete from then on (all but the CTA's last): a consumer that leaves the stream for an epilogue (a few
-    // microseconds with the ticket and a pair's final combination) costs its CTA an extra round of chunks.  While
-    // chunks are still to be issued the consumers keep them, or the ring would run dry meanwhile.  A claim word per
-    // deposit buffer decides who runs one.  Segments complete in order, so a second walker names the next one.
-    // d = 128 only (5 agents x 4097 tokens: 20.2 -> 19.2 us per launch, 2 agents: 18.4 -> 15.9 us; 40 agents: 1.8 %
-    // slower): in the other instantiations the second copy of the epilogue's code slowed the chunk loop of long
-    // launches by 5-9 %, as one shared non-inlined copy did through its spills.
-    // (A segment is the CTA's last when its chunks end the CTA's range: no count of the segments is needed.)
-    Walker wke = wk;
-    Segment sge;
-    int epi_idx = 0;
-    bool epi_more = false, epi_started = false;          // sge names a segment that is not the CTA's last
-    bool waited = false, bad_block = false, more = wk.next(seg), all_out = false;
-    int tq_head = 0, tq_tail = 0;            // patch queue: entries tq_head .. tq_tail-1 (indices taken modulo kTailQ)
-    int kb = 0;                              // chunks of `seg` already planned
-    int planned = 0;                         // chunks of the CTA that have their table entry
-    int next_k = lane < kSlots ? lane : INT_MAX, round = 0;   // this lane's next chunk and its round in the slot
-    const volatile int* my_released = &sm.released[lane < kSlots ? lane : 0];
-    uint32_t idle = 0;
-    for (;;) {
-      // ---- plan as far as the table allows: entries below every lane's next chunk are dead ----
-      if (more) {
-        int lo = next_k;
+  const int my_chunks = n_chunks > warp ? (n_chunks - warp + NW - 1) / NW : 0;
+  const int g = lane >> 2, tid = lane & 3;
+  // this warp's row of a segment's query; the new row's groups are quantized by the warps behind the query's (from 4 on)
+  constexpr int kNewWarps = NW - 4, kNewRounds = (G + Gv + kNewWarps - 1) / kNewWarps;
+  auto query_row = [&](const Segment& s) { return P.q + ((size_t)s.a * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
+  auto new_pair = [&](const Segment& s, int grp) {
+    const size_t head = (size_t)s.a * y.Hkv + s.hk;
+    return (grp < G ? P.k_new + head * D + 64 * grp : P.v_new + head * Dv + 64 * (grp - G)) + 2 * lane;
+  };
+  // the segment's last chunk holds the agent's newest position, and the token is appended by this launch
+  auto has_tail = [&](const Segment& s) { return P.k_new != nullptr && s.c1 == s.cf + s.nc; };
+  uint4 qv = make_uint4(0u, 0u, 0u, 0u);                 // the next segment's query row and new-row groups, on their way
+  uint32_t nv[kNewRounds];
+  auto fetch_rows = [&](const Segment& s) {
+    if (warp < n_rep && lane < D / 8) qv = *reinterpret_cast<const uint4*>(query_row(s));
+    if (warp >= 4 && has_tail(s)) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        while (more && planned + 32 <= lo + kOffCap && tq_tail - tq_head < kTailQ) {
-          const int cnt = seg.c1 - seg.c0;
-          if (kb == 0 && seg.tail_pos >= 0) {
-            // this segment ends with the agent's newest position: queue the patch, ask for the new rows
-            if (lane == 0) sm.tail_q[tq_tail % kTailQ] = make_int4(seg.k0 + seg.tail_pos, seg.a, seg.hk, (seg.n - 1) & 31);
-            ++tq_tail;
-            prefetch_new_token<G>(P.k_new, P.v_new, y.Hkv, seg.a, seg.hk, lane);
-          }
-          if (kb + lane < cnt) {
-            const int c = seg.chunk_at(kb + lane);
-            const int blk = P.tables[(size_t)seg.ar * P.max_blocks + (c >> 3)];
-            uint32_t off = kOffBad;
-            if (blk >= 0 && blk < P.n_blocks)
-              off = (uint32_t)(((uint64_t)seg.li * y.layer_bytes + (uint64_t)blk * y.block_bytes + (uint64_t)seg.hk * y.head_block_bytes +
-                                (uint64_t)(c & 7) * kChunkBytes) >> 4);
-            else
-              bad_block = true;
-            sm.src_off[(seg.k0 + kb + lane) % kOffCap] = off;
-          }
-          kb += 32;
-          if (kb >= cnt) { planned = seg.k0 + cnt; kb = 0; more = wk.next(seg); } else { planned = seg.k0 + kb; }
-        }
-        __syncwarp();
+      for (int r = 0; r < kNewRounds; ++r) {
+        const int grp = warp - 4 + kNewWarps * r;
+        if (grp < G + Gv) nv[r] = *reinterpret_cast<const uint32_t*>(new_pair(s, grp));
       }
-      if (!waited) {
-        // While the preceding kernel drains, ask L2 for the chunks of the first ring fill (more than that was measured
-        // and is no faster; the same prefetch in the MLA-latent kernel gains nothing).  A prefetch returns nothing
-        // to the kernel, and L2 is where the preceding kernel's writes land, so what the copies read after the wait
-        // is current whatever that kernel still writes.
-        if (lane < kSlots && next_k < planned) {
-          const uint32_t off = sm.src_off[next_k % kOffCap];
-          if (off != kOffBad) prefetch_l2_bulk(layer_base + (uint64_t)off * 16u, kChunkBytes);
-        }
-        grid_dependency_wait();
-        waited = true;
+    }
+  };
+  // While the preceding kernel drains, ask L2 for the first chunks and rows.  A prefetch returns nothing to the kernel, and
+  // L2 is where the preceding kernel's writes land, so what is read after the wait is current whatever it still writes.
+  if (n_chunks > 0) {
+    if (lane < 3 && lane < my_chunks && off != kOffBad) prefetch_l2_bulk(layer_base + (uint64_t)off * 16u, S::kChunkBytes);
+    if (warp < n_rep && lane < D / 8 && (lane & 7) == 0) prefetch_l2(query_row(sm.seg[0]));
+    if (warp >= 4 && has_tail(sm.seg[0]) && lane == 0)
+      for (int grp = warp - 4; grp < G + Gv; grp += kNewWarps) prefetch_l2(new_pair(sm.seg[0], grp));
+  }
+  // Everything written here (outputs, records, tickets) may still be in use by the preceding kernels of the stream until
+  // they have completed, and they may have written the pool, the queries and the new rows.
+  grid_dependency_wait();
+  if (n_chunks > 0) fetch_rows(sm.seg[0]);               // before the bulk copies, or the rows queue behind them
+  if (lane < kSlots && lane < my_chunks) {
+    issue_keys(lane, off);
+    if (kHalves && lane < kValSlots) issue_values(lane, off);
+  }
+
+  if (cta * NW + warp < P.n_agents) clear_empty_agents(P, cta * NW + warp, gridDim.x * NW, Dv, lane);
+  if (n_chunks == 0) return;                             // uniform over the CTA
+
+  const int hcol[2] = {(2 * tid) & (H - 1), (2 * tid + 1) & (H - 1)};   // this lane's two score columns
+  const uint32_t split_mask = tid >= 2 ? 0xFFFFE000u : 0u;
+  const float margin = my_chunks > 1 ? kMargin : 0.f;
+  bool aborted = false;
+  uint32_t cur = __shfl_sync(0xffffffffu, off, 0), nxt = __shfl_sync(0xffffffffu, off, 1);   // offsets of the chunks in the two slots
+  int i = 0;                                             // this warp's chunk counter: chunk k = warp + NW * i of the CTA
+  const uint4* qb = &sm.qfrag[0][lane];
+  for (int si = 0;; ++si) {
+    const Segment& seg = sm.seg[si % 3];
+    const int k0 = seg.k0, c0 = seg.c0, c1 = seg.c1, k1 = k0 + (c1 - c0);
+    const int key_lo = seg.lo, key_n = seg.n;
+    const bool newest = has_tail(seg);
+    const bool tail = newest && (k1 - 1) % NW == warp;                  // this warp holds the chunk of the newest position
+    if (warp < n_rep) stage_query_row<G, H>(sm.qfrag, sm.qsum, sm.kappa, qv, P.scale_log2, warp, lane);
+    if (warp >= 4 && newest) {
+#pragma unroll
+      for (int r = 0; r < kNewRounds; ++r)
+        if (warp - 4 + kNewWarps * r < G + Gv) quantize_new_group<G, H>(sm, nv[r], warp - 4 + kNewWarps * r, kBf, lane);
+    }
+    __syncthreads();
+    const float* const qs0 = sm.qsum[hcol[0]];
+    const float* const qs1 = sm.qsum[hcol[1]];
+    const float kap[2] = {sm.kappa[hcol[0]], sm.kappa[hcol[1]]};
+    WarpState<G> st;
+    st.reset();
+    bool poisoned = false;
+    bool have = false;
+#pragma unroll 1
+    for (int k = warp + NW * i; k < k1; k += NW, ++i) {
+      const int slot = i % kSlots;
+      const uint32_t parity = (uint32_t)(i / kSlots) & 1u;
+      const int j = i + kSlots;                          // the chunk this slot takes next
+      const bool refill = j < my_chunks && !aborted;
+      uint32_t noff = kOffBad;
+      if (refill) {
+        if ((j & 31) == 0) off = batch_offsets(P, sm.range, NW, warp, j >> 5, S::kChunkBytes);
+        noff = __shfl_sync(0xffffffffu, off, j & 31);
       }
-      // ---- issue: a short polling loop, left from time to time to plan further ----
-      bool any_left = true;
-      for (int it = 0; it < 64 && any_left; ++it) {
-        // the fused append: quantize the new token into the oldest queued chunk once that chunk has landed (the whole
-        // warp works on it; its consumer waits for sm.patched)
-        if (tq_head < tq_tail) {
-          const int4 t = sm.tail_q[tq_head % kTailQ];
-          const int tslot = t.x % kSlots, tround = t.x / kSlots;
-          const int issued = __shfl_sync(0xffffffffu, round, tslot);      // copies this slot's lane has issued so far
-          if (issued > tround && mbar_test_wait(&sm.full[tslot], (uint32_t)tround & 1u)) {
-            if (!sm.bad[tslot]) {
-              uint8_t* gchunk = const_cast<uint8_t*>(layer_base) + (uint64_t)sm.src_off[t.x % kOffCap] * 16u;
-              append_new_token<G>(sm.ring + (size_t)tslot * kChunkBytes, gchunk, y, P.k_new, P.v_new, t.y, t.z, t.w, lane);
-            }
-            __threadfence_block();
-            __syncwarp();
-            if (lane == 0) *(volatile int*)&sm.patched[tslot] = tround + 1;
-            ++tq_head;
-            idle = 0;
-          }
+      const bool bad = cur == kOffBad;
+      uint8_t* const chunk = ring + slot * (kHalves ? S::kKeyBytes : S::kChunkBytes);
+      uint8_t* const vhalf = kHalves ? ring + kSlots * S::kKeyBytes : chunk + S::kKeyBytes;
+      static_assert(!kHalves || kValSlots == 1, "");
+      const bool patch = tail && k == k1 - 1;
+      bool ok = mbar_wait(&sm.full[warp][slot], parity, &sm.abort_flag);
+      if (kHalves && patch && ok) ok = mbar_wait(&sm.full_v[warp][0], (uint32_t)i & 1u, &sm.abort_flag);
+      if (!ok) {
+        // giving up: the copies this warp has in flight land (or are waited for long enough) before it goes on
+        sm.abort_flag = 1;
+        aborted = true;
+        for (int s = 0; s < kSlots; ++s) {
+          const int last = i + (s - slot + kSlots) % kSlots;
+          if (last < my_chunks)
+            for (uint32_t t = 0; t < 4096u && !mbar_try_wait(&sm.full[warp][s], (uint32_t)(last / kSlots) & 1u); ++t) {}
         }
-        if (G == 2 && epi_more) {
-          const int eb = epi_idx % kMBufs, euse = epi_idx / kMBufs;
-          if (*(volatile int*)&sm.deposits[eb] >= (euse + 1) * NW) {
-            int state = 0;                               // 1: a consumer has it, 2: this warp takes it
-            if (lane == 0) {
-              if (*(volatile int*)&sm.epi_claim[eb] > euse) state = 1;
-              else if (all_out) state = atomicCAS(&sm.epi_claim[eb], euse, euse + 1) == euse ? 2 : 1;
-            }
-            state = __shfl_sync(0xffffffffu, state, 0);
-            if (state == 2) {
-              __threadfence_block();
-              segment_epilogue<G, NW>(&sm.merge[eb][0][0][0], &sm.epilogues[eb], euse, P, sge, cta, rs.part, lane);
-            }
-            if (state != 0) {
-              epi_more = wke.next(sge) && sge.k0 + (sge.c1 - sge.c0) < n_chunks;
-              ++epi_idx;
-              idle = 0;
-            }
-          }
-        }
-        const bool can = next_k < planned && *my_released >= round;
-        if (can) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the consumer's reads and patches of the slot come first
-          issue_copy(lane, sm.src_off[next_k % kOffCap]);
-          next_k += kSlots;
-          ++round;
-        }
-        if (G == 2 && !epi_started) {                    // the first segment is named here, after the first copies are out
-          epi_started = true;
-          epi_more = wke.next(sge) && sge.k0 + (sge.c1 - sge.c0) < n_chunks;
-        }
-        if (!all_out && !__any_sync(0xffffffffu, next_k < n_chunks)) {
-          all_out = true;
-          if (lane == 0) *(volatile int*)&sm.all_issued = 1;
-        }
-        any_left = !all_out || tq_head < tq_tail || (G == 2 && epi_more);
-        if (__any_sync(0xffffffffu, can)) { idle = 0; continue; }
-        if (more && tq_tail - tq_head < kTailQ && __all_sync(0xffffffffu, next_k >= planned)) break;   // plan further first
-        ++idle;
-        __nanosleep(200);
-      }
-      if (!any_left) break;                  // every chunk has been issued, every epilogue but the last is done
-      if (idle > (kSpinLimit >> 2) || *(volatile int*)&sm.abort_flag) {
-        if (lane == 0) { sm.abort_flag = 1; raise_flag(P.flags, Q4KV_FLAG_INTERNAL); }
-        // giving up: each lane lets the last copy it issued into its slot land before the CTA lets go of shared memory
-        if (lane < kSlots && round > 0)
-          for (uint32_t i = 0; i < 4096u && !mbar_try_wait(&sm.full[lane], (uint32_t)(round - 1) & 1u); ++i) {}
+        if (kHalves)
+          for (uint32_t t = 0; t < 4096u && !mbar_try_wait(&sm.full_v[warp][0], (uint32_t)i & 1u); ++t) {}
+        i = my_chunks;                                   // nothing is issued or read any more
         break;
       }
-    }
-    if (bad_block) raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK);
-    return;
-  }
-
-  // =============================== consumer warps ==============================================
-  // Everything the consumers write (output rows, partial records, tickets) may still be in use by
-  // the preceding kernels of the stream until they have completed.
-  grid_dependency_wait();
-  const int g = lane >> 2, tid = lane & 3;
-  // this lane's two score columns 2 tid, 2 tid + 1 of eight: columns 0..3 are the query heads of the KV head, 4..7
-  // repeat them and carry p*s minus its binary16 truncation
-  const int hcol[2] = {(2 * tid) & 3, (2 * tid + 1) & 3};
-  const bool live[2] = {hcol[0] < n_rep, hcol[1] < n_rep};
-  const uint32_t split_mask = tid >= 2 ? 0xFFFFE000u : 0u;
-
-  // agents without any key (kv_len == 0 or a rejected length): zeros, lse = -inf
-  for (int a = cta * NW + warp; a < P.n_agents; a += gridDim.x * NW) {
-    bool bad_len;
-    if (agent_range(P, a, bad_len).nc > 0) continue;
-    for (int i = lane; i < y.Hq * Dv; i += 32) store_out(P, (size_t)a * y.Hq * Dv + i, 0.f);
-    if (P.lse) for (int i = lane; i < y.Hq; i += 32) P.lse[(size_t)a * y.Hq + i] = -INFINITY;
-  }
-  if (n_chunks == 0) return;
-
-  // ---- the first segments' queries are staged up front, one warp each ----
-  {
-    Walker w2 = wk;
-    Segment s2;
-    for (int s = 0; s < kQBufs && w2.next(s2); ++s) {
-      if (s % NW != warp) continue;
-      stage_query<G>(sm.qfrag[s], sm.qsum[s], sm.kappa[s], P.q, y.Hq, n_rep, P.scale_log2, s2.a, s2.hk, lane);
-      __threadfence_block();
-      __syncwarp();
-      if (lane == 0) *(volatile int*)&sm.q_tag[s] = s + 1;
-    }
-  }
-
-  bool aborted = false, poisoned = false;
-  int cur = -1;                 // index of the segment `seg` describes (-1: none yet)
-  bool have_seg = false;        // this warp holds state for segment `cur`
-  const uint4* qa = nullptr;    // this lane's A registers of the segment's query, in shared memory
-  float qs[2][G], kap[2] = {0.f, 0.f};
-  WarpState<G> st;
-  st.reset();
-
-  // Deposit this warp's state for segment `cur` (described by `seg`); the warp that completes the
-  // count combines the deposits and runs the segment's epilogue.
-  auto deposit_and_maybe_finish = [&](bool real) {
-    const int b = cur % kMBufs, use = cur / kMBufs;
-    // the buffer is free once the epilogue of its previous use is done
-    if (!aborted && !spin_until_ge(&sm.epilogues[b], use, &sm.abort_flag)) aborted = true;
-    float (*mg)[S::kMergeStride] = sm.merge[b][warp];
-    if (real) {
-      // sums over the lane's tokens -> sums over the chunk's tokens (the eight lanes of equal tid)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float l = st.l_e[c] + 16.f * st.l_o[c];
-        l += __shfl_xor_sync(0xffffffffu, l, 4);
-        l += __shfl_xor_sync(0xffffffffu, l, 8);
-        l += __shfl_xor_sync(0xffffffffu, l, 16);
-        float bias[Gv];
-#pragma unroll
-        for (int gi = 0; gi < Gv; ++gi) {
-          float bb = st.bias_e[c][gi] + 16.f * st.bias_o[c][gi];
-          bb += __shfl_xor_sync(0xffffffffu, bb, 4);
-          bb += __shfl_xor_sync(0xffffffffu, bb, 8);
-          bb += __shfl_xor_sync(0xffffffffu, bb, 16);
-          bias[gi] = bb;
-        }
-        if (g == 0 && tid < 2) {
-          float* row = mg[2 * tid + c];
-          row[Dv] = st.m[c];
-          row[Dv + 1] = (poisoned || aborted) ? -1.f : l;
-#pragma unroll
-          for (int gi = 0; gi < Gv; ++gi) row[Dv + 2 + gi] = bias[gi];
-        }
-      }
-      // columns 4..7 (lanes tid 2,3) hold the low-part products of heads 0..3
-#pragma unroll
-      for (int mt = 0; mt < Dv / 16; ++mt) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float v = st.o[mt][r] + __shfl_xor_sync(0xffffffffu, st.o[mt][r], 2);
-          if (tid < 2) mg[2 * tid + (r & 1)][16 * mt + g + 8 * (r >> 1)] = v * 16777216.f;
-        }
-      }
-    } else if (lane < 4) {
-      mg[lane][Dv] = -INFINITY;
-      mg[lane][Dv + 1] = aborted ? -1.f : 0.f;
-    }
-    __threadfence_block();
-    __syncwarp();
-    int last = 0;
-    if (lane == 0) last = atomicAdd(&sm.deposits[b], 1) == (use + 1) * NW - 1;
-    last = __shfl_sync(0xffffffffu, last, 0);
-    const bool last_seg = seg.k0 + (seg.c1 - seg.c0) >= n_chunks;     // this segment's chunks end the CTA's range
-    if (G != 3 && last_seg) {
-      // the CTA's last segment: nothing is left to stream, so the head warps wait for the last deposit and share the
-      // epilogue; the other warps are done.  (Not in the d_qk 192 instantiation, where it measured 0.4 % slower.  On the
-      // d-128 kernel it cost 1.2 us while a consumer still ran the epilogues of earlier segments; since the planner
-      // warp takes those it saves 0.5 us per launch at 5 agents and 0.8 us at 2.)
-      if (warp >= n_rep) return;
-      {
-        bool ok = false;
-        for (uint32_t i = 0; i < (kSpinLimit << 2); ++i) {
-          if (*(volatile int*)&sm.deposits[b] >= (use + 1) * NW) { ok = true; break; }
-          __nanosleep(100);
-          if ((i & 63u) == 63u && *(volatile int*)&sm.abort_flag) break;
-        }
-        if (!ok) return;
-      }
-      __threadfence_block();
-      last_segment_by_heads<G, NW>(&sm.merge[b][0][0][0], &sm.fin_arrived, &sm.fin_ticket, &sm.abort_flag, P, seg, cta,
-                                   rs.part, warp, lane);
-      return;
-    }
-    if (!last) return;
-    if (G == 2 && !last_seg) {
-      // an earlier segment: the planner warp takes it if it has nothing left to issue
-      int mine = 0;
-      if (lane == 0 && !*(volatile int*)&sm.all_issued) mine = atomicCAS(&sm.epi_claim[b], use, use + 1) == use;
-      if (!__shfl_sync(0xffffffffu, mine, 0)) return;
-    }
-    __threadfence_block();
-    segment_epilogue<G, NW>(&sm.merge[b][0][0][0], &sm.epilogues[b], use, P, seg, cta, rs.part, lane);
-  };
-
-  // A chunk is claimed only when the warp is free to work on it: a warp that is away in a segment's epilogue (a few
-  // microseconds when it merges a pair's records) must not sit on a claimed chunk meanwhile.
-  bool out_of_chunks = false;
-  for (;;) {
-    int k = 0;
-    if (!out_of_chunks) {
-      if (lane == 0) k = atomicAdd(&sm.next_chunk, 1);
-      k = __shfl_sync(0xffffffffu, k, 0);
-      out_of_chunks = k >= n_chunks;
-    }
-    // move to the segment that holds chunk k (to the end of the list when out of chunks), leaving a
-    // deposit in every segment passed
-    bool finished = false;
-    while (cur < 0 || out_of_chunks || k >= seg.k0 + (seg.c1 - seg.c0)) {
-      if (cur >= 0) deposit_and_maybe_finish(have_seg);
-      have_seg = false;
-      poisoned = false;
-      if (!wk.next(seg)) { finished = true; break; }
-      ++cur;
-    }
-    if (finished) break;
-    if (!have_seg) {
-      // entering segment `cur`: its query fragments
-      const int qb = cur % kQBufs;
-      if (cur >= kQBufs && k == seg.k0) {
-        // later segments are staged by whoever claims their first chunk, once the buffer's previous
-        // segment has been left by every warp (its epilogue is done)
-        const int prev = cur - kQBufs;
-        if (!aborted && !spin_until_ge(&sm.epilogues[prev % kMBufs], prev / kMBufs + 1, &sm.abort_flag)) aborted = true;
-        stage_query<G>(sm.qfrag[qb], sm.qsum[qb], sm.kappa[qb], P.q, y.Hq, n_rep, P.scale_log2, seg.a, seg.hk, lane);
-        __threadfence_block();
+      const int pos0 = (c0 + (k - k0)) * 32;
+      const bool edge = pos0 < key_lo || pos0 + 32 > key_n;
+      if (bad) {
+        poisoned = true;
+      } else if (patch) {
+        patch_new_row<G, H>(sm, chunk, vhalf, const_cast<uint8_t*>(layer_base) + (uint64_t)cur * 16u,
+                            (key_n - 1) & 31, lane);
         __syncwarp();
-        if (lane == 0) *(volatile int*)&sm.q_tag[qb] = cur + 1;
       }
-      if (!aborted && !spin_until_ge(&sm.q_tag[qb], cur + 1, &sm.abort_flag)) aborted = true;
-      __threadfence_block();
-      qa = &sm.qfrag[qb][0][lane];
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-#pragma unroll
-        for (int gi = 0; gi < G; ++gi) qs[c][gi] = live[c] ? sm.qsum[qb][hcol[c]][gi] : 0.f;
-        kap[c] = live[c] ? sm.kappa[qb][hcol[c]] : 0.f;
+      float sc[4][2];
+      if (!bad) chunk_scores<G, kBf>(chunk, g, tid, qb, qs0, qs1, sc);
+      if (kHalves) {
+        __syncwarp();
+        if (refill && lane == 0) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the warp's reads and patches of the slot come first
+          issue_keys(slot, noff);
+        }
+        if (!mbar_wait(&sm.full_v[warp][0], (uint32_t)i & 1u, &sm.abort_flag)) { sm.abort_flag = 1; poisoned = true; }
+        __syncwarp();
       }
-      st.reset();
-      have_seg = true;
+      if (!bad) {
+        if (edge) {
+          clear_outside<G>(vhalf + 32 * (Dv / 2), pos0, key_lo, key_n, lane);
+          __syncwarp();
+        }
+        have = true;
+        chunk_values<G, H, kBf>(vhalf, edge, pos0, key_lo, key_n, g, tid, kap, split_mask, margin, sc, st);
+      }
+      __syncwarp();
+      if (kHalves) {
+        if (i + 1 < my_chunks && lane == 0) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          issue_values(0, nxt);
+        }
+      } else if (refill && lane == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue_keys(slot, noff);
+      }
+      cur = nxt;
+      nxt = noff;
     }
-    const int slot = k % kSlots;
-    const int round = k / kSlots;
-    // the slot's previous chunk must have been consumed (then its fill is complete and the parity wait is exact)
-    if (aborted || !spin_until_ge(&sm.released[slot], round, &sm.abort_flag) ||
-        !mbar_wait(&sm.full[slot], (uint32_t)round & 1u, &sm.abort_flag)) {
-      aborted = true;
-      continue;
+
+    // ---- end of the segment: deposit, combine ----
+    const bool more = sm.seg[(si + 1) % 3].a >= 0;
+    if (more) fetch_rows(sm.seg[(si + 1) % 3]);
+    if (have) {
+      deposit<G, H>(sm, warp, lane, st, poisoned || aborted);
+    } else if (lane < H) {
+      sm.dep_m[warp][lane] = -INFINITY;
+      sm.dep_l[warp][lane] = (poisoned || aborted) ? -1.f : 0.f;
     }
-    if (sm.bad[slot]) {
-      poisoned = true;
-    } else {
-      const int j = k - seg.k0;
-      // the chunk that receives the step's new token is usable once the planner warp has quantized the token into it
-      if (j == seg.tail_pos && !spin_until_ge(&sm.patched[slot], round + 1, &sm.abort_flag)) { aborted = true; continue; }
-      __threadfence_block();
-      process_chunk<G, kBf>(sm.ring + (size_t)slot * kChunkBytes, seg.chunk_at(j) * 32, seg.lo, seg.n, g, tid, qa, qs, kap,
-                       split_mask, st);
+    __syncthreads();
+    for (int unit = warp; unit < S::kDepUnits; unit += NW) combine_deposits<G, H>(sm, P, seg, cta, unit, lane);
+    if (warp == NW - 1 && lane == 0) {
+      if (seg.c1 - c0 != seg.nc) {                       // only the first and the last segment can be parts of a pair
+        int* f = sm.fin[k0 == 0 ? 0 : 1];
+        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = seg.a * y.Hq + seg.hk * n_rep;
+      }
+      if (more) sm.walker.next(P, sm.range, sm.seg[(si + 2) % 3]);       // never where the CTA holds one segment
     }
-    __syncwarp();
-    if (lane == 0) { __threadfence_block(); *(volatile int*)&sm.released[slot] = round + 1; }
+    if (!more) break;
+    __syncthreads();
   }
   if (aborted && lane == 0) raise_flag(P.flags, Q4KV_FLAG_INTERNAL);
+
+  // ---- tickets: all CTAs end at about the same time, so the first segment's is drawn here too, beside the last one's.
+  // The CTA's record stores are ordered before the atomic by the barrier, other CTAs' record loads after it by the second:
+  // one acquire-release atomic takes the place of a fence on either side. ----
+  __syncthreads();
+  if (lane == 0 && warp % (NW / 2) == 0) {
+    const int x = warp / (NW / 2);
+    int last = 0;
+    if (sm.fin[x][0] >= 0) {
+      int old;
+      asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(&P.tickets[sm.fin[x][0]]) : "memory");
+      last = old == sm.fin[x][2] - sm.fin[x][1];
+      if (last) P.tickets[sm.fin[x][0]] = 0;             // ready for the next call
+    }
+    sm.fin_last[x] = last;
+  }
+  __syncthreads();
+  const bool both = (sm.fin_last[0] & sm.fin_last[1]) != 0;
+#pragma unroll 1
+  for (int x = 0; x < 2; ++x) {
+    if (!sm.fin_last[x]) continue;
+    // one warp per head and 128 elements: all warps when one pair is to be combined, half of them each when there are two
+    const int first = both ? NW / 2 * x : 0, count = both ? NW / 2 : NW;
+    if (warp < first || warp >= first + count) continue;
+    const size_t rstride = (size_t)n_rep * kRecStride(Dv);
+    for (int t = warp - first; t < n_rep * (Dv / 128); t += count) {
+      const int h = t / (Dv / 128), d = (t % (Dv / 128)) * 128 + 4 * lane;
+      combine_records(P, P.partials + (size_t)(sm.fin[x][0] + sm.fin[x][1]) * rstride + (size_t)h * kRecStride(Dv), rstride,
+                      sm.fin[x][2] - sm.fin[x][1] + 1, Dv, d, (size_t)sm.fin[x][3] + h, lane);
+    }
+  }
 }
 
-template <int G, int NW, bool kBf>
-cudaError_t launch_g(const DecodeParams& P, int grid, bool pdl, cudaStream_t st) {
-  static bool configured[64] = {};     // the attribute is per function and device: set it once for each
-  const size_t smem = sizeof(Smem<G, NW>);
+template <int G, int H, bool kBf>
+cudaError_t launch_g(const DecodeParams& P, int grid, cudaStream_t st) {
+  static bool configured[64] = {};     // the attributes are per function and device: set them once for each
+  constexpr size_t smem = sizeof(Smem<G, H>);
+  static_assert(smem <= 227 * 1024 / kCtasPerSm - 1024, "two CTAs per SM");
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(decode_mma_kernel<G, NW, kBf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3((NW + 1) * 32);
+  cfg.blockDim = dim3(warps_of(G) * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, decode_mma_kernel<G, NW, kBf>, P);
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, decode_mma_kernel<G, H, kBf>, P);
+}
+template <int G, int H>
+cudaError_t launch_gh(const DecodeParams& P, int grid, cudaStream_t st) {
+  return P.y.sb_bf16 ? launch_g<G, H, true>(P, grid, st) : launch_g<G, H, false>(P, grid, st);
+}
+
+// Sets of query heads a KV head's heads are cut into: the kernel's columns take four of them, or eight at d = 128
+int head_sets(const Layout& y) {
+  const int most = y.D == 128 ? 8 : 4;
+  int sets = (y.n_rep + most - 1) / most;
+  while (y.n_rep % sets) ++sets;
+  return sets;
 }
 
 }  // namespace
 
-// Number of SMs of the current device (one persistent CTA each), looked up once per device.
+// Number of SMs of the current device, looked up once per device.
 int sm_count() {
   static int cached[64] = {};
   int dev = 0;
@@ -1493,21 +1328,22 @@ int sm_count() {
 }
 
 bool decode_mma_supported(const Layout& y) {
-  return !y.alias && y.n_rep <= 4 && ((y.D == y.Dv && (y.D == 128 || y.D == 256)) || (y.D == 192 && y.Dv == 128));
+  return !y.alias && ((y.D == y.Dv && (y.D == 128 || y.D == 256)) || (y.D == 192 && y.Dv == 128));
 }
 
-// the kernel counts work units in 32 bits and keeps one arrival counter per (layer of the call, agent, KV head) in
+// the kernel counts work units in 32 bits and keeps one arrival counter per (layer of the call, agent, head set) in
 // the workspace header; chunk offsets inside the call's layers are kept in 16-byte units in 32 bits
 bool decode_mma_fits(const Layout& y, int n_agents, int max_blocks, int layer_count) {
-  const long long v = (long long)n_agents * layer_count;
+  const long long v = (long long)n_agents * layer_count * head_sets(y);
   return layer_count >= 1 && layer_count <= kMaxLayersPerCall && v * y.Hkv * (max_blocks * 8ll) < (1ll << 30) &&
          v * y.Hkv <= kMaxTicketPairs && (unsigned long long)layer_count * y.layer_bytes < (1ull << 36);
 }
 
-// bytes behind the workspace header: one record per (layer, agent, KV head) and per CTA of the largest grid
+// bytes behind the workspace header: one record per (layer, agent, head set) and per CTA of the largest grid
 size_t decode_mma_workspace_bytes(const Layout& y, int n_agents, int layer_count) {
-  const size_t pairs = (size_t)n_agents * layer_count * y.Hkv;
-  return (pairs + kMaxGrid) * y.n_rep * kRecStride(y.Dv) * sizeof(float);
+  const int sets = head_sets(y);
+  const size_t pairs = (size_t)n_agents * layer_count * y.Hkv * sets;
+  return (pairs + kMaxGrid) * (y.n_rep / sets) * kRecStride(y.Dv) * sizeof(float);
 }
 
 // layer_count == 1: `windows` points at the one window.  Otherwise q, out, lse and the new rows hold layer_count
@@ -1520,12 +1356,13 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   DecodeParams P;
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents * layer_count;
   P.n_real = b.n_agents; P.layer_count = layer_count;
+  P.sets = head_sets(y); P.Hkv = y.Hkv * P.sets; P.n_rep = y.n_rep / P.sets;
   long long units = 0;
   for (int i = 0; i < kMaxLayersPerCall; ++i) {
     P.windows[i] = i < layer_count ? windows[i] : 0;
     if (i < layer_count) {
       const int span = (windows[i] > 0 && windows[i] + 32 < max_kv_len) ? windows[i] + 32 : max_kv_len;
-      units += (long long)b.n_agents * y.Hkv * ((span + 31) / 32 + 1);
+      units += (long long)b.n_agents * P.Hkv * ((span + 31) / 32 + 1);
     }
   }
   P.max_blocks = b.max_blocks; P.len_cap = max_kv_len; P.tables = b.block_tables; P.kv_lens = kv_lens;
@@ -1533,15 +1370,12 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   P.tickets = (int32_t*)ws; P.partials = (float*)((uint8_t*)ws + kWorkspaceHeaderBytes);
   P.out = out; P.out_dtype = out_dtype; P.lse = lse; P.flags = flags;
   P.k_new = (const uint16_t*)k_new; P.v_new = (const uint16_t*)v_new;
-  const int n_sm = sm_count();
-  const int grid = (int)(units < n_sm ? (units < 1 ? 1 : units) : n_sm);
-  if (y.sb_bf16)
-    return y.G == 2   ? launch_g<2, Q4KV_DECODE_WARPS_D128, true>(P, grid, true, st)
-           : y.G == 3 ? launch_g<3, Q4KV_DECODE_WARPS_D128, true>(P, grid, true, st)
-                      : launch_g<4, Q4KV_DECODE_WARPS_D256, true>(P, grid, true, st);
-  return y.G == 2   ? launch_g<2, Q4KV_DECODE_WARPS_D128, false>(P, grid, true, st)
-         : y.G == 3 ? launch_g<3, Q4KV_DECODE_WARPS_D128, false>(P, grid, true, st)
-                    : launch_g<4, Q4KV_DECODE_WARPS_D256, false>(P, grid, true, st);
+  const long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
+  const int nw = warps_of(y.G);
+  const long long wanted = (units + nw - 1) / nw;        // a chunk per warp at least
+  const int grid = (int)(wanted < slots ? (wanted < 1 ? 1 : wanted) : slots);
+  if (y.G == 2) return P.n_rep > 4 ? launch_gh<2, 8>(P, grid, st) : launch_gh<2, 4>(P, grid, st);
+  return y.G == 3 ? launch_gh<3, 4>(P, grid, st) : launch_gh<4, 4>(P, grid, st);
 }
 
 }  // namespace q4kv

@@ -163,7 +163,8 @@ int q4kv_append_decode_attention(const q4kv_spec* spec, void* pool, int32_t n_bl
                                             (cudaStream_t)stream, k_new, !tiles_allowed(spec, softmax_scale));
     return e == cudaSuccess ? Q4KV_OK : Q4KV_ECUDA;
   }
-  if (!decode_mma_supported(y) || !decode_mma_fits(y, batch->n_agents, batch->max_blocks)) return Q4KV_EUNSUPPORTED;
+  if (!decode_mma_supported(y) || y.n_rep > 4 || !decode_mma_fits(y, batch->n_agents, batch->max_blocks))
+    return Q4KV_EUNSUPPORTED;
   if (workspace_bytes < workspace_need(y, batch->n_agents, max_kv_len, 0)) return Q4KV_EWORKSPACE;
   const cudaError_t e = launch_decode_mma(y, pool, n_blocks, layer, *batch, kv_lens, max_kv_len, &window, 1, q, softmax_scale,
                                           out, out_dtype, lse, workspace, status_flags, (cudaStream_t)stream, k_new, v_new);
@@ -173,7 +174,7 @@ int q4kv_append_decode_attention(const q4kv_spec* spec, void* pool, int32_t n_bl
 size_t q4kv_workspace_bytes_layers(const q4kv_spec* spec, int32_t n_agents, int32_t max_kv_len, int32_t layer_count) {
   if (check_spec(spec) != Q4KV_OK || n_agents < 0 || max_kv_len < 0 || layer_count < 1) return 0;
   const Layout y = make_layout(*spec, 1);
-  if (!decode_mma_supported(y)) return 0;
+  if (!decode_mma_supported(y) || y.n_rep > 4) return 0;
   const size_t one = workspace_need(y, n_agents > 0 ? n_agents : 1, max_kv_len > 0 ? max_kv_len : 1, 0);
   const size_t all = kWorkspaceHeaderBytes + decode_mma_workspace_bytes(y, n_agents > 0 ? n_agents : 1, layer_count);
   return all > one ? all : one;
@@ -200,7 +201,8 @@ int q4kv_decode_attention_layers(const q4kv_spec* spec, void* pool, int32_t n_bl
   const int cap = batch->max_blocks * kBlockTokens;
   if (max_kv_len == 0 || max_kv_len > cap) max_kv_len = cap;
   const Layout y = make_layout(*spec, n_blocks);
-  if (!decode_mma_supported(y) || !decode_mma_fits(y, batch->n_agents, batch->max_blocks, layer_count)) return Q4KV_EUNSUPPORTED;
+  if (!decode_mma_supported(y) || y.n_rep > 4 || !decode_mma_fits(y, batch->n_agents, batch->max_blocks, layer_count))
+    return Q4KV_EUNSUPPORTED;
   if (workspace_bytes < kWorkspaceHeaderBytes + decode_mma_workspace_bytes(y, batch->n_agents, layer_count)) return Q4KV_EWORKSPACE;
   const cudaError_t e = launch_decode_mma(y, pool, n_blocks, layer_begin, *batch, kv_lens, max_kv_len, windows, layer_count, q,
                                           softmax_scale, out, out_dtype, lse, workspace, status_flags, (cudaStream_t)stream,

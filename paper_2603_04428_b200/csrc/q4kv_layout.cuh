@@ -132,7 +132,7 @@ cudaError_t launch_attention_generic(const Layout& y, const void* pool, int n_bl
                                      int max_kv_len, int window, const void* q, float scale, void* out,
                                      int out_dtype, float* lse, void* ws, int32_t* flags, cudaStream_t st);
 
-// tensor-core decode path (GQA shapes with d_qk = d_v in {128, 256}, at most 4 query heads per KV head)
+// tensor-core decode path (GQA shapes with d_qk = d_v in {128, 256}, and d_qk 192 with d_v 128)
 bool decode_mma_supported(const Layout& y);
 bool decode_mma_fits(const Layout& y, int n_agents, int max_blocks, int layer_count = 1);
 int sm_count();   // SMs of the current device (148 when no device can be asked)

@@ -46,6 +46,18 @@ __device__ inline GroupScale group_scale(float mn, float mx, bool bf16) {
   return gs;
 }
 
+// code = clamp(rne(fl((x - b) / s))), inv = fl(1 / s), s != 0.  The IEEE division would dominate the quantizer, so the
+// quotient is taken as t * (1/s) with one fused residual correction (within an ulp of the correctly rounded quotient, 1/s
+// being correctly rounded), which rounds to the same integer unless the quotient sits within a few ulps of k + 1/2; only
+// there is the division itself evaluated.
+__device__ inline uint32_t quantize_code(float x, const GroupScale& gs, float inv) {
+  const float t = __fsub_rn(x, gs.bf);
+  float q = __fmul_rn(t, inv);
+  q = __fmaf_rn(__fmaf_rn(-gs.sf, q, t), inv, q);
+  if (fabsf(q - (floorf(q) + 0.5f)) < 1e-5f) q = __fdiv_rn(t, gs.sf);
+  return (uint32_t)min(max(__float2int_rn(q), 0), 15);
+}
+
 // A (scale, bias) pair of the cache as two binary32 numbers.
 template <bool kBf16>
 __device__ __forceinline__ float2 sb_to_f2(uint32_t u) {
@@ -64,24 +76,11 @@ __device__ inline QuantOut quantize_eight(const float x[8], bool bf16) {
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
   const GroupScale gs = group_scale(mn, mx, bf16);
-  const float bf = gs.bf, sf = gs.sf;
   uint32_t w = 0;
-  if (sf != 0.0f) {
-    // code = clamp(rne(fl((x - b) / s))).  The eight IEEE divisions dominate this function, so the quotient is
-    // taken as t * (1/s) with one fused residual correction (within an ulp of the correctly rounded quotient,
-    // 1/s being correctly rounded), which rounds to the same integer unless the quotient sits within a few ulps
-    // of k + 1/2; only there is the division itself evaluated.
-    const float inv = __frcp_rn(sf);
+  if (gs.sf != 0.0f) {
+    const float inv = __frcp_rn(gs.sf);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float t = __fsub_rn(x[i], bf);
-      float q = __fmul_rn(t, inv);
-      q = __fmaf_rn(__fmaf_rn(-sf, q, t), inv, q);
-      if (fabsf(q - (floorf(q) + 0.5f)) < 1e-5f) q = __fdiv_rn(t, sf);
-      int c = __float2int_rn(q);
-      c = min(max(c, 0), 15);
-      w |= (uint32_t)c << (4 * i);
-    }
+    for (int i = 0; i < 8; ++i) w |= quantize_code(x[i], gs, inv) << (4 * i);
   }
   QuantOut o;
   o.word = w;

@@ -516,6 +516,26 @@ def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("spec_args,lens,window", [
+    ((1, 10, 2, 128, 128, False), [700, 0, 33], 0),          # five query heads per KV head: three columns stay empty
+    ((1, 16, 2, 128, 128, False), [1, 31, 32, 257, 3000], 0),
+    ((1, 16, 2, 128, 128, False), [1, 31, 32, 257, 3000], 100),
+    ((1, 24, 2, 128, 128, False), [513, 40], 0),             # twelve: two sets of six
+    ((1, 16, 2, 256, 256, False), [300, 64, 2000], 0),       # eight at d = 256: two sets of four
+    ((1, 7, 1, 192, 128, False), [300, 65], 0),              # seven at d_qk 192: no set of two to four divides it
+])
+@pytest.mark.parametrize("sb_dtype", [0, 1])
+def test_decode_more_than_four_query_heads_per_kv_head(H, spec_args, lens, window, sb_dtype):
+    p = Pair(H, spec_args, lens, seed=46, sb_dtype=sb_dtype).fill()
+    q = p.q(7, len(lens))
+    scale = 1.0 / math.sqrt(spec_args[3])
+    out, lse = p.dc.decode(0, lens, window, q, scale)
+    ref, rlse = O.decode_attention(p.opool, 0, p.tabs, lens, window, f32(q), scale)
+    assert_attention_close(out.cpu().numpy(), ref, "decode")
+    assert_lse_close(lse.cpu().numpy(), rlse)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("window", [0, 150])
 def test_decode_latent_cache_at_a_sharp_scale_takes_the_exact_kernel(H, window):
     """scale^2 * d_qk > 4 on the V-aliasing cache: routed to the kernel that keeps the values exact."""
