@@ -1,0 +1,466 @@
+// q4kv_prefill_attention on the MLA-latent cache in absorbed form (V aliasing K, d_qk 576, d_v 512): the queries of a new
+// phase over the cached latents plus the causal new tokens, read from the Q4 cache in place (Sections 3.4, 3.5, 3.6).
+//
+// A dense contraction (1088 multiply-adds per query head and key), so it runs on the fifth-generation tensor cores.  Every
+// key is key and value of all the heads, which decides the shape:
+//   * A 128-row tile (128 / n_rep consecutive queries x the n_rep heads) has a 512-column accumulator, which is all of the
+//     tensor memory.  So two CTAs share a tile: both take the scores over all 576 dims, each accumulates 256 of the 512 value
+//     dims (832 instead of 544 multiply-adds per head, key and CTA: the price of not exchanging scores between SMs).
+//     Tensor memory: O 256 columns, S 2 x 64, and the first 256 dims of the queries as packed binary16 (128); the other 320
+//     dims of the queries are 80 KB of shared memory.
+//   * Keys are walked 64 at a time.  Eight "dequantize" warps load a block's codes straight into registers, one block
+//     ahead (the raw bytes would not fit beside the tiles, and each is used once), and write the binary16 tile K^ [64
+//     keys][576 dims] (72 KB, two stages): x^ = c * s + b in one binary16 fma per pair of codes, one rounding per value.
+//     The tile is the K-major B operand of the score product and, read the other way (MN-major), the B operand of the value
+//     product: values are never written.  A packed word is one 16-byte row of a core matrix, elements in the order
+//     0,4,1,5,2,6,3,7; the queries are stored in that order and the output columns are put back in place at the end.
+//   * One thread issues the MMAs: S_b = Q K^T (M 128, N 64: 16 instructions with the queries in tensor memory at 33 clocks, 20
+//     with them in shared memory at 55) and O += P_b V^ (M 128, N 256: 4 at 129): 2140 clocks of tensor pipe per block.
+//   * Eight softmax warps, two threads per score row, as in the one-tile kernel: two score buffers, lazily updated reference
+//     maximum, P_b as packed binary16 over S_b.
+//   * With few tiles the keys of a tile are cut over several CTAs as well (plan_prefill_splits); these leave (acc, m, l)
+//     records that merge_prefill_kernel combines.
+// Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads: see launch_prefill_mla.
+// All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises Q4KV_FLAG_INTERNAL, drains the tensor
+// pipe and frees the tensor memory before the CTA returns.
+#include "prefill_common.cuh"
+
+namespace q4kv {
+
+namespace {
+
+using namespace tc;
+using namespace prefill;
+
+constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
+constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps;
+constexpr int kThreads = (kMmaWarp + 1) * 32;            // 544
+constexpr int kStages = 2;
+constexpr int kG = 9, kD = 576, kDv = 512, kDvCta = 256;
+constexpr int kQTmem = 256, kQSmem = kD - kQTmem;        // query dims in tensor memory and in shared memory
+constexpr int kSboK = (kD / 8) * 128, kSboQ = (kQSmem / 8) * 128;
+constexpr int kChunkBytes = 32 * (kD / 2 + 4 * kG);      // [Kc 9216 | Ksb 1152]
+constexpr uint32_t kColO = 0, kColS = 256, kColQ = 384;
+
+struct MlaPrefillParams {
+  Layout y;
+  const uint8_t* pool;
+  int n_blocks, layer, n_agents, max_blocks;
+  const int32_t* tables;
+  const int32_t* kv_lens;
+  const int32_t* q_offs;
+  int window;
+  const uint16_t* q;          // bf16 [total_q][Hq][576]
+  float scale_log2;
+  void* out;
+  int out_dtype;
+  float* lse;
+  int32_t* flags;
+  int n_splits;
+  float* records;             // n_splits > 1: [total_q][Hq][n_splits][kRecord]
+};
+
+struct MlaSmem {
+  alignas(128) uint8_t khat[kStages][64 * kD * 2];       // [key][dim]: (n%8)*16 + (n/8)*kSboK + (k/8)*128
+  alignas(128) uint8_t qs[128 * kQSmem * 2];             // [row][dim - 256]: (m%8)*16 + (m/8)*kSboQ + (k/8)*128
+  alignas(8) uint64_t k_full[kStages], k_free[kStages], s_full[2], p_full[2], o_done, q_ready, drain;
+  uint32_t tmem_base;
+  float xchg[2][2][128];                                 // [parity][column half][row]: maxima / sums of the two threads of a row
+  int stop[3], spoiled;
+  int abort_flag, poisoned;
+};
+
+template <bool kBf>
+__global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_constant__ MlaPrefillParams P) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  MlaSmem& sm = *reinterpret_cast<MlaSmem*>(smem_raw);
+
+  const Layout& y = P.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n_rep = y.n_rep;
+  // grid: x = (tile, value half), y = (KV head, split), z = agent
+  const int qt = blockIdx.x >> 1, hv = blockIdx.x & 1, hk = blockIdx.y / P.n_splits, split = blockIdx.y % P.n_splits, a = blockIdx.z;
+  const int tile_q = 128 / n_rep;                        // queries of the CTA's 128-row tile
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // ---- this CTA's queries and key range (inputs no kernel writes) ----
+  const int q0 = P.q_offs[a], q_len = P.q_offs[a + 1] - q0;
+  const int kv_len = P.kv_lens[a];
+  const int i_min = qt * tile_q;
+  if (i_min >= q_len) return;                            // uniform: nothing allocated, no barrier passed
+  const bool bad_len = kv_len < 0 || kv_len > P.max_blocks * kBlockTokens || q_len > kv_len;
+  const int i_max = min(q_len, i_min + tile_q) - 1;
+  const int prefix = kv_len - q_len;                     // query i sits at position prefix + i
+  const int W = P.window;
+  const int c_end = bad_len ? 0 : (prefix + i_max) / 32 + 1;
+  const int c_begin = (bad_len || W == 0) ? 0 : max(0, prefix + i_min - W + 1) >> 5;
+  const int all0 = c_begin >> 1, n_all = max(0, ((c_end + 1) >> 1) - all0);
+  const int it0 = all0 + n_all * split / P.n_splits;     // 64-key blocks it0 .. it0 + n_iter - 1
+  const int n_iter = all0 + n_all * (split + 1) / P.n_splits - it0;
+
+  if (threadIdx.x == 0) {
+    if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
+    for (int s = 0; s < kStages; ++s) { mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.k_free[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&sm.s_full[b], 1); mbar_init(&sm.p_full[b], kSoftmaxWarps * 32); }
+    mbar_init(&sm.o_done, 1);
+    mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
+    for (int i = 0; i < 3; ++i) sm.stop[i] = 0;
+    sm.spoiled = 0;
+    mbar_init(&sm.drain, 1);
+    sm.abort_flag = 0; sm.poisoned = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  if (warp == kMmaWarp) { tmem_alloc(&sm.tmem_base, 512); tmem_relinquish(); }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tb = sm.tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // the new tokens were appended by the preceding kernel
+  volatile int* abort_flag = &sm.abort_flag;
+
+  if (warp >= kSoftmaxWarps && warp < kMmaWarp) {
+    // =============================== dequantize warps ==========================================
+    // Thread (chunk c1 of the block, token tau = 4 kg + ki, kt): the words 4 p + kt, p = 0..17, of its token (four 16-byte
+    // pieces and an 8-byte one) and the token's nine (scale, bias) pairs.  A lane group of eight holds the eight tokens of
+    // a core matrix at one kt: its stores fill a 128-byte line, its loads are two pieces of each of four lines.
+    const int x = threadIdx.x - kSoftmaxWarps * 32;      // 0..255
+    const int c1 = x >> 7, kt = (x >> 3) & 3, ki = x & 3, kg = 2 * ((x >> 5) & 3) + ((x >> 2) & 1);
+    const int ktau = 4 * kg + ki;
+    const int read16 = ki * (256 * kG) + kg * 64 + kt * 16, read8 = ki * (256 * kG) + 2048 + kg * 32 + kt * 8;
+    const int read_sb = 1024 * kG + (((ktau & 3) * 4 + (ktau >> 3)) * 2 + ((ktau >> 2) & 1)) * (4 * kG);
+    const int n = c1 * 32 + ktau;
+    const int write = (n & 7) * 16 + (n >> 3) * kSboK + kt * 128;         // + p * 512
+    uint4 w16[4];
+    uint2 w8;
+    uint32_t sb[kG];
+    auto fetch = [&](int j) {                            // this thread's part of block it0 + j (bytes past the end: zeros)
+      const int c = 2 * (it0 + j) + c1;
+      const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
+      const bool bad = blk < 0 || blk >= P.n_blocks;
+      if (bad && lane == 0) { sm.poisoned = 1; raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK); }
+      if (bad || c * 32 + ktau >= kv_len) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w16[i] = make_uint4(0u, 0u, 0u, 0u);
+        w8 = make_uint2(0u, 0u);
+#pragma unroll
+        for (int i = 0; i < kG; ++i) sb[i] = 0u;
+        return;
+      }
+      const uint8_t* chunk = head_block(P.pool, y, P.layer, blk, hk) + (size_t)(c & 7) * kChunkBytes;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w16[i] = __ldcg(reinterpret_cast<const uint4*>(chunk + read16 + 512 * i));
+      w8 = __ldcg(reinterpret_cast<const uint2*>(chunk + read8));
+#pragma unroll
+      for (int i = 0; i < kG; ++i) sb[i] = *reinterpret_cast<const volatile uint32_t*>(chunk + read_sb + 4 * i);
+    };
+    if (n_iter > 0) fetch(0);
+    for (int j = 0; j < n_iter; ++j) {
+      const int s = j % kStages;
+      if (j >= kStages && !mbar_wait(&sm.k_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
+      if (kBf) {
+        bool overflow = false;
+#pragma unroll
+        for (int i = 0; i < kG; ++i) sb[i] = bf16_pair_to_h2(sb[i], overflow);
+        if (overflow) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
+      }
+      uint8_t* dst = sm.khat[s] + write;
+#pragma unroll
+      for (int p = 0; p < 18; ++p) {
+        const uint4& v = w16[(p >> 2) & 3];
+        const uint32_t w = p >= 16 ? (p == 16 ? w8.x : w8.y) : (p & 3) == 0 ? v.x : (p & 3) == 1 ? v.y : (p & 3) == 2 ? v.z : v.w;
+        const uint32_t sp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x1010), bp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x3232);
+        *reinterpret_cast<uint4*>(dst + p * 512) = dequant8(w, sp, bp, sp, bp, sp, bp, sp, bp);
+      }
+      if (j + 1 < n_iter) fetch(j + 1);
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.k_full[s]);
+    }
+  } else if (warp == kMmaWarp) {
+    // =============================== MMA issue ==================================================
+    // The whole warp runs this code, so that operands are computed once for the warp, and one elected
+    // lane (always the same) issues the MMAs and the commits.
+    if (n_iter > 0) {
+      constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, kDvCta, 0, 1);
+      const uint64_t qd = smem_desc(smem_u32(sm.qs), 128, kSboQ);
+      auto issue_qk = [&](int b, int s) {                // S_b = Q K^T
+        const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, kSboK);
+#pragma unroll
+        for (int k = 0; k < kQTmem / 16; ++k)
+          if (elect_one()) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, k > 0);
+#pragma unroll
+        for (int k = 0; k < kQSmem / 16; ++k)
+          if (elect_one()) mma_f16_ss(tb + kColS + 64 * b, qd + 16 * k, kd + 16 * (kQTmem / 16 + k), kIdescS, 1u);
+        if (elect_one()) commit(&sm.s_full[b]);
+      };
+      auto issue_pv = [&](int b, int s, bool first) {    // O (+)= P_b V^; afterwards the stage is free
+        const uint64_t vd = smem_desc(smem_u32(sm.khat[s]) + hv * (kDvCta / 8) * 128, kSboK, 128);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (elect_one()) mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + (2 * kSboK / 16) * k, kIdescO, (!first || k > 0) ? 1u : 0u);
+        if (elect_one()) { commit(&sm.o_done); commit(&sm.k_free[s]); }
+      };
+      bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        fence_after_sync();
+        issue_qk(0, 0);
+      }
+      for (int j = 0; ok && j < n_iter; ++j) {
+        if (j + 1 < n_iter) {                            // the next block's scores before this block's values
+          const int s1 = (j + 1) % kStages;
+          ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s1], (uint32_t)((j + 1) / kStages), abort_flag));
+          if (!ok) break;
+          fence_after_sync();
+          issue_qk((j + 1) & 1, s1);                     // S of block j - 1 (as P) was read by the product issued before it
+        }
+        ok = __all_sync(0xffffffffu, mbar_wait(&sm.p_full[j & 1], (uint32_t)(j >> 1), abort_flag));
+        if (!ok) break;
+        fence_after_sync();
+        issue_pv(j & 1, j % kStages, j == 0);
+      }
+    }
+  } else if (warp < kSoftmaxWarps) {
+    // =============================== softmax warps: two threads per score row ===================
+    // Warp w: column half = w / 4, tensor-memory lanes 32 (w % 4) ...  The two threads of a row exchange their block
+    // maxima (and at the end their sums) through shared memory; the 256 threads meet at a named barrier once per
+    // block, and they leave the loop together (one of them samples the give-up flag before the barrier).
+    const int half = (warp >> 2) & 1;
+    const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
+    const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
+    const int h = row / tile_q, i = i_min + row % tile_q;
+    const bool mine = i < q_len && h < n_rep;            // a row of the output
+    const bool valid = mine && !bad_len;
+    const int pq = prefix + i;                           // this row's position
+    const bool sampler = warp == 0 && lane == 0;
+    auto tile_barrier = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
+    float kappa;                                         // score in log2 units = S * kappa
+    {
+      // ---- stage the query row: bf16 -> binary16 times a power of two; pieces of eight dims 0..31 go to tensor memory
+      //      (sixteen by each thread of the row), 32..71 to shared memory (twenty by each) ----
+      const uint16_t* qrow = P.q + (valid ? row_index : 0) * kD;
+      const int p0 = 16 * half, p1 = 32 + 20 * half;
+      float mx = 0.f;
+      if (valid) {
+#pragma unroll 4
+        for (int p = 0; p < 36; ++p) mx = fmaxf(mx, max_abs8(*reinterpret_cast<const uint4*>(qrow + 8 * (p < 16 ? p0 + p : p1 + p - 16))));
+      }
+      sm.xchg[1][half][row] = mx;                        // slot 1: block 0 of the loop below writes slot 0
+      tile_barrier();
+      mx = fmaxf(mx, sm.xchg[1][half ^ 1][row]);
+      int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
+      if (mx == 0.f) ex = 0;
+      ex = min(max(ex, -100), 100);
+      const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
+      kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
+      const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+      for (int c = 0; c < 2; ++c) {                      // 32 columns (64 dims) at a time
+        uint32_t qa[32];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * (p0 + 8 * c + p)) : zero4, sf);
+          qa[4 * p] = v.x; qa[4 * p + 1] = v.y; qa[4 * p + 2] = v.z; qa[4 * p + 3] = v.w;
+        }
+        tmem_st32(lane_addr + kColQ + 64 * half + 32 * c, qa);
+      }
+#pragma unroll 4
+      for (int p = p1; p < p1 + 20; ++p) {
+        const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : zero4, sf);
+        *reinterpret_cast<uint4*>(sm.qs + (row & 7) * 16 + (row >> 3) * kSboQ + (p - 32) * 128) = v;
+      }
+      wait_st();
+      fence_async_smem();
+      fence_before_sync();
+      mbar_arrive(&sm.q_ready);
+    }
+    float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most kLazy
+    for (int j = 0; j < n_iter; ++j) {
+      const int b = j & 1;
+      mbar_wait(&sm.s_full[b], (uint32_t)(j >> 1), abort_flag);   // a wait that runs out raises the give-up flag; all leave below
+      fence_after_sync();
+      uint32_t sr[32];
+      tmem_ld32(lane_addr + kColS + 64 * b + 32 * half, sr);
+      wait_ld();
+      const int pos0 = (it0 + j) * 64 + 32 * half;
+      // column c of this half is key pos0 + c; causal and window masks on edge blocks only
+      if (pos0 + 31 > pq || (W > 0 && pos0 <= pq - W)) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+          if (pos0 + c > pq || (W > 0 && pos0 + c <= pq - W)) sr[c] = 0xff800000u;   // -inf
+      }
+      // Probabilities against the current reference, and the block maximum beside them (independent instruction
+      // streams); only when some row's maximum has outgrown its reference is the reference moved, the accumulator
+      // rescaled and the probabilities taken again.  The scores stay in registers meanwhile.
+      float sum = 0.f;
+      uint32_t pr[16];
+      auto probabilities = [&](float neg_m) {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+        for (int c = 0; c < 16; c += 2) {
+          const float p0 = fast_exp2(fmaf(__uint_as_float(sr[2 * c]), kappa, neg_m));
+          const float p1 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 1]), kappa, neg_m));
+          const float p2 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 2]), kappa, neg_m));
+          const float p3 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 3]), kappa, neg_m));
+          s0 += p0; s1 += p1; s2 += p2; s3 += p3;
+          pr[c] = f32x2_to_h2(p0, p1);
+          pr[c + 1] = f32x2_to_h2(p2, p3);
+        }
+        sum = (s0 + s1) + (s2 + s3);
+      };
+      probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
+      float cm4[4] = {__uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2]), __uint_as_float(sr[3])};
+#pragma unroll
+      for (int c = 4; c < 32; ++c) cm4[c & 3] = fmaxf(cm4[c & 3], __uint_as_float(sr[c]));
+      float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
+      sm.xchg[j & 1][half][row] = cm;
+      if (sampler) sm.stop[j % 3] = *abort_flag;
+      tile_barrier();                                    // also: every score of the block has been read (P overlays S)
+      if (sm.stop[j % 3]) break;
+      cm = fmaxf(cm, sm.xchg[j & 1][half ^ 1][row]);
+      if (cm != -INFINITY) cm *= kappa;                  // kappa > 0
+      const float m_new = fmaxf(m_ref, cm);
+      const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
+      if (__any_sync(0xffffffffu, grow)) {
+        if (j > 0) {
+          // rescale this thread's half of the accumulator row: the previous block's value product must have landed
+          mbar_wait(&sm.o_done, (uint32_t)(j - 1), abort_flag);
+          fence_after_sync();
+          const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;           // m_ref = -inf: 0
+#pragma unroll 1
+          for (int part = 0; part < kDvCta / 64; ++part) {
+            uint32_t orow[32];
+            tmem_ld32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+            wait_ld();
+#pragma unroll
+            for (int c = 0; c < 32; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
+            tmem_st32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+          }
+          if (grow) l *= f;
+        }
+        if (grow) m_ref = m_new;
+        probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
+      }
+      l += sum;
+      tmem_st16(lane_addr + kColS + 64 * b + 16 * half, pr);   // P_b overlays the first 32 columns of S_b
+      wait_st();
+      fence_before_sync();
+      mbar_arrive(&sm.p_full[b]);
+    }
+    // ---- normalise and write this thread's half of the row, or leave it as a record ----
+    bool ok = !*abort_flag;
+    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_done, (uint32_t)(n_iter - 1), abort_flag);
+    const int slot = n_iter & 1;                         // not the slot the last block used
+    sm.xchg[slot][half][row] = l;
+    if (!ok) sm.spoiled = 1;                             // anyone who gave up spoils the tile
+    tile_barrier();
+    ok = sm.spoiled == 0;                                // uniform over the tile: the loads below are warp-wide
+    l += sm.xchg[slot][half ^ 1][row];
+    if (ok) fence_after_sync();
+    const bool bad = !ok || sm.poisoned != 0;
+    const bool zero = bad || n_iter == 0 || l <= 0.f;
+    const bool final = P.n_splits == 1;
+    const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
+    float* rec = final ? nullptr : P.records + (row_index * P.n_splits + split) * prefill_record(kDv);
+#pragma unroll 1
+    for (int part = 0; part < kDvCta / 64; ++part) {
+      uint32_t orow[32];
+      if (ok && n_iter > 0) {
+        tmem_ld32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+        wait_ld();
+      }
+      if (!mine) continue;
+      const int d0 = kDvCta * hv + (kDvCta / 2) * half + 32 * part;
+      // slot j of every eight columns is value dim elem_of(j)
+      if (final && P.out_dtype == Q4KV_OUT_BF16) {
+        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + row_index * kDv + d0;
+#pragma unroll
+        for (int c = 0; c < 32; c += 8) {
+          uint4 v;
+          uint32_t* vv = reinterpret_cast<uint32_t*>(&v);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 bb = __floats2bfloat162_rn(zero ? 0.f : __uint_as_float(orow[c + slot_of(2 * e)]) * inv,
+                                                            zero ? 0.f : __uint_as_float(orow[c + slot_of(2 * e + 1)]) * inv);
+            vv[e] = *reinterpret_cast<const uint32_t*>(&bb);
+          }
+          *reinterpret_cast<uint4*>(o + c) = v;
+        }
+      } else {
+        float* o = (final ? reinterpret_cast<float*>(P.out) + row_index * kDv : rec) + d0;
+#pragma unroll
+        for (int c = 0; c < 32; c += 4)
+          *reinterpret_cast<float4*>(o + c) =
+              zero ? make_float4(0.f, 0.f, 0.f, 0.f)
+                   : make_float4(__uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 0)]) * inv, __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 1)]) * inv,
+                                 __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 2)]) * inv, __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 3)]) * inv);
+      }
+    }
+    if (half == 0 && hv == 0 && mine) {
+      if (!final) *reinterpret_cast<float2*>(rec + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
+      else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
+    }
+  }
+
+  // ---- teardown: nothing may be in flight in the tensor pipe when the columns are given back ----
+  fence_before_sync();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    if (sm.abort_flag) {
+      if (elect_one()) {                                 // the lane that issued the MMAs
+        commit(&sm.drain);
+        for (uint32_t k = 0; k < kSpinLimit && !mbar_try_wait(&sm.drain, 0); ++k) {}
+        raise_flag(P.flags, Q4KV_FLAG_INTERNAL);
+      }
+      __syncwarp();
+    }
+    fence_after_sync();
+    tmem_dealloc(tb, 512);
+  }
+}
+
+}  // namespace
+
+bool prefill_mla_supported(const Layout& y) { return y.alias && y.D == kD && y.Dv == kDv && y.n_rep <= 128; }
+
+cudaError_t launch_prefill_mla(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
+                               const int32_t* kv_lens, const int32_t* q_offs, int total_q, int max_q_len, int max_kv_len,
+                               int window, const void* q, float scale, void* out, int out_dtype, float* lse, void* ws,
+                               size_t ws_bytes, int32_t* flags, cudaStream_t st) {
+  if (b.n_agents <= 0 || max_q_len <= 0) return cudaSuccess;
+  MlaPrefillParams P;
+  P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents;
+  P.max_blocks = b.max_blocks; P.tables = b.block_tables; P.kv_lens = kv_lens; P.q_offs = q_offs; P.window = window;
+  P.q = (const uint16_t*)q; P.scale_log2 = scale * kLog2e; P.out = out; P.out_dtype = out_dtype; P.lse = lse; P.flags = flags;
+  const int tile_q = 128 / y.n_rep;
+  P.n_splits = plan_prefill_splits(y, tile_q, 2, b.n_agents, total_q, max_q_len, max_kv_len, window, ws_bytes);
+  P.records = (float*)ws;
+  static bool configured[64][2] = {};
+  const int bf = y.sb_bf16 ? 1 : 0;
+  void (*kernel)(const MlaPrefillParams) = bf ? prefill_mla_kernel<true> : prefill_mla_kernel<false>;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !configured[dev][bf]) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlaSmem));
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) configured[dev][bf] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * ((max_q_len + tile_q - 1) / tile_q), y.Hkv * P.n_splits, b.n_agents);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sizeof(MlaSmem);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, kernel, P);
+  if (e != cudaSuccess || P.n_splits == 1) return e;
+  return launch_merge_prefill(y, total_q, P.n_splits, P.records, out, out_dtype, lse, st);
+}
+
+}  // namespace q4kv

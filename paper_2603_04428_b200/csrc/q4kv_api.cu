@@ -28,7 +28,7 @@ int check_batch(const q4kv_batch* b) {
 // Every decode kernel keeps its partial records behind a header of fixed size (the arrival counters
 // of the kernels that merge in the same launch), so that one workspace serves any sequence of calls.
 size_t workspace_need(const Layout& y, int n_agents, int max_kv_len, int total_q) {
-  if (total_q > 0) return 16;   // the prefill path keeps no partials
+  if (total_q > 0) return 16;   // the prefill kernels need none; what they make use of is prefill_workspace
   const DecodePlan p = plan_decode(y, n_agents, max_kv_len, 0);
   size_t need = (size_t)n_agents * y.Hq * p.n_splits * (y.Dv + 2) * sizeof(float) + 16;
   if (decode_mla_supported(y)) {
@@ -40,6 +40,15 @@ size_t workspace_need(const Layout& y, int n_agents, int max_kv_len, int total_q
     if (mma > need) need = mma;
   }
   return kWorkspaceHeaderBytes + need;
+}
+
+// What a prefill call can make use of: records of the query tiles whose keys it cuts into parts.  The call makes do with
+// less (fewer parts), so this size is not a condition.
+size_t prefill_workspace(const Layout& y, int n_agents, int max_kv_len, int total_q) {
+  int splits = 1;
+  if (prefill_mla_supported(y))
+    splits = plan_prefill_splits(y, 128 / y.n_rep, 2, n_agents, total_q, total_q, max_kv_len, 0, (size_t)-1);
+  return splits > 1 ? prefill_record_bytes(y, total_q, splits) : 16;
 }
 
 // The kernels that expand the cache into binary16 tiles round each dequantized element once; they are taken only when
@@ -82,7 +91,9 @@ size_t q4kv_packed_bytes(const q4kv_spec* spec, int32_t n_tokens) {
 size_t q4kv_workspace_bytes(const q4kv_spec* spec, int32_t n_agents, int32_t max_kv_len, int32_t total_q) {
   if (check_spec(spec) != Q4KV_OK || n_agents < 0 || max_kv_len < 0 || total_q < 0) return 0;
   const Layout y = make_layout(*spec, 1);
-  return workspace_need(y, n_agents > 0 ? n_agents : 1, max_kv_len > 0 ? max_kv_len : 1, total_q);
+  if (n_agents == 0) n_agents = 1;
+  if (max_kv_len == 0) max_kv_len = 1;
+  return total_q > 0 ? prefill_workspace(y, n_agents, max_kv_len, total_q) : workspace_need(y, n_agents, max_kv_len, 0);
 }
 
 int q4kv_quantize_append(const q4kv_spec* spec, void* pool, int32_t n_blocks, int32_t layer,
@@ -239,6 +250,9 @@ int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_bl
   else if (prefill_umma_1tile_supported(y) && tiles_allowed(spec, softmax_scale))
     e = launch_prefill_umma_1tile(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale,
                                   out, out_dtype, lse, status_flags, (cudaStream_t)stream);
+  else if (prefill_mla_supported(y) && tiles_allowed(spec, softmax_scale))
+    e = launch_prefill_mla(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, total_q, max_q_len, max_kv_len, window, q,
+                           softmax_scale, out, out_dtype, lse, workspace, workspace_bytes, status_flags, (cudaStream_t)stream);
   else if (prefill_mma_supported(y))
     e = launch_prefill_mma(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale, out,
                            out_dtype, lse, status_flags, (cudaStream_t)stream);

@@ -163,6 +163,24 @@ cudaError_t launch_prefill_umma_1tile(const Layout& y, const void* pool, int n_b
                                    const void* q, float scale, void* out, int out_dtype, float* lse, int32_t* flags,
                                    cudaStream_t st);
 
+// tcgen05 prefill path for the MLA-latent cache (V aliasing K, d_qk 576, d_v 512)
+bool prefill_mla_supported(const Layout& y);
+cudaError_t launch_prefill_mla(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
+                               const int32_t* kv_lens, const int32_t* q_offs, int total_q, int max_q_len, int max_kv_len,
+                               int window, const void* q, float scale, void* out, int out_dtype, float* lse, void* ws,
+                               size_t ws_bytes, int32_t* flags, cudaStream_t st);
+// Prefill launches that cut the keys of a query tile into parts: their number (at most what fits ws_bytes), and the
+// combination of the records [total_q][Hq][n_splits][acc, m, l, pad]
+constexpr int kMaxPrefillSplits = 16;
+__host__ __device__ constexpr int prefill_record(int Dv) { return Dv + 4; }
+inline size_t prefill_record_bytes(const Layout& y, int total_q, int n_splits) {
+  return (size_t)total_q * y.Hq * n_splits * prefill_record(y.Dv) * sizeof(float);
+}
+int plan_prefill_splits(const Layout& y, int tile_q, int per_tile, int n_agents, int total_q, int max_q_len, int max_kv_len,
+                        int window, size_t ws_bytes);
+cudaError_t launch_merge_prefill(const Layout& y, int total_q, int n_splits, const float* records, void* out, int out_dtype,
+                                 float* lse, cudaStream_t st);
+
 // Decode on the MLA-latent cache (d_qk 576, d_v 512 aliasing K, one KV head, at most 16 query heads): a key-split
 // attention kernel -- on a binary16 tile of the dequantized keys, or, with on_codes, on the 4-bit codes themselves
 // (exact products) -- followed by the combination of the records.
