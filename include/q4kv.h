@@ -120,8 +120,8 @@ enum { Q4KV_OUT_F32 = 0, Q4KV_OUT_BF16 = 1 };
  *     at most 2e-5 * M + 1e-5, i.e. within 2e-3 for any cache with M <= 64.  (An absolute bound:
  *     the tensor-core kernels carry probability x scale in binary16, so contributions of groups
  *     whose scale is below 2^-24 vanish; only bfloat16 caches can hold such scales.)
- *   - Kernels that expand the cache into binary16 tiles (prefill with d_qk = d_v in {128, 256} or d_qk 192 / d_v 128 and 1, 2 or 4
- *     query heads per KV head; decode on the MLA-latent cache: V aliasing K, d_qk 576, d_v 512, one
+ *   - Kernels that expand the cache into binary16 tiles (prefill with d_qk = d_v in {128, 256}, d_qk 192 / d_v 128 or, V
+ *     aliasing K, d_qk 576 / d_v 512; decode on the MLA-latent cache: V aliasing K, d_qk 576, d_v 512, one
  *     KV head, at most 16 query heads) round every dequantized value once to binary16, a relative
  *     error of 2^-11 at most, and the probabilities likewise.  They are chosen only when
  *     exact_products == 0 and softmax_scale <= 2/sqrt(d_qk).  Their error is at most
@@ -271,7 +271,9 @@ int q4kv_decode_attention_static(const q4kv_spec* spec, const void* pool, int32_
  *                  (and j > position - window when window > 0)
  *   total_q, max_q_len, max_kv_len   host copies / upper bounds (size the grid)
  *   q bf16 [total_q][n_q_heads][d_qk];  out [total_q][n_q_heads][d_v];  lse optional
- *   workspace  at least q4kv_workspace_bytes(spec, A, max_kv_len, total_q) bytes
+ *   workspace  at least 16 bytes, better q4kv_workspace_bytes(spec, A, max_kv_len, total_q): with that much the call can cut
+ *              the keys of a query tile over several SMs when there are few tiles, and take agents that bring a single
+ *              query (in a batch where others bring more) as a decode step.  Its contents need not be cleared.
  * Accuracy: see "Accuracy of the attention entry points" above (spec->exact_products selects
  * between the binary16-tile kernel and the kernel that multiplies the codes). */
 int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_blocks, int32_t layer,

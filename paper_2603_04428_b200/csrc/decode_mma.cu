@@ -169,6 +169,7 @@ struct DecodeParams {
   int32_t* flags;
   const uint16_t* k_new;      // fused append: bf16 [A][Hkv][D] rows of the token at position kv_len - 1 (null: none)
   const uint16_t* v_new;
+  const int32_t* q_offs;      // prefill batch: attend for the agents with exactly one query, row q_offs[a]; or null
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -183,6 +184,11 @@ __device__ inline AgentRange agent_range(const DecodeParams& P, int a, bool& bad
   const int window = P.windows[li];
   r.n = P.kv_lens[a - li * P.n_real];
   bad = r.n < 0 || r.n > P.len_cap;
+  if (P.q_offs) {
+    const bool one = P.q_offs[a + 1] - P.q_offs[a] == 1;
+    bad = one && (bad || r.n < 1);
+    if (!one) r.n = 0;
+  }
   if (bad) r.n = 0;
   r.lo = window > 0 ? max(0, r.n - window) : 0;
   r.cf = r.lo >> 5;
@@ -342,6 +348,7 @@ struct Segment {
   int a, hk, c0, c1;      // (virtual) agent, head set, logical chunk indices [c0, c1) of the agent
   int ar, li;             // real agent (lengths, block table) and layer of the call (pool layer)
   int n, lo;              // key range of the agent
+  int row;                // query row of the agent
   int cf, nc;             // the pair's whole chunk range
   int k0;                 // running chunk counter of the CTA at c0
   int first, last;        // CTAs that hold the pair's first and last chunk
@@ -352,6 +359,7 @@ __device__ inline void whole_segment(const DecodeParams& P, const RangeStart& rs
   s.li = P.layer_count > 1 ? rs.agent / P.n_real : 0; s.ar = rs.agent - s.li * P.n_real;
   s.a = rs.agent; s.hk = rs.pair; s.c0 = rs.r.cf + (int)rs.u_begin; s.c1 = rs.r.cf + (int)rs.u_end;
   s.n = rs.r.n; s.lo = rs.r.lo; s.cf = rs.r.cf; s.nc = rs.r.nc; s.k0 = 0;
+  s.row = P.q_offs ? P.q_offs[rs.agent] : rs.agent;
   s.first = (int)blockIdx.x - rs.split;
   s.last = s.first + rs.splits - 1;
 }
@@ -384,6 +392,7 @@ struct Walker {
     const int c1 = (uint32_t)(pair_end - c) <= left ? pair_end : c + (int)left;
     s.li = P.layer_count > 1 ? a / P.n_real : 0; s.ar = a - s.li * P.n_real;
     s.a = a; s.hk = hk; s.c0 = c; s.c1 = c1; s.n = r.n; s.lo = r.lo; s.cf = r.cf; s.nc = r.nc; s.k0 = k;
+    s.row = P.q_offs ? P.q_offs[a] : a;
     const int cnt = c1 - c;
     s.first = s.last = 0;
     if (cnt != r.nc) {
@@ -893,7 +902,7 @@ __device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const Dec
   }
   const float L0 = __shfl_sync(0xffffffffu, L, h0), L1 = __shfl_sync(0xffffffffu, L, h0 + 1);
   const int d = H == 4 ? 32 * unit + g + 8 * (tid >> 1) : 16 * unit + g, step = H == 4 ? 16 : 8;
-  const size_t row0 = (size_t)seg.a * P.y.Hq + (size_t)seg.hk * n_rep;
+  const size_t row0 = (size_t)seg.row * P.y.Hq + (size_t)seg.hk * n_rep;
   if (whole) {
     const float i0 = L0 > 0.f ? 1.f / L0 : 0.f, i1 = L1 > 0.f ? 1.f / L1 : 0.f;
     if (h0 < n_rep) { store_out(P, (row0 + h0) * Dv + d, a[0] * i0); store_out(P, (row0 + h0) * Dv + d + step, a[2] * i0); }
@@ -964,11 +973,12 @@ __device__ __forceinline__ void clear_empty_agents(const DecodeParams& P, int fi
 #pragma unroll 1
   for (int a = first; a < P.n_agents; a += step) {
     bool bad_len;
-    if (agent_range(P, a, bad_len).nc > 0) continue;
+    if (agent_range(P, a, bad_len).nc > 0 || (P.q_offs && P.q_offs[a + 1] - P.q_offs[a] != 1)) continue;
+    const size_t row = P.q_offs ? P.q_offs[a] : a;
 #pragma unroll 1
-    for (int i = lane; i < P.y.Hq * Dv; i += 32) store_out(P, (size_t)a * P.y.Hq * Dv + i, 0.f);
+    for (int i = lane; i < P.y.Hq * Dv; i += 32) store_out(P, row * P.y.Hq * Dv + i, 0.f);
 #pragma unroll 1
-    for (int i = lane; i < P.y.Hq && P.lse; i += 32) P.lse[(size_t)a * P.y.Hq + i] = -INFINITY;
+    for (int i = lane; i < P.y.Hq && P.lse; i += 32) P.lse[row * P.y.Hq + i] = -INFINITY;
   }
 }
 
@@ -1013,6 +1023,11 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   const int n_rep = P.n_rep;
 
   grid_launch_dependents();
+  if (P.q_offs) {                                        // a prefill batch need not hold an agent with one query
+    bool any = false;
+    for (int a = threadIdx.x; a < P.n_agents; a += NW * 32) any |= P.q_offs[a + 1] - P.q_offs[a] == 1;
+    if (!__syncthreads_or(any)) return;
+  }
   // ---- this CTA's unit range and its first two segments: one warp, the others set up shared memory (lengths and block
   // tables are inputs that no kernel writes) ----
   if (warp == 0) {
@@ -1077,7 +1092,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   const int g = lane >> 2, tid = lane & 3;
   // this warp's row of a segment's query; the new row's groups are quantized by the warps behind the query's (from 4 on)
   constexpr int kNewWarps = NW - 4, kNewRounds = (G + Gv + kNewWarps - 1) / kNewWarps;
-  auto query_row = [&](const Segment& s) { return P.q + ((size_t)s.a * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
+  auto query_row = [&](const Segment& s) { return P.q + ((size_t)s.row * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
   auto new_pair = [&](const Segment& s, int grp) {
     const size_t head = (size_t)s.a * y.Hkv + s.hk;
     return (grp < G ? P.k_new + head * D + 64 * grp : P.v_new + head * Dv + 64 * (grp - G)) + 2 * lane;
@@ -1231,7 +1246,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
     if (warp == NW - 1 && lane == 0) {
       if (seg.c1 - c0 != seg.nc) {                       // only the first and the last segment can be parts of a pair
         int* f = sm.fin[k0 == 0 ? 0 : 1];
-        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = seg.a * y.Hq + seg.hk * n_rep;
+        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = seg.row * y.Hq + seg.hk * n_rep;
       }
       if (more) sm.walker.next(P, sm.range, sm.seg[(si + 2) % 3]);       // never where the CTA holds one segment
     }
@@ -1339,6 +1354,8 @@ bool decode_mma_fits(const Layout& y, int n_agents, int max_blocks, int layer_co
          v * y.Hkv <= kMaxTicketPairs && (unsigned long long)layer_count * y.layer_bytes < (1ull << 36);
 }
 
+int decode_mma_tickets(const Layout& y, int n_agents) { return n_agents * y.Hkv * head_sets(y); }
+
 // bytes behind the workspace header: one record per (layer, agent, head set) and per CTA of the largest grid
 size_t decode_mma_workspace_bytes(const Layout& y, int n_agents, int layer_count) {
   const int sets = head_sets(y);
@@ -1351,7 +1368,7 @@ size_t decode_mma_workspace_bytes(const Layout& y, int n_agents, int layer_count
 cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
                               const int32_t* kv_lens, int max_kv_len, const int32_t* windows, int layer_count,
                               const void* q, float scale, void* out, int out_dtype, float* lse, void* ws, int32_t* flags,
-                              cudaStream_t st, const void* k_new, const void* v_new) {
+                              cudaStream_t st, const void* k_new, const void* v_new, const int32_t* q_offs, int32_t* tickets) {
   if (b.n_agents <= 0 || layer_count <= 0) return cudaSuccess;
   DecodeParams P;
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents * layer_count;
@@ -1367,9 +1384,10 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   }
   P.max_blocks = b.max_blocks; P.len_cap = max_kv_len; P.tables = b.block_tables; P.kv_lens = kv_lens;
   P.q = (const uint16_t*)q; P.scale_log2 = scale * kLog2e;
-  P.tickets = (int32_t*)ws; P.partials = (float*)((uint8_t*)ws + kWorkspaceHeaderBytes);
+  P.tickets = tickets ? tickets : (int32_t*)ws; P.partials = (float*)((uint8_t*)ws + kWorkspaceHeaderBytes);
   P.out = out; P.out_dtype = out_dtype; P.lse = lse; P.flags = flags;
   P.k_new = (const uint16_t*)k_new; P.v_new = (const uint16_t*)v_new;
+  P.q_offs = q_offs;
   const long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
   const int nw = warps_of(y.G);
   const long long wanted = (units + nw - 1) / nw;        // a chunk per warp at least

@@ -60,5 +60,12 @@ __device__ inline uint4 query8(uint4 v, float sf) {
                     f32x2_to_h2(hi(v.y), hi(v.w)));
 }
 
+// The agents that bring one query in a batch where others bring more are left to the decode kernel, which is launched next
+// on the same stream; its arrival counters are cleared here, so that the caller need not hand over a cleared workspace.
+__device__ inline void clear_tickets(const PrefillExtra& x) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int i = threadIdx.x; i < x.n_tickets; i += blockDim.x) x.tickets[i] = 0;
+}
+
 }  // namespace prefill
 }  // namespace q4kv

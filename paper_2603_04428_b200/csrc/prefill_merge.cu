@@ -52,15 +52,14 @@ merge_prefill_kernel(int rows, int Dv, int n_splits, const float* __restrict__ r
 }  // namespace
 
 // Parts the keys of every query tile are cut into.  tile_q: queries per CTA tile; per_tile: CTAs that share a tile.  The
-// number of CTAs is only bounded here (lengths are on the device): all tiles full except the last of each agent.  A launch
+// number of CTAs is estimated (lengths are on the device): the queries spread over as few agents as they can be.  A launch
 // of c CTAs in s parts takes about ceil(c s / SMs) / s of a whole tile's time plus a fixed cost per part (start-up and
 // records: about four 64-key blocks), so few tiles on long contexts are cut, many tiles or short contexts are not.
 int plan_prefill_splits(const Layout& y, int tile_q, int per_tile, int n_agents, int total_q, int max_q_len, int max_kv_len,
                         int window, size_t ws_bytes) {
   const long long sms = sm_count();
-  const long long tiles = (long long)total_q / tile_q + n_agents;
-  const long long all = (long long)n_agents * ((max_q_len + tile_q - 1) / tile_q);
-  const long long ctas = (tiles < all ? tiles : all) * y.Hkv * per_tile;
+  const long long full = (total_q + max_q_len - 1) / max_q_len;      // agents it takes at least
+  const long long ctas = ((long long)total_q / tile_q + full) * y.Hkv * per_tile;
   const int span = window > 0 && window + tile_q < max_kv_len ? window + tile_q : max_kv_len;
   const double blocks = (span + 63) / 64;
   int best = 1;

@@ -16,13 +16,22 @@
 //     0,4,1,5,2,6,3,7; the queries are stored in that order and the output columns are put back in place at the end.
 //   * One thread issues the MMAs: S_b = Q K^T (M 128, N 64: 16 instructions with the queries in tensor memory at 33 clocks, 20
 //     with them in shared memory at 55) and O += P_b V^ (M 128, N 256: 4 at 129): 2140 clocks of tensor pipe per block.
-//   * Eight softmax warps, two threads per score row, as in the one-tile kernel: two score buffers, lazily updated reference
-//     maximum, P_b as packed binary16 over S_b.
+//     A CTA's value product reads 256 of a block's 576 dims; the other 320 can be overwritten as soon as the block's scores
+//     are complete, and the next scores can start on them.  So a stage has two parts: part A (the 320), part B (the 256).
+//     Score and value products are issued as their inputs become ready, not in a fixed order: a value product that waited
+//     for the next scores would hold the K^ stage that the block after them needs (6200 clocks per block that way).
+//   * Four softmax warps, one thread per score row: mask, online softmax with a lazily updated reference maximum (rescaling
+//     only when the row maximum has grown by more than 2^8), P_b as packed binary16 over S_b.  Nothing is exchanged between
+//     threads, so a row's softmax waits for nothing but its scores.
 //   * With few tiles the keys of a tile are cut over several CTAs as well (plan_prefill_splits); these leave (acc, m, l)
 //     records that merge_prefill_kernel combines.
-// Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads: see launch_prefill_mla.
+// Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads (102 GFLOP): 36 ms on the shape-agnostic kernel,
+// 0.25 ms here = 405 TFLOP/s; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
+// products share the shared-memory bandwidth (256 KB per block: 2000 clocks) and the issue slots.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises Q4KV_FLAG_INTERNAL, drains the tensor
 // pipe and frees the tensor memory before the CTA returns.
+#include <type_traits>
+
 #include "prefill_common.cuh"
 
 namespace q4kv {
@@ -32,9 +41,9 @@ namespace {
 using namespace tc;
 using namespace prefill;
 
-constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
+constexpr int kSoftmaxWarps = 4, kDequantWarps = 8;
 constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps;
-constexpr int kThreads = (kMmaWarp + 1) * 32;            // 544
+constexpr int kThreads = (kMmaWarp + 1) * 32;            // 416: four warps on one scheduler at most, 128 registers
 constexpr int kStages = 2;
 constexpr int kG = 9, kD = 576, kDv = 512, kDvCta = 256;
 constexpr int kQTmem = 256, kQSmem = kD - kQTmem;        // query dims in tensor memory and in shared memory
@@ -63,10 +72,8 @@ struct MlaPrefillParams {
 struct MlaSmem {
   alignas(128) uint8_t khat[kStages][64 * kD * 2];       // [key][dim]: (n%8)*16 + (n/8)*kSboK + (k/8)*128
   alignas(128) uint8_t qs[128 * kQSmem * 2];             // [row][dim - 256]: (m%8)*16 + (m/8)*kSboQ + (k/8)*128
-  alignas(8) uint64_t k_full[kStages], k_free[kStages], s_full[2], p_full[2], o_done, q_ready, drain;
+  alignas(8) uint64_t a_full[kStages], b_full[kStages], a_free[kStages], b_free[kStages], s_full[2], p_full[2], o_done, q_ready, drain;
   uint32_t tmem_base;
-  float xchg[2][2][128];                                 // [parity][column half][row]: maxima / sums of the two threads of a row
-  int stop[3], spoiled;
   int abort_flag, poisoned;
 };
 
@@ -100,12 +107,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
 
   if (threadIdx.x == 0) {
     if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
-    for (int s = 0; s < kStages; ++s) { mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.k_free[s], 1); }
+    for (int s = 0; s < kStages; ++s) { 
+      mbar_init(&sm.a_full[s], kDequantWarps); mbar_init(&sm.b_full[s], kDequantWarps);
+      mbar_init(&sm.a_free[s], 1); mbar_init(&sm.b_free[s], 1);
+    }
     for (int b = 0; b < 2; ++b) { mbar_init(&sm.s_full[b], 1); mbar_init(&sm.p_full[b], kSoftmaxWarps * 32); }
     mbar_init(&sm.o_done, 1);
     mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
-    for (int i = 0; i < 3; ++i) sm.stop[i] = 0;
-    sm.spoiled = 0;
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0; sm.poisoned = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -134,122 +142,159 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     uint4 w16[4];
     uint2 w8;
     uint32_t sb[kG];
-    auto fetch = [&](int j) {                            // this thread's part of block it0 + j (bytes past the end: zeros)
+    // this thread's part of a block, piece by piece; nullptr (no pool block, or a token past the end): zeros
+    auto locate = [&](int j) {
       const int c = 2 * (it0 + j) + c1;
-      const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
+      const int blk = __ldg(&P.tables[(size_t)a * P.max_blocks + (c >> 3)]);
       const bool bad = blk < 0 || blk >= P.n_blocks;
       if (bad && lane == 0) { sm.poisoned = 1; raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK); }
-      if (bad || c * 32 + ktau >= kv_len) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w16[i] = make_uint4(0u, 0u, 0u, 0u);
-        w8 = make_uint2(0u, 0u);
-#pragma unroll
-        for (int i = 0; i < kG; ++i) sb[i] = 0u;
-        return;
-      }
-      const uint8_t* chunk = head_block(P.pool, y, P.layer, blk, hk) + (size_t)(c & 7) * kChunkBytes;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) w16[i] = __ldcg(reinterpret_cast<const uint4*>(chunk + read16 + 512 * i));
-      w8 = __ldcg(reinterpret_cast<const uint2*>(chunk + read8));
-#pragma unroll
-      for (int i = 0; i < kG; ++i) sb[i] = *reinterpret_cast<const volatile uint32_t*>(chunk + read_sb + 4 * i);
+      if (bad || c * 32 + ktau >= kv_len) return (const uint8_t*)nullptr;
+      return head_block(P.pool, y, P.layer, blk, hk) + (size_t)(c & 7) * kChunkBytes;
     };
-    if (n_iter > 0) fetch(0);
-    for (int j = 0; j < n_iter; ++j) {
-      const int s = j % kStages;
-      if (j >= kStages && !mbar_wait(&sm.k_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
-      if (kBf) {
-        bool overflow = false;
+    auto fetch16 = [&](const uint8_t* chunk, int i) {
+      w16[i] = chunk ? __ldcg(reinterpret_cast<const uint4*>(chunk + read16 + 512 * i)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto fetch8 = [&](const uint8_t* chunk) { w8 = chunk ? __ldcg(reinterpret_cast<const uint2*>(chunk + read8)) : make_uint2(0u, 0u); };
+    auto fetch_sb = [&](const uint8_t* chunk, int i) {
+      sb[i] = chunk ? __ldg(reinterpret_cast<const uint32_t*>(chunk + read_sb + 4 * i)) : 0u;
+    };
+    const uint8_t* next = nullptr;
+    if (n_iter > 0) {
+      next = locate(0);
 #pragma unroll
-        for (int i = 0; i < kG; ++i) sb[i] = bf16_pair_to_h2(sb[i], overflow);
-        if (overflow) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
-      }
-      uint8_t* dst = sm.khat[s] + write;
+      for (int i = 0; i < 4; ++i) fetch16(next, i);
+      fetch8(next);
 #pragma unroll
-      for (int p = 0; p < 18; ++p) {
-        const uint4& v = w16[(p >> 2) & 3];
-        const uint32_t w = p >= 16 ? (p == 16 ? w8.x : w8.y) : (p & 3) == 0 ? v.x : (p & 3) == 1 ? v.y : (p & 3) == 2 ? v.z : v.w;
-        const uint32_t sp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x1010), bp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x3232);
-        *reinterpret_cast<uint4*>(dst + p * 512) = dequant8(w, sp, bp, sp, bp, sp, bp, sp, bp);
-      }
-      if (j + 1 < n_iter) fetch(j + 1);
-      fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.k_full[s]);
+      for (int i = 0; i < kG; ++i) fetch_sb(next, i);
+      next = n_iter > 1 ? locate(1) : nullptr;
     }
+    // Word p of a token belongs to part B if it is one of the CTA's value dims (words 8 hv .. 8 hv + 7), else to part A.
+    auto run = [&](auto half) {
+      constexpr int kHv = decltype(half)::value;
+      for (int j = 0; j < n_iter; ++j) {
+        const int s = j % kStages;
+        uint8_t* dst = sm.khat[s] + write;
+        bool overflow = false;
+        // a register that has been used takes the next block's bytes at once, so that the loads are spread over the block
+        const uint8_t* const chunk = next;
+        auto word = [&](int p) {
+          if (kBf && (p & 1) == 0) sb[p >> 1] = bf16_pair_to_h2(sb[p >> 1], overflow);
+          const uint4& v = w16[(p >> 2) & 3];
+          const uint32_t w = p >= 16 ? (p == 16 ? w8.x : w8.y) : (p & 3) == 0 ? v.x : (p & 3) == 1 ? v.y : (p & 3) == 2 ? v.z : v.w;
+          const uint32_t sp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x1010), bp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x3232);
+          *reinterpret_cast<uint4*>(dst + p * 512) = dequant8(w, sp, bp, sp, bp, sp, bp, sp, bp);
+          if (p & 1) fetch_sb(chunk, p >> 1);
+          if (p < 16 && (p & 3) == 3) fetch16(chunk, p >> 2);
+          if (p == 17) fetch8(chunk);
+        };
+        if (j >= kStages && !mbar_wait(&sm.a_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
+#pragma unroll
+        for (int p = 0; p < 18; ++p)
+          if (p / 8 != kHv) word(p);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.a_full[s]);
+        if (j >= kStages && !mbar_wait(&sm.b_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
+#pragma unroll
+        for (int p = 8 * kHv; p < 8 * kHv + 8; ++p) word(p);
+        if (kBf && overflow) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.b_full[s]);
+        next = j + 2 < n_iter ? locate(j + 2) : nullptr;
+      }
+    };
+    if (hv == 0) run(std::integral_constant<int, 0>()); else run(std::integral_constant<int, 1>());
   } else if (warp == kMmaWarp) {
     // =============================== MMA issue ==================================================
-    // The whole warp runs this code, so that operands are computed once for the warp, and one elected
-    // lane (always the same) issues the MMAs and the commits.
+    // The whole warp runs this code, and one elected lane (always the same) issues: one election for a whole product
+    // (an election per MMA made the issue of a block 20 % longer than its execution).
     if (n_iter > 0) {
       constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, kDvCta, 0, 1);
       const uint64_t qd = smem_desc(smem_u32(sm.qs), 128, kSboQ);
-      auto issue_qk = [&](int b, int s) {                // S_b = Q K^T
+      // part A or B of S_b = Q K^T: the 16-dim steps outside / inside the CTA's value dims
+      auto issue_qk = [&](int b, int s, auto half, auto part_b) {
+        constexpr int kHv = decltype(half)::value;
+        constexpr bool kB = decltype(part_b)::value;
+        constexpr int kFirst = kHv == 0 ? 16 : 0;        // of part A
         const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, kSboK);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < kQTmem / 16; ++k)
-          if (elect_one()) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, k > 0);
-#pragma unroll
-        for (int k = 0; k < kQSmem / 16; ++k)
-          if (elect_one()) mma_f16_ss(tb + kColS + 64 * b, qd + 16 * k, kd + 16 * (kQTmem / 16 + k), kIdescS, 1u);
-        if (elect_one()) commit(&sm.s_full[b]);
+          for (int k = 0; k < kD / 16; ++k) {
+            if ((k / 16 == kHv) != kB) continue;
+            const uint32_t accumulate = !kB && k == kFirst ? 0u : 1u;
+            if (k < kQTmem / 16)
+              mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, accumulate);
+            else
+              mma_f16_ss(tb + kColS + 64 * b, qd + 16 * (k - kQTmem / 16), kd + 16 * k, kIdescS, accumulate);
+          }
+          if (kB) { commit(&sm.s_full[b]); commit(&sm.a_free[s]); }
+        }
+        __syncwarp();
       };
       auto issue_pv = [&](int b, int s, bool first) {    // O (+)= P_b V^; afterwards the stage is free
         const uint64_t vd = smem_desc(smem_u32(sm.khat[s]) + hv * (kDvCta / 8) * 128, kSboK, 128);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (elect_one()) mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + (2 * kSboK / 16) * k, kIdescO, (!first || k > 0) ? 1u : 0u);
-        if (elect_one()) { commit(&sm.o_done); commit(&sm.k_free[s]); }
-      };
-      bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
-        fence_after_sync();
-        issue_qk(0, 0);
-      }
-      for (int j = 0; ok && j < n_iter; ++j) {
-        if (j + 1 < n_iter) {                            // the next block's scores before this block's values
-          const int s1 = (j + 1) % kStages;
-          ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s1], (uint32_t)((j + 1) / kStages), abort_flag));
-          if (!ok) break;
-          fence_after_sync();
-          issue_qk((j + 1) & 1, s1);                     // S of block j - 1 (as P) was read by the product issued before it
+          for (int k = 0; k < 4; ++k)
+            mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + (2 * kSboK / 16) * k, kIdescO, (!first || k > 0) ? 1u : 0u);
+          commit(&sm.o_done);
+          commit(&sm.b_free[s]);
         }
-        ok = __all_sync(0xffffffffu, mbar_wait(&sm.p_full[j & 1], (uint32_t)(j >> 1), abort_flag));
-        if (!ok) break;
-        fence_after_sync();
-        issue_pv(j & 1, j % kStages, j == 0);
-      }
+        __syncwarp();
+      };
+      bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.q_ready, 0, abort_flag));
+      int na = 0, nb = 0, np = 0;                        // blocks whose scores (parts A, B) / values have been issued
+      uint32_t idle = 0;
+      auto run = [&](auto half) {
+        while (ok && np < n_iter) {
+          if (np < nb && __all_sync(0xffffffffu, mbar_test_wait(&sm.p_full[np & 1], (uint32_t)(np >> 1) & 1u))) {
+            fence_after_sync();
+            issue_pv(np & 1, np % kStages, np == 0);
+            ++np;
+            idle = 0;
+          }
+          // part A of block na: its keys are there, and the probabilities that its buffer held have been used
+          if (na < n_iter && na < np + 2 && __all_sync(0xffffffffu, mbar_test_wait(&sm.a_full[na % kStages], (uint32_t)(na / kStages) & 1u))) {
+            fence_after_sync();
+            issue_qk(na & 1, na % kStages, half, std::false_type());
+            ++na;
+            idle = 0;
+          }
+          if (nb < na && __all_sync(0xffffffffu, mbar_test_wait(&sm.b_full[nb % kStages], (uint32_t)(nb / kStages) & 1u))) {
+            fence_after_sync();
+            issue_qk(nb & 1, nb % kStages, half, std::true_type());
+            ++nb;
+            idle = 0;
+          }
+          if (++idle > 64) {
+            __nanosleep(64);
+            ok = __all_sync(0xffffffffu, idle < (1u << 25) && !*abort_flag);
+            if (!ok) *abort_flag = 1;
+          }
+        }
+      };
+      if (hv == 0) run(std::integral_constant<int, 0>()); else run(std::integral_constant<int, 1>());
     }
   } else if (warp < kSoftmaxWarps) {
-    // =============================== softmax warps: two threads per score row ===================
-    // Warp w: column half = w / 4, tensor-memory lanes 32 (w % 4) ...  The two threads of a row exchange their block
-    // maxima (and at the end their sums) through shared memory; the 256 threads meet at a named barrier once per
-    // block, and they leave the loop together (one of them samples the give-up flag before the barrier).
-    const int half = (warp >> 2) & 1;
-    const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
-    const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
+    // =============================== softmax warps: one thread per score row ===================
+    const int row = warp * 32 + lane;                    // tensor-memory lane
+    const uint32_t lane_addr = tb + ((uint32_t)(warp * 32) << 16);
     const int h = row / tile_q, i = i_min + row % tile_q;
     const bool mine = i < q_len && h < n_rep;            // a row of the output
     const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
-    const bool sampler = warp == 0 && lane == 0;
-    auto tile_barrier = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
     const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
     float kappa;                                         // score in log2 units = S * kappa
     {
-      // ---- stage the query row: bf16 -> binary16 times a power of two; pieces of eight dims 0..31 go to tensor memory
-      //      (sixteen by each thread of the row), 32..71 to shared memory (twenty by each) ----
+      // ---- stage the query row: bf16 -> binary16 times a power of two; pieces of eight dims 0..31 go to tensor memory,
+      //      32..71 to shared memory ----
       const uint16_t* qrow = P.q + (valid ? row_index : 0) * kD;
-      const int p0 = 16 * half, p1 = 32 + 20 * half;
       float mx = 0.f;
       if (valid) {
-#pragma unroll 4
-        for (int p = 0; p < 36; ++p) mx = fmaxf(mx, max_abs8(*reinterpret_cast<const uint4*>(qrow + 8 * (p < 16 ? p0 + p : p1 + p - 16))));
+#pragma unroll 8
+        for (int p = 0; p < kD / 8; ++p) mx = fmaxf(mx, max_abs8(*reinterpret_cast<const uint4*>(qrow + 8 * p)));
       }
-      sm.xchg[1][half][row] = mx;                        // slot 1: block 0 of the loop below writes slot 0
-      tile_barrier();
-      mx = fmaxf(mx, sm.xchg[1][half ^ 1][row]);
       int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
       if (mx == 0.f) ex = 0;
       ex = min(max(ex, -100), 100);
@@ -257,19 +302,19 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
       kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
       const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
-      for (int c = 0; c < 2; ++c) {                      // 32 columns (64 dims) at a time
+      for (int c = 0; c < kQTmem / 64; ++c) {            // 32 columns (64 dims) at a time
         uint32_t qa[32];
 #pragma unroll
         for (int p = 0; p < 8; ++p) {
-          const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * (p0 + 8 * c + p)) : zero4, sf);
+          const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * (8 * c + p)) : zero4, sf);
           qa[4 * p] = v.x; qa[4 * p + 1] = v.y; qa[4 * p + 2] = v.z; qa[4 * p + 3] = v.w;
         }
-        tmem_st32(lane_addr + kColQ + 64 * half + 32 * c, qa);
+        tmem_st32(lane_addr + kColQ + 32 * c, qa);
       }
 #pragma unroll 4
-      for (int p = p1; p < p1 + 20; ++p) {
+      for (int p = kQTmem / 8; p < kD / 8; ++p) {
         const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : zero4, sf);
-        *reinterpret_cast<uint4*>(sm.qs + (row & 7) * 16 + (row >> 3) * kSboQ + (p - 32) * 128) = v;
+        *reinterpret_cast<uint4*>(sm.qs + (row & 7) * 16 + (row >> 3) * kSboQ + (p - kQTmem / 8) * 128) = v;
       }
       wait_st();
       fence_async_smem();
@@ -279,85 +324,70 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most kLazy
     for (int j = 0; j < n_iter; ++j) {
       const int b = j & 1;
-      mbar_wait(&sm.s_full[b], (uint32_t)(j >> 1), abort_flag);   // a wait that runs out raises the give-up flag; all leave below
+      if (!mbar_wait(&sm.s_full[b], (uint32_t)(j >> 1), abort_flag)) break;
       fence_after_sync();
-      uint32_t sr[32];
-      tmem_ld32(lane_addr + kColS + 64 * b + 32 * half, sr);
+      __syncwarp();
+      uint32_t sr[64];
+      tmem_ld32(lane_addr + kColS + 64 * b, sr);
+      tmem_ld32(lane_addr + kColS + 64 * b + 32, sr + 32);
       wait_ld();
-      const int pos0 = (it0 + j) * 64 + 32 * half;
-      // column c of this half is key pos0 + c; causal and window masks on edge blocks only
-      if (pos0 + 31 > pq || (W > 0 && pos0 <= pq - W)) {
+      const int pos0 = (it0 + j) * 64;
+      // column c is key pos0 + c; causal and window masks on edge blocks only
+      if (pos0 + 63 > pq || (W > 0 && pos0 <= pq - W)) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < 64; ++c)
           if (pos0 + c > pq || (W > 0 && pos0 + c <= pq - W)) sr[c] = 0xff800000u;   // -inf
       }
-      // Probabilities against the current reference, and the block maximum beside them (independent instruction
-      // streams); only when some row's maximum has outgrown its reference is the reference moved, the accumulator
-      // rescaled and the probabilities taken again.  The scores stay in registers meanwhile.
-      float sum = 0.f;
-      uint32_t pr[16];
-      auto probabilities = [&](float neg_m) {
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-        for (int c = 0; c < 16; c += 2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sr[2 * c]), kappa, neg_m));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 1]), kappa, neg_m));
-          const float p2 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 2]), kappa, neg_m));
-          const float p3 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 3]), kappa, neg_m));
-          s0 += p0; s1 += p1; s2 += p2; s3 += p3;
-          pr[c] = f32x2_to_h2(p0, p1);
-          pr[c + 1] = f32x2_to_h2(p2, p3);
-        }
-        sum = (s0 + s1) + (s2 + s3);
-      };
-      probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
       float cm4[4] = {__uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2]), __uint_as_float(sr[3])};
 #pragma unroll
-      for (int c = 4; c < 32; ++c) cm4[c & 3] = fmaxf(cm4[c & 3], __uint_as_float(sr[c]));
+      for (int c = 4; c < 64; ++c) cm4[c & 3] = fmaxf(cm4[c & 3], __uint_as_float(sr[c]));
       float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
-      sm.xchg[j & 1][half][row] = cm;
-      if (sampler) sm.stop[j % 3] = *abort_flag;
-      tile_barrier();                                    // also: every score of the block has been read (P overlays S)
-      if (sm.stop[j % 3]) break;
-      cm = fmaxf(cm, sm.xchg[j & 1][half ^ 1][row]);
       if (cm != -INFINITY) cm *= kappa;                  // kappa > 0
       const float m_new = fmaxf(m_ref, cm);
       const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
       if (__any_sync(0xffffffffu, grow)) {
         if (j > 0) {
-          // rescale this thread's half of the accumulator row: the previous block's value product must have landed
-          mbar_wait(&sm.o_done, (uint32_t)(j - 1), abort_flag);
+          // rescale the accumulator row: the previous block's value product must have landed
+          if (!mbar_wait(&sm.o_done, (uint32_t)(j - 1), abort_flag)) break;
           fence_after_sync();
+          __syncwarp();
           const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;           // m_ref = -inf: 0
 #pragma unroll 1
-          for (int part = 0; part < kDvCta / 64; ++part) {
-            uint32_t orow[32];
-            tmem_ld32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+          for (int part = 0; part < kDvCta / 16; ++part) {
+            uint32_t orow[16];
+            tmem_ld16(lane_addr + kColO + 16 * part, orow);
             wait_ld();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
-            tmem_st32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+            for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
+            tmem_st16(lane_addr + kColO + 16 * part, orow);
           }
           if (grow) l *= f;
         }
         if (grow) m_ref = m_new;
-        probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
       }
-      l += sum;
-      tmem_st16(lane_addr + kColS + 64 * b + 16 * half, pr);   // P_b overlays the first 32 columns of S_b
+      const float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+      uint32_t pr[32];
+#pragma unroll
+      for (int c = 0; c < 32; c += 2) {
+        const float p0 = fast_exp2(fmaf(__uint_as_float(sr[2 * c]), kappa, neg_m));
+        const float p1 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 1]), kappa, neg_m));
+        const float p2 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 2]), kappa, neg_m));
+        const float p3 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 3]), kappa, neg_m));
+        s0 += p0; s1 += p1; s2 += p2; s3 += p3;
+        pr[c] = f32x2_to_h2(p0, p1);
+        pr[c + 1] = f32x2_to_h2(p2, p3);
+      }
+      l += (s0 + s1) + (s2 + s3);
+      tmem_st32(lane_addr + kColS + 64 * b, pr);         // P_b overlays the first 32 columns of S_b
       wait_st();
       fence_before_sync();
       mbar_arrive(&sm.p_full[b]);
     }
-    // ---- normalise and write this thread's half of the row, or leave it as a record ----
+    // ---- normalise and write the row, or leave it as a record ----
     bool ok = !*abort_flag;
     if (ok && n_iter > 0) ok = mbar_wait(&sm.o_done, (uint32_t)(n_iter - 1), abort_flag);
-    const int slot = n_iter & 1;                         // not the slot the last block used
-    sm.xchg[slot][half][row] = l;
-    if (!ok) sm.spoiled = 1;                             // anyone who gave up spoils the tile
-    tile_barrier();
-    ok = sm.spoiled == 0;                                // uniform over the tile: the loads below are warp-wide
-    l += sm.xchg[slot][half ^ 1][row];
+    ok = __all_sync(0xffffffffu, ok);                    // the loads below are warp-wide
     if (ok) fence_after_sync();
     const bool bad = !ok || sm.poisoned != 0;
     const bool zero = bad || n_iter == 0 || l <= 0.f;
@@ -365,14 +395,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
     float* rec = final ? nullptr : P.records + (row_index * P.n_splits + split) * prefill_record(kDv);
 #pragma unroll 1
-    for (int part = 0; part < kDvCta / 64; ++part) {
+    for (int part = 0; part < kDvCta / 32; ++part) {
       uint32_t orow[32];
       if (ok && n_iter > 0) {
-        tmem_ld32(lane_addr + kColO + (kDvCta / 2) * half + 32 * part, orow);
+        tmem_ld32(lane_addr + kColO + 32 * part, orow);
         wait_ld();
       }
       if (!mine) continue;
-      const int d0 = kDvCta * hv + (kDvCta / 2) * half + 32 * part;
+      const int d0 = kDvCta * hv + 32 * part;
       // slot j of every eight columns is value dim elem_of(j)
       if (final && P.out_dtype == Q4KV_OUT_BF16) {
         __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + row_index * kDv + d0;
@@ -398,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
                                  __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 2)]) * inv, __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 3)]) * inv);
       }
     }
-    if (half == 0 && hv == 0 && mine) {
+    if (hv == 0 && mine) {
       if (!final) *reinterpret_cast<float2*>(rec + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
       else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
     }

@@ -1,6 +1,6 @@
 // q4kv_prefill_attention, tcgen05 path with one query tile per CTA, for the head shapes whose
 // accumulator leaves no room for two: d_qk = d_v = 256 (the sliding-window model of Section 3.6) and
-// d_qk 192 / d_v 128 (the per-head MLA cache of Section 3.6); 1, 2 or 4 query heads per KV head.  The
+// d_qk 192 / d_v 128 (the per-head MLA cache of Section 3.6).  The
 // queries of a new phase over the cached Q4 prefix plus the causal new tokens, read from the Q4
 // cache in place (Sections 3.4 "chunked prefill" and 3.5 "cross-phase context injection").
 //
@@ -28,14 +28,14 @@
 //   * One warp streams the raw blocks through a three-slot ring with bulk asynchronous copies.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
 // Q4KV_FLAG_INTERNAL, drains the tensor pipe and frees the tensor memory before the CTA returns.
-#include "q4kv_layout.cuh"
-#include "tcgen05.cuh"
+#include "prefill_common.cuh"
 
 namespace q4kv {
 
 namespace {
 
 using namespace tc;
+using namespace prefill;
 
 constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
 constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps, kLoadWarp = kMmaWarp + 1;
@@ -53,8 +53,6 @@ struct Shape {
   static constexpr int kTileK = 64 * D * 2, kTileV = Dv * 64 * 2;   // binary16 tiles
   static constexpr int kSboK = (D / 8) * 128;            // bytes between 8-key groups of K^
 };
-constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLazy = 8.f;                             // rescale when the row maximum grew by more than this (log2)
 
 struct UmmaParams {
   Layout y;
@@ -70,6 +68,7 @@ struct UmmaParams {
   int out_dtype;
   float* lse;
   int32_t* flags;
+  PrefillExtra x;
 };
 
 template <int G, int Gv>
@@ -88,44 +87,6 @@ struct UmmaSmem {
   int abort_flag, poisoned;
 };
 
-// Eight codes of one packed word -> eight binary16 values c * s + b, as the pairs (0,4) (1,5) (2,6)
-// (3,7) with the scale and bias pair given for each.  Masking a nibble into the mantissa of 1024
-// (ulp 1) or of 64 (ulp 1/16, for a nibble sitting four bits up) gives 1024 + c or 64 + c exactly.
-__device__ inline uint4 dequant8(uint32_t w, uint32_t s04, uint32_t b04, uint32_t s15, uint32_t b15, uint32_t s26,
-                                 uint32_t b26, uint32_t s37, uint32_t b37) {
-  const uint32_t wh = w >> 8;
-  const __half2 k1024 = __half2half2(__ushort_as_half((unsigned short)0x6400));
-  const __half2 k64 = __half2half2(__ushort_as_half((unsigned short)0x5400));
-  auto as_h2 = [](uint32_t u) { return *reinterpret_cast<__half2*>(&u); };
-  auto as_u = [](__half2 h) { return *reinterpret_cast<uint32_t*>(&h); };
-  const __half2 c04 = __hsub2(as_h2((w & 0x000F000Fu) | 0x64006400u), k1024);
-  const __half2 c15 = __hsub2(as_h2((w & 0x00F000F0u) | 0x54005400u), k64);
-  const __half2 c26 = __hsub2(as_h2((wh & 0x000F000Fu) | 0x64006400u), k1024);
-  const __half2 c37 = __hsub2(as_h2((wh & 0x00F000F0u) | 0x54005400u), k64);
-  return make_uint4(as_u(__hfma2(c04, as_h2(s04), as_h2(b04))), as_u(__hfma2(c15, as_h2(s15), as_h2(b15))),
-                    as_u(__hfma2(c26, as_h2(s26), as_h2(b26))), as_u(__hfma2(c37, as_h2(s37), as_h2(b37))));
-}
-// position inside a row's eight elements of element u (the inverse of 0,4,1,5,2,6,3,7)
-__device__ inline int slot_of(int u) { return ((u & 3) << 1) | (u >> 2); }
-// element held by slot j of a row
-__device__ inline int elem_of(int j) { return ((j & 1) << 2) | (j >> 1); }
-__device__ inline float fast_exp2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ inline uint32_t f32x2_to_h2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-// A bfloat16 (scale, bias) pair as a binary16 pair: exact while the magnitude is a binary16 normal number (bfloat16
-// has 8 significant bits), within 2^-25 below that; a magnitude beyond binary16's largest number is reported.
-__device__ inline uint32_t bf16_pair_to_h2(uint32_t u, bool& overflow) {
-  const uint32_t h = f32x2_to_h2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
-  overflow |= (((h & 0x7C007C00u) + 0x04000400u) & 0x80008000u) != 0u;     // an exponent field of all ones
-  return h;
-}
-
 template <int G, int Gv, bool kBf>
 __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const __grid_constant__ UmmaParams P) {
   using Sh = Shape<G, Gv>;
@@ -136,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
 
   const Layout& y = P.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qt = blockIdx.x, hk = blockIdx.y, a = blockIdx.z;
+  const int qt = blockIdx.x, hk = blockIdx.y / P.x.n_splits, split = blockIdx.y % P.x.n_splits, a = blockIdx.z;
   const int n_rep = y.n_rep;
   const int tile_q = 128 / n_rep;                        // queries of the CTA's 128-row tile
 
@@ -145,15 +106,17 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
   const int q0 = P.q_offs[a], q_len = P.q_offs[a + 1] - q0;
   const int kv_len = P.kv_lens[a];
   const int i_min = qt * tile_q;
-  if (i_min >= q_len) return;                            // uniform: nothing allocated, no barrier passed
+  if (P.x.tickets && qt == 0 && blockIdx.y == 0 && a == 0) clear_tickets(P.x);
+  if (i_min >= q_len || (P.x.tickets && q_len == 1)) return;   // uniform: nothing allocated, no barrier passed
   const bool bad_len = kv_len < 0 || kv_len > P.max_blocks * kBlockTokens || q_len > kv_len;
   const int i_max = min(q_len, i_min + tile_q) - 1;
   const int prefix = kv_len - q_len;                     // query i sits at position prefix + i
   const int W = P.window;
   const int c_end = bad_len ? 0 : (prefix + i_max) / 32 + 1;
   const int c_begin = (bad_len || W == 0) ? 0 : max(0, prefix + i_min - W + 1) >> 5;
-  const int it0 = c_begin >> 1;                          // 64-key blocks it0 .. it0 + n_iter - 1
-  const int n_iter = max(0, ((c_end + 1) >> 1) - it0);
+  const int all0 = c_begin >> 1, n_all = max(0, ((c_end + 1) >> 1) - all0);
+  const int it0 = all0 + n_all * split / P.x.n_splits;   // 64-key blocks it0 .. it0 + n_iter - 1
+  const int n_iter = all0 + n_all * (split + 1) / P.x.n_splits - it0;
 
   if (threadIdx.x == 0) {
     if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
@@ -315,27 +278,30 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     }
   } else if (warp == kMmaWarp) {
     // =============================== MMA issue ==================================================
-    // The whole warp runs this code, so that operands are computed once for the warp, and one elected
-    // lane (always the same) issues the MMAs and the commits.
+    // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
     if (n_iter > 0) {
       constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, kDv);
+      // one election for a whole product: an election per MMA costs more issue time than the MMA takes
       auto issue_qk = [&](int b, int s) {                // S_b = Q K^T; afterwards the K^ stage is free
-        const uint32_t kb = smem_u32(sm.khat[s]);
+        const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, Sh::kSboK);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < kD / 16; ++k) {
-          const uint64_t bd = smem_desc(kb + 256 * k, 128, Sh::kSboK);
-          if (elect_one()) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, bd, kIdescS, k > 0);
+          for (int k = 0; k < kD / 16; ++k) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, k > 0);
+          commit(&sm.s_full[b]);
+          commit(&sm.k_free[s]);
         }
-        if (elect_one()) { commit(&sm.s_full[b]); commit(&sm.k_free[s]); }
+        __syncwarp();
       };
       auto issue_pv = [&](int b, int s, bool first) {    // O (+)= P_b V^; afterwards the V^ stage is free
-        const uint32_t vb = smem_u32(sm.vhat[s]);
+        const uint64_t vd = smem_desc(smem_u32(sm.vhat[s]), 128, 1024);
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t bd = smem_desc(vb + 256 * k, 128, 1024);
-          if (elect_one()) mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, bd, kIdescO, (!first || k > 0) ? 1u : 0u);
+          for (int k = 0; k < 4; ++k)
+            mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + 16 * k, kIdescO, (!first || k > 0) ? 1u : 0u);
+          commit(&sm.o_done);
+          commit(&sm.v_free[s]);
         }
-        if (elect_one()) { commit(&sm.o_done); commit(&sm.v_free[s]); }
+        __syncwarp();
       };
       bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
@@ -374,7 +340,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
     const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
     const int h = row / tile_q, i = i_min + row % tile_q;
-    const bool valid = i < q_len && !bad_len;
+    const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
+    const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
     const bool sampler = warp == 0 && lane == 0;
     auto tile_barrier = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
@@ -519,9 +486,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     ok = sm.spoiled == 0;                                // uniform over the tile: the loads below are warp-wide
     l += sm.xchg[slot][half ^ 1][row];
     if (ok) fence_after_sync();
-    const bool zero = !ok || n_iter == 0 || sm.poisoned != 0 || l <= 0.f;
-    const float inv = zero ? 0.f : 1.f / l;
-    const size_t orow_index = ((size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h) * kDv + (kDv / 2) * half;
+    const bool bad = !ok || sm.poisoned != 0;
+    const bool zero = bad || n_iter == 0 || l <= 0.f;
+    const bool final = P.x.n_splits == 1;                // else the row is left as a record
+    const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
+    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
+    const size_t orow_index = row_index * kDv + (kDv / 2) * half;
+    float* rec = final ? nullptr : P.x.records + (row_index * P.x.n_splits + split) * prefill_record(kDv);
 #pragma unroll 1
     for (int part = 0; part < kDv / 64; ++part) {
       uint32_t orow[32];
@@ -529,8 +500,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         tmem_ld32(lane_addr + kColO + (kDv / 2) * half + 32 * part, orow);
         wait_ld();
       }
-      if (i >= q_len) continue;
-      if (P.out_dtype == Q4KV_OUT_BF16) {
+      if (!mine) continue;
+      if (final && P.out_dtype == Q4KV_OUT_BF16) {
         __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + orow_index + 32 * part;
 #pragma unroll
         for (int c = 0; c < 32; c += 8) {
@@ -545,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
           *reinterpret_cast<uint4*>(o + c) = v;
         }
       } else {
-        float* o = reinterpret_cast<float*>(P.out) + orow_index + 32 * part;
+        float* o = (final ? reinterpret_cast<float*>(P.out) + orow_index : rec + (kDv / 2) * half) + 32 * part;
 #pragma unroll
         for (int c = 0; c < 32; c += 4)
           *reinterpret_cast<float4*>(o + c) =
@@ -554,8 +525,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
                                  __uint_as_float(orow[c + 2]) * inv, __uint_as_float(orow[c + 3]) * inv);
       }
     }
-    if (half == 0 && i < q_len && P.lse)
-      P.lse[(size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
+    if (half == 0 && mine) {
+      if (!final) *reinterpret_cast<float2*>(rec + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
+      else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
+    }
   }
 
   // ---- teardown: nothing may be in flight in the tensor pipe when the columns are given back ----
@@ -579,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
 
 bool prefill_umma_1tile_supported(const Layout& y) {
   const bool shape = (y.D == 256 && y.Dv == 256) || (y.D == 192 && y.Dv == 128);
-  return !y.alias && shape && (y.n_rep == 1 || y.n_rep == 2 || y.n_rep == 4);
+  return !y.alias && shape && y.n_rep <= 128;
 }
 
 namespace {
@@ -597,7 +570,7 @@ cudaError_t launch_shape(const UmmaParams& P, int max_q_len, cudaStream_t st) {
   }
   const int cta_q = 128 / P.y.n_rep;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((max_q_len + cta_q - 1) / cta_q, P.y.Hkv, P.n_agents);
+  cfg.gridDim = dim3((max_q_len + cta_q - 1) / cta_q, P.y.Hkv * P.x.n_splits, P.n_agents);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -613,12 +586,13 @@ cudaError_t launch_shape(const UmmaParams& P, int max_q_len, cudaStream_t st) {
 cudaError_t launch_prefill_umma_1tile(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
                                       const int32_t* kv_lens, const int32_t* q_offs, int max_q_len, int window,
                                       const void* q, float scale, void* out, int out_dtype, float* lse, int32_t* flags,
-                                      cudaStream_t st) {
+                                      cudaStream_t st, const PrefillExtra& x) {
   if (b.n_agents <= 0 || max_q_len <= 0) return cudaSuccess;
   UmmaParams P;
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents;
   P.max_blocks = b.max_blocks; P.tables = b.block_tables; P.kv_lens = kv_lens; P.q_offs = q_offs; P.window = window;
   P.q = (const uint16_t*)q; P.scale_log2 = scale * kLog2e; P.out = out; P.out_dtype = out_dtype; P.lse = lse; P.flags = flags;
+  P.x = x;
   if (y.D == 256) return y.sb_bf16 ? launch_shape<4, 4, true>(P, max_q_len, st) : launch_shape<4, 4, false>(P, max_q_len, st);
   return y.sb_bf16 ? launch_shape<3, 2, true>(P, max_q_len, st) : launch_shape<3, 2, false>(P, max_q_len, st);
 }

@@ -42,13 +42,32 @@ size_t workspace_need(const Layout& y, int n_agents, int max_kv_len, int total_q
   return kWorkspaceHeaderBytes + need;
 }
 
-// What a prefill call can make use of: records of the query tiles whose keys it cuts into parts.  The call makes do with
-// less (fewer parts), so this size is not a condition.
+// The tcgen05 prefill kernels: the query rows of a CTA and the CTAs that share them (0: no such kernel for the shape).
+int prefill_rows(const Layout& y) { return prefill_umma_supported(y) ? 256 : prefill_umma_1tile_supported(y) || prefill_mla_supported(y) ? 128 : 0; }
+int prefill_tile_q(const Layout& y) { return prefill_rows(y) == 256 ? 2 * (128 / y.n_rep) : 128 / y.n_rep; }
+size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
+
+// Agents that bring one query while others bring more go to the decode kernel.  The counts are on the device; what the host
+// sees is that one such agent leaves the batch max_q_len - 1 rows short of n_agents * max_q_len.  A launch that finds none
+// costs 2 us, so it is made only where an average agent brings at most a third of the longest: chunks of one schedule lie
+// closer together, decoding agents pull the average down.
+bool may_decode_singles(const Layout& y, int n_agents, int max_blocks, int total_q, int max_q_len) {
+  const long long all = (long long)n_agents * max_q_len;
+  return max_q_len > 1 && all - total_q >= max_q_len - 1 && 3ll * total_q <= all && decode_mma_supported(y) &&
+         decode_mma_fits(y, n_agents, max_blocks);
+}
+size_t singles_bytes(const Layout& y, int n_agents) {
+  return align256(sizeof(int32_t) * decode_mma_tickets(y, n_agents)) + decode_mma_workspace_bytes(y, n_agents);
+}
+
+// What a prefill call can make use of: the records of the query tiles whose keys it cuts into parts, and the workspace of
+// the decode launch for agents with one query.  The call makes do with less, so this size is not a condition.
 size_t prefill_workspace(const Layout& y, int n_agents, int max_kv_len, int total_q) {
-  int splits = 1;
-  if (prefill_mla_supported(y))
-    splits = plan_prefill_splits(y, 128 / y.n_rep, 2, n_agents, total_q, total_q, max_kv_len, 0, (size_t)-1);
-  return splits > 1 ? prefill_record_bytes(y, total_q, splits) : 16;
+  if (!prefill_rows(y)) return 16;
+  const int splits = plan_prefill_splits(y, prefill_tile_q(y), prefill_mla_supported(y) ? 2 : 1, n_agents, total_q, total_q, max_kv_len, 0, (size_t)-1);
+  size_t need = splits > 1 ? align256(prefill_record_bytes(y, total_q, splits)) : 0;
+  if (n_agents > 1 && total_q > n_agents && decode_mma_supported(y)) need += align256(singles_bytes(y, n_agents));
+  return need > 16 ? need : 16;
 }
 
 // The kernels that expand the cache into binary16 tiles round each dequantized element once; they are taken only when
@@ -244,12 +263,29 @@ int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_bl
   const Layout y = make_layout(*spec, n_blocks);
   if (workspace_bytes < workspace_need(y, batch->n_agents, max_kv_len, total_q)) return Q4KV_EWORKSPACE;
   cudaError_t e;
-  if (prefill_umma_supported(y) && tiles_allowed(spec, softmax_scale))
-    e = launch_prefill_umma(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale, out,
-                            out_dtype, lse, status_flags, (cudaStream_t)stream);
-  else if (prefill_umma_1tile_supported(y) && tiles_allowed(spec, softmax_scale))
-    e = launch_prefill_umma_1tile(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale,
-                                  out, out_dtype, lse, status_flags, (cudaStream_t)stream);
+  if ((prefill_umma_supported(y) || prefill_umma_1tile_supported(y)) && tiles_allowed(spec, softmax_scale)) {
+    PrefillExtra x = {};
+    uint8_t* at = (uint8_t*)workspace;
+    size_t left = workspace_bytes;
+    if (may_decode_singles(y, batch->n_agents, batch->max_blocks, total_q, max_q_len) && left >= singles_bytes(y, batch->n_agents)) {
+      x.tickets = (int32_t*)at;
+      x.n_tickets = decode_mma_tickets(y, batch->n_agents);
+      at += align256(singles_bytes(y, batch->n_agents));
+      left -= left < align256(singles_bytes(y, batch->n_agents)) ? left : align256(singles_bytes(y, batch->n_agents));
+    }
+    x.n_splits = plan_prefill_splits(y, prefill_tile_q(y), 1, batch->n_agents, total_q, max_q_len, max_kv_len, window, left);
+    x.records = (float*)at;
+    const auto launch = prefill_umma_supported(y) ? launch_prefill_umma : launch_prefill_umma_1tile;
+    e = launch(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale, out, out_dtype, lse,
+               status_flags, (cudaStream_t)stream, x);
+    if (e == cudaSuccess && x.n_splits > 1)
+      e = launch_merge_prefill(y, total_q, x.n_splits, x.records, out, out_dtype, lse, (cudaStream_t)stream);
+    // after the merge, which leaves something or other in the rows of these agents
+    if (e == cudaSuccess && x.tickets)
+      e = launch_decode_mma(y, pool, n_blocks, layer, *batch, kv_lens, cap, &window, 1, q, softmax_scale, out, out_dtype, lse,
+                            (uint8_t*)x.tickets + align256(sizeof(int32_t) * x.n_tickets) - kWorkspaceHeaderBytes, status_flags,
+                            (cudaStream_t)stream, nullptr, nullptr, q_offs, x.tickets);
+  }
   else if (prefill_mla_supported(y) && tiles_allowed(spec, softmax_scale))
     e = launch_prefill_mla(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, total_q, max_q_len, max_kv_len, window, q,
                            softmax_scale, out, out_dtype, lse, workspace, workspace_bytes, status_flags, (cudaStream_t)stream);

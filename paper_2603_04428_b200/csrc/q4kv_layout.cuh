@@ -140,7 +140,18 @@ size_t decode_mma_workspace_bytes(const Layout& y, int n_agents, int layer_count
 cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
                               const int32_t* kv_lens, int max_kv_len, const int32_t* windows, int layer_count,
                               const void* q, float scale, void* out, int out_dtype, float* lse, void* ws, int32_t* flags,
-                              cudaStream_t st, const void* k_new = nullptr, const void* v_new = nullptr);
+                              cudaStream_t st, const void* k_new = nullptr, const void* v_new = nullptr,
+                              // q_offs: only the agents with exactly one query row; tickets: counters of their own
+                              const int32_t* q_offs = nullptr, int32_t* tickets = nullptr);
+int decode_mma_tickets(const Layout& y, int n_agents);
+
+// What a tcgen05 prefill launch does beside the attention of its tiles
+struct PrefillExtra {
+  int n_splits;               // parts the keys of a tile are cut into; above 1 the parts leave records
+  float* records;             // [total_q][Hq][n_splits][acc, m, l, pad]
+  int32_t* tickets;           // arrival counters to clear for the decode launch that takes the agents with one query; or null
+  int n_tickets;
+};
 
 // tensor-core prefill path (d_qk = d_v = 128, at most 4 query heads per KV head)
 bool prefill_mma_supported(const Layout& y);
@@ -149,19 +160,20 @@ cudaError_t launch_prefill_mma(const Layout& y, const void* pool, int n_blocks, 
                                float scale, void* out, int out_dtype, float* lse, int32_t* flags, cudaStream_t st);
 
 
-// tcgen05 prefill path (d_qk = d_v = 128; 1, 2 or 4 query heads per KV head)
+// tcgen05 prefill path (d_qk = d_v = 128)
 bool prefill_umma_supported(const Layout& y);
 cudaError_t launch_prefill_umma(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
                                 const int32_t* kv_lens, const int32_t* q_offs, int max_q_len, int window, const void* q,
-                                float scale, void* out, int out_dtype, float* lse, int32_t* flags, cudaStream_t st);
+                                float scale, void* out, int out_dtype, float* lse, int32_t* flags, cudaStream_t st,
+                                const PrefillExtra& x);
 
-// tcgen05 prefill path for d_qk = d_v = 256 and for d_qk 192 / d_v 128 (1, 2 or 4 query heads per KV head): one 128-row
+// tcgen05 prefill path for d_qk = d_v = 256 and for d_qk 192 / d_v 128: one 128-row
 // tile per CTA, two score buffers
 bool prefill_umma_1tile_supported(const Layout& y);
 cudaError_t launch_prefill_umma_1tile(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
                                    const int32_t* kv_lens, const int32_t* q_offs, int max_q_len, int window,
                                    const void* q, float scale, void* out, int out_dtype, float* lse, int32_t* flags,
-                                   cudaStream_t st);
+                                   cudaStream_t st, const PrefillExtra& x);
 
 // tcgen05 prefill path for the MLA-latent cache (V aliasing K, d_qk 576, d_v 512)
 bool prefill_mla_supported(const Layout& y);
