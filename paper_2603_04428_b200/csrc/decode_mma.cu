@@ -1026,7 +1026,10 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   if (P.q_offs) {                                        // a prefill batch need not hold an agent with one query
     bool any = false;
     for (int a = threadIdx.x; a < P.n_agents; a += NW * 32) any |= P.q_offs[a + 1] - P.q_offs[a] == 1;
-    if (!__syncthreads_or(any)) return;
+    if (!__syncthreads_or(any)) {
+      grid_dependency_wait();                            // or this grid could complete before the one it follows
+      return;
+    }
   }
   // ---- this CTA's unit range and its first two segments: one warp, the others set up shared memory (lengths and block
   // tables are inputs that no kernel writes) ----
