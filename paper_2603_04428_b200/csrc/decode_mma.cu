@@ -169,7 +169,13 @@ struct DecodeParams {
   int32_t* flags;
   const uint16_t* k_new;      // fused append: bf16 [A][Hkv][D] rows of the token at position kv_len - 1 (null: none)
   const uint16_t* v_new;
-  const int32_t* q_offs;      // prefill batch: attend for the agents with exactly one query, row q_offs[a]; or null
+  const int32_t* q_offs;      // kSingles: see Params
+};
+// kSingles: the batch of a prefill call, in which this launch takes the agents with exactly one query (row q_offs[a]).  An
+// instantiation of its own: the look-ups cost the others 1-4 % as a run-time branch.
+template <bool kSinglesOnly>
+struct Params : DecodeParams {
+  static constexpr bool kSingles = kSinglesOnly;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -178,13 +184,14 @@ struct DecodeParams {
 struct AgentRange { int n, lo, cf, nc; };   // keys [lo, n); chunks cf .. cf+nc-1
 
 // len_cap: the host's bound on every length (at most max_blocks * 256); longer or negative lengths are rejected
-__device__ inline AgentRange agent_range(const DecodeParams& P, int a, bool& bad) {
+template <class Par>
+__device__ inline AgentRange agent_range(const Par& P, int a, bool& bad) {
   AgentRange r;
   const int li = P.layer_count > 1 ? a / P.n_real : 0;
   const int window = P.windows[li];
   r.n = P.kv_lens[a - li * P.n_real];
   bad = r.n < 0 || r.n > P.len_cap;
-  if (P.q_offs) {
+  if (Par::kSingles) {
     const bool one = P.q_offs[a + 1] - P.q_offs[a] == 1;
     bad = one && (bad || r.n < 1);
     if (!one) r.n = 0;
@@ -221,7 +228,8 @@ struct RangeStart {
 
 // The agent that contains the CTA's first unit, among more than 32 of them (out of line: instruction fetches are what a
 // launch starts with).
-__device__ __noinline__ void find_agent(const DecodeParams& P, RangeStart& rs) {
+template <class Par>
+__device__ __noinline__ void find_agent(const Par& P, RangeStart& rs) {
   const int lane = threadIdx.x & 31;
   uint32_t cum = 0;
 #pragma unroll 1
@@ -247,7 +255,8 @@ __device__ __noinline__ void find_agent(const DecodeParams& P, RangeStart& rs) {
   }
 }
 
-__device__ inline RangeStart find_range(const DecodeParams& P, int cta, int grid, uint32_t nw) {
+template <class Par>
+__device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_t nw) {
   const int lane = threadIdx.x & 31;
   const int n_agents = P.n_agents, Hkv = P.Hkv;
   RangeStart rs;
@@ -348,18 +357,19 @@ struct Segment {
   int a, hk, c0, c1;      // (virtual) agent, head set, logical chunk indices [c0, c1) of the agent
   int ar, li;             // real agent (lengths, block table) and layer of the call (pool layer)
   int n, lo;              // key range of the agent
-  int row;                // query row of the agent
+  int row;                // query row of the agent (kSingles)
   int cf, nc;             // the pair's whole chunk range
   int k0;                 // running chunk counter of the CTA at c0
   int first, last;        // CTAs that hold the pair's first and last chunk
 };
 
 // The one segment of a CTA that holds a part of one pair.
-__device__ inline void whole_segment(const DecodeParams& P, const RangeStart& rs, Segment& s) {
+template <class Par>
+__device__ inline void whole_segment(const Par& P, const RangeStart& rs, Segment& s) {
   s.li = P.layer_count > 1 ? rs.agent / P.n_real : 0; s.ar = rs.agent - s.li * P.n_real;
   s.a = rs.agent; s.hk = rs.pair; s.c0 = rs.r.cf + (int)rs.u_begin; s.c1 = rs.r.cf + (int)rs.u_end;
   s.n = rs.r.n; s.lo = rs.r.lo; s.cf = rs.r.cf; s.nc = rs.r.nc; s.k0 = 0;
-  s.row = P.q_offs ? P.q_offs[rs.agent] : rs.agent;
+  if (Par::kSingles) s.row = P.q_offs[rs.agent];
   s.first = (int)blockIdx.x - rs.split;
   s.last = s.first + rs.splits - 1;
 }
@@ -370,7 +380,8 @@ struct Walker {
   int k, a, hk, c;
   AgentRange r;
 
-  __device__ __forceinline__ void init(const DecodeParams& P_, const RangeStart& rs) {
+  template <class Par>
+  __device__ __forceinline__ void init(const Par& P_, const RangeStart& rs) {
     n_agents = P_.n_agents; Hkv = P_.Hkv;
     u = rs.u_begin; u_end = rs.u_end; k = 0;
     a = rs.agent; hk = 0; c = 0;
@@ -385,14 +396,15 @@ struct Walker {
       }
     }
   }
-  __device__ __forceinline__ bool next(const DecodeParams& P, const RangeStart& rs, Segment& s) {
+  template <class Par>
+  __device__ __forceinline__ bool next(const Par& P, const RangeStart& rs, Segment& s) {
     if (u >= u_end || a < 0) { s.a = -1; return false; }
     const int pair_end = r.cf + r.nc;
     const uint32_t left = u_end - u;
     const int c1 = (uint32_t)(pair_end - c) <= left ? pair_end : c + (int)left;
     s.li = P.layer_count > 1 ? a / P.n_real : 0; s.ar = a - s.li * P.n_real;
     s.a = a; s.hk = hk; s.c0 = c; s.c1 = c1; s.n = r.n; s.lo = r.lo; s.cf = r.cf; s.nc = r.nc; s.k0 = k;
-    s.row = P.q_offs ? P.q_offs[a] : a;
+    if (Par::kSingles) s.row = P.q_offs[a];
     const int cnt = c1 - c;
     s.first = s.last = 0;
     if (cnt != r.nc) {
@@ -857,8 +869,8 @@ __device__ __forceinline__ void deposit(Smem<G, H>& sm, int warp, int lane, Warp
 
 // Combine the eight warps' deposits of a segment: unit `unit` (one warp each).  A pair that lies wholly inside this CTA is
 // normalised and written out, otherwise the combination becomes this CTA's partial record.
-template <int G, int H>
-__device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const DecodeParams& P, const Segment& seg, int cta, int unit,
+template <int G, int H, class Par>
+__device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const Par& P, const Segment& seg, int cta, int unit,
                                                  int lane) {
   constexpr int Dv = Smem<G, H>::Dv, NW = Smem<G, H>::NW;
   const int g = lane >> 2, tid = lane & 3, n_rep = P.n_rep;
@@ -902,7 +914,7 @@ __device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const Dec
   }
   const float L0 = __shfl_sync(0xffffffffu, L, h0), L1 = __shfl_sync(0xffffffffu, L, h0 + 1);
   const int d = H == 4 ? 32 * unit + g + 8 * (tid >> 1) : 16 * unit + g, step = H == 4 ? 16 : 8;
-  const size_t row0 = (size_t)seg.row * P.y.Hq + (size_t)seg.hk * n_rep;
+  const size_t row0 = (size_t)(Par::kSingles ? seg.row : seg.a) * P.y.Hq + (size_t)seg.hk * n_rep;
   if (whole) {
     const float i0 = L0 > 0.f ? 1.f / L0 : 0.f, i1 = L1 > 0.f ? 1.f / L1 : 0.f;
     if (h0 < n_rep) { store_out(P, (row0 + h0) * Dv + d, a[0] * i0); store_out(P, (row0 + h0) * Dv + d + step, a[2] * i0); }
@@ -969,12 +981,13 @@ __device__ __forceinline__ void combine_records(const DecodeParams& P, const flo
 }
 
 // Agents first, first + step, ... without any key (kv_len == 0 or a rejected length): zeros, lse = -inf.
-__device__ __forceinline__ void clear_empty_agents(const DecodeParams& P, int first, int step, int Dv, int lane) {
+template <class Par>
+__device__ __forceinline__ void clear_empty_agents(const Par& P, int first, int step, int Dv, int lane) {
 #pragma unroll 1
   for (int a = first; a < P.n_agents; a += step) {
     bool bad_len;
-    if (agent_range(P, a, bad_len).nc > 0 || (P.q_offs && P.q_offs[a + 1] - P.q_offs[a] != 1)) continue;
-    const size_t row = P.q_offs ? P.q_offs[a] : a;
+    if (agent_range(P, a, bad_len).nc > 0 || (Par::kSingles && P.q_offs[a + 1] - P.q_offs[a] != 1)) continue;
+    const size_t row = Par::kSingles ? P.q_offs[a] : a;
 #pragma unroll 1
     for (int i = lane; i < P.y.Hq * Dv; i += 32) store_out(P, row * P.y.Hq * Dv + i, 0.f);
 #pragma unroll 1
@@ -990,7 +1003,8 @@ __device__ __forceinline__ uint32_t chunk_offset(const DecodeParams& P, const Se
   return (uint32_t)(((uint64_t)s.li * P.y.layer_bytes + (uint64_t)blk * P.y.block_bytes +
                      (uint64_t)(s.hk / P.sets) * P.y.head_block_bytes + (uint64_t)(c & 7) * chunk_bytes) >> 4);
 }
-__device__ __noinline__ uint32_t batch_offsets(const DecodeParams& P, const RangeStart& rs, int nw, int warp, int b, uint32_t chunk_bytes) {
+template <class Par>
+__device__ __noinline__ uint32_t batch_offsets(const Par& P, const RangeStart& rs, int nw, int warp, int b, uint32_t chunk_bytes) {
   Segment s;
   uint32_t off = kOffBad;
   const int my_k = warp + nw * (32 * b + (int)(threadIdx.x & 31)), end = min((int)(rs.u_end - rs.u_begin), nw * 32 * (b + 1));
@@ -1009,8 +1023,8 @@ __device__ __noinline__ uint32_t batch_offsets(const DecodeParams& P, const Rang
   return off;
 }
 
-template <int G, int H, bool kBf>
-__global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kernel(const __grid_constant__ DecodeParams P) {
+template <int G, int H, bool kBf, bool kSingles>
+__global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kernel(const __grid_constant__ Params<kSingles> P) {
   using S = Smem<G, H>;
   constexpr int NW = S::NW, D = S::D, Gv = S::Gv, Dv = S::Dv, kSlots = S::kSlots, kValSlots = S::kValSlots;
   constexpr bool kHalves = S::kHalves;
@@ -1023,7 +1037,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   const int n_rep = P.n_rep;
 
   grid_launch_dependents();
-  if (P.q_offs) {                                        // a prefill batch need not hold an agent with one query
+  if (kSingles) {                                        // a prefill batch need not hold an agent with one query
     bool any = false;
     for (int a = threadIdx.x; a < P.n_agents; a += NW * 32) any |= P.q_offs[a + 1] - P.q_offs[a] == 1;
     if (!__syncthreads_or(any)) {
@@ -1095,7 +1109,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   const int g = lane >> 2, tid = lane & 3;
   // this warp's row of a segment's query; the new row's groups are quantized by the warps behind the query's (from 4 on)
   constexpr int kNewWarps = NW - 4, kNewRounds = (G + Gv + kNewWarps - 1) / kNewWarps;
-  auto query_row = [&](const Segment& s) { return P.q + ((size_t)s.row * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
+  auto query_row = [&](const Segment& s) { return P.q + ((size_t)(kSingles ? s.row : s.a) * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
   auto new_pair = [&](const Segment& s, int grp) {
     const size_t head = (size_t)s.a * y.Hkv + s.hk;
     return (grp < G ? P.k_new + head * D + 64 * grp : P.v_new + head * Dv + 64 * (grp - G)) + 2 * lane;
@@ -1249,7 +1263,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
     if (warp == NW - 1 && lane == 0) {
       if (seg.c1 - c0 != seg.nc) {                       // only the first and the last segment can be parts of a pair
         int* f = sm.fin[k0 == 0 ? 0 : 1];
-        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = seg.row * y.Hq + seg.hk * n_rep;
+        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = (kSingles ? seg.row : seg.a) * y.Hq + seg.hk * n_rep;
       }
       if (more) sm.walker.next(P, sm.range, sm.seg[(si + 2) % 3]);       // never where the CTA holds one segment
     }
@@ -1290,8 +1304,8 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   }
 }
 
-template <int G, int H, bool kBf>
-cudaError_t launch_g(const DecodeParams& P, int grid, cudaStream_t st) {
+template <int G, int H, bool kBf, bool kSingles>
+cudaError_t launch_g(const DecodeParams& P_, int grid, cudaStream_t st) {
   static bool configured[64] = {};     // the attributes are per function and device: set them once for each
   constexpr size_t smem = sizeof(Smem<G, H>);
   static_assert(smem <= 227 * 1024 / kCtasPerSm - 1024, "two CTAs per SM");
@@ -1299,9 +1313,9 @@ cudaError_t launch_g(const DecodeParams& P, int grid, cudaStream_t st) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf, kSingles>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    e = cudaFuncSetAttribute(decode_mma_kernel<G, H, kBf, kSingles>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
@@ -1315,11 +1329,14 @@ cudaError_t launch_g(const DecodeParams& P, int grid, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_mma_kernel<G, H, kBf>, P);
+  Params<kSingles> P;
+  static_cast<DecodeParams&>(P) = P_;
+  return cudaLaunchKernelEx(&cfg, decode_mma_kernel<G, H, kBf, kSingles>, P);
 }
 template <int G, int H>
 cudaError_t launch_gh(const DecodeParams& P, int grid, cudaStream_t st) {
-  return P.y.sb_bf16 ? launch_g<G, H, true>(P, grid, st) : launch_g<G, H, false>(P, grid, st);
+  if (P.q_offs) return P.y.sb_bf16 ? launch_g<G, H, true, true>(P, grid, st) : launch_g<G, H, false, true>(P, grid, st);
+  return P.y.sb_bf16 ? launch_g<G, H, true, false>(P, grid, st) : launch_g<G, H, false, false>(P, grid, st);
 }
 
 // Sets of query heads a KV head's heads are cut into: the kernel's columns take four of them, or eight at d = 128

@@ -72,7 +72,7 @@ struct MlaPrefillParams {
 struct MlaSmem {
   alignas(128) uint8_t khat[kStages][64 * kD * 2];       // [key][dim]: (n%8)*16 + (n/8)*kSboK + (k/8)*128
   alignas(128) uint8_t qs[128 * kQSmem * 2];             // [row][dim - 256]: (m%8)*16 + (m/8)*kSboQ + (k/8)*128
-  alignas(8) uint64_t a_full[kStages], b_full[kStages], a_free[kStages], b_free[kStages], s_full[2], p_full[2], o_done, q_ready, drain;
+  alignas(8) uint64_t a_full[kStages], b_full[kStages], a_free[kStages], b_free[kStages], s_full[2], p_full[2], o_done, o_last, q_ready, drain;
   uint32_t tmem_base;
   int abort_flag, poisoned;
 };
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     }
     for (int b = 0; b < 2; ++b) { mbar_init(&sm.s_full[b], 1); mbar_init(&sm.p_full[b], kSoftmaxWarps * 32); }
     mbar_init(&sm.o_done, 1);
+    mbar_init(&sm.o_last, 1);
     mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0; sm.poisoned = 0;
@@ -232,13 +233,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
         }
         __syncwarp();
       };
-      auto issue_pv = [&](int b, int s, bool first) {    // O (+)= P_b V^; afterwards the stage is free
+      auto issue_pv = [&](int b, int s, bool first, bool last) {    // O (+)= P_b V^; afterwards the stage is free
         const uint64_t vd = smem_desc(smem_u32(sm.khat[s]) + hv * (kDvCta / 8) * 128, kSboK, 128);
         if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + (2 * kSboK / 16) * k, kIdescO, (!first || k > 0) ? 1u : 0u);
           commit(&sm.o_done);
+          if (last) commit(&sm.o_last);
           commit(&sm.b_free[s]);
         }
         __syncwarp();
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
         while (ok && np < n_iter) {
           if (np < nb && __all_sync(0xffffffffu, mbar_test_wait(&sm.p_full[np & 1], (uint32_t)(np >> 1) & 1u))) {
             fence_after_sync();
-            issue_pv(np & 1, np % kStages, np == 0);
+            issue_pv(np & 1, np % kStages, np == 0, np + 1 == n_iter);
             ++np;
             idle = 0;
           }
@@ -330,7 +332,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
       uint32_t sr[64];
       tmem_ld32(lane_addr + kColS + 64 * b, sr);
       tmem_ld32(lane_addr + kColS + 64 * b + 32, sr + 32);
-      wait_ld();
+      wait_ld32(sr);
+      wait_ld32(sr + 32);
       const int pos0 = (it0 + j) * 64;
       // column c is key pos0 + c; causal and window masks on edge blocks only
       if (pos0 + 63 > pq || (W > 0 && pos0 <= pq - W)) {
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
           for (int part = 0; part < kDvCta / 16; ++part) {
             uint32_t orow[16];
             tmem_ld16(lane_addr + kColO + 16 * part, orow);
-            wait_ld();
+            wait_ld16(orow);
 #pragma unroll
             for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
             tmem_st16(lane_addr + kColO + 16 * part, orow);
@@ -386,7 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     }
     // ---- normalise and write the row, or leave it as a record ----
     bool ok = !*abort_flag;
-    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_done, (uint32_t)(n_iter - 1), abort_flag);
+    // (the last two value products may both be under way, and a wait on o_done could not tell which phase it sees)
+    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_last, 0, abort_flag);
     ok = __all_sync(0xffffffffu, ok);                    // the loads below are warp-wide
     if (ok) fence_after_sync();
     const bool bad = !ok || sm.poisoned != 0;
@@ -399,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
       uint32_t orow[32];
       if (ok && n_iter > 0) {
         tmem_ld32(lane_addr + kColO + 32 * part, orow);
-        wait_ld();
+        wait_ld32(orow);
       }
       if (!mine) continue;
       const int d0 = kDvCta * hv + 32 * part;

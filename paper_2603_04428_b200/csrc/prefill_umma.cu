@@ -5,24 +5,28 @@
 //
 // Prefill is a dense contraction, so it runs on the fifth-generation tensor cores, and the 4-bit
 // cache is expanded exactly once per CTA and key block, not once per query row:
-//   * A CTA owns 256 score rows = two tiles of 128 rows (128 / n_rep consecutive queries x the n_rep
-//     heads of one KV head) and walks the keys 64 at a time (two 32-token chunks, one bulk copy).
-//   * Four "dequantize" warps turn each raw block into binary16 tiles K^ [64 keys][128 dims] and
-//     V^ [128 dims][64 keys] in shared memory, in the core-matrix order a K-major tcgen05 operand
-//     wants: x^ = c * s + b in one binary16 fma per pair of codes (the code is made a binary16
-//     integer by or-ing the masked nibble into the mantissa of 1024 or 64 and subtracting), i.e.
-//     each value is rounded once, to 11 significant bits.  A packed word becomes one 16-byte row of
-//     a core matrix; the order of the eight elements inside a row (0,4,1,5,2,6,3,7) is absorbed by
-//     storing the queries, and the key rows, in the same order.
-//   * One thread issues the MMAs: S_t = Q_t K^T (M 128, N 64, K 128) with Q_t resident in tensor
-//     memory as packed binary16 (each bf16 query row scaled by a power of two, so nothing is
-//     rounded), and O_t += P_t V^ (M 128, N 128, K 64) with P_t read from tensor memory too; the
-//     f32 accumulators S_t and O_t live in tensor memory (512 columns: O 2 x 128, S 2 x 64, Q 2 x 64;
-//     P_t overlays S_t).  Only the B operands come from shared memory, which keeps the operand
-//     traffic at half of the shared-memory bandwidth and leaves the rest to the dequantize warps.
-//   * Sixteen softmax warps, two threads per score row (a tensor-memory lane; each takes 32 of the
-//     64 scores): mask, online softmax with a lazily updated reference maximum (the accumulator is
-//     rescaled only when the maximum has grown by more than 2^8), write P_t as packed binary16.
+//   * A CTA owns 256 score rows = two tiles of 128 rows (128 / n_rep consecutive queries x the n_rep heads of one KV head)
+//     and walks the keys 128 at a time.  Per such step the tensor pipe is needed for 2100 clocks, the exponential unit for
+//     2050, shared memory for 2300 (operands 1570, tiles written 510, raw blocks 150) and the issue slots for 1700, so what
+//     matters is that all of them work at once: few, long hand-offs.  (Steps of 64 keys with the queries in tensor memory and
+//     two threads per row, which exchanged their maxima, took 2 x 3000 clocks.)  Measured on 8 agents x (8192 + 1024 tokens),
+//     32 / 8 heads: 5300 clocks per step, 1616 -> 1290 us per launch = 905 TFLOP/s (723 before).  What is left is the chain of
+//     a tile's step -- scores 330 clocks after their product, exponentials 2 x 1500, value and score products 1700 -- of which
+//     the two tiles overlap a half.  Measured without gain: four softmax warps per row pair (16 in all), score buffers of 64
+//     keys issued two blocks ahead, an issuing warp per tile (the tiles then fall into step), scores fetched ahead.
+//   * Eight "dequantize" warps turn each raw 64-key block into binary16 tiles K^ [64 keys][128 dims] and V^ [128 dims][64
+//     keys] in shared memory (four of each), in the core-matrix order a K-major tcgen05 operand wants: x^ = c * s + b in one
+//     binary16 fma per pair of codes (the code is made a binary16 integer by or-ing the masked nibble into the mantissa of
+//     1024 or 64 and subtracting), i.e. each value is rounded once, to 11 significant bits.  A packed word becomes one 16-byte
+//     row of a core matrix; the order of the eight elements inside a row (0,4,1,5,2,6,3,7) is absorbed by storing the queries,
+//     and the key rows, in the same order.
+//   * One thread issues the MMAs: S_t = Q_t K^T (M 128, N 128, K 128) with Q_t in shared memory as binary16 (each bf16 query
+//     row scaled by a power of two, so nothing is rounded), and O_t += P_t V^ (M 128, N 128, K 128) with P_t read from tensor
+//     memory.  The f32 accumulators fill the tensor memory (O 2 x 128, S 2 x 128); P_t overlays S_t.  At
+//     N = 128 a product whose A operand is in shared memory runs at the full rate (66 clocks per instruction).
+//   * Eight softmax warps, one thread per score row (a tensor-memory lane): mask, online softmax with a lazily updated
+//     reference maximum (the accumulator is rescaled only when the maximum has grown by more than 2^8), P_t as packed
+//     binary16, in halves of 64 keys, so that the first half's value product runs under the second half's exponentials.
 //     The two tiles alternate, so one tile's softmax overlaps the other tile's MMAs.
 //   * One warp streams the raw blocks through a small ring with bulk asynchronous copies.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
@@ -36,15 +40,18 @@ namespace {
 using namespace tc;
 using namespace prefill;
 
-constexpr int kSoftmaxWarps = 16, kDequantWarps = 4;
+constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
 constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps, kLoadWarp = kMmaWarp + 1;
-constexpr int kThreads = (kLoadWarp + 1) * 32;           // 704
-constexpr int kStages = 3;                               // K^ / V^ tiles in flight
-constexpr int kRawSlots = 4;                             // raw 64-key blocks in flight
+constexpr int kThreads = (kMmaWarp + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps), ...
+// ... launched with 96 registers per thread; the softmax warpgroups take 144, the others keep 64 (61440 in all)
+constexpr int kRegsSoftmax = 144, kRegsOther = 64;
+static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * 96, "");
+constexpr int kStages = 4;                               // K^ / V^ tiles of 64 keys in flight: two steps
+constexpr int kRawSlots = 3;                             // raw 64-key blocks in flight
 constexpr int kChunkBytes = 4608;                        // d = 128: [Kc 2048 | Ksb 256 | Vc 2048 | Vsb 256]
 constexpr int kRawBytes = 2 * kChunkBytes;
 constexpr int kTileBytes = 64 * 128 * 2;                 // one binary16 tile
-constexpr uint32_t kColO = 0, kColS = 256, kColQ = 384;  // tensor-memory columns (+128 t, +64 t, +64 t)
+constexpr uint32_t kColO = 0, kColS = 256;               // tensor-memory columns (+128 t; P inside S)
 
 struct UmmaParams {
   Layout y;
@@ -64,16 +71,15 @@ struct UmmaParams {
 };
 
 struct UmmaSmem {
+  alignas(128) uint8_t qs[2][128 * 128 * 2];             // [row][dim]: (m%8)*16 + (m/8)*2048 + (k/8)*128
   alignas(128) uint8_t khat[kStages][kTileBytes];        // [key 64][dim 128]: (n%8)*16 + (n/8)*2048 + (k/8)*128
   alignas(128) uint8_t vhat[kStages][kTileBytes];        // [dim 128][key 64]: (n%8)*16 + (n/8)*1024 + (k/8)*128
   alignas(128) uint8_t raw[kRawSlots][kRawBytes];
   alignas(8) uint64_t raw_full[kRawSlots], raw_free[kRawSlots], sb_done[kRawSlots];
-  uint64_t k_full[kStages], v_full[kStages], kv_free[kStages];
-  uint64_t s_full[2], p_full[2], o_done[2], q_ready, drain;
+  uint64_t k_full[kStages], v_full[kStages], k_free[kStages / 2], v_free[kStages / 2];   // free: a step's two tiles
+  uint64_t s_full[2], p_full[2][2], o_half[2], o_done[2], q_ready, drain;    // p_full: [tile][half of the step]
   uint32_t tmem_base;
   int bad[kRawSlots];
-  float xchg[2][2][2][128];                              // [tile][parity][column half][row]: maxima / sums of the two threads of a row
-  int stop[2][3], spoiled[2];
   int abort_flag, poisoned;
 };
 
@@ -101,20 +107,22 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
   const int W = P.window;
   const int c_end = bad_len ? 0 : (prefix + i_max) / 32 + 1;
   const int c_begin = (bad_len || W == 0) ? 0 : max(0, prefix + i_min - W + 1) >> 5;
-  const int all0 = c_begin >> 1, n_all = max(0, ((c_end + 1) >> 1) - all0);
-  const int it0 = all0 + n_all * split / P.x.n_splits;   // 64-key blocks it0 .. it0 + n_iter - 1
-  const int n_iter = all0 + n_all * (split + 1) / P.x.n_splits - it0;
+  // steps of 128 keys (the last one may reach past the end, inside its pool block: zeros)
+  const int all0 = c_begin >> 2, n_all = max(0, ((c_end + 3) >> 2) - all0);
+  const int st0 = all0 + n_all * split / P.x.n_splits;   // steps st0 .. st0 + n_step - 1
+  const int n_step = all0 + n_all * (split + 1) / P.x.n_splits - st0;
+  const int it0 = 2 * st0, n_iter = 2 * n_step;          // 64-key blocks
 
   if (threadIdx.x == 0) {
     if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
     for (int s = 0; s < kRawSlots; ++s) { mbar_init(&sm.raw_full[s], 1); mbar_init(&sm.raw_free[s], kDequantWarps); mbar_init(&sm.sb_done[s], kDequantWarps); sm.bad[s] = 0; }
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.v_full[s], kDequantWarps); mbar_init(&sm.kv_free[s], 1);
+    for (int s = 0; s < kStages; ++s) { mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.v_full[s], kDequantWarps); }
+    for (int s = 0; s < kStages / 2; ++s) { mbar_init(&sm.k_free[s], 1); mbar_init(&sm.v_free[s], 1); }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(&sm.s_full[t], 1); mbar_init(&sm.o_half[t], 1); mbar_init(&sm.o_done[t], 1);
+      mbar_init(&sm.p_full[t][0], 4); mbar_init(&sm.p_full[t][1], 4);
     }
-    for (int t = 0; t < 2; ++t) { mbar_init(&sm.s_full[t], 1); mbar_init(&sm.p_full[t], 256); mbar_init(&sm.o_done[t], 1); }
-    mbar_init(&sm.q_ready, 512);
-    for (int i = 0; i < 6; ++i) (&sm.stop[0][0])[i] = 0;
-    sm.spoiled[0] = 0; sm.spoiled[1] = 0;
+    mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0; sm.poisoned = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -128,13 +136,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the new tokens were appended by the preceding kernel
   volatile int* abort_flag = &sm.abort_flag;
 
-  if (warp == kLoadWarp) {
+  if (warp >= kMmaWarp) {
+    fewer_registers<kRegsOther>();
+    if (warp == kLoadWarp) {
     // =============================== raw block loader ==========================================
     if (lane == 0) {
       int issued = 0;
       for (int j = 0; j < n_iter; ++j) {
         const int r = j % kRawSlots;
-        if (j >= kRawSlots && !mbar_wait(&sm.raw_free[r], (uint32_t)(j / kRawSlots - 1), abort_flag)) break;
+        if (j >= kRawSlots && !mbar_doze(&sm.raw_free[r], (uint32_t)(j / kRawSlots - 1), abort_flag)) break;
         const int c = 2 * (it0 + j);
         const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
         if (blk < 0 || blk >= P.n_blocks) {
@@ -158,54 +168,110 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         }
       }
     }
-  } else if (warp >= kSoftmaxWarps && warp < kMmaWarp) {
+    } else if (warp == kMmaWarp) {
+    // =============================== MMA issue ==================================================
+    // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
+    if (n_step > 0) {
+      constexpr uint32_t kIdesc = idesc_f16(128, 128);
+      // one election for a whole product: an election per MMA costs more issue time than the MMA takes
+      auto issue_qk = [&](int t, int s) {                // S_t = Q_t K^T over the tiles 2 s, 2 s + 1
+        const uint64_t qd = smem_desc(smem_u32(sm.qs[t]), 128, 2048), kd = smem_desc(smem_u32(sm.khat[2 * s]), 128, 2048);
+        if (elect_one()) {
+#pragma unroll                                           // rolled, every MMA waits for its own operand arithmetic: 2x slower
+          for (int k = 0; k < 8; ++k) mma_f16_ss(tb + kColS + 128 * t, qd + 16 * k, kd + 16 * k, kIdesc, k > 0);
+          commit(&sm.s_full[t]);
+          if (t == 1) commit(&sm.k_free[s]);             // both tiles' products have been issued
+        }
+        __syncwarp();
+      };
+      auto issue_pv = [&](int t, int s, int half, bool first) {    // O_t (+)= P_t V^ over half of the step's keys
+        const uint64_t vd = smem_desc(smem_u32(sm.vhat[2 * s + half]), 128, 1024);
+        if (elect_one()) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_f16_ts(tb + kColO + 128 * t, tb + kColS + 128 * t + 64 * half + 8 * k, vd + 16 * k, kIdesc, (!first || k > 0) ? 1u : 0u);
+          commit(half == 0 ? &sm.o_half[t] : &sm.o_done[t]);
+          if (t == 1 && half == 1) commit(&sm.v_free[s]);
+        }
+        __syncwarp();
+      };
+      auto wait = [&](uint64_t* bar, int use) {
+        const bool ok = mbar_wait(bar, (uint32_t)use, abort_flag);
+        if (ok) fence_after_sync();
+        return ok;
+      };
+      auto wait_tiles = [&](uint64_t* bars, int j) {     // both tiles of step j
+        const int s = 2 * (j & 1);
+        return wait(&bars[s], j >> 1) && wait(&bars[s + 1], j >> 1);
+      };
+      bool ok = wait(&sm.q_ready, 0) && wait_tiles(sm.k_full, 0);
+      if (ok) {
+        issue_qk(0, 0);
+        issue_qk(1, 0);
+      }
+      for (int j = 0; ok && j < n_step; ++j) {
+#pragma unroll 1
+        for (int t = 0; t < 2 && ok; ++t) {
+          ok = wait(&sm.p_full[t][0], j) && (t == 1 || wait(&sm.v_full[2 * (j & 1)], j >> 1));
+          if (!ok) break;
+          issue_pv(t, j & 1, 0, j == 0);
+          ok = wait(&sm.p_full[t][1], j) && (t == 1 || wait(&sm.v_full[2 * (j & 1) + 1], j >> 1));
+          if (!ok) break;
+          issue_pv(t, j & 1, 1, false);
+          if (j + 1 < n_step) {
+            if (t == 0) ok = wait_tiles(sm.k_full, j + 1);
+            if (!ok) break;
+            issue_qk(t, (j + 1) & 1);
+          }
+        }
+      }
+    }
+    }
+  } else if (warp >= kSoftmaxWarps) {
+    fewer_registers<kRegsOther>();
     // =============================== dequantize warps ==========================================
-    const int x = threadIdx.x - kSoftmaxWarps * 32;      // 0..127
-    // K: one 16-byte piece (words w = 4j + kt, j = 0..3) of token tau = 4 kg + ki per chunk.  The eight lanes
+    const int x = threadIdx.x - kSoftmaxWarps * 32, ci = x >> 7, x7 = x & 127;     // ci: the thread's chunk of the block
+    // K: one 16-byte piece (words w = 4j + kt, j = 0..3) of token tau = 4 kg + ki.  The eight lanes
     // of a shared-memory phase read eight different 16-byte columns and write eight different rows.
-    const int ki = x & 3, kg = 2 * ((x >> 3) & 3) + ((x >> 2) & 1), kt = (ki + (x >> 5)) & 3;
+    const int ki = x & 3, kg = 2 * ((x >> 3) & 3) + ((x >> 2) & 1), kt = (ki + (x7 >> 5)) & 3;
     const int ktau = 4 * kg + ki;
-    const int k_read = (ki * 32 + kg * 4 + kt) * 16;
-    const int k_sb = 2048 + (((ktau & 3) * 4 + (ktau >> 3)) * 2 + ((ktau >> 2) & 1)) * 8;
-    const int k_row = 8 * (ktau >> 3) + slot_of(ktau & 7);       // row of the token inside its chunk's 32 rows
-    // V: one 16-byte piece (dims 32 vq + 8 k + vr, k = 0..3) of token octet vo per chunk.
-    const int vr = x & 7, vq = (x >> 3) & 3, vo = ((vr >> 1) + (x >> 5)) & 3;
-    const int v_read = 2304 + ((vq * 8 + vr) * 4 + vo) * 16;
-    const int v_sb = 4352 + (vo * 2 * 2 + (vq >> 1)) * 4;        // + i * 64 + e * 8: token 8 vo + 4 e + i, group vq / 2
+    const int k_read = ci * kChunkBytes + (ki * 32 + kg * 4 + kt) * 16;
+    const int k_sb = ci * kChunkBytes + 2048 + (((ktau & 3) * 4 + (ktau >> 3)) * 2 + ((ktau >> 2) & 1)) * 8;
+    const int k_row = ci * 32 + 8 * (ktau >> 3) + slot_of(ktau & 7);      // row of the token in the tile
+    const int k_write = (k_row & 7) * 16 + (k_row >> 3) * 2048 + kt * 128;
+    // V: one 16-byte piece (dims 32 vq + 8 k + vr, k = 0..3) of token octet vo.
+    const int vr = x & 7, vq = (x >> 3) & 3, vo = ((vr >> 1) + (x7 >> 5)) & 3;
+    const int v_read = ci * kChunkBytes + 2304 + ((vq * 8 + vr) * 4 + vo) * 16;
+    const int v_sb = ci * kChunkBytes + 4352 + (vo * 2 * 2 + (vq >> 1)) * 4;        // + i * 64 + e * 8: token 8 vo + 4 e + i, group vq / 2
+    const int v_write = vr * 16 + (4 * vq) * 1024 + (ci * 4 + vo) * 128;
     for (int j = 0; j < n_iter; ++j) {
       const int s = j % kStages, r = j % kRawSlots;
-      if (j >= kStages && !mbar_wait(&sm.kv_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
-      if (!mbar_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
+      if (j >= kStages && !mbar_doze(&sm.k_free[s >> 1], (uint32_t)(j / kStages - 1), abort_flag)) break;
+      if (!mbar_doze(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
       const bool bad = sm.bad[r] != 0;
-      const int pos_base = (it0 + j) * 64;
+      const int pos_base = (it0 + j) * 64 + ci * 32;
+      const uint8_t* raw = sm.raw[r];
       if (kBf) {
-        // bfloat16 scales and biases become binary16 in place, once per block (the tiles are binary16); only the
-        // tokens below the agent's length count for the range report (bytes past the end are whatever was there)
-        bool overflow = false;
-        for (int w = x; w < 256; w += kDequantWarps * 32) {              // per chunk: 64 words of Ksb, 64 of Vsb
-          const int ci = w >> 7, o = w & 127;
-          const int row = (o & 63) >> 1;                                 // (i * 4 + tid) * 2 + e: token 8 tid + 4 e + i
-          const int tau = 8 * ((row >> 1) & 3) + 4 * (row & 1) + (row >> 3);
-          uint32_t* at = reinterpret_cast<uint32_t*>(sm.raw[r] + ci * kChunkBytes + (o < 64 ? 2048 + 4 * o : 4352 + 4 * (o - 64)));
-          bool over = false;
-          *at = bf16_pair_to_h2(*at, over);
-          overflow |= over && pos_base + ci * 32 + tau < kv_len;
-        }
-        if (overflow && !bad) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
+        // bfloat16 scales and biases become binary16 in place, once per block (the tiles are binary16), one word per thread;
+        // only the tokens below the agent's length count for the range report (bytes past the end are whatever was there)
+        const int o = x7;                                // 64 words of Ksb, 64 of Vsb
+        const int row = (o & 63) >> 1;                   // (i * 4 + tid) * 2 + e: token 8 tid + 4 e + i
+        const int tau = 8 * ((row >> 1) & 3) + 4 * (row & 1) + (row >> 3);
+        uint32_t* at = reinterpret_cast<uint32_t*>(sm.raw[r] + ci * kChunkBytes + (o < 64 ? 2048 + 4 * o : 4352 + 4 * (o - 64)));
+        bool over = false;
+        *at = bf16_pair_to_h2(*at, over);
+        if (over && !bad && pos_base + tau < kv_len) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.sb_done[r]);
         if (!mbar_wait(&sm.sb_done[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
       }
-#pragma unroll
-      for (int ci = 0; ci < 2; ++ci) {
-        const uint8_t* chunk = sm.raw[r] + ci * kChunkBytes;
-        const uint4 kw = *reinterpret_cast<const uint4*>(chunk + k_read);
-        uint2 sb = *reinterpret_cast<const uint2*>(chunk + k_sb);          // (scale, bias) of groups 0 and 1
-        if (bad || pos_base + ci * 32 + ktau >= kv_len) sb = make_uint2(0u, 0u);   // stale bytes past the end
+      {
+        const uint4 kw = *reinterpret_cast<const uint4*>(raw + k_read);
+        uint2 sb = *reinterpret_cast<const uint2*>(raw + k_sb);            // (scale, bias) of groups 0 and 1
+        if (bad || pos_base + ktau >= kv_len) sb = make_uint2(0u, 0u);     // stale bytes past the end
         const uint32_t s0 = __byte_perm(sb.x, sb.x, 0x1010), b0 = __byte_perm(sb.x, sb.x, 0x3232);
         const uint32_t s1 = __byte_perm(sb.y, sb.y, 0x1010), b1 = __byte_perm(sb.y, sb.y, 0x3232);
-        const int n = ci * 32 + k_row;
-        uint8_t* dst = sm.khat[s] + (n & 7) * 16 + (n >> 3) * 2048 + kt * 128;
+        uint8_t* dst = sm.khat[s] + k_write;
         *reinterpret_cast<uint4*>(dst + 0 * 512) = dequant8(kw.x, s0, b0, s0, b0, s0, b0, s0, b0);
         *reinterpret_cast<uint4*>(dst + 1 * 512) = dequant8(kw.y, s0, b0, s0, b0, s0, b0, s0, b0);
         *reinterpret_cast<uint4*>(dst + 2 * 512) = dequant8(kw.z, s1, b1, s1, b1, s1, b1, s1, b1);
@@ -214,22 +280,21 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.k_full[s]);
-#pragma unroll
-      for (int ci = 0; ci < 2; ++ci) {
-        const uint8_t* chunk = sm.raw[r] + ci * kChunkBytes;
-        const uint4 vw = *reinterpret_cast<const uint4*>(chunk + v_read);
+      if (j >= kStages && !mbar_doze(&sm.v_free[s >> 1], (uint32_t)(j / kStages - 1), abort_flag)) break;
+      {
+        const uint4 vw = *reinterpret_cast<const uint4*>(raw + v_read);
         uint32_t sp[4], bp[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          uint32_t e0 = *reinterpret_cast<const uint32_t*>(chunk + v_sb + i * 64);
-          uint32_t e1 = *reinterpret_cast<const uint32_t*>(chunk + v_sb + i * 64 + 8);
-          const int pos = pos_base + ci * 32 + 8 * vo + i;
+          uint32_t e0 = *reinterpret_cast<const uint32_t*>(raw + v_sb + i * 64);
+          uint32_t e1 = *reinterpret_cast<const uint32_t*>(raw + v_sb + i * 64 + 8);
+          const int pos = pos_base + 8 * vo + i;
           if (bad || pos >= kv_len) e0 = 0u;
           if (bad || pos + 4 >= kv_len) e1 = 0u;
           sp[i] = __byte_perm(e0, e1, 0x5410);                             // scales of tokens i and i + 4
           bp[i] = __byte_perm(e0, e1, 0x7632);                             // biases
         }
-        uint8_t* dst = sm.vhat[s] + vr * 16 + (4 * vq) * 1024 + (ci * 4 + vo) * 128;
+        uint8_t* dst = sm.vhat[s] + v_write;
         *reinterpret_cast<uint4*>(dst + 0 * 1024) = dequant8(vw.x, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
         *reinterpret_cast<uint4*>(dst + 1 * 1024) = dequant8(vw.y, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
         *reinterpret_cast<uint4*>(dst + 2 * 1024) = dequant8(vw.z, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
@@ -239,218 +304,156 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
       __syncwarp();
       if (lane == 0) { mbar_arrive(&sm.v_full[s]); mbar_arrive(&sm.raw_free[r]); }
     }
-  } else if (warp == kMmaWarp) {
-    // =============================== MMA issue ==================================================
-    // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
-    if (n_iter > 0) {
-      constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, 128);
-      // one election for a whole product: an election per MMA costs more issue time than the MMA takes
-      auto issue_qk = [&](int t, int s) {                // S_t = Q_t K^T
-        const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, 2048);
-        if (elect_one()) {
-#pragma unroll                                           // rolled, every MMA waits for its own operand arithmetic: 2x slower
-          for (int k = 0; k < 8; ++k) mma_f16_ts(tb + kColS + 64 * t, tb + kColQ + 64 * t + 8 * k, kd + 16 * k, kIdescS, k > 0);
-          commit(&sm.s_full[t]);
-        }
-        __syncwarp();
-      };
-      auto issue_pv = [&](int t, int s, bool first) {    // O_t (+)= P_t V^
-        const uint64_t vd = smem_desc(smem_u32(sm.vhat[s]), 128, 1024);
-        if (elect_one()) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_f16_ts(tb + kColO + 128 * t, tb + kColS + 64 * t + 8 * k, vd + 16 * k, kIdescO, (!first || k > 0) ? 1u : 0u);
-          commit(&sm.o_done[t]);
-          if (t == 1) commit(&sm.kv_free[s]);            // every MMA that reads stage s has been issued
-        }
-        __syncwarp();
-      };
-      bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
-        fence_after_sync();
-        issue_qk(0, 0);
-        issue_qk(1, 0);
-      }
-      for (int j = 0; ok && j < n_iter; ++j) {
-        const int s = j % kStages, sn = (j + 1) % kStages;
-        for (int t = 0; t < 2 && ok; ++t) {
-          ok = mbar_wait(&sm.p_full[t], (uint32_t)j, abort_flag);
-          if (ok && t == 0) ok = mbar_wait(&sm.v_full[s], (uint32_t)(j / kStages), abort_flag);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          fence_after_sync();
-          issue_pv(t, s, j == 0);
-          if (j + 1 < n_iter) {
-            if (t == 0) ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[sn], (uint32_t)((j + 1) / kStages), abort_flag));
-            if (!ok) break;
-            fence_after_sync();
-            issue_qk(t, sn);
-          }
-        }
-      }
-    }
   } else {
-    // =============================== softmax warps: two threads per score row ===================
-    // Warp w: tile t = w / 8, column half = (w / 4) % 2, tensor-memory lanes 32 (w % 4) ...  The two threads of a
-    // row exchange their block maxima (and at the end their sums) through shared memory; the 256 threads of a
-    // tile meet at a named barrier once per block, and they leave the loop together (one of them samples the
-    // give-up flag before the barrier).
-    const int t = warp >> 3, half = (warp >> 2) & 1;
+    more_registers<kRegsSoftmax>();
+    // =============================== softmax warps: one thread per score row ===================
+    const int t = warp >> 2;
     const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
     const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_addr = lane_addr + kColS + 128 * t, o_addr = lane_addr + kColO + 128 * t;
     const int h = row / tile_q, i = i_min + t * tile_q + row % tile_q;
     const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
     const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
-    const bool sampler = (warp & 7) == 0 && lane == 0;   // one thread per tile
-    auto tile_barrier = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + t) : "memory"); };
+    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
     float kappa;                                         // score in log2 units = S * kappa
     {
-      // ---- stage this thread's half of the query row: bf16 -> binary16 times a power of two, element order
-      //      (0,4,1,5,2,6,3,7) inside every eight ----
-      const uint16_t* qrow = P.q + ((size_t)(q0 + (valid ? i : 0)) * y.Hq + (size_t)hk * n_rep + h) * 128 + 64 * half;
-      uint32_t qa[32];
+      // ---- stage the query row: bf16 -> binary16 times a power of two ----
+      const uint16_t* qrow = P.q + (valid ? row_index : 0) * 128;
+      auto piece = [&](int p) { return valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : make_uint4(0u, 0u, 0u, 0u); };
       float mx = 0.f;
-      if (valid) {
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-          const uint4 v = *reinterpret_cast<const uint4*>(qrow + 8 * w);
-          qa[4 * w] = v.x; qa[4 * w + 1] = v.y; qa[4 * w + 2] = v.z; qa[4 * w + 3] = v.w;
-          mx = fmaxf(mx, fmaxf(fmaxf(fabsf(__uint_as_float(v.x << 16)), fabsf(__uint_as_float(v.x & 0xffff0000u))),
-                               fmaxf(fabsf(__uint_as_float(v.y << 16)), fabsf(__uint_as_float(v.y & 0xffff0000u)))));
-          mx = fmaxf(mx, fmaxf(fmaxf(fabsf(__uint_as_float(v.z << 16)), fabsf(__uint_as_float(v.z & 0xffff0000u))),
-                               fmaxf(fabsf(__uint_as_float(v.w << 16)), fabsf(__uint_as_float(v.w & 0xffff0000u)))));
-        }
-      } else {
-#pragma unroll
-        for (int w = 0; w < 32; ++w) qa[w] = 0u;
-      }
-      sm.xchg[t][1][half][row] = mx;                     // slot 1: block 0 of the loop below writes slot 0
-      tile_barrier();
-      mx = fmaxf(mx, sm.xchg[t][1][half ^ 1][row]);
+#pragma unroll 8
+      for (int p = 0; p < 16; ++p) mx = fmaxf(mx, max_abs8(piece(p)));
       int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
       if (mx == 0.f) ex = 0;
       ex = min(max(ex, -100), 100);
       const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
       kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
-#pragma unroll
-      for (int w = 0; w < 8; ++w) {
-        // elements 8w..8w+7 arrive as bf16 pairs (0,1) (2,3) (4,5) (6,7); columns hold (0,4) (1,5) (2,6) (3,7)
-        const uint32_t u01 = qa[4 * w], u23 = qa[4 * w + 1], u45 = qa[4 * w + 2], u67 = qa[4 * w + 3];
-        const float x0 = __uint_as_float(u01 << 16) * sf, x1 = __uint_as_float(u01 & 0xffff0000u) * sf;
-        const float x2 = __uint_as_float(u23 << 16) * sf, x3 = __uint_as_float(u23 & 0xffff0000u) * sf;
-        const float x4 = __uint_as_float(u45 << 16) * sf, x5 = __uint_as_float(u45 & 0xffff0000u) * sf;
-        const float x6 = __uint_as_float(u67 << 16) * sf, x7 = __uint_as_float(u67 & 0xffff0000u) * sf;
-        qa[4 * w] = f32x2_to_h2(x0, x4); qa[4 * w + 1] = f32x2_to_h2(x1, x5);
-        qa[4 * w + 2] = f32x2_to_h2(x2, x6); qa[4 * w + 3] = f32x2_to_h2(x3, x7);
-      }
-      tmem_st32(lane_addr + kColQ + 64 * t + 32 * half, qa);
-      wait_st();
-      fence_before_sync();
+#pragma unroll 8
+      for (int p = 0; p < 16; ++p)
+        *reinterpret_cast<uint4*>(sm.qs[t] + (row & 7) * 16 + (row >> 3) * 2048 + p * 128) = query8(piece(p), sf);
+      fence_async_smem();
       mbar_arrive(&sm.q_ready);
     }
     float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most kLazy
-    for (int j = 0; j < n_iter; ++j) {
-      mbar_wait(&sm.s_full[t], (uint32_t)j, abort_flag); // a wait that runs out raises the give-up flag; all leave below
+    for (int j = 0; j < n_step; ++j) {
+      // one warp of the tile polls and the others sleep at a barrier: polling takes issue slots from the other tile's warps
+      // (6 % of the kernel's time, like the sleeping waits of the dequantize warps)
+      if ((warp & 3) == 0) mbar_spin(&sm.s_full[t], (uint32_t)j, abort_flag);
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
       fence_after_sync();
-      uint32_t sr[32];
-      tmem_ld32(lane_addr + kColS + 64 * t + 32 * half, sr);
-      wait_ld();
-      const int pos0 = (it0 + j) * 64 + 32 * half;
-      // column c of this half is key pos0 + (c & ~7) + elem_of(c & 7); causal and window masks on edge blocks only
-      if (pos0 + 31 > pq || (W > 0 && pos0 <= pq - W)) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          const int pos = pos0 + (c & ~7) + elem_of(c & 7);
-          if (pos > pq || (W > 0 && pos <= pq - W)) sr[c] = 0xff800000u;   // -inf
-        }
-      }
-      // Probabilities against the current reference, and the block maximum beside them (independent instruction
-      // streams); only when some row's maximum has outgrown its reference is the reference moved, the accumulator
-      // rescaled and the probabilities taken again.  The scores stay in registers meanwhile.
-      float sum = 0.f;
-      uint32_t pr[16];
-      auto probabilities = [&](float neg_m) {
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-        for (int c = 0; c < 16; c += 2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sr[2 * c]), kappa, neg_m));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 1]), kappa, neg_m));
-          const float p2 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 2]), kappa, neg_m));
-          const float p3 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 3]), kappa, neg_m));
-          s0 += p0; s1 += p1; s2 += p2; s3 += p3;
-          pr[c] = f32x2_to_h2(p0, p1);
-          pr[c + 1] = f32x2_to_h2(p2, p3);
-        }
-        sum = (s0 + s1) + (s2 + s3);
-      };
-      probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
-      float cm4[4] = {__uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2]), __uint_as_float(sr[3])};
-#pragma unroll
-      for (int c = 4; c < 32; ++c) cm4[c & 3] = fmaxf(cm4[c & 3], __uint_as_float(sr[c]));
-      float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
-      sm.xchg[t][j & 1][half][row] = cm;
-      if (sampler) sm.stop[t][j % 3] = *abort_flag;
-      tile_barrier();                                    // also: every score of the tile has been read (P overlays S)
-      if (sm.stop[t][j % 3]) break;
-      cm = fmaxf(cm, sm.xchg[t][j & 1][half ^ 1][row]);
-      if (cm != -INFINITY) cm *= kappa;                  // kappa > 0
-      const float m_new = fmaxf(m_ref, cm);
-      const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
-      if (__any_sync(0xffffffffu, grow)) {
-        if (j > 0) {
-          // rescale this thread's half of the accumulator row: the previous block's value product must have landed
-          mbar_wait(&sm.o_done[t], (uint32_t)(j - 1), abort_flag);
-          fence_after_sync();
-          const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;           // m_ref = -inf: 0
+      const int pos0 = (st0 + j) * 128;
+      const bool edge = pos0 + 127 > pq || (W > 0 && pos0 <= pq - W);
 #pragma unroll 1
-          for (int part = 0; part < 2; ++part) {
-            uint32_t orow[32];
-            tmem_ld32(lane_addr + kColO + 128 * t + 64 * half + 32 * part, orow);
-            wait_ld();
+      for (int half = 0; half < 2; ++half) {             // 64 keys at a time: the first half's value product starts meanwhile
+        const uint32_t half_addr = s_addr + 64 * half;
+        // column c is key pos0 + 64 half + (c & ~7) + elem_of(c & 7); causal and window masks on edge steps only
+        auto mask = [&](uint32_t* x, int c0) {
+          const int last = pq - (pos0 + 64 * half + c0), first = W > 0 ? last - W + 1 : -1000;     // columns [first, last] count
 #pragma unroll
-            for (int c = 0; c < 32; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
-            tmem_st32(lane_addr + kColO + 128 * t + 64 * half + 32 * part, orow);
+          for (int c = 0; c < 32; ++c) {
+            const int k = (c & ~7) + elem_of(c & 7);
+            if (k > last || k < first) x[c] = 0xff800000u;   // -inf
           }
-          if (grow) l *= f;
+        };
+        // Probabilities against the current reference, and the maximum beside them (independent instruction streams); only
+        // when some row's maximum has outgrown its reference is the reference moved, the accumulator rescaled and the
+        // probabilities taken again.
+        uint32_t pr[32];
+        uint64_t sum0, sum1;
+        auto probabilities = [&](const uint32_t* x, uint32_t* p, uint64_t kk, uint64_t nn) {
+#pragma unroll
+          for (int c = 0; c < 16; c += 2) {
+            const float2 a = unpair64(fma2(pair64(__uint_as_float(x[2 * c]), __uint_as_float(x[2 * c + 1])), kk, nn));
+            const float2 b = unpair64(fma2(pair64(__uint_as_float(x[2 * c + 2]), __uint_as_float(x[2 * c + 3])), kk, nn));
+            const float a0 = fast_exp2(a.x), a1 = fast_exp2(a.y), b0 = fast_exp2(b.x), b1 = fast_exp2(b.y);
+            sum0 = add2(sum0, pair64(a0, a1));
+            sum1 = add2(sum1, pair64(b0, b1));
+            p[c] = f32x2_to_h2(a0, a1);
+            p[c + 1] = f32x2_to_h2(b0, b1);
+          }
+        };
+        float cm0 = -INFINITY, cm1 = -INFINITY;
+        auto maximum = [&](const uint32_t* x) {
+#pragma unroll
+          for (int c = 0; c < 32; c += 4) {
+            cm0 = fmaxf(cm0, fmaxf(__uint_as_float(x[c]), __uint_as_float(x[c + 1])));
+            cm1 = fmaxf(cm1, fmaxf(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])));
+          }
+        };
+        uint32_t x[64];
+        float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+        sum0 = sum1 = 0ull;
+        const uint64_t kk = pair64(kappa, kappa);
+        uint64_t nn = pair64(neg_m, neg_m);
+        tmem_ld32(half_addr, x);
+        wait_ld32(x);
+        tmem_ld32(half_addr + 32, x + 32);
+        if (edge) mask(x, 0);
+        probabilities(x, pr, kk, nn);
+        maximum(x);
+        wait_ld32(x + 32);
+        if (edge) mask(x + 32, 32);
+        probabilities(x + 32, pr + 16, kk, nn);
+        maximum(x + 32);
+        float cm = fmaxf(cm0, cm1);
+        if (cm != -INFINITY) cm *= kappa;                // kappa > 0
+        const float m_new = fmaxf(m_ref, cm);
+        const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
+        if (__any_sync(0xffffffffu, grow)) {
+          if (j + half > 0) {
+            // rescale the accumulator row once the value products issued so far have landed (those of earlier steps have: the
+            // scores were issued behind them)
+            if (half == 1 && !__all_sync(0xffffffffu, mbar_wait(&sm.o_half[t], (uint32_t)j, abort_flag))) break;
+            fence_after_sync();
+            const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;         // m_ref = -inf: 0
+#pragma unroll 1
+            for (int part = 0; part < 8; ++part) {
+              uint32_t orow[16];
+              tmem_ld16(o_addr + 16 * part, orow);
+              wait_ld16(orow);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
+              tmem_st16(o_addr + 16 * part, orow);
+            }
+            if (grow) l *= f;
+          }
+          if (grow) m_ref = m_new;
+          neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+          nn = pair64(neg_m, neg_m);
+          sum0 = sum1 = 0ull;
+          probabilities(x, pr, kk, nn);
+          probabilities(x + 32, pr + 16, kk, nn);
         }
-        if (grow) m_ref = m_new;
-        probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
+        tmem_st32(half_addr, pr);                        // P overlays the half's first 32 columns of S
+        const float2 u = unpair64(add2(sum0, sum1));
+        l += u.x + u.y;
+        wait_st();
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.p_full[t][half]);
       }
-      l += sum;
-      tmem_st16(lane_addr + kColS + 64 * t + 16 * half, pr);   // P_t overlays the first 32 columns of S_t
-      wait_st();
-      fence_before_sync();
-      mbar_arrive(&sm.p_full[t]);
     }
-    // ---- normalise and write this thread's half of the row ----
+    // ---- normalise and write the row, or leave it as a record ----
     bool ok = !*abort_flag;
-    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_done[t], (uint32_t)(n_iter - 1), abort_flag);
-    const int slot = n_iter & 1;                         // not the slot the last block used
-    sm.xchg[t][slot][half][row] = l;
-    if (!ok) sm.spoiled[t] = 1;                          // anyone who gave up spoils the tile
-    tile_barrier();
-    ok = sm.spoiled[t] == 0;                             // uniform over the tile: the loads below are warp-wide
-    l += sm.xchg[t][slot][half ^ 1][row];
+    if (ok && n_step > 0) ok = mbar_wait(&sm.o_done[t], (uint32_t)(n_step - 1), abort_flag);
+    ok = __all_sync(0xffffffffu, ok);                    // the loads below are warp-wide
     if (ok) fence_after_sync();
     const bool bad = !ok || sm.poisoned != 0;
-    const bool zero = bad || n_iter == 0 || l <= 0.f;
+    const bool zero = bad || n_step == 0 || l <= 0.f;
     const bool final = P.x.n_splits == 1;                // else the row is left as a record
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
-    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
-    const size_t orow_index = row_index * 128 + 64 * half;
     float* rec = final ? nullptr : P.x.records + (row_index * P.x.n_splits + split) * prefill_record(128);
 #pragma unroll 1
-    for (int part = 0; part < 2; ++part) {
+    for (int part = 0; part < 4; ++part) {
       uint32_t orow[32];
-      if (ok && n_iter > 0) {
-        tmem_ld32(lane_addr + kColO + 128 * t + 64 * half + 32 * part, orow);
-        wait_ld();
+      if (ok && n_step > 0) {
+        tmem_ld32(o_addr + 32 * part, orow);
+        wait_ld32(orow);
       }
       if (!mine) continue;
       if (final && P.out_dtype == Q4KV_OUT_BF16) {
-        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + orow_index + 32 * part;
+        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + row_index * 128 + 32 * part;
 #pragma unroll
         for (int c = 0; c < 32; c += 8) {
           uint4 v;
@@ -464,7 +467,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
           *reinterpret_cast<uint4*>(o + c) = v;
         }
       } else {
-        float* o = (final ? reinterpret_cast<float*>(P.out) + orow_index : rec + 64 * half) + 32 * part;
+        float* o = (final ? reinterpret_cast<float*>(P.out) + row_index * 128 : rec) + 32 * part;
 #pragma unroll
         for (int c = 0; c < 32; c += 4)
           *reinterpret_cast<float4*>(o + c) =
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                                  __uint_as_float(orow[c + 2]) * inv, __uint_as_float(orow[c + 3]) * inv);
       }
     }
-    if (half == 0 && mine) {
+    if (mine) {
       if (!final) *reinterpret_cast<float2*>(rec + 128) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
       else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
     }

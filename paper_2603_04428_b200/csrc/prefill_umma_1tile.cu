@@ -79,7 +79,7 @@ struct UmmaSmem {
   alignas(128) uint8_t raw[kRawSlots][Sh::kRawBytes];
   alignas(8) uint64_t raw_full[kRawSlots], raw_free[kRawSlots], sb_done[kRawSlots];
   uint64_t k_full[kStages], v_full[kStages], k_free[kStages], v_free[kStages];
-  uint64_t s_full[2], p_full[2], o_done, q_ready, drain;
+  uint64_t s_full[2], p_full[2], o_done, o_last, q_ready, drain;
   uint32_t tmem_base;
   int bad[kRawSlots];
   float xchg[2][2][128];                                 // [parity][column half][row]: maxima / sums of the two threads of a row
@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     }
     for (int b = 0; b < 2; ++b) { mbar_init(&sm.s_full[b], 1); mbar_init(&sm.p_full[b], kSoftmaxWarps * 32); }
     mbar_init(&sm.o_done, 1);
+    mbar_init(&sm.o_last, 1);
     mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
     for (int i = 0; i < 3; ++i) sm.stop[i] = 0;
     sm.spoiled = 0;
@@ -292,13 +293,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         }
         __syncwarp();
       };
-      auto issue_pv = [&](int b, int s, bool first) {    // O (+)= P_b V^; afterwards the V^ stage is free
+      auto issue_pv = [&](int b, int s, bool first, bool last) {    // O (+)= P_b V^; afterwards the V^ stage is free
         const uint64_t vd = smem_desc(smem_u32(sm.vhat[s]), 128, 1024);
         if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + 16 * k, kIdescO, (!first || k > 0) ? 1u : 0u);
           commit(&sm.o_done);
+          if (last) commit(&sm.o_last);
           commit(&sm.v_free[s]);
         }
         __syncwarp();
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         fence_after_sync();
-        issue_pv(b, s, j == 0);
+        issue_pv(b, s, j == 0, j + 1 == n_iter);
         if (j + 2 < n_iter) {                            // the scores of block j + 2 replace P_b once the product above has read it
           ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s], (uint32_t)((j + 2) / kStages), abort_flag));
           if (!ok) break;
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       fence_after_sync();
       uint32_t sr[32];
       tmem_ld32(lane_addr + kColS + 64 * b + 32 * half, sr);
-      wait_ld();
+      wait_ld32(sr);
       const int pos0 = (it0 + j) * 64 + 32 * half;
       // column c of this half is key pos0 + (c & ~7) + elem_of(c & 7); causal and window masks on edge blocks only
       if (pos0 + 31 > pq || (W > 0 && pos0 <= pq - W)) {
@@ -460,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
           for (int part = 0; part < kDv / 64; ++part) {
             uint32_t orow[32];
             tmem_ld32(lane_addr + kColO + (kDv / 2) * half + 32 * part, orow);
-            wait_ld();
+            wait_ld32(orow);
 #pragma unroll
             for (int c = 0; c < 32; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
             tmem_st32(lane_addr + kColO + (kDv / 2) * half + 32 * part, orow);
@@ -478,7 +480,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     }
     // ---- normalise and write this thread's half of the row ----
     bool ok = !*abort_flag;
-    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_done, (uint32_t)(n_iter - 1), abort_flag);
+    // (the last two value products may both be under way, and a wait on o_done could not tell which phase it sees)
+    if (ok && n_iter > 0) ok = mbar_wait(&sm.o_last, 0, abort_flag);
     const int slot = n_iter & 1;                         // not the slot the last block used
     sm.xchg[slot][half][row] = l;
     if (!ok) sm.spoiled = 1;                             // anyone who gave up spoils the tile
@@ -498,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       uint32_t orow[32];
       if (ok && n_iter > 0) {
         tmem_ld32(lane_addr + kColO + (kDv / 2) * half + 32 * part, orow);
-        wait_ld();
+        wait_ld32(orow);
       }
       if (!mine) continue;
       if (final && P.out_dtype == Q4KV_OUT_BF16) {

@@ -64,6 +64,27 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t use, volatile int* abor
   *abort_flag = 1;
   return false;
 }
+// The same without suspending: for the few warps whose wake-up is on the critical path.
+__device__ inline bool mbar_spin(uint64_t* bar, uint32_t use, volatile int* abort_flag) {
+  const uint32_t parity = use & 1u;
+  for (uint32_t i = 0; i < (1u << 26); ++i) {
+    if (mbar_test_wait(bar, parity)) return true;
+    if ((i & 255u) == 255u && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+// The same with sleeps in between: for warps that run ahead of the others, so that they do not take issue slots meanwhile.
+__device__ inline bool mbar_doze(uint64_t* bar, uint32_t use, volatile int* abort_flag) {
+  const uint32_t parity = use & 1u;
+  for (uint32_t i = 0; i < (1u << 23); ++i) {
+    if (mbar_test_wait(bar, parity)) return true;
+    __nanosleep(200);
+    if ((i & 15u) == 15u && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
 __device__ inline void bulk_load(void* dst_smem, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(dst_smem)),
@@ -71,6 +92,13 @@ __device__ inline void bulk_load(void* dst_smem, const void* src, uint32_t bytes
                : "memory");
 }
 __device__ inline void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Registers per thread of a warpgroup (all four warps call it): the sum over the CTA must stay within what it was launched
+// with, and every warpgroup that gives some up must do so without waiting for one that asks for more.
+template <int N>
+__device__ __forceinline__ void more_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void fewer_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // ---- tensor memory ----
 __device__ inline void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {      // one whole warp
@@ -86,6 +114,25 @@ __device__ inline void tmem_dealloc(uint32_t taddr, uint32_t ncols) {        // 
 __device__ inline void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ inline void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ inline void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// the same, and nothing that uses these registers may move above it (loads with other work between them and the wait)
+__device__ inline void wait_ld32(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                 "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]),
+                 "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]),
+                 "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
+__device__ inline void wait_ld16(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                 "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
 __device__ inline void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // the mbarrier gets one arrival when every MMA this thread has issued so far is complete
 __device__ inline void commit(uint64_t* bar) {
