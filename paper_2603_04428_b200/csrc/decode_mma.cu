@@ -357,7 +357,6 @@ struct Segment {
   int a, hk, c0, c1;      // (virtual) agent, head set, logical chunk indices [c0, c1) of the agent
   int ar, li;             // real agent (lengths, block table) and layer of the call (pool layer)
   int n, lo;              // key range of the agent
-  int row;                // query row of the agent (kSingles)
   int cf, nc;             // the pair's whole chunk range
   int k0;                 // running chunk counter of the CTA at c0
   int first, last;        // CTAs that hold the pair's first and last chunk
@@ -369,7 +368,6 @@ __device__ inline void whole_segment(const Par& P, const RangeStart& rs, Segment
   s.li = P.layer_count > 1 ? rs.agent / P.n_real : 0; s.ar = rs.agent - s.li * P.n_real;
   s.a = rs.agent; s.hk = rs.pair; s.c0 = rs.r.cf + (int)rs.u_begin; s.c1 = rs.r.cf + (int)rs.u_end;
   s.n = rs.r.n; s.lo = rs.r.lo; s.cf = rs.r.cf; s.nc = rs.r.nc; s.k0 = 0;
-  if (Par::kSingles) s.row = P.q_offs[rs.agent];
   s.first = (int)blockIdx.x - rs.split;
   s.last = s.first + rs.splits - 1;
 }
@@ -404,7 +402,6 @@ struct Walker {
     const int c1 = (uint32_t)(pair_end - c) <= left ? pair_end : c + (int)left;
     s.li = P.layer_count > 1 ? a / P.n_real : 0; s.ar = a - s.li * P.n_real;
     s.a = a; s.hk = hk; s.c0 = c; s.c1 = c1; s.n = r.n; s.lo = r.lo; s.cf = r.cf; s.nc = r.nc; s.k0 = k;
-    if (Par::kSingles) s.row = P.q_offs[a];
     const int cnt = c1 - c;
     s.first = s.last = 0;
     if (cnt != r.nc) {
@@ -914,7 +911,7 @@ __device__ __forceinline__ void combine_deposits(const Smem<G, H>& sm, const Par
   }
   const float L0 = __shfl_sync(0xffffffffu, L, h0), L1 = __shfl_sync(0xffffffffu, L, h0 + 1);
   const int d = H == 4 ? 32 * unit + g + 8 * (tid >> 1) : 16 * unit + g, step = H == 4 ? 16 : 8;
-  const size_t row0 = (size_t)(Par::kSingles ? seg.row : seg.a) * P.y.Hq + (size_t)seg.hk * n_rep;
+  const size_t row0 = (size_t)(Par::kSingles ? P.q_offs[seg.a] : seg.a) * P.y.Hq + (size_t)seg.hk * n_rep;
   if (whole) {
     const float i0 = L0 > 0.f ? 1.f / L0 : 0.f, i1 = L1 > 0.f ? 1.f / L1 : 0.f;
     if (h0 < n_rep) { store_out(P, (row0 + h0) * Dv + d, a[0] * i0); store_out(P, (row0 + h0) * Dv + d + step, a[2] * i0); }
@@ -1109,7 +1106,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   const int g = lane >> 2, tid = lane & 3;
   // this warp's row of a segment's query; the new row's groups are quantized by the warps behind the query's (from 4 on)
   constexpr int kNewWarps = NW - 4, kNewRounds = (G + Gv + kNewWarps - 1) / kNewWarps;
-  auto query_row = [&](const Segment& s) { return P.q + ((size_t)(kSingles ? s.row : s.a) * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
+  auto query_row = [&](const Segment& s) { return P.q + ((size_t)(kSingles ? P.q_offs[s.a] : s.a) * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
   auto new_pair = [&](const Segment& s, int grp) {
     const size_t head = (size_t)s.a * y.Hkv + s.hk;
     return (grp < G ? P.k_new + head * D + 64 * grp : P.v_new + head * Dv + 64 * (grp - G)) + 2 * lane;
@@ -1263,7 +1260,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
     if (warp == NW - 1 && lane == 0) {
       if (seg.c1 - c0 != seg.nc) {                       // only the first and the last segment can be parts of a pair
         int* f = sm.fin[k0 == 0 ? 0 : 1];
-        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = (kSingles ? seg.row : seg.a) * y.Hq + seg.hk * n_rep;
+        f[0] = seg.a * P.Hkv + seg.hk; f[1] = seg.first; f[2] = seg.last; f[3] = (kSingles ? P.q_offs[seg.a] : seg.a) * y.Hq + seg.hk * n_rep;
       }
       if (more) sm.walker.next(P, sm.range, sm.seg[(si + 2) % 3]);       // never where the CTA holds one segment
     }
