@@ -1,6 +1,7 @@
 // What the tcgen05 prefill kernels share: the expansion of packed codes into binary16, small conversions, and the plan and
 // records of launches that cut the keys of a query tile over several CTAs.
 #pragma once
+#include "f32x2.cuh"
 #include "q4kv_layout.cuh"
 #include "tcgen05.cuh"
 
@@ -39,27 +40,6 @@ __device__ inline float fast_exp2(float x) {
 __device__ inline uint32_t f32x2_to_h2(float lo, float hi) {
   const __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
-}
-// two binary32 operations in one instruction
-__device__ __forceinline__ uint64_t pair64(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unpair64(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
 }
 // A bfloat16 (scale, bias) pair as a binary16 pair: exact while the magnitude is a binary16 normal number (bfloat16
 // has 8 significant bits), within 2^-25 below that; a magnitude beyond binary16's largest number is reported.

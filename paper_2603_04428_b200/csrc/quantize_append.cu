@@ -7,6 +7,7 @@
 // Eight consecutive lanes own one 64-element group (eight elements each) and reduce
 // min/max with three shuffles.  Every arithmetic step is a single rounded binary32
 // operation in the documented order so that codes/scales/biases are reproducible.
+#include "f32x2.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
 
@@ -154,19 +155,19 @@ quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_a
 }
 
 // ---------------------------------------------------------------------------------------------
-// Bulk form (a prefill phase: many new tokens per agent).  One warp owns one (32-token chunk, KV head) unit and walks
-// its items -- (octet of eight positions, pass of four groups: K groups first, then V groups) -- with the loads of the
+// Bulk form (a prefill phase: many new tokens per agent).  kWpc warps own one (32-token chunk, KV head) unit and walk its
+// items -- (octet of eight positions, pass of four groups: K groups first, then V groups) -- with the loads of the
 // next item in flight while the current one is quantized.  Within an item a lane owns one of the eight positions and
 // one 64-element group: it loads its 64 elements as eight 16-byte words, takes minimum and maximum with packed bf16
-// instructions (no cross-lane step at all), and quantizes them: the quotient as t * (1/scale), rounded by adding
-// 1.5 * 2^23 (the code is then in the low bits), and only a quotient within 4e-6 of a tie goes through the division
-// itself, so that the codes equal those of the fixed sequence bit for bit.  V words are first exchanged between the
-// eight lanes of a group (an 8 x 8 transposition of words by twelve shuffles), which leaves in each lane the
-// 8 positions x 8 elements block of nibbles that an in-register transposition turns into eight token-packed words.
-// The chunk is assembled in shared memory and stored as whole 16-byte pieces; a chunk that the phase fills only in
+// instructions (no cross-lane step at all), and quantizes them two at a time (packed binary32): t = x - bias, c = t *
+// (1/scale) rounded by adding 1.5 * 2^23 in the same fma, and the distance of t * (1/scale) from c; a word with a quotient
+// within 4e-6 of a tie is decided from exact residuals, so that the codes equal those of the fixed sequence bit for bit.  V words
+// are first exchanged between the eight lanes of a group (an 8 x 8 transposition of words by twelve shuffles), which leaves
+// in each lane the 8 positions x 8 elements block of nibbles that an in-register transposition turns into eight token-packed
+// words.  The chunk is assembled in shared memory and stored as whole 16-byte pieces; a chunk that the phase fills only in
 // part (an unaligned start or end) starts from its present bytes.
-// Measured on 8 x 1024 tokens (43 MB): 20.1 us, bound by instruction issue (about 1230 warp instructions per item of
-// 32 x 64 elements at 0.5 issued per scheduler and clock); the same time with one warp per octet and direct stores.
+// kWpc = 1 where the units fill the GPU; 4 for smaller phases, whose time is one unit's chain of items.
+// Bound by instruction issue: see launch_quantize_append for the times.
 // ---------------------------------------------------------------------------------------------
 __device__ inline void transpose_nibbles_8x8_regs(uint32_t (&r)[8]) {
   // rows = registers, columns = nibbles: three rounds of block swaps
@@ -183,10 +184,26 @@ __device__ inline void transpose_nibbles_8x8_regs(uint32_t (&r)[8]) {
   }
 }
 
-// Code of one element by the division itself (the rare element whose quotient is within a few ulps of a tie).  A call, so
-// that the compiler keeps the division out of the common path.
-__device__ __noinline__ float exact_code(float x, float bf, float sf) {
-  return fminf(rintf(__fdiv_rn(__fsub_rn(x, bf), sf)), 15.0f);
+// The eight codes of a word with a quotient within a few ulps of a tie, without dividing.  With k = floor(t * inv) and v = k +
+// 1/2 the residual t - s v is exact (s v has at most 16 significant bits, and t is close to it); the rounded quotient of the
+// fixed sequence is v itself where the residual is at most half an ulp of v times s, and then goes to the even neighbour.
+// Rows of bf16 numbers meet exact ties often (7e-4 of all elements), so this is not rare: one warp in six per word.
+__device__ __noinline__ uint32_t exact_word(uint4 raw, float bf, float sf, float inv) {
+  const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
+  uint32_t word = 0u;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float x = (e & 1) ? __uint_as_float(wv[e >> 1] & 0xffff0000u) : __uint_as_float(wv[e >> 1] << 16);
+    const float t = __fsub_rn(x, bf);
+    const float k = floorf(t * inv), v = k + 0.5f;
+    const float rr = __fmaf_rn(-sf, v, t);
+    // half an ulp of v; below 1/2, a power of two, the spacing is half as wide
+    float lim = sf * (__uint_as_float(__float_as_uint(v) & 0x7f800000u) * 5.9604644775390625e-8f);
+    if (k == 0.f && rr < 0.f) lim *= 0.5f;
+    const uint32_t ki = (uint32_t)k;
+    word |= min(ki + (fabsf(rr) <= lim ? (ki & 1u) : rr > 0.f ? 1u : 0u), 15u) << (4 * e);
+  }
+  return word;
 }
 
 // Unit of the bulk kernel: one 32-token chunk of one agent's new range (up to four octets, all in one pool block).
@@ -234,8 +251,7 @@ __device__ inline void find_chunk_unit(int u, int n_agents, int max_blocks, int 
   if (!found && lane == 0) out->agent = -1;
 }
 
-// One warp owns one (chunk, KV head) unit and walks its items -- (octet, pass of four groups) -- with the loads of
-// the next item in flight while the current one is quantized.
+template <int kWpc>
 __global__ void __launch_bounds__(kThreads, 2)
 quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                             const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
@@ -245,14 +261,18 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
   extern __shared__ __align__(16) uint8_t stage_all[];  // one chunk per warp
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * (kThreads / 32) + warp;
+  const int sub = warp % kWpc;                           // this warp of the unit
+  const int gw = (blockIdx.x * (kThreads / 32) + warp) / kWpc;
   const int u = gw / y.Hkv, hk = gw - u * y.Hkv;
   if (u >= units) return;
-  find_chunk_unit(u, n_agents, max_blocks, n_blocks, tables, pos, new_offs, flags, gw == 0, &s_unit[warp]);
+  find_chunk_unit(u, n_agents, max_blocks, n_blocks, tables, pos, new_offs, flags, gw == 0 && sub == 0, &s_unit[warp]);
   __syncwarp();
   const ChunkUnit un = s_unit[warp];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (un.agent < 0) return;
+  auto unit_sync = [&]() {
+    if (kWpc == 1) __syncwarp(); else asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / kWpc), "n"(32 * kWpc) : "memory");
+  };
 
   const int s = lane & 7, gq0 = lane >> 3;             // position slot inside an octet, group inside a pass
   const int c0 = un.chunk << 5;                          // first cache position of the chunk
@@ -262,11 +282,11 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
   // over the chunk: stored one by one they would reach L2 as a million and a half partial sectors per phase).  A
   // chunk that this phase fills only in part starts from its present bytes; this warp is its only writer.
   uint8_t* gchunk = head_block(pool, y, layer, un.block, hk) + (size_t)(un.chunk & 7) * y.chunk_bytes;
-  uint8_t* chunk = stage_all + (size_t)warp * y.chunk_bytes;
+  uint8_t* chunk = stage_all + (size_t)(warp / kWpc) * y.chunk_bytes;
   const int n16 = y.chunk_bytes / 16;
   if (lo != c0 || hi != c0 + 32) {
-    for (int q = lane; q < n16; q += 32) reinterpret_cast<uint4*>(chunk)[q] = reinterpret_cast<const uint4*>(gchunk)[q];
-    __syncwarp();
+    for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(chunk)[q] = reinterpret_cast<const uint4*>(gchunk)[q];
+    unit_sync();
   }
   const int n_groups = y.G + (y.alias ? 0 : y.Gv);
   const int n_pass = (n_groups + 3) >> 2;
@@ -296,9 +316,9 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
   };
 
   uint4 raw[8], nxt[8];
-  load_item(0, raw);
-  for (int t = 0; t < n_items; ++t) {
-    if (t + 1 < n_items) load_item(t + 1, nxt);
+  if (sub < n_items) load_item(sub, raw);
+  for (int t = sub; t < n_items; t += kWpc) {
+    if (t + kWpc < n_items) load_item(t + kWpc, nxt);
     const int o = o_first + t / n_pass, pass = t - (t / n_pass) * n_pass;
     const int first = max(lo, c0 + 8 * o), cnt = min(hi, c0 + 8 * o + 8) - first;
     const int k0 = first & 7;
@@ -332,31 +352,26 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
     for (int j = 0; j < 8; ++j) cw[j] = 0u;
     if (gs.sf != 0.0f) {
       const float inv = __frcp_rn(gs.sf);
+      const uint64_t nb2 = pair64(-gs.bf, -gs.bf), inv2 = pair64(inv, inv), ninv2 = pair64(-inv, -inv);
+      const uint64_t up2 = pair64(kMagic, kMagic), down2 = pair64(-kMagic, -kMagic), k256 = pair64(256.f, 256.f);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint32_t wv[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
-        // t = x - bias, q = t / scale (as t * inv), c = q rounded to nearest even by adding and subtracting 1.5 * 2^23;
-        // q <= 15 + a few ulps by construction of the scale, so no clamp is needed.  The eight codes are assembled in
-        // floating point (two exact 16-bit halves) instead of by shifts.
-        float c[8], far = 0.f;
+        // t = x - bias, c = t / scale (as t * inv) rounded to nearest even by adding and subtracting 1.5 * 2^23;
+        // the quotient is at most 15 + a few ulps by construction of the scale, so no clamp is needed.  The eight codes
+        // are assembled in floating point (two exact 16-bit halves) instead of by shifts.
+        uint64_t c[4];
+        float far = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float x = (e & 1) ? __uint_as_float(wv[e >> 1] & 0xffff0000u) : __uint_as_float(wv[e >> 1] << 16);
-          const float q = __fmul_rn(__fsub_rn(x, gs.bf), inv);
-          c[e] = __fsub_rn(__fadd_rn(q, kMagic), kMagic);
-          far = fmaxf(far, fabsf(__fsub_rn(q, c[e])));
+        for (int e = 0; e < 4; ++e) {
+          const uint64_t t = add2(pair64(__uint_as_float(wv[e] << 16), __uint_as_float(wv[e] & 0xffff0000u)), nb2);
+          c[e] = add2(fma2(t, inv2, up2), down2);
+          const float2 d = unpair64(fma2(t, ninv2, c[e]));
+          far = fmaxf(far, fmaxf(fabsf(d.x), fabsf(d.y)));
         }
-        if (far > kTieZone) {                            // rare: some quotient is too close to a tie for t * inv to decide
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float x = (e & 1) ? __uint_as_float(wv[e >> 1] & 0xffff0000u) : __uint_as_float(wv[e >> 1] << 16);
-            const float q = __fmul_rn(__fsub_rn(x, gs.bf), inv);
-            if (fabsf(__fsub_rn(q, c[e])) > kTieZone) c[e] = exact_code(x, gs.bf, gs.sf);
-          }
-        }
-        const float lo4 = fmaf(fmaf(fmaf(c[3], 16.f, c[2]), 16.f, c[1]), 16.f, c[0]);
-        const float hi4 = fmaf(fmaf(fmaf(c[7], 16.f, c[6]), 16.f, c[5]), 16.f, c[4]);
-        cw[j] = __byte_perm(__float_as_uint(lo4 + 8388608.0f), __float_as_uint(hi4 + 8388608.0f), 0x5410);
+        const float2 a = unpair64(fma2(c[1], k256, c[0])), b = unpair64(fma2(c[3], k256, c[2]));
+        cw[j] = far > kTieZone ? exact_word(raw[j], gs.bf, gs.sf, inv) :
+                __byte_perm(__float_as_uint(fmaf(a.y, 16.f, a.x) + 8388608.0f), __float_as_uint(fmaf(b.y, 16.f, b.x) + 8388608.0f), 0x5410);
       }
     }
     const uint32_t sb = gs.hs | (gs.hb << 16);
@@ -395,8 +410,36 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
 #pragma unroll
     for (int j = 0; j < 8; ++j) raw[j] = nxt[j];
   }
-  __syncwarp();
-  for (int q = lane; q < n16; q += 32) reinterpret_cast<uint4*>(gchunk)[q] = reinterpret_cast<const uint4*>(chunk)[q];
+  unit_sync();
+  for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(gchunk)[q] = reinterpret_cast<const uint4*>(chunk)[q];
+}
+
+template <int kWpc>
+cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer, const q4kv_batch& b, const int32_t* pos,
+                        const int32_t* new_offs, int chunk_units, const void* k_new, const void* v_new, int32_t* flags,
+                        cudaStream_t st) {
+  const long long warps = (long long)chunk_units * y.Hkv * kWpc;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((warps + kThreads / 32 - 1) / (kThreads / 32)));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = (size_t)(kThreads / 32 / kWpc) * y.chunk_bytes;
+  cfg.stream = st;
+  static bool configured[64] = {};     // the attribute is per function and device: set it once for each
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !configured[dev]) {
+    e = cudaFuncSetAttribute(quantize_append_bulk_kernel<kWpc>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) configured[dev] = true;
+  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel<kWpc>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
+                            b.block_tables, pos, new_offs, (const uint16_t*)k_new, (const uint16_t*)v_new, flags, chunk_units);
 }
 
 template <int M>
@@ -427,29 +470,10 @@ cudaError_t launch_quantize_append(const Layout& y, void* pool, int n_blocks, in
   if (total_new >= 8 * b.n_agents && (size_t)(kThreads / 32) * y.chunk_bytes <= 112 * 1024) {
     // a phase of many tokens per agent: one warp per (32-token chunk, KV head)
     const int chunk_units = total_new / 32 + 2 * b.n_agents;   // >= sum over agents of the chunks their new range touches
-    const long long warps = (long long)chunk_units * y.Hkv;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((warps + kThreads / 32 - 1) / (kThreads / 32)));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = (size_t)(kThreads / 32) * y.chunk_bytes;
-    cfg.stream = st;
-    static bool configured[64] = {};     // the attribute is per function and device: set it once for each
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !configured[dev]) {
-      e = cudaFuncSetAttribute(quantize_append_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) configured[dev] = true;
-    }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel, y, (uint8_t*)pool, n_blocks, layer, b.n_agents,
-                              b.max_blocks, b.block_tables, pos, new_offs, (const uint16_t*)k_new,
-                              (const uint16_t*)v_new, flags, chunk_units);
+    // four warps per unit while one warp each would leave half of the resident warps (sixteen per SM) without work
+    if ((long long)chunk_units * y.Hkv < 8ll * sm_count())
+      return launch_bulk<4>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
+    return launch_bulk<1>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
   }
   return launch_m<1>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, units, k_new, v_new, flags, st);
 }
