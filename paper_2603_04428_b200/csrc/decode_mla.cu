@@ -3,32 +3,35 @@
 // agent in absorbed form over the Q4 latent cache, read in place (Section 3.4 "Batched Quantized
 // Inference"; the MLA cache of Section 3.6).
 //
-// Every key serves all 16 heads and is both key and value, so the cache bytes are expanded once
-// per 64-key block into a binary16 tile that the tensor cores read twice:
-//   * Work is split along the keys: CTA (split, agent) walks its share of the agent's keys 64 at a
-//     time (two 32-token chunks = one bulk copy of 20736 bytes into a two-slot ring, issued two
-//     blocks ahead by one thread), leaves an (acc, m, l) record per head, and a second kernel combines the
-//     records of an agent.
-//   * The eight compute warps first turn the raw block into the tile K^ [64 keys][576 dims] in
-//     shared memory (x^ = c * s + b, one binary16 fma per pair of codes, rounded once), stored as
-//     8 x 16-byte core matrices: 8 keys x 8 dims each, 128 contiguous bytes -- exactly one ldmatrix
-//     8x8 tile, read without bank conflicts either way.
-//   * Scores: warp w owns keys 8w..8w+7 of the block: S[16 heads][8 keys] by 36 mma.sync m16n8k16
-//     (A = the queries, staged once as binary16 scaled by a power of two per head; B = K^ through
-//     plain ldmatrix).  Values: warp w owns dims 64w..64w+63: O[16 heads][64 dims] += P V^ by 32
-//     mma.sync, with V^ = the same tile read through ldmatrix.trans and P exchanged through a 2 KB
-//     shared tile.  544 tensor instructions per block over eight warps; the accumulators of the
-//     whole share stay in registers.  (A tcgen05 version of this kernel was measured at 40 us per
-//     call: with only 16 heads every tensor-memory MMA is tiny, and an MMA whose A operand comes
-//     from shared memory costs ~110 clocks whatever its size.)
-//   * Softmax with a lazily moved reference maximum per head, shared by the CTA: a block whose
-//     scores exceed it by more than 2^8 triggers an exact per-head maximum (shuffles + shared
-//     memory) and a rescale of the register accumulators; otherwise a block costs four
-//     exponentials per thread.  Row sums stay per-thread until the end.
-// Three CTA-wide named barriers per block (tile ready, growth agreed, probabilities ready); the raw
-// blocks arrive on mbarriers with bounded waits (Q4KV_FLAG_INTERNAL when one runs out; the 256
-// threads then leave together).  Eight warps, not nine: with a ninth the register allocation drops
-// to 168 per thread, and the queries' fragments alone take 144.
+// Every key serves all 16 heads and is both key and value: its words are expanded once, used as tensor-core operands for the
+// scores from the registers that expanded them, and stored once as binary16 for the value product.
+//   * Work is split along the keys: CTA (split, agent) walks its share of the agent's keys 64 at a time (two 32-token chunks =
+//     one bulk copy of 20736 bytes into a three-slot ring, issued three blocks ahead by one thread), leaves an (acc, m, l)
+//     record per head, and a second kernel combines the records of an agent.
+//   * Scores: the two warps of a pair own two key octets and half of the words each.  A lane expands a word of its key
+//     (x^ = c * s + b, one binary16 fma per pair of codes, rounded once); the four pairs of elements are the B fragments of
+//     two mma.sync m16n8k16 whose A operand, the queries (staged once as binary16 scaled by a power of two per head), has its
+//     columns in the same order and stays in registers.  The pair's halves meet through 4 KB of shared memory.
+//   * Values: the same registers are stored as one 16-byte row per (key, word), two stages deep; warp w owns dims 64w..64w+63:
+//     O[16 heads][64 dims] += P V^ by 32 mma.sync, with V^ read through ldmatrix.trans and P through a 2 KB shared tile.  The
+//     value product of a block is interleaved with the expansion and the scores of the next one.  (A tcgen05 version of this
+//     kernel was measured at 40 us per call: with only 16 heads every tensor-memory MMA is tiny, and one whose A operand comes
+//     from shared memory costs 55 to 110 clocks whatever its N.)
+//   * Softmax with a lazily moved reference maximum per head, shared by the CTA: a block whose scores exceed it by more than
+//     2^8 triggers an exact per-head maximum (shuffles + shared memory), a rescale of the register accumulators and the
+//     probabilities anew; otherwise a block costs four exponentials per thread.  Row sums stay per-thread until the end.
+// One CTA-wide barrier per block, and one per pair of warps; the raw blocks arrive on mbarriers with bounded waits
+// (Q4KV_FLAG_INTERNAL when one runs out; the 256 threads then leave together).
+//
+// What bounds it: 2800 clocks per block, of which 2050 are the expansion with both products (the tensor instructions of a
+// scheduler's two warps alone take 1150), 250 the softmax, 500 the barrier and the wait for the block; and per launch about
+// 6 us of prologue, first block, record and merge.  Eight warps because the queries' fragments, the accumulators and two
+// words in flight need the registers: sixteen warps of 128 registers (four per group of octets) took 22.1 us where this
+// takes 20.2 (4 agents x 16384 tokens with the merge), two groups of four warps with separate chunks 20.9.  The first form,
+// with an expanded key tile read through ldmatrix for the scores and three barriers per block, took 21.3 (23.8 with bfloat16
+// scales, now 20.6); 32 agents x 8192 tokens 110 us, now 60.
+#include <algorithm>
+
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
 #include "tcgen05.cuh"
@@ -44,9 +47,10 @@ constexpr int kComputeWarps = 8;
 constexpr int kThreads = kComputeWarps * 32;            // 256
 constexpr int kChunkBytes = 32 * (kD / 2 + 4 * (kD / 64));   // 10368: [Kc 9216 | Ksb 1152]
 constexpr int kRawBytes = 2 * kChunkBytes;               // one 64-key block
-constexpr int kTileBytes = 64 * kD * 2;                  // 73728
+constexpr int kOctetBytes = (kDv / 8) * 128;             // 8192: one key octet of the value tile
+constexpr int kTileBytes = 8 * kOctetBytes;              // 65536
 constexpr int kGroupStride = (kD / 8) * 128;             // 9216: bytes between 8-row groups of a [rows][576] tile
-constexpr int kStages = 2, kRawSlots = 2;
+constexpr int kStages = 2, kRawSlots = 3;
 constexpr int kRecStride = kDv + 2;                      // acc[512], m, l
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLazy = 8.f;
@@ -54,38 +58,38 @@ constexpr float kLazy = 8.f;
 using MlaParams = MlaDecodeParams;
 
 struct MlaSmem {
-  alignas(128) uint8_t khat[kStages][kTileBytes];        // [key 64][dim 576]: (key%8)*16 + (key/8)*9216 + (dim/8)*128
+  // [key octet = warp][word of 8 dims][8 keys x 16 bytes]; key k of the octet sits in slot k ^ 2 * (word % 4)
+  alignas(128) uint8_t vhat[kStages][kTileBytes];
   alignas(128) uint8_t raw[kRawSlots][kRawBytes];
   alignas(128) uint8_t qtile[kHeads * kD * 2];           // [head 16][dim 576], same form
-  alignas(128) uint8_t ptile[kHeads * 64 * 2];           // [head 16][key 64]: (h%8)*16 + (h/8)*1024 + (key/8)*128
+  alignas(128) uint8_t ptile[2][kHeads * 64 * 2];         // [head 16][key 64]: (h%8)*16 + (h/8)*1024 + (key/8)*128
   float kappa[kHeads];                                   // score in log2 units = S * kappa[head]
-  float wmax[kComputeWarps][kHeads];
-  float wsum[kComputeWarps][kHeads];
+  float wmax[8][kHeads];                                 // per key octet
+  float wsum[8][kHeads];
+  float4 exch[kComputeWarps][32];                        // half scores on their way to the other warp of a pair
   alignas(8) uint64_t raw_full[kRawSlots];
-  int grow[3], stop[3];
   int bad[kRawSlots];
   int abort_flag, poisoned;
+  uint32_t masks[2];
   uint32_t new_words[kD / 8], new_sb[kD / 64];           // the new token's codes and (scale, bias) pairs (update-and-fetch)
 };
 
 // Eight codes of one packed word -> eight binary16 values c * s + b in the order (0,4) (1,5) (2,6) (3,7),
 // one (scale, bias) for all (s2 = (s, s), b2 = (b, b)).  Or-ing a masked nibble into the mantissa of 1024
 // (ulp 1), or of 64 for a nibble four bits up (ulp 1/16), gives 1024 + c or 64 + c exactly.
-__device__ inline uint4 dequant8(uint32_t w, uint32_t s2, uint32_t b2) {
+__device__ inline uint4 dequant8(uint32_t w, uint32_t s2, uint32_t b2, uint32_t mask_lo, uint32_t mask_hi) {
   const uint32_t wh = w >> 8;
   const __half2 k1024 = __half2half2(__ushort_as_half((unsigned short)0x6400));
   const __half2 k64 = __half2half2(__ushort_as_half((unsigned short)0x5400));
   auto as_h2 = [](uint32_t u) { return *reinterpret_cast<__half2*>(&u); };
   auto as_u = [](__half2 h) { return *reinterpret_cast<uint32_t*>(&h); };
   const __half2 s = as_h2(s2), b = as_h2(b2);
-  const __half2 c04 = __hsub2(as_h2((w & 0x000F000Fu) | 0x64006400u), k1024);
-  const __half2 c15 = __hsub2(as_h2((w & 0x00F000F0u) | 0x54005400u), k64);
-  const __half2 c26 = __hsub2(as_h2((wh & 0x000F000Fu) | 0x64006400u), k1024);
-  const __half2 c37 = __hsub2(as_h2((wh & 0x00F000F0u) | 0x54005400u), k64);
+  const __half2 c04 = __hsub2(as_h2((w & mask_lo) | 0x64006400u), k1024);
+  const __half2 c15 = __hsub2(as_h2((w & mask_hi) | 0x54005400u), k64);
+  const __half2 c26 = __hsub2(as_h2((wh & mask_lo) | 0x64006400u), k1024);
+  const __half2 c37 = __hsub2(as_h2((wh & mask_hi) | 0x54005400u), k64);
   return make_uint4(as_u(__hfma2(c04, s, b)), as_u(__hfma2(c15, s, b)), as_u(__hfma2(c26, s, b)), as_u(__hfma2(c37, s, b)));
 }
-// element held by slot j of a 16-byte row
-__device__ inline int elem_of(int j) { return ((j & 1) << 2) | (j >> 1); }
 __device__ inline float fast_exp2(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -102,20 +106,47 @@ __device__ inline uint32_t bf16_pair_to_h2(uint32_t u, bool& overflow) {
   overflow |= (((h & 0x7C007C00u) + 0x04000400u) & 0x80008000u) != 0u;     // an exponent field of all ones
   return h;
 }
-__device__ inline void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // the eight compute warps
+__device__ inline void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // all eight warps
+// the same, and whether the predicate holds for any of the threads
+__device__ inline bool compute_any(bool p) {
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, 1, 256, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(any) : "r"((uint32_t)p) : "memory");
+  return any != 0u;
+}
+__device__ inline uint4 lds128(uint32_t at) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
+  return v;
+}
+__device__ inline uint32_t lds32(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at));
+  return v;
+}
+__device__ inline void sts128(uint32_t at, uint4 v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ inline uint2 lds64(uint32_t at) {
+  uint2 v;
+  asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at));
+  return v;
+}
+__device__ inline void pair_barrier(int op) { asm volatile("bar.sync %0, 64;" ::"r"(2 + op) : "memory"); }
+// (the two loads below carry no memory clobber: they stay between the barriers, which are volatile and do)
 // four 8x8 b16 matrices; lane l supplies the address of row l % 8 of matrix l / 8; register i <- matrix i,
 // thread (g, t) of the warp receiving the elements (row g, columns 2t, 2t+1)
 __device__ inline void ldmatrix_x4(uint32_t (&r)[4], uint32_t smem_addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr) : "memory");
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr));
 }
 // the same with every matrix transposed: thread (g, t) receives the elements (rows 2t, 2t+1, column g)
 __device__ inline void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t smem_addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr) : "memory");
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr));
 }
 __device__ inline void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -150,8 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kRawSlots; ++s) { mbar_init(&sm.raw_full[s], 1); sm.bad[s] = 0; }
-    for (int i = 0; i < 3; ++i) { sm.grow[i] = 0; sm.stop[i] = 0; }
     sm.abort_flag = 0; sm.poisoned = 0;
+    sm.masks[0] = 0x000F000Fu; sm.masks[1] = 0x00F000F0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -170,10 +201,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
 
   // Raw 64-key blocks: one bulk copy each into a two-slot ring, issued by thread 0 -- blocks 0 and 1 here, block
   // j + 2 once every warp has left block j's raw bytes (the barrier after the dequantize step).
-  auto issue_block = [&](int j) {
+  auto block_of = [&](int j) { return P.tables[(size_t)a * P.max_blocks + ((2 * (b0 + j)) >> 3)]; };
+  auto issue_block = [&](int j, int blk) {
     const int r = j % kRawSlots;
     const int c = 2 * (b0 + j);
-    const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
     if (blk < 0 || blk >= P.n_blocks) {
       sm.bad[r] = 1;
       sm.poisoned = 1;
@@ -187,9 +218,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   };
   int issued = 0;                                        // thread 0: blocks whose copy has been issued
   if (threadIdx.x == 0) {
-    issue_block(0);
-    if (n_iter > 1) issue_block(1);
+    issue_block(0, block_of(0));
     issued = min(n_iter, kRawSlots);
+    for (int j = 1; j < issued; ++j) issue_block(j, block_of(j));
   }
 
   // Update-and-fetch: the CTA whose share ends with the agent's last block quantizes the row of position n - 1
@@ -250,46 +281,70 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
       const float x2 = __uint_as_float(u23 << 16) * sf, x3 = __uint_as_float(u23 & 0xffff0000u) * sf;
       const float x4 = __uint_as_float(u45 << 16) * sf, x5 = __uint_as_float(u45 & 0xffff0000u) * sf;
       const float x6 = __uint_as_float(u67 << 16) * sf, x7 = __uint_as_float(u67 & 0xffff0000u) * sf;
-      *reinterpret_cast<uint4*>(sm.qtile + (h & 7) * 16 + (h >> 3) * kGroupStride + w * 128) =
+      *reinterpret_cast<uint4*>(sm.qtile + ((h & 7) ^ (2 * (w & 3))) * 16 + (h >> 3) * kGroupStride + w * 128) =
           make_uint4(f32x2_to_h2(x0, x4), f32x2_to_h2(x1, x5), f32x2_to_h2(x2, x6), f32x2_to_h2(x3, x7));
     }
   }
   compute_barrier();                                     // queries and kappa are complete
 
-  // per-chunk dequantize coordinates: thread xx of 128 owns token tau = 4 kg + ki of chunk ci and, of its 72 words,
-  // those with w % 4 == kt (four 16-byte pieces and one 8-byte piece).  The eight lanes of a shared-memory phase
-  // read eight different 16-byte columns and write eight different rows.
-  const int ci = tq >> 7, xx = tq & 127;
-  const int ki = xx & 3, kg = 2 * ((xx >> 3) & 3) + ((xx >> 2) & 1), kt = (ki + (xx >> 5)) & 3;
-  const int tau = 4 * kg + ki;
-  const int rd16 = ci * kChunkBytes + (ki * 144 + kg * 4 + kt) * 16;        // + j * 512
-  const int rd8 = ci * kChunkBytes + (ki * 576 + 512) * 4 + (kg * 4 + kt) * 8;
-  const int sb_at = ci * kChunkBytes + 9216 + ((((tau & 3) * 4 + (tau >> 3)) * 2 + ((tau >> 2) & 1)) * 9) * 4;   // + 4 * group
-  const int krow = ci * 32 + tau;
-  const int wr_at = (krow & 7) * 16 + (krow >> 3) * kGroupStride + kt * 128;
+  // Dequantize and score coordinates: the warps h = 0, 1 of pair op own the key octets 2 op and 2 op + 1 -- octet e is key
+  // tile e % 4 of chunk e / 4, the tokens 4 g + e % 4.  Lane (g, tid) of warp h takes the words 4 p + tid of token g of both
+  // octets for p = 8 h + i, i < 8 (two 16-byte pieces each), and of its own octet, 2 op + h, for p = 16 and 17 (an 8-byte
+  // one): eighteen words, which are the score product's B fragments once they are expanded.
+  const int op = warp & 3, hh = warp >> 2;               // the warps of a pair share a scheduler
+  const int ci = op >> 1, tile0 = 2 * (op & 1) + hh;     // own octet; the other one is tile0 ^ 1
+  const int oct = 4 * ci + tile0;
+  const uint32_t raw0 = smem_u32(sm.raw[0]) + ci * kChunkBytes;
+  const uint32_t rd_a = raw0 + (tile0 * 144 + hh * 64 + lane) * 16, rd_b = raw0 + ((tile0 ^ 1) * 144 + hh * 64 + lane) * 16;
+  const uint32_t rd8 = raw0 + (tile0 * 576 + 512) * 4 + lane * 8;
+  auto sb_row = [&](int t) { return raw0 + 9216 + (((t * 4 + (g >> 1)) * 2 + (g & 1)) * 9) * 4; };
+  const uint32_t sb_a = sb_row(tile0) + 16 * hh, sb_b = sb_row(tile0 ^ 1) + 16 * hh;    // + 4 (i / 2)
+  const uint32_t sb_8 = sb_row(tile0) + 32;
+  const uint32_t wr = smem_u32(sm.vhat[0]) + oct * kOctetBytes + (32 * hh + tid) * 128 + (g ^ (2 * tid)) * 16;   // + 512 i
+  const int wr_b = (oct & 1) ? -kOctetBytes : kOctetBytes;
+
+  // from memory, so that the compiler does not know them: (w & mask) | magic is one instruction with one immediate
+  const uint32_t mask_lo = sm.masks[0], mask_hi = sm.masks[1];
 
   // ldmatrix lane addresses (lane l: matrix l / 8, row l % 8)
   const int lm = lane >> 3, lr = lane & 7;
-  const uint32_t q_lane = smem_u32(sm.qtile) + lr * 16 + (lm & 1) * kGroupStride + (lm >> 1) * 128;   // + 256 per k-step
-  const uint32_t p_lane = smem_u32(sm.ptile) + lr * 16 + (lm & 1) * 1024 + (lm >> 1) * 128;           // + 256 per k-step
-  const uint32_t kq_lane = lr * 16 + warp * kGroupStride + lm * 128;        // scores: key octet = warp; + 512 per two k-steps
-  const uint32_t kv_lane = lr * 16 + (lm & 1) * kGroupStride + (8 * warp + (lm >> 1)) * 128;   // values: + 2 ks octets, + 256 per dim-core pair
+  const uint32_t p_lane = smem_u32(sm.ptile[0]) + lr * 16 + (lm & 1) * 1024 + (lm >> 1) * 128;        // + 256 per k-step
+  // values: key octets 2 ks + lm % 2, words 8 warp + 2 cc + lm / 2; from an even to an odd cc the slot's bit 2 flips
+  const uint32_t v_lane = smem_u32(sm.vhat[0]) + (lm & 1) * kOctetBytes + (8 * warp + (lm >> 1)) * 128 + (lr ^ (2 * (lm >> 1))) * 16;
+  const int v_step = 256 + ((lr & 4) ? -64 : 64);
 
-  // The queries never change: their A fragments (36 k-steps x 4 registers) live in registers for the whole launch.
-  uint32_t qa[kD / 16][4];
+  // The queries never change: the A fragments that meet this warp's words (20 k-steps x 4 registers) live in registers for
+  // the whole launch.  A k-step's 16 columns are elements 0, 4 | 1, 5 (or 2, 6 | 3, 7) of the four words 4 p + tid, so that
+  // what a lane has expanded from its own word is its B fragment.
+  uint32_t qa[20][4];
 #pragma unroll
-  for (int ks = 0; ks < kD / 16; ++ks) ldmatrix_x4(qa[ks], q_lane + ks * 256);
-  float kap[2], m_ref[2], l_part[2];                     // heads g and g + 8
-  kap[0] = sm.kappa[g]; kap[1] = sm.kappa[g + 8];
-  m_ref[0] = -INFINITY; m_ref[1] = -INFINITY; l_part[0] = 0.f; l_part[1] = 0.f;
-  float o[8][4];                                         // [dim core 8 warp + c][head g: slots 2 tid, 2 tid + 1 | head g + 8: same]
+  for (int i = 0; i < 10; ++i) {
+    const int w = 4 * (i < 8 ? 8 * hh + i : 8 + i) + tid;                   // of heads g and g + 8
+    const uint4 q0 = *reinterpret_cast<const uint4*>(sm.qtile + (g ^ (2 * tid)) * 16 + w * 128);
+    const uint4 q1 = *reinterpret_cast<const uint4*>(sm.qtile + kGroupStride + (g ^ (2 * tid)) * 16 + w * 128);
+    qa[2 * i][0] = q0.x; qa[2 * i][1] = q1.x; qa[2 * i][2] = q0.y; qa[2 * i][3] = q1.y;
+    qa[2 * i + 1][0] = q0.z; qa[2 * i + 1][1] = q1.z; qa[2 * i + 1][2] = q0.w; qa[2 * i + 1][3] = q1.w;
+  }
+  const float kap[2] = {sm.kappa[g], sm.kappa[g + 8]};
+  float m_ref[2] = {-INFINITY, -INFINITY}, l_part[2] = {0.f, 0.f};          // heads g and g + 8
+  float o[8][4];                                         // [word 8 warp + c][head g: slots 2 tid, 2 tid + 1 | head g + 8: same]
 #pragma unroll
   for (int c = 0; c < 8; ++c) { o[c][0] = 0.f; o[c][1] = 0.f; o[c][2] = 0.f; o[c][3] = 0.f; }
 
+  // Units of the value product, u = 4 ks + cc: 16 keys (k-step ks) x 16 dims (words 2 cc, 2 cc + 1 of this warp's eight)
+  auto load_values = [&](uint32_t (&bv)[4], uint32_t v_tile, int u) {
+    ldmatrix_x4_trans(bv, v_tile + (u >> 2) * 2 * kOctetBytes + ((u >> 1) & 1) * 512 + ((u & 1) ? v_step : 0));
+  };
+  auto values = [&](int u, const uint32_t (&pa)[4], const uint32_t (&bv)[4]) {
+    mma_f16(o[2 * (u & 3)], pa, bv[0], bv[1]);
+    mma_f16(o[2 * (u & 3) + 1], pa, bv[2], bv[3]);
+  };
+
   bool stopped = false;
   for (int j = 0; j < n_iter; ++j) {
-    const int s = j % kStages, r = j % kRawSlots;
-    // ---- raw block -> binary16 tile (every thread: one token of one chunk, 18 words) ----
+    const int r = j % kRawSlots;
+    int next_blk = 0;
+    if (tq == 0 && j + kRawSlots < n_iter) next_blk = block_of(j + kRawSlots);
     mbar_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag);     // a wait that runs out raises the give-up flag
     if (has_new && j == n_iter - 1) {
       // words 0..71 and the nine (scale, bias) pairs of position n - 1, one per thread
@@ -307,124 +362,118 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
       }
       compute_barrier();
     }
-    if (kBf) {
-      // bfloat16 scales and biases become binary16 in place, once per block (the tile is binary16); only the tokens
-      // below the agent's length count for the range report (bytes past the end are whatever was there)
-      bool overflow = false;
-      for (int w = tq; w < 2 * 288; w += kThreads) {     // per chunk: 32 tokens x 9 groups
-        const int cw = w >= 288 ? 1 : 0, o = w - 288 * cw;
-        const int row = o / 9;                           // (i * 4 + tid) * 2 + e: token 8 tid + 4 e + i
-        const int tok = 8 * ((row >> 1) & 3) + 4 * (row & 1) + (row >> 3);
-        uint32_t* at = reinterpret_cast<uint32_t*>(sm.raw[r] + cw * kChunkBytes + 9216 + 4 * o);
-        bool over = false;
-        *at = bf16_pair_to_h2(*at, over);
-        overflow |= over && (b0 + j) * 64 + cw * 32 + tok < n;
-      }
-      if (overflow && sm.bad[r] == 0) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
-      compute_barrier();
-    }
-    {
-      const uint8_t* raw = sm.raw[r];
-      const bool dead = sm.bad[r] != 0 || (b0 + j) * 64 + krow >= n;       // stale bytes past the end
-      uint8_t* dst = sm.khat[s] + wr_at;
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const uint4 kw = *reinterpret_cast<const uint4*>(raw + rd16 + jj * 512);
-        uint32_t sb0 = *reinterpret_cast<const uint32_t*>(raw + sb_at + 8 * jj);            // group 2 jj
-        uint32_t sb1 = *reinterpret_cast<const uint32_t*>(raw + sb_at + 8 * jj + 4);        // group 2 jj + 1
-        if (dead) { sb0 = 0u; sb1 = 0u; }
-        const uint32_t s0 = __byte_perm(sb0, sb0, 0x1010), c0 = __byte_perm(sb0, sb0, 0x3232);
-        const uint32_t s1 = __byte_perm(sb1, sb1, 0x1010), c1 = __byte_perm(sb1, sb1, 0x3232);
-        *reinterpret_cast<uint4*>(dst + (16 * jj + 0) * 128) = dequant8(kw.x, s0, c0);
-        *reinterpret_cast<uint4*>(dst + (16 * jj + 4) * 128) = dequant8(kw.y, s0, c0);
-        *reinterpret_cast<uint4*>(dst + (16 * jj + 8) * 128) = dequant8(kw.z, s1, c1);
-        *reinterpret_cast<uint4*>(dst + (16 * jj + 12) * 128) = dequant8(kw.w, s1, c1);
-      }
-      {
-        const uint2 kw = *reinterpret_cast<const uint2*>(raw + rd8);
-        uint32_t sb8 = *reinterpret_cast<const uint32_t*>(raw + sb_at + 32);                // group 8
-        if (dead) sb8 = 0u;
-        const uint32_t s8 = __byte_perm(sb8, sb8, 0x1010), c8 = __byte_perm(sb8, sb8, 0x3232);
-        *reinterpret_cast<uint4*>(dst + 64 * 128) = dequant8(kw.x, s8, c8);
-        *reinterpret_cast<uint4*>(dst + 68 * 128) = dequant8(kw.y, s8, c8);
-      }
-    }
-    if (tq == 0) sm.stop[j % 3] = *abort_flag;           // sampled by one thread: all 256 leave in the same block
-    compute_barrier();                                   // the tile is complete, and nobody reads the raw slot any more
-    if (sm.stop[j % 3]) { stopped = true; break; }
-    if (tq == 0 && j + kRawSlots < n_iter) { issue_block(j + kRawSlots); issued = j + kRawSlots + 1; }
-
-    // ---- scores of this warp's eight keys: S[16 heads][8 keys], 36 k-steps ----
+    // ---- expand this warp's share of eight keys; scores from the registers, the value part to shared memory; meanwhile the
+    //      value product of the block before (its probabilities are complete since the barrier at the end of its turn) ----
     float sc[4];
     {
-      // four independent accumulation chains (the tensor instruction's latency, not its rate, would bound one chain)
-      float acc[4][4];
+      const uint32_t at = r * kRawBytes, dst = wr + (j & 1) * kTileBytes;
+      const uint32_t p_prev = p_lane + ((j - 1) & 1) * (kHeads * 64 * 2), v_prev = v_lane + ((j - 1) & 1) * kTileBytes;
+      const int live = sm.bad[r] != 0 ? 0 : n - ((b0 + j) * 64 + ci * 32 + 4 * g);   // tokens from 4 g on; stale bytes past the end
+      bool overflow = false;
+      uint32_t sb[9];                                    // [own octet's four groups, the other one's, the own one's last]
+      uint4 k4[2] = {lds128(rd_a + at), lds128(rd_b + at)};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f; }
-      const uint32_t kb = smem_u32(sm.khat[s]) + kq_lane;
+      for (int i = 0; i < 4; ++i) { sb[i] = lds32(sb_a + at + 4 * i); sb[4 + i] = lds32(sb_b + at + 4 * i); }
+      sb[8] = lds32(sb_8 + at);
+      const uint2 k8 = lds64(rd8 + at);
+      uint32_t pa[2][4], bv[2][4];
+      ldmatrix_x4(pa[0], p_prev);
+      load_values(bv[0], v_prev, 0);
 #pragma unroll
-      for (int kk = 0; kk < kD / 32; ++kk) {
-        uint32_t bq[4];
-        ldmatrix_x4(bq, kb + kk * 512);
-        mma_f16(acc[(2 * kk) & 3], qa[2 * kk], bq[0], bq[1]);
-        mma_f16(acc[(2 * kk + 1) & 3], qa[2 * kk + 1], bq[2], bq[3]);
+      for (int i = 0; i < 9; ++i) {
+        if (live <= (i >= 4 && i < 8 ? tile0 ^ 1 : tile0)) sb[i] = 0u;
+        if (kBf) sb[i] = bf16_pair_to_h2(sb[i], overflow);
       }
+      auto expand = [&](uint32_t w, uint32_t pair) {
+        return dequant8(w, __byte_perm(pair, pair, 0x1010), __byte_perm(pair, pair, 0x3232), mask_lo, mask_hi);
+      };
+      float acc[2][4];                                   // [own octet, the other one]
 #pragma unroll
-      for (int e = 0; e < 4; ++e) sc[e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
+      for (int i = 0; i < 2; ++i) { acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f; }
+      uint4 next[2] = {};
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {                     // one word's expansion and scores, one unit of the value product
+        const int i = u >> 1, l = u & 1;
+        if (u == 4) { next[0] = lds128(rd_a + at + 512); next[1] = lds128(rd_b + at + 512); }
+        if (u == 8) { k4[0] = next[0]; k4[1] = next[1]; }
+        if ((u & 3) == 2 && u < 14) ldmatrix_x4(pa[((u >> 2) + 1) & 1], p_prev + ((u >> 2) + 1) * 256);
+        if (u < 15) load_values(bv[(u + 1) & 1], v_prev, u + 1);
+        const uint4 x = expand((i & 3) == 0 ? k4[l].x : (i & 3) == 1 ? k4[l].y : (i & 3) == 2 ? k4[l].z : k4[l].w, sb[4 * l + (i >> 1)]);
+        values(u, pa[(u >> 2) & 1], bv[u & 1]);
+        sts128(dst + (l ? wr_b : 0) + i * 512, x);
+        mma_f16(acc[l], qa[2 * i], x.x, x.y);
+        mma_f16(acc[l], qa[2 * i + 1], x.z, x.w);
+      }
+      // the halves of the words meet: each warp takes its own octet
+      sm.exch[warp ^ 4][lane] = make_float4(acc[1][0], acc[1][1], acc[1][2], acc[1][3]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const uint4 x = expand(i ? k8.y : k8.x, sb[8]);
+        mma_f16(acc[0], qa[16 + 2 * i], x.x, x.y);
+        mma_f16(acc[0], qa[17 + 2 * i], x.z, x.w);
+      }
+      if (j == 0) {                                      // there was no block before: what was summed is no product
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { o[c][0] = 0.f; o[c][1] = 0.f; o[c][2] = 0.f; o[c][3] = 0.f; }
+      }
+      if (kBf && overflow && sm.bad[r] == 0) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
+      pair_barrier(op);
+      const float4 e = sm.exch[warp][lane];
+      sc[0] = acc[0][0] + e.x; sc[1] = acc[0][1] + e.y; sc[2] = acc[0][2] + e.z; sc[3] = acc[0][3] + e.w;
     }
-    // this thread: heads g (sc[0], sc[1]) and g + 8 (sc[2], sc[3]), keys 8 warp + 2 tid, + 1
-    const int pos = (b0 + j) * 64 + 8 * warp + 2 * tid;
-    const bool v0 = pos >= lo && pos < n, v1 = pos + 1 >= lo && pos + 1 < n;
+    // this thread: heads g (sc[0], sc[1]) and g + 8 (sc[2], sc[3]), keys 2 tid and 2 tid + 1 of the own octet
+    const int pos = (b0 + j) * 64 + ci * 32 + 8 * tid + tile0;
+    const bool v0 = pos >= lo && pos < n, v1 = pos + 4 >= lo && pos + 4 < n;
     sc[0] = v0 ? sc[0] * kap[0] : -INFINITY; sc[1] = v1 ? sc[1] * kap[0] : -INFINITY;
     sc[2] = v0 ? sc[2] * kap[1] : -INFINITY; sc[3] = v1 ? sc[3] * kap[1] : -INFINITY;
     const float mx0 = fmaxf(sc[0], sc[1]), mx1 = fmaxf(sc[2], sc[3]);
     const bool grow = mx0 > m_ref[0] + kLazy || (m_ref[0] == -INFINITY && mx0 != -INFINITY) ||
                       mx1 > m_ref[1] + kLazy || (m_ref[1] == -INFINITY && mx1 != -INFINITY);
-    if (__any_sync(0xffffffffu, grow) && lane == 0) sm.grow[j % 3] = 1;
-    compute_barrier();                                   // growth agreed (and every warp has left the previous block's P)
-    if (tq == 0) sm.grow[(j + 2) % 3] = 0;               // not touched again before the barrier after next
-    if (sm.grow[j % 3]) {
-      // ---- exact per-head maxima of the block, new reference, rescale of what has been accumulated ----
+    // ---- probabilities relative to the references so far (a head without any key yet: reference -inf and p = 0) ----
+    float p[4];
+    uint32_t* pt = reinterpret_cast<uint32_t*>(sm.ptile[j & 1] + g * 16 + oct * 128 + 4 * tid);
+    auto probabilities = [&]() {
+      p[0] = v0 ? fast_exp2(sc[0] - m_ref[0]) : 0.f; p[1] = v1 ? fast_exp2(sc[1] - m_ref[0]) : 0.f;
+      p[2] = v0 ? fast_exp2(sc[2] - m_ref[1]) : 0.f; p[3] = v1 ? fast_exp2(sc[3] - m_ref[1]) : 0.f;
+      pt[0] = f32x2_to_h2(p[0], p[1]);
+      pt[256] = f32x2_to_h2(p[2], p[3]);
+    };
+    probabilities();
+    // The block's only barrier: the probabilities of all 64 keys and their value tile are in place; nobody reads the raw
+    // slot, or the tile and the probabilities of the block before, any more; growth (or a wait that ran out) is agreed.
+    if (compute_any(grow || *abort_flag != 0)) {
+      // ---- exact per-head maxima of the block, new references, rescale of what has been accumulated, probabilities anew ----
       float w0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)), w1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
       w0 = fmaxf(w0, __shfl_xor_sync(0xffffffffu, w0, 2)); w1 = fmaxf(w1, __shfl_xor_sync(0xffffffffu, w1, 2));
-      if (tid == 0) { sm.wmax[warp][g] = w0; sm.wmax[warp][g + 8] = w1; }
-      compute_barrier();
+      if (tid == 0) { sm.wmax[oct][g] = w0; sm.wmax[oct][g + 8] = w1; }
+      if (compute_any(*abort_flag != 0)) { stopped = true; break; }        // all leave in the same block
       float f[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         float m_new = m_ref[e];
 #pragma unroll
-        for (int w = 0; w < kComputeWarps; ++w) m_new = fmaxf(m_new, sm.wmax[w][g + 8 * e]);
+        for (int w = 0; w < 8; ++w) m_new = fmaxf(m_new, sm.wmax[w][g + 8 * e]);
         f[e] = m_new == -INFINITY ? 1.f : fast_exp2(m_ref[e] - m_new);     // m_ref = -inf: 0
         l_part[e] *= f[e];
         m_ref[e] = m_new;
       }
 #pragma unroll
       for (int c = 0; c < 8; ++c) { o[c][0] *= f[0]; o[c][1] *= f[0]; o[c][2] *= f[1]; o[c][3] *= f[1]; }
+      probabilities();
+      compute_barrier();
     }
-    // ---- probabilities (a head without any key yet keeps the reference at -inf and p = 0) ----
-    const float p0 = v0 ? fast_exp2(sc[0] - m_ref[0]) : 0.f, p1 = v1 ? fast_exp2(sc[1] - m_ref[0]) : 0.f;
-    const float p2 = v0 ? fast_exp2(sc[2] - m_ref[1]) : 0.f, p3 = v1 ? fast_exp2(sc[3] - m_ref[1]) : 0.f;
-    l_part[0] += p0 + p1; l_part[1] += p2 + p3;
-    *reinterpret_cast<uint32_t*>(sm.ptile + (g & 7) * 16 + 0 * 1024 + warp * 128 + 4 * tid) = f32x2_to_h2(p0, p1);
-    *reinterpret_cast<uint32_t*>(sm.ptile + (g & 7) * 16 + 1 * 1024 + warp * 128 + 4 * tid) = f32x2_to_h2(p2, p3);
-    compute_barrier();                                   // the probabilities of all 64 keys are in place
-
-    // ---- values: O[16 heads][dims 64 warp ..] += P V^, four k-steps of 16 keys ----
-    {
-      const uint32_t vb = smem_u32(sm.khat[s]) + kv_lane;
+    l_part[0] += p[0] + p[1]; l_part[1] += p[2] + p[3];
+    if (tq == 0 && j + kRawSlots < n_iter) { issue_block(j + kRawSlots, next_blk); issued = j + kRawSlots + 1; }
+  }
+  if (!stopped) {                                        // the last block's value product
+    const uint32_t p_last = p_lane + ((n_iter - 1) & 1) * (kHeads * 64 * 2), v_last = v_lane + ((n_iter - 1) & 1) * kTileBytes;
+    uint32_t pa[4], bv[2][4];
+    load_values(bv[0], v_last, 0);
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        uint32_t pa[4];
-        ldmatrix_x4(pa, p_lane + ks * 256);
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-          uint32_t bv[4];
-          ldmatrix_x4_trans(bv, vb + ks * 2 * kGroupStride + c * 128);
-          mma_f16(o[c], pa, bv[0], bv[1]);
-          mma_f16(o[c + 1], pa, bv[2], bv[3]);
-        }
-      }
+    for (int u = 0; u < 16; ++u) {
+      if ((u & 3) == 0) ldmatrix_x4(pa, p_last + (u >> 2) * 256);
+      if (u < 15) load_values(bv[(u + 1) & 1], v_last, u + 1);
+      values(u, pa, bv[u & 1]);
     }
   }
 
@@ -434,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
     float lh = l_part[e];
     lh += __shfl_xor_sync(0xffffffffu, lh, 1);
     lh += __shfl_xor_sync(0xffffffffu, lh, 2);
-    if (tid == 0) sm.wsum[warp][g + 8 * e] = lh;
+    if (tid == 0) sm.wsum[oct][g + 8 * e] = lh;
   }
   compute_barrier();
   const bool spoiled = stopped || sm.poisoned != 0;
@@ -444,14 +493,18 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
       for (uint32_t i = 0; i < 64 && !mbar_try_wait(&sm.raw_full[jj % kRawSlots], (uint32_t)(jj / kRawSlots) & 1u); ++i) {}
     raise_flag(P.flags, Q4KV_FLAG_INTERNAL);
   }
+  // Slots 2 tid and 2 tid + 1 of a word's row are its elements tid and tid + 4: even and odd lanes exchange one of the two, so
+  // that an even lane stores the elements tid and tid + 1, an odd one tid + 3 and tid + 4 (whole sectors of eight floats).
+  const int d_lane = 8 * 8 * warp + ((tid & 1) ? tid + 3 : tid);
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    // dim core 8 warp + c, slots 2 tid and 2 tid + 1 of its 16-byte row
-    const int d0 = 8 * (8 * warp + c) + elem_of(2 * tid), d1 = 8 * (8 * warp + c) + elem_of(2 * tid + 1);
-    rec[g * kRecStride + d0] = spoiled ? 0.f : o[c][0];
-    rec[g * kRecStride + d1] = spoiled ? 0.f : o[c][1];
-    rec[(g + 8) * kRecStride + d0] = spoiled ? 0.f : o[c][2];
-    rec[(g + 8) * kRecStride + d1] = spoiled ? 0.f : o[c][3];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float got = __shfl_xor_sync(0xffffffffu, (tid & 1) ? o[c][2 * e] : o[c][2 * e + 1], 1);
+      float2 v = (tid & 1) ? make_float2(got, o[c][2 * e + 1]) : make_float2(o[c][2 * e], got);
+      if (spoiled) v = make_float2(0.f, 0.f);
+      *reinterpret_cast<float2*>(rec + (g + 8 * e) * kRecStride + d_lane + 8 * c) = v;      // 514 floats a head: 8-byte aligned
+    }
   }
   if (warp == 0 && tid == 0) {
 #pragma unroll
@@ -466,19 +519,22 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   }
 }
 
-// grid: (16 heads, n_agents, 4 quarters of the value dims), 512 threads; combines the records of one (agent, head)
-// for 128 output dims.  The records sit in L2 a microsecond away, so nothing here is a chain of dependent loads: thread
-// s fetches (m, l) of split s, the block agrees on the weights, while sixteen groups of 32 threads each take every
-// sixteenth split with their loads issued together (up to 64 splits are in flight before the weights are known),
-// and the groups' sums meet in shared memory.  Four CTAs per (agent, head) rather than one: a quarter of the record
-// bytes per CTA and four times the SMs pulling them (4.1 -> see the profile).
-constexpr int kMergeThreads = 512, kMaxSplits = 512, kMergeGroups = kMergeThreads / 32, kMergeQuarters = 4;
+// grid: (16 heads, n_agents, 128 / kLanes slices of the value dims), 512 threads; combines the records of one (agent, head)
+// for 4 kLanes output dims.  The records sit in L2 a microsecond away, so nothing here is a chain of dependent loads: thread
+// s fetches (m, l) of split s, the block agrees on the weights, while the 512 / kLanes groups of threads each take every
+// so-many-th split with their loads issued together before the weights are known, and the groups' sums meet in registers
+// (groups of one warp) and shared memory.  How narrow the slices are depends on the count of splits: with four of them
+// sixteen groups would leave most threads idle (and make four times the CTAs), with 148 each group would walk nine.
+constexpr int kMergeThreads = 512, kMaxSplits = 512;
+template <int kLanes>
 __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_splits, const float* __restrict__ records,
                                                                   void* __restrict__ out, int out_dtype,
                                                                   float* __restrict__ lse) {
   __shared__ float s_w[kMaxSplits];                      // weight of each split (0: empty)
   __shared__ float s_red[kMergeThreads / 32][2];
-  __shared__ float4 s_acc[kMergeGroups - 1][32];
+  constexpr int kGroups = kMergeThreads / kLanes;
+  constexpr int kRows = kLanes < 32 ? kMergeThreads / 32 : kGroups;         // sums that meet in shared memory
+  __shared__ float4 s_acc[kRows - 1][kLanes];
   __shared__ float s_ml[2];
   const int h = blockIdx.x, a = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -486,14 +542,14 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
   if (h >= Hq) return;
   const float* rec = records + ((size_t)a * n_splits * kHeads + h) * kRecStride;
   const size_t step = (size_t)kHeads * kRecStride;       // between the splits of one head
-  // The record loads of the first 16 * kPre splits do not wait for the weights: they are issued first and overlap the
+  // The record loads of the first kGroups * kPre splits do not wait for the weights: they are issued first and overlap the
   // round trip of the (m, l) loads (an empty split's data is whatever an earlier call left there; it is dropped below).
   constexpr int kPre = 4;
-  const int grp = warp, d = (kDv / kMergeQuarters) * blockIdx.z + 4 * lane;   // 32 lanes x 4 consecutive dims per group
+  const int grp = tid / kLanes, gl = tid % kLanes, d = 4 * (kLanes * blockIdx.z + gl);   // 4 consecutive dims per thread
   float4 pre[kPre];
 #pragma unroll
   for (int u = 0; u < kPre; ++u) {
-    const int sp = grp + kMergeGroups * u;
+    const int sp = grp + kGroups * u;
     pre[u] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (sp < n_splits) {
       const float2 lo2 = *reinterpret_cast<const float2*>(rec + sp * step + d);       // records are 8-byte aligned
@@ -527,14 +583,14 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
   for (int u = 0; u < kPre; ++u) {
-    const int sp = grp + kMergeGroups * u;
+    const int sp = grp + kGroups * u;
     const float wu = sp < n_splits ? s_w[sp] : 0.f;
     if (wu > 0.f) {                                      // an empty split's record holds no data
       acc.x = fmaf(wu, pre[u].x, acc.x); acc.y = fmaf(wu, pre[u].y, acc.y);
       acc.z = fmaf(wu, pre[u].z, acc.z); acc.w = fmaf(wu, pre[u].w, acc.w);
     }
   }
-  for (int sp = grp + kMergeGroups * kPre; sp < n_splits; sp += kMergeGroups) {
+  for (int sp = grp + kGroups * kPre; sp < n_splits; sp += kGroups) {
     const float wu = s_w[sp];
     if (wu > 0.f) {
       const float2 lo2 = *reinterpret_cast<const float2*>(rec + sp * step + d);
@@ -543,13 +599,21 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
       acc.z = fmaf(wu, hi2.x, acc.z); acc.w = fmaf(wu, hi2.y, acc.w);
     }
   }
-  if (grp > 0) s_acc[grp - 1][lane] = acc;
+  if (kLanes < 32) {
+#pragma unroll
+    for (int o = kLanes; o < 32; o *= 2) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+    }
+  }
+  const int row = kLanes < 32 ? warp : grp;
+  if (row > 0 && (kLanes >= 32 || lane < kLanes)) s_acc[row - 1][gl] = acc;
   __syncthreads();
-  if (grp > 0) return;
+  if (tid >= kLanes) return;
   const float Lsum = s_ml[1];
   const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
 #pragma unroll
-  for (int g = 0; g < kMergeGroups - 1; ++g) { const float4 o = s_acc[g][lane]; acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w; }
+  for (int g = 0; g < kRows - 1; ++g) { const float4 o = s_acc[g][gl]; acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w; }
   acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
   const size_t out_index = ((size_t)a * Hq + h) * kDv;
   if (out_dtype == Q4KV_OUT_BF16) {
@@ -568,10 +632,14 @@ struct MlaPlan { int n_splits, blocks_per_split; };
 MlaPlan plan_mla(int n_agents, int max_kv_len, int window) {
   const int span = (window > 0 && window + 64 < max_kv_len) ? window + 64 : max_kv_len;
   const int blocks = (span + 63) / 64 + 1;               // a window may straddle one more 64-key block
-  int n_splits = (sm_count() + n_agents - 1) / n_agents;   // about one CTA per SM
+  // One CTA per SM, in as few waves as the count of agents allows: rounding the shares of an agent up puts up to n_agents - 1
+  // CTAs into a second wave, which pays only where the shares get that much shorter.  A wave costs its blocks and about
+  // four more for its prologue and its record.
+  const int sms = sm_count(), up = (sms + n_agents - 1) / n_agents, down = sms / n_agents;
+  auto cost = [&](int n) { return ((long long)n * n_agents + sms - 1) / sms * ((blocks + n - 1) / n + 4); };
+  int n_splits = down > 0 && cost(down) <= cost(up) ? down : up;
   if (n_splits > blocks) n_splits = blocks;
   if (n_splits > kMaxSplits) n_splits = kMaxSplits;
-  if (n_splits < 1) n_splits = 1;
   MlaPlan p;
   p.blocks_per_split = (blocks + n_splits - 1) / n_splits;
   p.n_splits = (blocks + p.blocks_per_split - 1) / p.blocks_per_split;
@@ -586,9 +654,9 @@ bool decode_mla_supported(const Layout& y) {
 
 size_t decode_mla_workspace_bytes(const Layout& y, int n_agents, int max_kv_len) {
   (void)y;
-  // the split count depends on the window only through a smaller span: size for the whole cache
-  const MlaPlan p = plan_mla(n_agents, max_kv_len, 0);
-  return (size_t)n_agents * p.n_splits * kHeads * kRecStride * sizeof(float);
+  // the split count depends on the window through the span: room for the most that any span gets
+  const int blocks = (max_kv_len + 63) / 64 + 1, most = (sm_count() + n_agents - 1) / n_agents;
+  return (size_t)n_agents * std::min(std::min(blocks, most), kMaxSplits) * kHeads * kRecStride * sizeof(float);
 }
 
 cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
@@ -596,9 +664,7 @@ cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, i
                               int out_dtype, float* lse, void* ws, int32_t* flags, cudaStream_t st, const void* k_new,
                               bool on_codes) {
   if (b.n_agents <= 0) return cudaSuccess;
-  MlaPlan plan = plan_mla(b.n_agents, max_kv_len, window);
-  const MlaPlan full = plan_mla(b.n_agents, max_kv_len, 0);
-  if (plan.n_splits > full.n_splits) plan = full;        // never more records than the workspace was sized for
+  const MlaPlan plan = plan_mla(b.n_agents, max_kv_len, window);
   MlaParams P;
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents;
   P.max_blocks = b.max_blocks; P.tables = b.block_tables; P.kv_lens = kv_lens; P.len_cap = max_kv_len; P.window = window;
@@ -634,12 +700,18 @@ cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, i
   }
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t mcfg = {};
-  mcfg.gridDim = dim3(kHeads, b.n_agents, kMergeQuarters);
+  // 4, 8, 16 or 64 groups of threads share the splits, so that a thread's loads are few and all in flight together.  Measured,
+  // merge and kernel: 4 splits x 32 agents 60.1 us on 128 lanes (66.2 on 32), 17 x 8 13.5 on 64 (14.4 on 32), 37 x 4 20.2 on
+  // 32 (21.6 on 64, 21.0 on 16), 148 x 1 22.4 on 8 (24.1 on 32).
+  const int lanes = plan.n_splits <= 8 ? 128 : plan.n_splits <= 24 ? 64 : plan.n_splits <= 64 ? 32 : 8;
+  void (*merge)(int, int, const float*, void*, int, float*) =
+      lanes == 128 ? merge_mla_kernel<128> : lanes == 64 ? merge_mla_kernel<64> : lanes == 32 ? merge_mla_kernel<32> : merge_mla_kernel<8>;
+  mcfg.gridDim = dim3(kHeads, b.n_agents, kDv / 4 / lanes);
   mcfg.blockDim = dim3(kMergeThreads);
   mcfg.stream = st;
   mcfg.attrs = attr;
   mcfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&mcfg, merge_mla_kernel, (int)y.Hq, plan.n_splits, (const float*)ws, out, out_dtype, lse);
+  return cudaLaunchKernelEx(&mcfg, merge, (int)y.Hq, plan.n_splits, (const float*)ws, out, out_dtype, lse);
 }
 
 }  // namespace q4kv
