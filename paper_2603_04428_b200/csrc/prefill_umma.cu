@@ -320,12 +320,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     {
       // ---- stage the query row: bf16 -> binary16 times a power of two ----
       const uint16_t* qrow = P.q + (valid ? row_index : 0) * 128;
-      uint4 v[16];
-#pragma unroll
-      for (int p = 0; p < 16; ++p) v[p] = valid ? __ldcg(reinterpret_cast<const uint4*>(qrow + 8 * p)) : make_uint4(0u, 0u, 0u, 0u);
+      auto piece = [&](int p) { return valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : make_uint4(0u, 0u, 0u, 0u); };
       float mx = 0.f;
 #pragma unroll
-      for (int p = 0; p < 16; ++p) mx = fmaxf(mx, max_abs8(v[p]));
+      for (int p = 0; p < 16; ++p) mx = fmaxf(mx, max_abs8(piece(p)));
       int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
       if (mx == 0.f) ex = 0;
       ex = min(max(ex, -100), 100);
@@ -333,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
       kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
 #pragma unroll
       for (int p = 0; p < 16; ++p)
-        *reinterpret_cast<uint4*>(sm.qs[t] + (row & 7) * 16 + (row >> 3) * 2048 + p * 128) = query8(v[p], sf);
+        *reinterpret_cast<uint4*>(sm.qs[t] + (row & 7) * 16 + (row >> 3) * 2048 + p * 128) = query8(piece(p), sf);
       fence_async_smem();
       mbar_arrive(&sm.q_ready);
     }
