@@ -536,6 +536,24 @@ def test_decode_more_than_four_query_heads_per_kv_head(H, spec_args, lens, windo
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("n_heads,lens,sb_dtype", [
+    (16, [9000, 70], 0),                                     # 74 key shares per agent
+    (16, [4800], 1),                                         # 38, one agent
+    (3, [700 + 9 * i for i in range(8)], 0),                 # twelve; 8 x 19 CTAs would not fit one wave
+    (16, [1 + 37 * i for i in range(40)], 1),                # three: 40 x 4 would not either
+    (16, [5 + i for i in range(150)], 0),                    # more agents than SMs
+])
+def test_latent_decode_shares_and_merges(H, n_heads, lens, sb_dtype):
+    p = Pair(H, (1, n_heads, 1, 576, 512, True), lens, seed=53, sb_dtype=sb_dtype).fill()
+    q = p.q(7, len(lens))
+    scale = 1.0 / math.sqrt(192)
+    out, lse = p.dc.decode(0, lens, 0, q, scale)
+    ref, rlse = O.decode_attention(p.opool, 0, p.tabs, lens, 0, f32(q), scale)
+    assert_attention_close(out.cpu().numpy(), ref, "decode")
+    assert_lse_close(lse.cpu().numpy(), rlse)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("window", [0, 150])
 def test_decode_latent_cache_at_a_sharp_scale_takes_the_exact_kernel(H, window):
     """scale^2 * d_qk > 4 on the V-aliasing cache: routed to the kernel that keeps the values exact."""
@@ -892,6 +910,83 @@ def test_prefill_tcgen05_path(H, spec_args, prefix, chunks, window, scale_mul):
     out16, _ = p.dc.prefill(0, lens, q_offs, window, q, scale, out_dtype=B.OUT_BF16)
     assert torch.allclose(out16.float(), out.to(torch.bfloat16).float(), atol=1e-5, rtol=2.0 ** -7)
     assert p.dc.read_flags() == 0
+
+
+def check_prefill(H, spec_args, prefix, chunks, window, sb_dtype=0, scale=None):
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = QuietStartPair(H, spec_args, lens, seed=59, sb_dtype=sb_dtype).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = p.q(9, int(q_offs[-1]))
+    scale = scale or 1.0 / math.sqrt(spec_args[3])
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, window, f32(q), scale)
+    out, lse = p.dc.prefill(0, lens, q_offs, window, q, scale)
+    assert_attention_close(out.cpu().numpy(), ref)
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    assert p.dc.read_flags() == 0
+    return p, lens, q_offs, q, scale, out
+
+
+@pytest.mark.parametrize("n_heads,prefix,chunks,window,sb_dtype", [
+    (16, [0, 33], [65, 8], 0, 0),                            # no prefix, a tile of eight queries exactly, one query over
+    (16, [300, 64, 0], [9, 64, 1], 0, 1),
+    (16, [3000], [40], 700, 0),                              # a window that starts inside a 64-key block
+    (16, [6000, 10], [7, 3], 0, 1),                          # few tiles: the keys are split
+    (5, [500], [70], 0, 0),                                  # heads that do not divide the tile
+])
+def test_prefill_over_the_latent_cache(H, n_heads, prefix, chunks, window, sb_dtype):
+    from paper_2603_04428_b200 import binding as B
+    p, lens, q_offs, q, scale, out = check_prefill(H, (1, n_heads, 1, 576, 512, True), prefix, chunks, window, sb_dtype,
+                                                   1.0 / math.sqrt(192))
+    out16, _ = p.dc.prefill(0, lens, q_offs, window, q, scale, out_dtype=B.OUT_BF16)
+    assert torch.allclose(out16.float(), out.to(torch.bfloat16).float(), atol=1e-5, rtol=2.0 ** -7)
+    tabs = p.tabs.copy()
+    tabs[0, (lens[0] - 1) // 256] = p.n_blocks + 3           # a block outside the pool: its agent's rows are zero
+    t = H.dev(tabs)
+    bad, lse_bad = p.dc.prefill(0, lens, q_offs, window, q, scale, bt=B.batch(t))
+    assert p.dc.read_flags() & B.FLAG_BAD_BLOCK
+    n0 = int(q_offs[1])
+    assert torch.all(bad[n0 - 1] == 0) and torch.isneginf(lse_bad[n0 - 1]).all()
+    assert torch.allclose(bad[n0:], out[n0:], atol=1e-5)
+
+
+@pytest.mark.parametrize("spec_args,prefix,chunks,window,sb_dtype", [
+    ((1, 8, 2, 128, 128, False), [9000], [40], 0, 0),        # two tiles of work: many splits of the keys
+    ((1, 8, 2, 128, 128, False), [9000, 3], [33, 2], 2500, 1),   # under a window; an agent whose splits are mostly empty
+    ((1, 4, 2, 256, 256, False), [5000], [65], 0, 0),
+    ((1, 4, 4, 192, 128, False), [5000, 0], [129, 30], 0, 1),
+    ((1, 10, 2, 128, 128, False), [300, 5], [30, 60], 0, 0),     # five query heads per KV head
+    ((1, 16, 2, 128, 128, False), [300], [70], 100, 0),          # eight
+    ((1, 16, 1, 256, 256, False), [200], [20], 0, 1),            # sixteen at d = 256
+    ((1, 7, 1, 192, 128, False), [100], [50], 0, 0),             # seven at d_qk 192
+])
+def test_prefill_key_splits_and_head_counts(H, spec_args, prefix, chunks, window, sb_dtype):
+    check_prefill(H, spec_args, prefix, chunks, window, sb_dtype)
+
+
+@pytest.mark.parametrize("spec_args,window", [
+    ((1, 8, 2, 128, 128, False), 0),
+    ((1, 8, 2, 128, 128, False), 90),
+    ((1, 4, 2, 256, 256, False), 0),
+    ((1, 4, 4, 192, 128, False), 0),
+    ((1, 16, 2, 128, 128, False), 0),
+])
+@pytest.mark.parametrize("chunks", [
+    [1, 70, 1, 1, 0, 1, 1],                                  # 3 x 75 rows < 7 agents x 70: the single queries leave the tiles
+    [1, 3, 1, 1, 1, 1],                                      # 3 x 8 > 6 x 3: they stay
+    [1, 1, 1, 1, 1, 1, 1],                                   # nothing but single queries
+])
+def test_prefill_of_mostly_single_queries(H, spec_args, window, chunks):
+    prefix = [0, 130, 255, 256, 40, 31, 2000][:len(chunks)]
+    check_prefill(H, spec_args, prefix, chunks, window)
+
+
+@pytest.mark.parametrize("spec_args,lens,sb_dtype", [
+    ((1, 16, 16, 192, 128, False), [2200, 31], 0),           # 16 x (69 + 4) units: four warps each
+    ((1, 16, 16, 192, 128, False), [2290, 31], 1),           # 16 x (72 + 4) units: one warp each
+    ((1, 16, 1, 576, 512, True), [38000], 0),                # latent rows, one warp per unit
+])
+def test_append_on_both_sides_of_the_unit_split(H, spec_args, lens, sb_dtype):
+    Pair(H, spec_args, lens, seed=61, sb_dtype=sb_dtype).fill().check_packed_equal()
 
 
 @pytest.mark.parametrize("gain,outlier_frac", [(8.0, 0.0), (1.0, 0.01)])
