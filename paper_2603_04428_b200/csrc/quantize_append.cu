@@ -159,15 +159,16 @@ quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_a
 // items -- (octet of eight positions, pass of four groups: K groups first, then V groups) -- with the loads of the
 // next item in flight while the current one is quantized.  Within an item a lane owns one of the eight positions and
 // one 64-element group: it loads its 64 elements as eight 16-byte words, takes minimum and maximum with packed bf16
-// instructions (no cross-lane step at all), and quantizes them two at a time (packed binary32): t = x - bias, c = t *
-// (1/scale) rounded by adding 1.5 * 2^23 in the same fma, and the distance of t * (1/scale) from c; a word with a quotient
-// within 4e-6 of a tie is decided from exact residuals, so that the codes equal those of the fixed sequence bit for bit.  V words
+// instructions (no cross-lane step at all), and quantizes them two at a time (packed binary32; see quantize_code for why the
+// codes equal those of the fixed sequence bit for bit).  V words
 // are first exchanged between the eight lanes of a group (an 8 x 8 transposition of words by twelve shuffles), which leaves
 // in each lane the 8 positions x 8 elements block of nibbles that an in-register transposition turns into eight token-packed
 // words.  The chunk is assembled in shared memory and stored as whole 16-byte pieces; a chunk that the phase fills only in
 // part (an unaligned start or end) starts from its present bytes.
-// kWpc = 1 where the units fill the GPU; 4 for smaller phases, whose time is one unit's chain of items.
-// Bound by instruction issue: see launch_quantize_append for the times.
+// Bound by instruction issue and, with the sixteen warps an SM has room for, by the latency of the loads: 14.4 instructions an
+// element (18.7 before ties were left to the corrected quotient), issued at 0.46 a clock.  Measured at d = 128, 8 KV heads:
+// 8 x 1024 tokens 20.4 -> 16.3 us, 8 x 4096 69 -> 56 us.  kWpc = 1 where the units fill the GPU; 4 for smaller phases, whose
+// time is one unit's chain of items: 5 x 64 tokens 12.8 -> 4.4 us, latent cache 8 x 1024 tokens 29 -> 10 us.
 // ---------------------------------------------------------------------------------------------
 __device__ inline void transpose_nibbles_8x8_regs(uint32_t (&r)[8]) {
   // rows = registers, columns = nibbles: three rounds of block swaps
@@ -184,25 +185,13 @@ __device__ inline void transpose_nibbles_8x8_regs(uint32_t (&r)[8]) {
   }
 }
 
-// The eight codes of a word with a quotient within a few ulps of a tie, without dividing.  With k = floor(t * inv) and v = k +
-// 1/2 the residual t - s v is exact (s v has at most 16 significant bits, and t is close to it); the rounded quotient of the
-// fixed sequence is v itself where the residual is at most half an ulp of v times s, and then goes to the even neighbour.
-// Rows of bf16 numbers meet exact ties often (7e-4 of all elements), so this is not rare: one warp in six per word.
-__device__ __noinline__ uint32_t exact_word(uint4 raw, float bf, float sf, float inv) {
+// The eight codes of a word for a (bfloat16) scale without a finite reciprocal.
+__device__ __noinline__ uint32_t divided_word(uint4 raw, GroupScale gs, float inv) {
   const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
   uint32_t word = 0u;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const float x = (e & 1) ? __uint_as_float(wv[e >> 1] & 0xffff0000u) : __uint_as_float(wv[e >> 1] << 16);
-    const float t = __fsub_rn(x, bf);
-    const float k = floorf(t * inv), v = k + 0.5f;
-    const float rr = __fmaf_rn(-sf, v, t);
-    // half an ulp of v; below 1/2, a power of two, the spacing is half as wide
-    float lim = sf * (__uint_as_float(__float_as_uint(v) & 0x7f800000u) * 5.9604644775390625e-8f);
-    if (k == 0.f && rr < 0.f) lim *= 0.5f;
-    const uint32_t ki = (uint32_t)k;
-    word |= min(ki + (fabsf(rr) <= lim ? (ki & 1u) : rr > 0.f ? 1u : 0u), 15u) << (4 * e);
-  }
+  for (int e = 0; e < 4; ++e)
+    word |= (quantize_code(__uint_as_float(wv[e] << 16), gs, inv) | (quantize_code(__uint_as_float(wv[e] & 0xffff0000u), gs, inv) << 4)) << (8 * e);
   return word;
 }
 
@@ -291,10 +280,8 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
   const int n_groups = y.G + (y.alias ? 0 : y.Gv);
   const int n_pass = (n_groups + 3) >> 2;
   const int n_items = (o_last - o_first + 1) * n_pass;
-  constexpr float kMagic = 12582912.0f;                  // 1.5 * 2^23: (q + kMagic) - kMagic is q rounded to nearest even
-  // t * inv is within 2 ulps (2e-6 at q < 16) of the quotient the fixed sequence rounds: beyond 4e-6 of a tie both round
-  // to the same code
-  constexpr float kTieZone = 0.499996f;
+  constexpr float kMagic = 12582912.0f;                  // 1.5 * 2^23: q + kMagic holds q rounded to nearest even in its low bits
+  constexpr uint32_t kMagicSum = 0x4B400000u * (1u + 16u + 256u);           // what eight of them add to a word (e > 2: shifted out)
 
   // item t: octet o_first + t / n_pass of the chunk, groups 4 * (t % n_pass) .. + 3
   auto load_item = [&](int t, uint4 (&raw)[8]) {
@@ -352,26 +339,27 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
     for (int j = 0; j < 8; ++j) cw[j] = 0u;
     if (gs.sf != 0.0f) {
       const float inv = __frcp_rn(gs.sf);
-      const uint64_t nb2 = pair64(-gs.bf, -gs.bf), inv2 = pair64(inv, inv), ninv2 = pair64(-inv, -inv);
-      const uint64_t up2 = pair64(kMagic, kMagic), down2 = pair64(-kMagic, -kMagic), k256 = pair64(256.f, 256.f);
+      const uint64_t nb2 = pair64(-gs.bf, -gs.bf), inv2 = pair64(inv, inv), ns2 = pair64(-gs.sf, -gs.sf), up2 = pair64(kMagic, kMagic);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint32_t wv[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
-        // t = x - bias, c = t / scale (as t * inv) rounded to nearest even by adding and subtracting 1.5 * 2^23;
-        // the quotient is at most 15 + a few ulps by construction of the scale, so no clamp is needed.  The eight codes
-        // are assembled in floating point (two exact 16-bit halves) instead of by shifts.
-        uint64_t c[4];
-        float far = 0.f;
+        // quantize_code, two elements at a time; the quotient is at most 15 + a few ulps by construction of the scale, hence
+        // no clamp
+        uint32_t m[8];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const uint64_t t = add2(pair64(__uint_as_float(wv[e] << 16), __uint_as_float(wv[e] & 0xffff0000u)), nb2);
-          c[e] = add2(fma2(t, inv2, up2), down2);
-          const float2 d = unpair64(fma2(t, ninv2, c[e]));
-          far = fmaxf(far, fmaxf(fabsf(d.x), fabsf(d.y)));
+          const uint64_t q = mul2(t, inv2);
+          const float2 r = unpair64(add2(fma2(fma2(ns2, q, t), inv2, q), up2));
+          m[2 * e] = __float_as_uint(r.x); m[2 * e + 1] = __float_as_uint(r.y);
         }
-        const float2 a = unpair64(fma2(c[1], k256, c[0])), b = unpair64(fma2(c[3], k256, c[2]));
-        cw[j] = far > kTieZone ? exact_word(raw[j], gs.bf, gs.sf, inv) :
-                __byte_perm(__float_as_uint(fmaf(a.y, 16.f, a.x) + 8388608.0f), __float_as_uint(fmaf(b.y, 16.f, b.x) + 8388608.0f), 0x5410);
+        // (m0 + 16 m1) + 256 (m2 + 16 m3) + ...: sums of the low bits, the rest being known
+        const uint32_t w01 = m[1] * 16u + m[0], w23 = m[3] * 16u + m[2], w45 = m[5] * 16u + m[4], w67 = m[7] * 16u + m[6];
+        cw[j] = (w67 * 256u + w45) * 65536u + (w23 * 256u + w01) - kMagicSum;
+      }
+      if (inv > 3.0e38f) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) cw[j] = divided_word(raw[j], gs, inv);
       }
     }
     const uint32_t sb = gs.hs | (gs.hb << 16);

@@ -47,14 +47,17 @@ __device__ inline GroupScale group_scale(float mn, float mx, bool bf16) {
 }
 
 // code = clamp(rne(fl((x - b) / s))), inv = fl(1 / s), s != 0.  The IEEE division would dominate the quantizer, so the
-// quotient is taken as t * (1/s) with one fused residual correction (within an ulp of the correctly rounded quotient, 1/s
-// being correctly rounded), which rounds to the same integer unless the quotient sits within a few ulps of k + 1/2; only
-// there is the division itself evaluated.
+// quotient is taken as q = t * inv with one correction by its residual.  The residual t - s q is exact, since s has at most 11
+// significant bits, and with inv correctly rounded the corrected quotient is within 2^-46 of itself of t / s before its own
+// rounding, while t / s, unless it is a binary32 number, is at least 2^-36 of itself away from the midpoint of two of them: it
+// is the correctly rounded quotient, ties of the code included.  Only a scale without a finite reciprocal (a bfloat16 scale
+// below 2^-128) is divided by.
+static __device__ __noinline__ float divided(float t, float s) { return __fdiv_rn(t, s); }
 __device__ inline uint32_t quantize_code(float x, const GroupScale& gs, float inv) {
   const float t = __fsub_rn(x, gs.bf);
   float q = __fmul_rn(t, inv);
   q = __fmaf_rn(__fmaf_rn(-gs.sf, q, t), inv, q);
-  if (fabsf(q - (floorf(q) + 0.5f)) < 1e-5f) q = __fdiv_rn(t, gs.sf);
+  if (inv > 3.0e38f) q = divided(t, gs.sf);
   return (uint32_t)min(max(__float2int_rn(q), 0), 15);
 }
 
