@@ -139,14 +139,28 @@ def lib() -> ctypes.CDLL:
 def _ptr(t):
     if t is None:
         return None
-    if isinstance(t, int):
-        return t
-    assert t.is_cuda and t.is_contiguous(), "device pointers come from contiguous CUDA tensors"
-    return t.data_ptr()
+    try:
+        if t.is_cuda and t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:
+        if isinstance(t, int):
+            return t
+        raise
+    raise AssertionError("device pointers come from contiguous CUDA tensors")
+
+
+_get_device = _raw_stream = None
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    """The current stream's handle.  torch.cuda.current_stream() builds a Stream object (3.2 us, a third of a small call's host
+    time), so it is asked once, which also initialises CUDA; after that the handle alone is read (0.2 us)."""
+    global _get_device, _raw_stream
+    if _raw_stream is not None:
+        return _raw_stream(_get_device())
+    handle = torch.cuda.current_stream().cuda_stream
+    _get_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+    return handle
 
 
 def _check(code, where):
