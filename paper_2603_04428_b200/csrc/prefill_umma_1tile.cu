@@ -22,12 +22,17 @@
 //     with P_b read from tensor memory too, where it overlays S_b.  The scores of block j + 1 are
 //     issued before the probabilities of block j exist, so the tensor pipe works through the softmax.
 //     Tensor memory: O d_v columns, S 2 x 64, Q d_qk / 2.
-//   * Eight softmax warps, two threads per score row (each takes 32 of the 64 scores and half of the
-//     accumulator columns): mask, online softmax with a lazily updated reference maximum, P_b as
-//     packed binary16.
+//   * Eight softmax warps, two threads per score row (each takes 32 of the 64 scores and half of the accumulator columns):
+//     mask, online softmax with a lazily updated reference maximum, P_b as packed binary16 over the half of S_b that the
+//     thread has read.  The two warps of a row meet once per block at a barrier that carries the vote whether the reference
+//     has to move; maxima are exchanged only then.
 //   * One warp streams the raw blocks through a three-slot ring with bulk asynchronous copies.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
 // Q4KV_FLAG_INTERNAL, drains the tensor pipe and frees the tensor memory before the CTA returns.
+//
+// Bound by the softmax chain of a block (about 2600 clocks per 64 keys; the two products take 1250).  With one barrier for all
+// eight softmax warps, maxima exchanged in every block and 96 registers for every warp (the d = 256 form spilled) it took
+// 3400: 8 agents x (4096 + 512) tokens, 16 query heads, d = 256: 508 -> 400 us (575 -> 731 TFLOP/s), 192 / 128: 350 -> 335.
 #include "prefill_common.cuh"
 
 namespace q4kv {
@@ -39,7 +44,9 @@ using namespace prefill;
 
 constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
 constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps, kLoadWarp = kMmaWarp + 1;
-constexpr int kThreads = (kLoadWarp + 1) * 32;           // 576
+constexpr int kThreads = (kMmaWarp + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps)
+constexpr int kRegsSoftmax = 144, kRegsOther = 64;       // of the 96 each thread is launched with
+static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * 96, "");
 constexpr int kStages = 2;                               // K^ tiles, and V^ tiles, in flight
 constexpr int kRawSlots = 3;                             // raw 64-key blocks in flight
 constexpr uint32_t kColO = 0, kColS = 256, kColQ = 384;  // tensor-memory columns (d_v <= 256, 2 x 64, d_qk / 2 <= 128)
@@ -83,7 +90,7 @@ struct UmmaSmem {
   uint32_t tmem_base;
   int bad[kRawSlots];
   float xchg[2][2][128];                                 // [parity][column half][row]: maxima / sums of the two threads of a row
-  int stop[3], spoiled;
+  int spoiled;
   int abort_flag, poisoned;
 };
 
@@ -129,7 +136,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     mbar_init(&sm.o_done, 1);
     mbar_init(&sm.o_last, 1);
     mbar_init(&sm.q_ready, kSoftmaxWarps * 32);
-    for (int i = 0; i < 3; ++i) sm.stop[i] = 0;
     sm.spoiled = 0;
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0; sm.poisoned = 0;
@@ -144,37 +150,97 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the new tokens were appended by the preceding kernel
   volatile int* abort_flag = &sm.abort_flag;
 
-  if (warp == kLoadWarp) {
-    // =============================== raw block loader ==========================================
-    if (lane == 0) {
-      int issued = 0;
-      for (int j = 0; j < n_iter; ++j) {
-        const int r = j % kRawSlots;
-        if (j >= kRawSlots && !mbar_wait(&sm.raw_free[r], (uint32_t)(j / kRawSlots - 1), abort_flag)) break;
-        const int c = 2 * (it0 + j);
-        const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
-        if (blk < 0 || blk >= P.n_blocks) {
-          sm.bad[r] = 1;
-          sm.poisoned = 1;
-          raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK);
-          mbar_arrive(&sm.raw_full[r]);
-        } else {
-          sm.bad[r] = 0;
-          mbar_arrive_expect_tx(&sm.raw_full[r], kRawBytes);
-          bulk_load(sm.raw[r], head_block(P.pool, y, P.layer, blk, hk) + (size_t)(c & 7) * kChunkBytes, kRawBytes,
-                    &sm.raw_full[r]);
-        }
-        issued = j + 1;
-      }
-      // a CTA that is giving up still lets its own copies land before shared memory is released
-      if (*abort_flag) {
-        for (int j = max(0, issued - kRawSlots); j < issued; ++j) {
+  if (warp >= kMmaWarp) {
+    fewer_registers<kRegsOther>();
+    if (warp == kLoadWarp) {
+      // =============================== raw block loader ==========================================
+      if (lane == 0) {
+        int issued = 0;
+        for (int j = 0; j < n_iter; ++j) {
           const int r = j % kRawSlots;
-          for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots) & 1u); ++i) {}
+          if (j >= kRawSlots && !mbar_wait(&sm.raw_free[r], (uint32_t)(j / kRawSlots - 1), abort_flag)) break;
+          const int c = 2 * (it0 + j);
+          const int blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
+          if (blk < 0 || blk >= P.n_blocks) {
+            sm.bad[r] = 1;
+            sm.poisoned = 1;
+            raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK);
+            mbar_arrive(&sm.raw_full[r]);
+          } else {
+            sm.bad[r] = 0;
+            mbar_arrive_expect_tx(&sm.raw_full[r], kRawBytes);
+            bulk_load(sm.raw[r], head_block(P.pool, y, P.layer, blk, hk) + (size_t)(c & 7) * kChunkBytes, kRawBytes,
+                      &sm.raw_full[r]);
+          }
+          issued = j + 1;
+        }
+        // a CTA that is giving up still lets its own copies land before shared memory is released
+        if (*abort_flag) {
+          for (int j = max(0, issued - kRawSlots); j < issued; ++j) {
+            const int r = j % kRawSlots;
+            for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots) & 1u); ++i) {}
+          }
+        }
+      }
+    } else if (warp == kMmaWarp) {
+      // =============================== MMA issue ==================================================
+      // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
+      if (n_iter > 0) {
+        constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, kDv);
+        // one election for a whole product: an election per MMA costs more issue time than the MMA takes
+        auto issue_qk = [&](int b, int s) {                // S_b = Q K^T; afterwards the K^ stage is free
+          const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, Sh::kSboK);
+          if (elect_one()) {
+  #pragma unroll
+            for (int k = 0; k < kD / 16; ++k) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, k > 0);
+            commit(&sm.s_full[b]);
+            commit(&sm.k_free[s]);
+          }
+          __syncwarp();
+        };
+        auto issue_pv = [&](int b, int s, bool first, bool last) {    // O (+)= P_b V^; afterwards the V^ stage is free
+          const uint64_t vd = smem_desc(smem_u32(sm.vhat[s]), 128, 1024);
+          if (elect_one()) {
+  #pragma unroll
+            for (int k = 0; k < 4; ++k)
+              mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 32 * (k >> 1) + 8 * (k & 1), vd + 16 * k, kIdescO, (!first || k > 0) ? 1u : 0u);
+            commit(&sm.o_done);
+            if (last) commit(&sm.o_last);
+            commit(&sm.v_free[s]);
+          }
+          __syncwarp();
+        };
+        bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+          fence_after_sync();
+          issue_qk(0, 0);
+          if (n_iter > 1) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[1], 0, abort_flag));
+            if (ok) {
+              fence_after_sync();
+              issue_qk(1, 1);
+            }
+          }
+        }
+        for (int j = 0; ok && j < n_iter; ++j) {
+          const int b = j & 1, s = j % kStages;
+          ok = mbar_wait(&sm.p_full[b], (uint32_t)(j >> 1), abort_flag) && mbar_wait(&sm.v_full[s], (uint32_t)(j / kStages), abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          fence_after_sync();
+          issue_pv(b, s, j == 0, j + 1 == n_iter);
+          if (j + 2 < n_iter) {                            // the scores of block j + 2 replace P_b once the product above has read it
+            ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s], (uint32_t)((j + 2) / kStages), abort_flag));
+            if (!ok) break;
+            fence_after_sync();
+            issue_qk(b, s);
+          }
         }
       }
     }
-  } else if (warp >= kSoftmaxWarps && warp < kMmaWarp) {
+  } else if (warp >= kSoftmaxWarps) {
+    fewer_registers<kRegsOther>();
     // =============================== dequantize warps ==========================================
     // 256 threads.  At 256 / 256 a thread takes one of the two 16-byte key pieces of a token row (kj) and one value
     // piece, in both chunks of the block; at 192 / 128 a token row is a 16-byte and an 8-byte key piece and there are
@@ -277,67 +343,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       __syncwarp();
       if (lane == 0) { mbar_arrive(&sm.v_full[s]); mbar_arrive(&sm.raw_free[r]); }
     }
-  } else if (warp == kMmaWarp) {
-    // =============================== MMA issue ==================================================
-    // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
-    if (n_iter > 0) {
-      constexpr uint32_t kIdescS = idesc_f16(128, 64), kIdescO = idesc_f16(128, kDv);
-      // one election for a whole product: an election per MMA costs more issue time than the MMA takes
-      auto issue_qk = [&](int b, int s) {                // S_b = Q K^T; afterwards the K^ stage is free
-        const uint64_t kd = smem_desc(smem_u32(sm.khat[s]), 128, Sh::kSboK);
-        if (elect_one()) {
-#pragma unroll
-          for (int k = 0; k < kD / 16; ++k) mma_f16_ts(tb + kColS + 64 * b, tb + kColQ + 8 * k, kd + 16 * k, kIdescS, k > 0);
-          commit(&sm.s_full[b]);
-          commit(&sm.k_free[s]);
-        }
-        __syncwarp();
-      };
-      auto issue_pv = [&](int b, int s, bool first, bool last) {    // O (+)= P_b V^; afterwards the V^ stage is free
-        const uint64_t vd = smem_desc(smem_u32(sm.vhat[s]), 128, 1024);
-        if (elect_one()) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_f16_ts(tb + kColO, tb + kColS + 64 * b + 8 * k, vd + 16 * k, kIdescO, (!first || k > 0) ? 1u : 0u);
-          commit(&sm.o_done);
-          if (last) commit(&sm.o_last);
-          commit(&sm.v_free[s]);
-        }
-        __syncwarp();
-      };
-      bool ok = mbar_wait(&sm.q_ready, 0, abort_flag) && mbar_wait(&sm.k_full[0], 0, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
-        fence_after_sync();
-        issue_qk(0, 0);
-        if (n_iter > 1) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[1], 0, abort_flag));
-          if (ok) {
-            fence_after_sync();
-            issue_qk(1, 1);
-          }
-        }
-      }
-      for (int j = 0; ok && j < n_iter; ++j) {
-        const int b = j & 1, s = j % kStages;
-        ok = mbar_wait(&sm.p_full[b], (uint32_t)(j >> 1), abort_flag) && mbar_wait(&sm.v_full[s], (uint32_t)(j / kStages), abort_flag);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        fence_after_sync();
-        issue_pv(b, s, j == 0, j + 1 == n_iter);
-        if (j + 2 < n_iter) {                            // the scores of block j + 2 replace P_b once the product above has read it
-          ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s], (uint32_t)((j + 2) / kStages), abort_flag));
-          if (!ok) break;
-          fence_after_sync();
-          issue_qk(b, s);
-        }
-      }
-    }
   } else {
+    more_registers<kRegsSoftmax>();
     // =============================== softmax warps: two threads per score row ===================
-    // Warp w: column half = w / 4, tensor-memory lanes 32 (w % 4) ...  The two threads of a row exchange their block
-    // maxima (and at the end their sums) through shared memory; the 256 threads meet at a named barrier once per
-    // block, and they leave the loop together (one of them samples the give-up flag before the barrier).
+    // Warp w: column half = w / 4, tensor-memory lanes 32 (w % 4) ...  The warps w and w + 4 share their rows: they meet at a
+    // named barrier once per block, which tells both whether a row's maximum has outgrown its reference (or a wait has run
+    // out: they leave the loop together); only then are maxima exchanged through shared memory, and at the end the sums.
     const int half = (warp >> 2) & 1;
     const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
     const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
@@ -345,8 +356,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
     const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
-    const bool sampler = warp == 0 && lane == 0;
     auto tile_barrier = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    auto pair_any = [&](bool p) {                        // of the 64 threads of the rows' two warps
+      uint32_t any;
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, %2, 64, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                   : "=r"(any) : "r"((uint32_t)p), "r"(2 + (warp & 3)) : "memory");
+      return any != 0u;
+    };
     float kappa;                                         // score in log2 units = S * kappa
     {
       // ---- stage this thread's half of the query row: bf16 -> binary16 times a power of two, element order
@@ -406,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most kLazy
     for (int j = 0; j < n_iter; ++j) {
       const int b = j & 1;
-      mbar_wait(&sm.s_full[b], (uint32_t)(j >> 1), abort_flag);   // a wait that runs out raises the give-up flag; all leave below
+      const bool quit = !mbar_wait(&sm.s_full[b], (uint32_t)(j >> 1), abort_flag);   // raises the give-up flag; both warps leave below
       fence_after_sync();
       uint32_t sr[32];
       tmem_ld32(lane_addr + kColS + 64 * b + 32 * half, sr);
@@ -425,34 +441,35 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       // rescaled and the probabilities taken again.  The scores stay in registers meanwhile.
       float sum = 0.f;
       uint32_t pr[16];
+      const uint64_t kk = pair64(kappa, kappa);
       auto probabilities = [&](float neg_m) {
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        const uint64_t nn = pair64(neg_m, neg_m);
+        uint64_t sum0 = 0u, sum1 = 0u;                   // (+0, +0)
 #pragma unroll
         for (int c = 0; c < 16; c += 2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sr[2 * c]), kappa, neg_m));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 1]), kappa, neg_m));
-          const float p2 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 2]), kappa, neg_m));
-          const float p3 = fast_exp2(fmaf(__uint_as_float(sr[2 * c + 3]), kappa, neg_m));
-          s0 += p0; s1 += p1; s2 += p2; s3 += p3;
+          const float2 u = unpair64(fma2(pair64(__uint_as_float(sr[2 * c]), __uint_as_float(sr[2 * c + 1])), kk, nn));
+          const float2 v = unpair64(fma2(pair64(__uint_as_float(sr[2 * c + 2]), __uint_as_float(sr[2 * c + 3])), kk, nn));
+          const float p0 = fast_exp2(u.x), p1 = fast_exp2(u.y), p2 = fast_exp2(v.x), p3 = fast_exp2(v.y);
+          sum0 = add2(sum0, pair64(p0, p1)); sum1 = add2(sum1, pair64(p2, p3));
           pr[c] = f32x2_to_h2(p0, p1);
           pr[c + 1] = f32x2_to_h2(p2, p3);
         }
-        sum = (s0 + s1) + (s2 + s3);
+        const float2 s01 = unpair64(sum0), s23 = unpair64(sum1);
+        sum = (s01.x + s01.y) + (s23.x + s23.y);
       };
       probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
       float cm4[4] = {__uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2]), __uint_as_float(sr[3])};
 #pragma unroll
       for (int c = 4; c < 32; ++c) cm4[c & 3] = fmaxf(cm4[c & 3], __uint_as_float(sr[c]));
       float cm = fmaxf(fmaxf(cm4[0], cm4[1]), fmaxf(cm4[2], cm4[3]));
-      sm.xchg[j & 1][half][row] = cm;
-      if (sampler) sm.stop[j % 3] = *abort_flag;
-      tile_barrier();                                    // also: every score of the block has been read (P overlays S)
-      if (sm.stop[j % 3]) break;
-      cm = fmaxf(cm, sm.xchg[j & 1][half ^ 1][row]);
-      if (cm != -INFINITY) cm *= kappa;                  // kappa > 0
-      const float m_new = fmaxf(m_ref, cm);
-      const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
-      if (__any_sync(0xffffffffu, grow)) {
+      // P_b overlays the half of S_b that this thread has read: 16 columns from column 32 half on
+      tmem_st16(lane_addr + kColS + 64 * b + 32 * half, pr);
+      const float cs = cm == -INFINITY ? cm : cm * kappa;                  // kappa > 0
+      if (pair_any(quit || cs > m_ref + kLazy || (m_ref == -INFINITY && cs != -INFINITY))) {
+        sm.xchg[j & 1][half][row] = cs;
+        if (pair_any(quit)) break;
+        const float m_new = fmaxf(m_ref, fmaxf(cs, sm.xchg[j & 1][half ^ 1][row]));
+        const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
         if (j > 0) {
           // rescale this thread's half of the accumulator row: the previous block's value product must have landed
           mbar_wait(&sm.o_done, (uint32_t)(j - 1), abort_flag);
@@ -471,9 +488,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         }
         if (grow) m_ref = m_new;
         probabilities(m_ref == -INFINITY ? 0.f : -m_ref);
+        wait_st();
+        tmem_st16(lane_addr + kColS + 64 * b + 32 * half, pr);
       }
       l += sum;
-      tmem_st16(lane_addr + kColS + 64 * b + 16 * half, pr);   // P_b overlays the first 32 columns of S_b
       wait_st();
       fence_before_sync();
       mbar_arrive(&sm.p_full[b]);
