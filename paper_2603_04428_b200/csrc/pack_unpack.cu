@@ -61,11 +61,20 @@ struct ExchangeView {
 // chunk c of the head-block through its own shared-memory copy of the chunk (dynamic smem: 8 * chunk_bytes).  Every
 // global access is a full 16- or 32-byte piece of a contiguous run: the pool chunk is one contiguous range, and each
 // head-dim-packed tensor's part of a chunk is too.
-template <bool kPack, bool kDense>
+//
+// kLatent: the latent cache (nine groups, values an alias of the keys), with its sizes known at compile time: the offsets of a
+// word cost shifts and adds instead of divisions (27 layers x 4000 tokens, packed and unpacked: 49 -> 46 us).  For the per-head
+// caches the same made the launches slower (d = 128, 32 layers x 4000 tokens: 115 -> 123 us, with any bound on the registers):
+// their chunks are four times as many, and more accesses in flight at once cost more in DRAM than the instructions saved.
+template <bool kPack, bool kDense, bool kLatent>
 __global__ void __launch_bounds__(kThreads)
 pack_unpack_kernel(Layout y, uint8_t* pool, int n_blocks, const int32_t* __restrict__ row, int n_tokens,
                    uint8_t* buf, int32_t* flags, ExchangeView xv) {
   extern __shared__ __align__(16) uint8_t stage_all[];
+  if (kLatent) {                                         // what make_layout computes
+    y.G = 9; y.Gv = 8; y.D = 576; y.Dv = 512; y.alias = 1;
+    y.off_kc = 0; y.off_ksb = kChunkTokens * 288; y.off_vc = y.off_vsb = y.chunk_bytes = kChunkTokens * (288 + 36);
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lb = blockIdx.x / y.Hkv, hk = blockIdx.x % y.Hkv;
   const int kw = y.D / 8, vw = y.Dv / 8;
@@ -198,23 +207,29 @@ pack_unpack_kernel(Layout y, uint8_t* pool, int n_blocks, const int32_t* __restr
 }  // namespace
 
 namespace {
-template <bool kPack, bool kDense>
-cudaError_t launch_pu(const Layout& y, uint8_t* pool, int n_blocks, const int32_t* row, int n_tokens, uint8_t* buf,
+template <bool kPack, bool kDense, bool kLatent>
+cudaError_t launch_pu_shape(const Layout& y, uint8_t* pool, int n_blocks, const int32_t* row, int n_tokens, uint8_t* buf,
                       int32_t* flags, cudaStream_t st, const ExchangeView& xv, int grid_y) {
   static bool configured[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(pack_unpack_kernel<kPack, kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    e = cudaFuncSetAttribute(pack_unpack_kernel<kPack, kDense, kLatent>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const int nblk = (n_tokens + kBlockTokens - 1) / kBlockTokens;   // mode 1: n_tokens is T, the dense row count
   dim3 grid(nblk * y.Hkv, grid_y);
-  pack_unpack_kernel<kPack, kDense><<<grid, kThreads, (size_t)kChunksPerBlock * y.chunk_bytes, st>>>(y, pool, n_blocks, row, n_tokens,
-                                                                                              buf, flags, xv);
+  pack_unpack_kernel<kPack, kDense, kLatent><<<grid, kThreads, (size_t)kChunksPerBlock * y.chunk_bytes, st>>>(
+      y, pool, n_blocks, row, n_tokens, buf, flags, xv);
   return cudaGetLastError();
+}
+template <bool kPack, bool kDense>
+cudaError_t launch_pu(const Layout& y, uint8_t* pool, int n_blocks, const int32_t* row, int n_tokens, uint8_t* buf,
+                      int32_t* flags, cudaStream_t st, const ExchangeView& xv, int grid_y) {
+  auto launch = y.alias && y.G == 9 && y.Gv == 8 ? launch_pu_shape<kPack, kDense, true> : launch_pu_shape<kPack, kDense, false>;
+  return launch(y, pool, n_blocks, row, n_tokens, buf, flags, st, xv, grid_y);
 }
 ExchangeView persisted_view(int layer0) {
   ExchangeView xv;
