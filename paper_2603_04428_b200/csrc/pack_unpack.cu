@@ -63,9 +63,10 @@ struct ExchangeView {
 // head-dim-packed tensor's part of a chunk is too.
 //
 // kLatent: the latent cache (nine groups, values an alias of the keys), with its sizes known at compile time: the offsets of a
-// word cost shifts and adds instead of divisions (27 layers x 4000 tokens, packed and unpacked: 49 -> 46 us).  For the per-head
-// caches the same made the launches slower (d = 128, 32 layers x 4000 tokens: 115 -> 123 us, with any bound on the registers):
-// their chunks are four times as many, and more accesses in flight at once cost more in DRAM than the instructions saved.
+// word cost shifts and adds instead of divisions (27 layers x 4000 tokens, packed and unpacked: 49 -> 45 us).  For the per-head
+// caches the same made the launches slower (d = 128, 32 layers x 4000 tokens: 115 -> 123 us): it wants 62 registers, which leave
+// room for four CTAs per SM where shared memory allows six, and held to 40 it spills (129 us); with fewer CTAs per SM the
+// general form is slower too (131 us on four, 149 on three).
 template <bool kPack, bool kDense, bool kLatent>
 __global__ void __launch_bounds__(kThreads)
 pack_unpack_kernel(Layout y, uint8_t* pool, int n_blocks, const int32_t* __restrict__ row, int n_tokens,
