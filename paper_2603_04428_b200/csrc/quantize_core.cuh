@@ -52,12 +52,11 @@ __device__ inline GroupScale group_scale(float mn, float mx, bool bf16) {
 // rounding, while t / s, unless it is a binary32 number, is at least 2^-36 of itself away from the midpoint of two of them: it
 // is the correctly rounded quotient, ties of the code included.  Only a scale without a finite reciprocal (a bfloat16 scale
 // below 2^-128) is divided by.
-static __device__ __noinline__ float divided(float t, float s) { return __fdiv_rn(t, s); }
 __device__ inline uint32_t quantize_code(float x, const GroupScale& gs, float inv) {
   const float t = __fsub_rn(x, gs.bf);
   float q = __fmul_rn(t, inv);
   q = __fmaf_rn(__fmaf_rn(-gs.sf, q, t), inv, q);
-  if (inv > 3.0e38f) q = divided(t, gs.sf);
+  if (inv > 3.0e38f) q = __fdiv_rn(t, gs.sf);
   return (uint32_t)min(max(__float2int_rn(q), 0), 15);
 }
 
