@@ -1,4 +1,4 @@
-"""Thin ctypes binding of libq4kv.so: argument marshalling only.
+"""Thin binding of libq4kv.so (ctypes; the per-layer entry points through csrc/py_call.c): argument marshalling only.
 
 Every function has the name and argument order of its C entry point
 (include/q4kv.h).  Tensors are torch CUDA tensors used purely as device
@@ -15,6 +15,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libq4kv.so")
+CALL_PATH = os.path.join(_HERE, "_call.so")
 
 OK, EINVAL, EUNSUPPORTED, EWORKSPACE, ECUDA = 0, -1, -2, -3, -4
 FLAG_BAD_BLOCK, FLAG_BAD_LENGTH, FLAG_INTERNAL, FLAG_SB_RANGE = 1, 2, 4, 8
@@ -56,14 +57,16 @@ class Batch(ctypes.Structure):
 
 
 _lib = None
+_call = None                     # the four per-layer entry points through native marshalling (csrc/py_call.c)
 
 
 def lib() -> ctypes.CDLL:
-    global _lib
+    global _lib, _call
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
+        missing = [p for p in (LIB_PATH, CALL_PATH) if not os.path.exists(p)]
+        if missing:
             raise RuntimeError(
-                f"{LIB_PATH} is missing: build it with `python -m paper_2603_04428_b200.build` "
+                f"{missing[0]} is missing: build it with `python -m paper_2603_04428_b200.build` "
                 "(there is no fallback path)")
         L = ctypes.CDLL(LIB_PATH)
         vp, i32, sz, f32 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_size_t, ctypes.c_float
@@ -132,8 +135,15 @@ def lib() -> ctypes.CDLL:
         L.q4kv_pack.argtypes = [sp, vp, i32, vp, i32, vp, sz, vp, vp]
         L.q4kv_unpack.restype = ctypes.c_int
         L.q4kv_unpack.argtypes = [sp, vp, sz, i32, vp, i32, vp, vp, vp]
-        _lib = L
+        from . import _call as call
+        call.bind(*(ctypes.cast(getattr(L, "q4kv_" + n), ctypes.c_void_p).value for n in (
+            "quantize_append", "decode_attention", "append_decode_attention", "prefill_attention")))
+        _lib, _call = L, call
     return _lib
+
+
+def _native():
+    return _call or (lib() and _call)
 
 
 def _ptr(t):
@@ -191,30 +201,22 @@ def q4kv_workspace_bytes(spec: Spec, n_agents: int, max_kv_len: int, total_q: in
 
 def q4kv_quantize_append(spec, pool, n_blocks, layer, bt: Batch, pos, new_offs, total_new, k_new, v_new,
                          status_flags=None):
-    _check(lib().q4kv_quantize_append(ctypes.byref(spec), _ptr(pool), n_blocks, layer, ctypes.byref(bt), _ptr(pos),
-                                      _ptr(new_offs), total_new, _ptr(k_new), _ptr(v_new), _ptr(status_flags),
-                                      _stream()), "q4kv_quantize_append")
+    _check(_native().append(spec, pool, n_blocks, layer, bt, pos, new_offs, total_new, k_new, v_new, status_flags, _stream()),
+           "q4kv_quantize_append")
 
 
 def q4kv_decode_attention(spec, pool, n_blocks, layer, bt: Batch, kv_lens, max_kv_len, window, q, softmax_scale,
                           out, out_dtype, lse, workspace, status_flags=None):
-    _check(lib().q4kv_decode_attention(ctypes.byref(spec), _ptr(pool), n_blocks, layer, ctypes.byref(bt),
-                                       _ptr(kv_lens), max_kv_len, window, _ptr(q), softmax_scale, _ptr(out),
-                                       out_dtype, _ptr(lse), _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _ptr(status_flags), _stream()),
-           "q4kv_decode_attention")
+    _check(_native().decode(spec, pool, n_blocks, layer, bt, kv_lens, max_kv_len, window, q, softmax_scale, out, out_dtype,
+                            lse, workspace, status_flags, _stream()), "q4kv_decode_attention")
 
 
 def q4kv_append_decode_attention(spec, pool, n_blocks, layer, bt: Batch, kv_lens, max_kv_len, window, k_new, v_new, q,
                                  softmax_scale, out, out_dtype, lse, workspace, status_flags=None):
     """Update-and-fetch in one launch: quantize one new token per agent into the cache (position kv_len - 1) and
     attend over the cache including it."""
-    _check(lib().q4kv_append_decode_attention(ctypes.byref(spec), _ptr(pool), n_blocks, layer, ctypes.byref(bt),
-                                              _ptr(kv_lens), max_kv_len, window, _ptr(k_new), _ptr(v_new), _ptr(q),
-                                              softmax_scale, _ptr(out), out_dtype, _ptr(lse), _ptr(workspace),
-                                              workspace.numel() * workspace.element_size(), _ptr(status_flags),
-                                              _stream()),
-           "q4kv_append_decode_attention")
+    _check(_native().append_decode(spec, pool, n_blocks, layer, bt, kv_lens, max_kv_len, window, k_new, v_new, q, softmax_scale,
+                                   out, out_dtype, lse, workspace, status_flags, _stream()), "q4kv_append_decode_attention")
 
 
 def q4kv_decode_attention_static(spec, pool, n_blocks, layer, bt: Batch, kv_lens, max_kv_len, window, q, softmax_scale,
@@ -229,20 +231,17 @@ def q4kv_decode_attention_static(spec, pool, n_blocks, layer, bt: Batch, kv_lens
 
 def q4kv_prefill_attention(spec, pool, n_blocks, layer, bt: Batch, kv_lens, q_offs, total_q, max_q_len, max_kv_len,
                            window, q, softmax_scale, out, out_dtype, lse, workspace, status_flags=None):
-    _check(lib().q4kv_prefill_attention(ctypes.byref(spec), _ptr(pool), n_blocks, layer, ctypes.byref(bt),
-                                        _ptr(kv_lens), _ptr(q_offs), total_q, max_q_len, max_kv_len, window, _ptr(q),
-                                        softmax_scale, _ptr(out), out_dtype, _ptr(lse), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _ptr(status_flags), _stream()),
-           "q4kv_prefill_attention")
+    _check(_native().prefill(spec, pool, n_blocks, layer, bt, kv_lens, q_offs, total_q, max_q_len, max_kv_len, window, q,
+                             softmax_scale, out, out_dtype, lse, workspace, status_flags, _stream()), "q4kv_prefill_attention")
 
 
 def q4kv_pack(spec, pool, n_blocks, block_table_row, n_tokens, dst, status_flags=None):
     _check(lib().q4kv_pack(ctypes.byref(spec), _ptr(pool), n_blocks, _ptr(block_table_row), n_tokens, _ptr(dst),
-                           dst.numel() * dst.element_size(), _ptr(status_flags), _stream()), "q4kv_pack")
+                           dst.nbytes, _ptr(status_flags), _stream()), "q4kv_pack")
 
 
 def q4kv_unpack(spec, src, n_tokens, pool, n_blocks, block_table_row, status_flags=None):
-    _check(lib().q4kv_unpack(ctypes.byref(spec), _ptr(src), src.numel() * src.element_size(), n_tokens, _ptr(pool),
+    _check(lib().q4kv_unpack(ctypes.byref(spec), _ptr(src), src.nbytes, n_tokens, _ptr(pool),
                              n_blocks, _ptr(block_table_row), _ptr(status_flags), _stream()), "q4kv_unpack")
 
 
@@ -355,5 +354,5 @@ def q4kv_decode_attention_layers(spec, pool, n_blocks, layer_begin, layer_count,
     _check(lib().q4kv_decode_attention_layers(ctypes.byref(spec), _ptr(pool), n_blocks, layer_begin, layer_count,
                                               ctypes.byref(bt), _ptr(kv_lens), max_kv_len, w, _ptr(k_new), _ptr(v_new),
                                               _ptr(q), softmax_scale, _ptr(out), out_dtype, _ptr(lse), _ptr(workspace),
-                                              workspace.numel() * workspace.element_size(), _ptr(status_flags), _stream()),
+                                              workspace.nbytes, _ptr(status_flags), _stream()),
            "q4kv_decode_attention_layers")

@@ -1,4 +1,5 @@
-"""Build libq4kv.so (sm_100a) in-tree with nvcc.  `python -m paper_2603_04428_b200.build`.
+"""Build libq4kv.so (sm_100a) in-tree with nvcc, and the binding's marshalling module _call.so with the host compiler.
+`python -m paper_2603_04428_b200.build`.
 
 Each .cu file is compiled to an object of its own (in parallel, and only when it or a header changed), then the
 objects are linked into the shared library next to this file.
@@ -10,11 +11,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libq4kv.so")
+CALL_SRC, CALL = os.path.join(CSRC, "py_call.c"), os.path.join(HERE, "_call.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -42,7 +45,7 @@ def _stale(target: str, deps) -> bool:
 
 
 def needs_build() -> bool:
-    return _stale(LIB, sources() + headers())
+    return _stale(LIB, sources() + headers()) or _stale(CALL, [CALL_SRC] + headers())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -70,6 +73,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         sys.stderr.write(res.stdout + res.stderr)
     if res.returncode != 0:
         raise RuntimeError("nvcc failed linking libq4kv.so")
+    res = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                          "-o", CALL, CALL_SRC], capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("the host compiler failed building _call.so")
     return LIB
 
 
