@@ -11,7 +11,7 @@
 //   * A CTA owns 128 score rows (128 / n_rep consecutive queries x the n_rep heads of one KV head)
 //     and walks the keys 64 at a time (two 32-token chunks, one bulk copy).
 //   * Eight "dequantize" warps turn each raw block into binary16 tiles K^ [64 keys][d_qk] and
-//     V^ [d_v][64 keys] in shared memory (two stages each), in the core-matrix order a K-major
+//     V^ [d_v][64 keys] in shared memory (two or three stages each), in the core-matrix order a K-major
 //     tcgen05 operand wants: x^ = c * s + b in one binary16 fma per pair of codes, each value rounded
 //     once to 11 significant bits.  A packed word becomes one 16-byte row of a core matrix; the order
 //     of the eight elements inside a row (0,4,1,5,2,6,3,7) is absorbed by storing the queries, and
@@ -30,9 +30,10 @@
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
 // Q4KV_FLAG_INTERNAL, drains the tensor pipe and frees the tensor memory before the CTA returns.
 //
-// Bound by the softmax chain of a block (about 2600 clocks per 64 keys; the two products take 1250).  With one barrier for all
-// eight softmax warps, maxima exchanged in every block and 96 registers for every warp (the d = 256 form spilled) it took
-// 3400: 8 agents x (4096 + 512) tokens, 16 query heads, d = 256: 508 -> 400 us (575 -> 731 TFLOP/s), 192 / 128: 350 -> 335.
+// Bound by the dequantize warps' chain per block (2750 clocks per 64 keys; the two products take 1250, and with the tiles left
+// as they are a block takes 2100).  With one barrier for all eight softmax warps, maxima exchanged in every block and 96
+// registers for every warp (the d = 256 form spilled) it took 3400.  8 agents x (4096 + 512) tokens, 16 query heads, d = 256:
+// 508 -> 392 us (575 -> 745 TFLOP/s); 192 / 128: 350 -> 322 (566).
 #include "prefill_common.cuh"
 
 namespace q4kv {
@@ -47,7 +48,7 @@ constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps, kLoadWarp = kMmaWarp + 1
 constexpr int kThreads = (kMmaWarp + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps)
 constexpr int kRegsSoftmax = 144, kRegsOther = 64;       // of the 96 each thread is launched with
 static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * 96, "");
-constexpr int kStages = 2;                               // K^ tiles, and V^ tiles, in flight
+constexpr int kStages = 2;                               // K^ tiles in flight
 constexpr int kRawSlots = 3;                             // raw 64-key blocks in flight
 constexpr uint32_t kColO = 0, kColS = 256, kColQ = 384;  // tensor-memory columns (d_v <= 256, 2 x 64, d_qk / 2 <= 128)
 // G, Gv: groups of 64 along the key and value head dims
@@ -58,6 +59,9 @@ struct Shape {
   static constexpr int kChunkBytes = kOffVsb + 128 * Gv; // [Kc | Ksb | Vc | Vsb]: 9216 at 256 / 256, 5760 at 192 / 128
   static constexpr int kRawBytes = 2 * kChunkBytes;
   static constexpr int kTileK = 64 * D * 2, kTileV = Dv * 64 * 2;   // binary16 tiles
+  // V^ tiles in flight.  The dequantize warps' value tile of a block waits for a value product and delays the next key tile; a
+  // third stage takes that wait out at 192 / 128 (335 -> 326 us); at 256 / 256 it costs more than it gives (399 -> 408).
+  static constexpr int kStagesV = G == 4 ? 2 : 3;
   static constexpr int kSboK = (D / 8) * 128;            // bytes between 8-key groups of K^
 };
 
@@ -82,10 +86,10 @@ template <int G, int Gv>
 struct UmmaSmem {
   using Sh = Shape<G, Gv>;
   alignas(128) uint8_t khat[kStages][Sh::kTileK];        // [key 64][dim d_qk]: (n%8)*16 + (n/8)*kSboK + (k/8)*128
-  alignas(128) uint8_t vhat[kStages][Sh::kTileV];        // [dim d_v][key 64]: (n%8)*16 + (n/8)*1024 + (k/8)*128
+  alignas(128) uint8_t vhat[Sh::kStagesV][Sh::kTileV];   // [dim d_v][key 64]: (n%8)*16 + (n/8)*1024 + (k/8)*128
   alignas(128) uint8_t raw[kRawSlots][Sh::kRawBytes];
   alignas(8) uint64_t raw_full[kRawSlots], raw_free[kRawSlots], sb_done[kRawSlots];
-  uint64_t k_full[kStages], v_full[kStages], k_free[kStages], v_free[kStages];
+  uint64_t k_full[kStages], v_full[Sh::kStagesV], k_free[kStages], v_free[Sh::kStagesV];
   uint64_t s_full[2], p_full[2], o_done, o_last, q_ready, drain;
   uint32_t tmem_base;
   int bad[kRawSlots];
@@ -128,10 +132,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
   if (threadIdx.x == 0) {
     if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
     for (int s = 0; s < kRawSlots; ++s) { mbar_init(&sm.raw_full[s], 1); mbar_init(&sm.raw_free[s], kDequantWarps); mbar_init(&sm.sb_done[s], kDequantWarps); sm.bad[s] = 0; }
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.v_full[s], kDequantWarps);
-      mbar_init(&sm.k_free[s], 1); mbar_init(&sm.v_free[s], 1);
-    }
+    for (int s = 0; s < kStages; ++s) { mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.k_free[s], 1); }
+    for (int s = 0; s < Sh::kStagesV; ++s) { mbar_init(&sm.v_full[s], kDequantWarps); mbar_init(&sm.v_free[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&sm.s_full[b], 1); mbar_init(&sm.p_full[b], kSoftmaxWarps * 32); }
     mbar_init(&sm.o_done, 1);
     mbar_init(&sm.o_last, 1);
@@ -224,12 +226,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
           }
         }
         for (int j = 0; ok && j < n_iter; ++j) {
-          const int b = j & 1, s = j % kStages;
-          ok = mbar_wait(&sm.p_full[b], (uint32_t)(j >> 1), abort_flag) && mbar_wait(&sm.v_full[s], (uint32_t)(j / kStages), abort_flag);
+          const int b = j & 1, s = j % kStages, sv = j % Sh::kStagesV;
+          ok = mbar_wait(&sm.p_full[b], (uint32_t)(j >> 1), abort_flag) && mbar_wait(&sm.v_full[sv], (uint32_t)(j / Sh::kStagesV), abort_flag);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           fence_after_sync();
-          issue_pv(b, s, j == 0, j + 1 == n_iter);
+          issue_pv(b, sv, j == 0, j + 1 == n_iter);
           if (j + 2 < n_iter) {                            // the scores of block j + 2 replace P_b once the product above has read it
             ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_full[s], (uint32_t)((j + 2) / kStages), abort_flag));
             if (!ok) break;
@@ -262,8 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     const int v_sb = kOffVsb + (vo * 2 * Gv + (vq >> 1)) * 4;    // + (i * 8 + e) * Gv * 4: token 8 vo + 4 e + i, group vq / 2
     constexpr int kChunksPerThread = G == 4 ? 2 : 1;
     for (int j = 0; j < n_iter; ++j) {
-      const int s = j % kStages, r = j % kRawSlots;
-      if (j >= kStages && !mbar_wait(&sm.k_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
+      const int s = j % kStages, sv = j % Sh::kStagesV, r = j % kRawSlots;
       if (!mbar_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
       const bool bad = sm.bad[r] != 0;
       const int pos_base = (it0 + j) * 64;
@@ -287,6 +288,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         if (lane == 0) mbar_arrive(&sm.sb_done[r]);
         if (!mbar_wait(&sm.sb_done[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
       }
+      uint4 kws[kChunksPerThread], vws[kChunksPerThread];    // the codes, read while the stages are not yet free
+#pragma unroll
+      for (int cc = 0; cc < kChunksPerThread; ++cc) {
+        const uint8_t* chunk = sm.raw[r] + (G == 4 ? cc : c1) * kChunkBytes;
+        kws[cc] = *reinterpret_cast<const uint4*>(chunk + k_read); vws[cc] = *reinterpret_cast<const uint4*>(chunk + v_read);
+      }
+      if (j >= kStages && !mbar_wait(&sm.k_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
 #pragma unroll
       for (int cc = 0; cc < kChunksPerThread; ++cc) {
         const int ci = G == 4 ? cc : c1;
@@ -294,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         const bool dead = bad || pos_base + ci * 32 + ktau >= kv_len;      // stale bytes past the end
         const int n = ci * 32 + k_row;
         uint8_t* dst = sm.khat[s] + (n & 7) * 16 + (n >> 3) * Sh::kSboK + (16 * kj + kt) * 128;
-        const uint4 kw = *reinterpret_cast<const uint4*>(chunk + k_read);
+        const uint4 kw = kws[cc];
         uint32_t e0 = *reinterpret_cast<const uint32_t*>(chunk + k_sb);       // (scale, bias) of groups 2 kj and 2 kj + 1
         uint32_t e1 = *reinterpret_cast<const uint32_t*>(chunk + k_sb + 4);
         if (dead) { e0 = 0u; e1 = 0u; }
@@ -316,12 +324,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.k_full[s]);
-      if (j >= kStages && !mbar_wait(&sm.v_free[s], (uint32_t)(j / kStages - 1), abort_flag)) break;
+      if (j >= Sh::kStagesV && !mbar_wait(&sm.v_free[sv], (uint32_t)(j / Sh::kStagesV - 1), abort_flag)) break;
 #pragma unroll
       for (int cc = 0; cc < kChunksPerThread; ++cc) {
         const int ci = G == 4 ? cc : c1;
         const uint8_t* chunk = sm.raw[r] + ci * kChunkBytes;
-        const uint4 vw = *reinterpret_cast<const uint4*>(chunk + v_read);
+        const uint4 vw = vws[cc];
         uint32_t sp[4], bp[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -333,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
           sp[i] = __byte_perm(e0, e1, 0x5410);                             // scales of tokens i and i + 4
           bp[i] = __byte_perm(e0, e1, 0x7632);                             // biases
         }
-        uint8_t* dst = sm.vhat[s] + vr * 16 + (4 * vq) * 1024 + (ci * 4 + vo) * 128;
+        uint8_t* dst = sm.vhat[sv] + vr * 16 + (4 * vq) * 1024 + (ci * 4 + vo) * 128;
         *reinterpret_cast<uint4*>(dst + 0 * 1024) = dequant8(vw.x, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
         *reinterpret_cast<uint4*>(dst + 1 * 1024) = dequant8(vw.y, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
         *reinterpret_cast<uint4*>(dst + 2 * 1024) = dequant8(vw.z, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
@@ -341,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
       }
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) { mbar_arrive(&sm.v_full[s]); mbar_arrive(&sm.raw_free[r]); }
+      if (lane == 0) { mbar_arrive(&sm.v_full[sv]); mbar_arrive(&sm.raw_free[r]); }
     }
   } else {
     more_registers<kRegsSoftmax>();
