@@ -26,7 +26,7 @@
 //   * With few tiles the keys of a tile are cut over several CTAs as well (plan_prefill_splits); these leave (acc, m, l)
 //     records that merge_prefill_kernel combines.
 // Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads (102 GFLOP): 36 ms on the shape-agnostic kernel,
-// 0.25 ms here = 405 TFLOP/s; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
+// 0.227 ms here = 449 TFLOP/s; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
 // products share the shared-memory bandwidth (256 KB per block: 2000 clocks) and the issue slots.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises Q4KV_FLAG_INTERNAL, drains the tensor
 // pipe and frees the tensor memory before the CTA returns.
@@ -67,6 +67,7 @@ struct MlaPrefillParams {
   int32_t* flags;
   int n_splits;
   float* records;             // n_splits > 1: [total_q][Hq][n_splits][kRecord]
+  CodeMasks masks;
 };
 
 struct MlaSmem {
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
           const uint4& v = w16[(p >> 2) & 3];
           const uint32_t w = p >= 16 ? (p == 16 ? w8.x : w8.y) : (p & 3) == 0 ? v.x : (p & 3) == 1 ? v.y : (p & 3) == 2 ? v.z : v.w;
           const uint32_t sp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x1010), bp = __byte_perm(sb[p >> 1], sb[p >> 1], 0x3232);
-          *reinterpret_cast<uint4*>(dst + p * 512) = dequant8(w, sp, bp, sp, bp, sp, bp, sp, bp);
+          *reinterpret_cast<uint4*>(dst + p * 512) = dequant8(w, sp, bp, sp, bp, sp, bp, sp, bp, P.masks);
           if (p & 1) fetch_sb(chunk, p >> 1);
           if (p < 16 && (p & 3) == 3) fetch16(chunk, p >> 2);
           if (p == 17) fetch8(chunk);

@@ -30,10 +30,10 @@
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
 // Q4KV_FLAG_INTERNAL, drains the tensor pipe and frees the tensor memory before the CTA returns.
 //
-// Bound by the dequantize warps' chain per block (2750 clocks per 64 keys; the two products take 1250, and with the tiles left
+// Bound by the dequantize warps' chain per block (2650 clocks per 64 keys; the two products take 1250, and with the tiles left
 // as they are a block takes 2100).  With one barrier for all eight softmax warps, maxima exchanged in every block and 96
 // registers for every warp (the d = 256 form spilled) it took 3400.  8 agents x (4096 + 512) tokens, 16 query heads, d = 256:
-// 508 -> 392 us (575 -> 745 TFLOP/s); 192 / 128: 350 -> 322 (566).
+// 508 -> 379 us (575 -> 771 TFLOP/s); 192 / 128: 350 -> 303 (601).
 #include "prefill_common.cuh"
 
 namespace q4kv {
@@ -80,6 +80,7 @@ struct UmmaParams {
   float* lse;
   int32_t* flags;
   PrefillExtra x;
+  CodeMasks masks;
 };
 
 template <int G, int Gv>
@@ -308,17 +309,17 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         if (dead) { e0 = 0u; e1 = 0u; }
         const uint32_t s0 = __byte_perm(e0, e0, 0x1010), b0 = __byte_perm(e0, e0, 0x3232);
         const uint32_t s1 = __byte_perm(e1, e1, 0x1010), b1 = __byte_perm(e1, e1, 0x3232);
-        *reinterpret_cast<uint4*>(dst + 0 * 512) = dequant8(kw.x, s0, b0, s0, b0, s0, b0, s0, b0);
-        *reinterpret_cast<uint4*>(dst + 1 * 512) = dequant8(kw.y, s0, b0, s0, b0, s0, b0, s0, b0);
-        *reinterpret_cast<uint4*>(dst + 2 * 512) = dequant8(kw.z, s1, b1, s1, b1, s1, b1, s1, b1);
-        *reinterpret_cast<uint4*>(dst + 3 * 512) = dequant8(kw.w, s1, b1, s1, b1, s1, b1, s1, b1);
+        *reinterpret_cast<uint4*>(dst + 0 * 512) = dequant8(kw.x, s0, b0, s0, b0, s0, b0, s0, b0, P.masks);
+        *reinterpret_cast<uint4*>(dst + 1 * 512) = dequant8(kw.y, s0, b0, s0, b0, s0, b0, s0, b0, P.masks);
+        *reinterpret_cast<uint4*>(dst + 2 * 512) = dequant8(kw.z, s1, b1, s1, b1, s1, b1, s1, b1, P.masks);
+        *reinterpret_cast<uint4*>(dst + 3 * 512) = dequant8(kw.w, s1, b1, s1, b1, s1, b1, s1, b1, P.masks);
         if (G == 3) {
           const uint2 kw2 = *reinterpret_cast<const uint2*>(chunk + k_read2);
           uint32_t e2 = *reinterpret_cast<const uint32_t*>(chunk + k_sb + 8);  // group 2
           if (dead) e2 = 0u;
           const uint32_t s2 = __byte_perm(e2, e2, 0x1010), b2 = __byte_perm(e2, e2, 0x3232);
-          *reinterpret_cast<uint4*>(dst + 4 * 512) = dequant8(kw2.x, s2, b2, s2, b2, s2, b2, s2, b2);
-          *reinterpret_cast<uint4*>(dst + 5 * 512) = dequant8(kw2.y, s2, b2, s2, b2, s2, b2, s2, b2);
+          *reinterpret_cast<uint4*>(dst + 4 * 512) = dequant8(kw2.x, s2, b2, s2, b2, s2, b2, s2, b2, P.masks);
+          *reinterpret_cast<uint4*>(dst + 5 * 512) = dequant8(kw2.y, s2, b2, s2, b2, s2, b2, s2, b2, P.masks);
         }
       }
       fence_async_smem();
@@ -342,10 +343,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
           bp[i] = __byte_perm(e0, e1, 0x7632);                             // biases
         }
         uint8_t* dst = sm.vhat[sv] + vr * 16 + (4 * vq) * 1024 + (ci * 4 + vo) * 128;
-        *reinterpret_cast<uint4*>(dst + 0 * 1024) = dequant8(vw.x, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
-        *reinterpret_cast<uint4*>(dst + 1 * 1024) = dequant8(vw.y, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
-        *reinterpret_cast<uint4*>(dst + 2 * 1024) = dequant8(vw.z, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
-        *reinterpret_cast<uint4*>(dst + 3 * 1024) = dequant8(vw.w, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3]);
+        *reinterpret_cast<uint4*>(dst + 0 * 1024) = dequant8(vw.x, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3], P.masks);
+        *reinterpret_cast<uint4*>(dst + 1 * 1024) = dequant8(vw.y, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3], P.masks);
+        *reinterpret_cast<uint4*>(dst + 2 * 1024) = dequant8(vw.z, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3], P.masks);
+        *reinterpret_cast<uint4*>(dst + 3 * 1024) = dequant8(vw.w, sp[0], bp[0], sp[1], bp[1], sp[2], bp[2], sp[3], bp[3], P.masks);
       }
       fence_async_smem();
       __syncwarp();
