@@ -273,7 +273,9 @@ int q4kv_decode_attention_static(const q4kv_spec* spec, const void* pool, int32_
  *   q bf16 [total_q][n_q_heads][d_qk];  out [total_q][n_q_heads][d_v];  lse optional
  *   workspace  at least 16 bytes, better q4kv_workspace_bytes(spec, A, max_kv_len, total_q): with that much the call can cut
  *              the keys of a query tile over several SMs when there are few tiles, and take agents that bring a single
- *              query (in a batch where others bring more) as a decode step.  Its contents need not be cleared.
+ *              query (in a batch where others bring more) as a decode step.  The call neither reads nor writes the first
+ *              Q4KV_WORKSPACE_HEADER_BYTES, so a workspace of the larger of the two sizes serves prefill and decode calls in
+ *              any order; for prefill alone its contents need not be cleared.
  * Accuracy: see "Accuracy of the attention entry points" above (spec->exact_products selects
  * between the binary16-tile kernel and the kernel that multiplies the codes). */
 int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_blocks, int32_t layer,

@@ -67,7 +67,15 @@ size_t prefill_workspace(const Layout& y, int n_agents, int max_kv_len, int tota
   const int splits = plan_prefill_splits(y, prefill_tile_q(y), prefill_mla_supported(y) ? 2 : 1, n_agents, total_q, total_q, max_kv_len, 0, (size_t)-1);
   size_t need = splits > 1 ? align256(prefill_record_bytes(y, total_q, splits)) : 0;
   if (n_agents > 1 && total_q > n_agents && decode_mma_supported(y)) need += align256(singles_bytes(y, n_agents));
-  return need > 16 ? need : 16;
+  return need > 0 ? kWorkspaceHeaderBytes + need : 16;
+}
+
+// The part of a workspace that a prefill call may write: what lies behind the arrival counters, which every decode call on
+// the same workspace expects to find at zero.
+struct Scratch { uint8_t* at; size_t bytes; };
+Scratch prefill_scratch(void* workspace, size_t bytes) {
+  if (bytes <= kWorkspaceHeaderBytes) return {nullptr, 0};
+  return {(uint8_t*)workspace + kWorkspaceHeaderBytes, bytes - kWorkspaceHeaderBytes};
 }
 
 // The kernels that expand the cache into binary16 tiles round each dequantized element once; they are taken only when
@@ -262,11 +270,12 @@ int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_bl
   if (max_q_len == 0 || max_q_len > total_q) max_q_len = total_q;
   const Layout y = make_layout(*spec, n_blocks);
   if (workspace_bytes < workspace_need(y, batch->n_agents, max_kv_len, total_q)) return Q4KV_EWORKSPACE;
+  const Scratch scratch = prefill_scratch(workspace, workspace_bytes);
   cudaError_t e;
   if ((prefill_umma_supported(y) || prefill_umma_1tile_supported(y)) && tiles_allowed(spec, softmax_scale)) {
     PrefillExtra x = {};
-    uint8_t* at = (uint8_t*)workspace;
-    size_t left = workspace_bytes;
+    uint8_t* at = scratch.at;
+    size_t left = scratch.bytes;
     if (may_decode_singles(y, batch->n_agents, batch->max_blocks, total_q, max_q_len) && left >= singles_bytes(y, batch->n_agents)) {
       x.tickets = (int32_t*)at;
       x.n_tickets = decode_mma_tickets(y, batch->n_agents);
@@ -288,7 +297,7 @@ int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_bl
   }
   else if (prefill_mla_supported(y) && tiles_allowed(spec, softmax_scale))
     e = launch_prefill_mla(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, total_q, max_q_len, max_kv_len, window, q,
-                           softmax_scale, out, out_dtype, lse, workspace, workspace_bytes, status_flags, (cudaStream_t)stream);
+                           softmax_scale, out, out_dtype, lse, scratch.at, scratch.bytes, status_flags, (cudaStream_t)stream);
   else if (prefill_mma_supported(y))
     e = launch_prefill_mma(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale, out,
                            out_dtype, lse, status_flags, (cudaStream_t)stream);

@@ -674,6 +674,53 @@ def test_one_workspace_serves_growing_batches_and_every_kernel(H):
     assert int(ws[:B.WORKSPACE_HEADER_BYTES].max()) == 0          # every call left the arrival counters at zero
 
 
+@pytest.mark.parametrize("spec_args,chunks", [
+    ((1, 8, 8, 128, 128, False), [100]),                     # one agent's chunk: its keys are split
+    ((1, 8, 8, 256, 256, False), [70]),
+    ((1, 8, 8, 192, 128, False), [70]),
+    ((1, 16, 1, 576, 512, True), [20]),
+    ((1, 8, 8, 128, 128, False), [1, 60, 1, 1, 0, 1, 1, 1, 1]),   # single queries on the decode kernel, and splits
+    ((1, 16, 2, 128, 128, False), [1, 60, 1, 1]),            # eight heads per KV head
+])
+def test_one_workspace_serves_prefill_and_decode(H, spec_args, chunks):
+    """A serving program's order of calls on one workspace, zero-filled once: prefill, decode, prefill, update-and-fetch.
+    Nine agents x 8 KV heads are 72 pairs, each cut over several CTAs that find the last one of them by an arrival counter;
+    prefill leaves the counters at zero, and every decode equals the oracle."""
+    from paper_2603_04428_b200 import binding as B
+    lens = [2100 + 37 * a for a in range(9)]
+    p = Pair(H, spec_args, lens, seed=63, extra_tokens=1).fill()
+    s, A, cap = p.ospec, len(lens), p.dc.bt.max_blocks * 256
+    scale = 1.0 / math.sqrt(192 if s.v_aliases_k else s.d_qk)
+    total_q = sum(chunks)
+    ws = p.dc._ws = torch.zeros(max(B.q4kv_workspace_bytes(p.dc.spec, A, cap, 0),
+                                    B.q4kv_workspace_bytes(p.dc.spec, len(chunks), cap, total_q)),
+                                dtype=torch.uint8, device="cuda")
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    table, sub = p.dc.sub_batch(0, len(chunks))
+    qp, qd = p.q(9, total_q), p.q(10, A)
+    ref_p, _ = O.prefill_attention(p.opool, 0, p.tabs[:len(chunks)], lens[:len(chunks)], q_offs, 0, f32(qp), scale)
+    ref_d, lse_d = O.decode_attention(p.opool, 0, p.tabs, lens, 0, f32(qd), scale)
+    fused = s.v_aliases_k or s.n_q_heads // s.n_kv_heads <= 4
+    for step in range(2):
+        out, _ = p.dc.prefill(0, lens[:len(chunks)], q_offs, 0, qp, scale, bt=sub)
+        assert int(ws[:B.WORKSPACE_HEADER_BYTES].max()) == 0, "prefill wrote the arrival counters"
+        assert_attention_close(out.cpu().numpy(), ref_p, "prefill")
+        if step == 0 or not fused:
+            out, lse = p.dc.decode(0, lens, 0, qd, scale)
+        else:
+            kb = synth.kv_bf16(63, 500, A, s.n_kv_heads, s.d_qk)
+            vb = None if s.v_aliases_k else synth.kv_bf16(63, 501, A, s.n_kv_heads, s.d_v)
+            O.quantize_append(p.opool, 0, p.tabs, lens, np.arange(A + 1), f32(kb), None if vb is None else f32(vb))
+            lens = [n + 1 for n in lens]
+            ref_d, lse_d = O.decode_attention(p.opool, 0, p.tabs, lens, 0, f32(qd), scale)
+            out, lse = p.dc.append_decode(0, lens, 0, kb, vb, qd, scale)
+        assert_attention_close(out.cpu().numpy(), ref_d, f"decode after prefill, step {step}")
+        assert_lse_close(lse.cpu().numpy(), lse_d)
+        assert int(ws[:B.WORKSPACE_HEADER_BYTES].max()) == 0
+        assert p.dc.read_flags() == 0
+    assert p.dc._ws is ws
+
+
 @pytest.mark.parametrize("name", ["gqa128", "mla", "asym"])
 def test_length_beyond_the_stated_maximum_is_flagged_on_every_kernel(H, name):
     """max_kv_len is the caller's bound on every length: an agent above it gets zeros and Q4KV_FLAG_BAD_LENGTH,
