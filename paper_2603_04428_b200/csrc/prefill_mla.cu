@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     };
     auto fetch8 = [&](const uint8_t* chunk) { w8 = chunk ? __ldcg(reinterpret_cast<const uint2*>(chunk + read8)) : make_uint2(0u, 0u); };
     auto fetch_sb = [&](const uint8_t* chunk, int i) {
-      sb[i] = chunk ? __ldg(reinterpret_cast<const uint32_t*>(chunk + read_sb + 4 * i)) : 0u;
+      // through L1 (a line holds several tokens' pairs), but not as read-only data: the append before writes them while this runs
+      sb[i] = chunk ? *reinterpret_cast<const uint32_t*>(chunk + read_sb + 4 * i) : 0u;
     };
     const uint8_t* next = nullptr;
     if (n_iter > 0) {

@@ -996,6 +996,29 @@ def test_prefill_over_the_latent_cache(H, n_heads, prefix, chunks, window, sb_dt
     assert torch.allclose(bad[n0:], out[n0:], atol=1e-5)
 
 
+def test_latent_prefill_back_to_back_reads_the_rows_just_appended(H):
+    """The attention launch overlaps the tail of the append before it, which rewrites the same slots (codes, scales and
+    biases of another magnitude) in every round: enqueued without a pause, each round gives what it gives on an idle GPU."""
+    prefix, chunks = [600, 20], [100, 70]
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = Pair(H, SPECS["mla"], lens, seed=64).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    total, scale = int(q_offs[-1]), 1.0 / math.sqrt(192)
+    q = H.bf16_dev(p.q(9, total))
+    rows = [H.bf16_dev(synth.f32_to_bf16_bits(f32(synth.kv_bf16(64, 700 + r, total, 1, 576)) * np.float32(4.0 ** (r % 3 - 1))))
+            for r in range(8)]
+
+    def one(k):
+        p.dc.append(0, prefix, q_offs, k, None)
+        return p.dc.prefill(0, lens, q_offs, 0, q, scale)[0]
+
+    together = [one(k) for k in rows]
+    for k, out in zip(rows, together):
+        torch.cuda.synchronize()
+        assert torch.equal(one(k), out)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("spec_args,prefix,chunks,window,sb_dtype", [
     ((1, 8, 2, 128, 128, False), [9000], [40], 0, 0),        # two tiles of work: many splits of the keys
     ((1, 8, 2, 128, 128, False), [9000, 3], [33, 2], 2500, 1),   # under a window; an agent whose splits are mostly empty
