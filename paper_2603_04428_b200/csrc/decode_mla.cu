@@ -525,11 +525,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
 // so-many-th split with their loads issued together before the weights are known, and the groups' sums meet in registers
 // (groups of one warp) and shared memory.  How narrow the slices are depends on the count of splits: with four of them
 // sixteen groups would leave most threads idle (and make four times the CTAs), with 148 each group would walk nine.
+// The pointers carry no __restrict__: the records are written by the preceding kernel while this one is already resident, and
+// read-only loads are not defined for such data.
 constexpr int kMergeThreads = 512, kMaxSplits = 512;
 template <int kLanes>
-__global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_splits, const float* __restrict__ records,
-                                                                  void* __restrict__ out, int out_dtype,
-                                                                  float* __restrict__ lse) {
+__global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_splits, const float* records, void* out, int out_dtype,
+                                                                  float* lse) {
   __shared__ float s_w[kMaxSplits];                      // weight of each split (0: empty)
   __shared__ float s_red[kMergeThreads / 32][2];
   constexpr int kGroups = kMergeThreads / kLanes;

@@ -11,8 +11,7 @@ using namespace prefill;
 // One warp per (query row, head): weights of the parts, then the weighted sum, 128 output elements at a time.  Bound by
 // the latency of the records in L2; the parts of a row are in flight together.
 __global__ void __launch_bounds__(128)
-merge_prefill_kernel(int rows, int Dv, int n_splits, const float* __restrict__ records, void* __restrict__ out, int out_dtype,
-                     float* __restrict__ lse) {
+merge_prefill_kernel(int rows, int Dv, int n_splits, const float* records, void* out, int out_dtype, float* lse) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);

@@ -73,10 +73,11 @@ template <int M>
 __global__ void __launch_bounds__(kThreads)
 quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                        const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
-                       const int32_t* __restrict__ new_offs, const void* __restrict__ k_new,
-                       const void* __restrict__ v_new, int32_t* flags) {
+                       const int32_t* __restrict__ new_offs, const void* k_new, const void* v_new, int32_t* flags) {
   extern __shared__ uint8_t vcodes_all[];   // [M][8][Dv]
   __shared__ UnitInfo s_unit[M];
+  // (k_new, v_new carry no __restrict__: the preceding kernel may write them while this one is resident, and read-only loads are
+  // not defined for such data.)
   // let the next kernel of the stream start its prologue; the unit is found from the lengths and block tables (inputs
   // that no kernel writes) while the preceding kernels drain, and the wait comes before the new rows and the pool
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -244,8 +245,8 @@ template <int kWpc>
 __global__ void __launch_bounds__(kThreads, 2)
 quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                             const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
-                            const int32_t* __restrict__ new_offs, const uint16_t* __restrict__ k_new,
-                            const uint16_t* __restrict__ v_new, int32_t* flags, int units) {
+                            const int32_t* __restrict__ new_offs, const uint16_t* k_new, const uint16_t* v_new,
+                            int32_t* flags, int units) {
   __shared__ ChunkUnit s_unit[kThreads / 32];
   extern __shared__ __align__(16) uint8_t stage_all[];  // one chunk per warp
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -295,7 +296,7 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
       const size_t row = (size_t)(un.r0 + (first - un.p) + i) * y.Hkv + hk;
       const uint16_t* src = is_v ? v_new + row * y.Dv + 64 * gi : k_new + row * y.D + 64 * gi;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) raw[j] = __ldg(reinterpret_cast<const uint4*>(src) + j);
+      for (int j = 0; j < 8; ++j) raw[j] = reinterpret_cast<const uint4*>(src)[j];
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) raw[j] = make_uint4(0u, 0u, 0u, 0u);

@@ -996,21 +996,23 @@ def test_prefill_over_the_latent_cache(H, n_heads, prefix, chunks, window, sb_dt
     assert torch.allclose(bad[n0:], out[n0:], atol=1e-5)
 
 
-def test_latent_prefill_back_to_back_reads_the_rows_just_appended(H):
-    """The attention launch overlaps the tail of the append before it, which rewrites the same slots (codes, scales and
-    biases of another magnitude) in every round: enqueued without a pause, each round gives what it gives on an idle GPU."""
+@pytest.mark.parametrize("call", ["prefill", "decode"])
+def test_latent_calls_back_to_back_read_what_the_call_before_wrote(H, call):
+    """Every launch overlaps the tail of the one before it.  The append rewrites the same slots (codes, scales and biases of
+    another magnitude) in every round, and the split records are rewritten too: enqueued without a pause, each round gives
+    what it gives on an idle GPU."""
     prefix, chunks = [600, 20], [100, 70]
     lens = [p0 + c for p0, c in zip(prefix, chunks)]
     p = Pair(H, SPECS["mla"], lens, seed=64).fill()
     q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
     total, scale = int(q_offs[-1]), 1.0 / math.sqrt(192)
-    q = H.bf16_dev(p.q(9, total))
+    q = H.bf16_dev(p.q(9, total if call == "prefill" else 2))
     rows = [H.bf16_dev(synth.f32_to_bf16_bits(f32(synth.kv_bf16(64, 700 + r, total, 1, 576)) * np.float32(4.0 ** (r % 3 - 1))))
             for r in range(8)]
 
     def one(k):
         p.dc.append(0, prefix, q_offs, k, None)
-        return p.dc.prefill(0, lens, q_offs, 0, q, scale)[0]
+        return p.dc.prefill(0, lens, q_offs, 0, q, scale)[0] if call == "prefill" else p.dc.decode(0, lens, 0, q, scale)[0]
 
     together = [one(k) for k in rows]
     for k, out in zip(rows, together):
