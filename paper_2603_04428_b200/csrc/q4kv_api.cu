@@ -282,14 +282,15 @@ int q4kv_prefill_attention(const q4kv_spec* spec, const void* pool, int32_t n_bl
       at += align256(singles_bytes(y, batch->n_agents));
       left -= left < align256(singles_bytes(y, batch->n_agents)) ? left : align256(singles_bytes(y, batch->n_agents));
     }
-    x.n_splits = plan_prefill_splits(y, prefill_tile_q(y), 1, batch->n_agents, total_q, max_q_len, max_kv_len, window, left);
+    x.n_splits = plan_prefill_splits(y, prefill_tile_q(y), 1, batch->n_agents, total_q, max_q_len, max_kv_len, window, left,
+                                     x.tickets != nullptr);
     x.records = (float*)at;
     const auto launch = prefill_umma_supported(y) ? launch_prefill_umma : launch_prefill_umma_1tile;
     e = launch(y, pool, n_blocks, layer, *batch, kv_lens, q_offs, max_q_len, window, q, softmax_scale, out, out_dtype, lse,
                status_flags, (cudaStream_t)stream, x);
     if (e == cudaSuccess && x.n_splits > 1)
-      e = launch_merge_prefill(y, total_q, x.n_splits, x.records, out, out_dtype, lse, (cudaStream_t)stream);
-    // after the merge, which leaves something or other in the rows of these agents
+      e = launch_merge_prefill(y, total_q, x.n_splits, x.records, out, out_dtype, lse, (cudaStream_t)stream,
+                               x.tickets ? q_offs : nullptr, batch->n_agents);
     if (e == cudaSuccess && x.tickets)
       e = launch_decode_mma(y, pool, n_blocks, layer, *batch, kv_lens, cap, &window, 1, q, softmax_scale, out, out_dtype, lse,
                             (uint8_t*)x.tickets + align256(sizeof(int32_t) * x.n_tickets) - kWorkspaceHeaderBytes, status_flags,

@@ -189,9 +189,11 @@ inline size_t prefill_record_bytes(const Layout& y, int total_q, int n_splits) {
   return (size_t)total_q * y.Hq * n_splits * prefill_record(y.Dv) * sizeof(float);
 }
 int plan_prefill_splits(const Layout& y, int tile_q, int per_tile, int n_agents, int total_q, int max_q_len, int max_kv_len,
-                        int window, size_t ws_bytes);
+                        int window, size_t ws_bytes, bool singles = false);   // singles: agents with one query are not in the launch
 cudaError_t launch_merge_prefill(const Layout& y, int total_q, int n_splits, const float* records, void* out, int out_dtype,
-                                 float* lse, cudaStream_t st);
+                                 float* lse, cudaStream_t st,
+                                 // q_offs: the rows of agents with one query are left as they are
+                                 const int32_t* q_offs = nullptr, int n_agents = 0);
 
 // Decode on the MLA-latent cache (d_qk 576, d_v 512 aliasing K, one KV head, at most 16 query heads): a key-split
 // attention kernel -- on a binary16 tile of the dequantized keys, or, with on_codes, on the 4-bit codes themselves

@@ -1052,6 +1052,29 @@ def test_prefill_of_mostly_single_queries(H, spec_args, window, chunks):
     check_prefill(H, spec_args, prefix, chunks, window)
 
 
+def test_one_wave_of_tiles_beside_single_queries_is_not_cut(H):
+    """Two chunks of 512 queries (32 / 8 heads: 128 tiles, one wave) among ten agents that decode: the tiles stay whole, so
+    nothing is written behind the scratch of the single queries, and the rows equal those of a call without scratch."""
+    from paper_2603_04428_b200 import binding as B
+    chunks = [1, 512, 1, 1, 1, 1, 512, 1, 1, 1, 1, 1]
+    lens = [700 + 431 * a for a in range(12)]
+    p = Pair(H, (1, 32, 8, 128, 128, False), lens, seed=65)
+    rows = sum(lens)
+    p.dc.append(0, [0] * 12, np.concatenate([[0], np.cumsum(lens)]), synth.kv_bf16(65, 1, rows, 8, 128),
+                synth.kv_bf16(65, 2, rows, 8, 128))
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q, scale = H.bf16_dev(p.q(9, sum(chunks))), 1.0 / math.sqrt(128)
+    p.dc._ws = ws = torch.full((256 << 20,), 0x5A, dtype=torch.uint8, device="cuda")
+    out, lse = p.dc.prefill(0, lens, q_offs, 0, q, scale, max_kv_len=max(lens))
+    used = torch.nonzero(ws != 0x5A).max().item()
+    assert used < B.q4kv_workspace_bytes(p.dc.spec, 12, max(lens), 0) + 4096
+    p.dc.workspace = lambda *sizes: torch.zeros(16, dtype=torch.uint8, device="cuda")
+    whole, lse_whole = p.dc.prefill(0, lens, q_offs, 0, q, scale, max_kv_len=max(lens))
+    assert_attention_close(out.cpu().numpy(), whole.cpu().numpy().astype(np.float64))
+    assert_lse_close(lse.cpu().numpy(), lse_whole.cpu().numpy().astype(np.float64))
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("spec_args,lens,sb_dtype", [
     ((1, 16, 16, 192, 128, False), [2200, 31], 0),           # 16 x (69 + 4) units: four warps each
     ((1, 16, 16, 192, 128, False), [2290, 31], 1),           # 16 x (72 + 4) units: one warp each
