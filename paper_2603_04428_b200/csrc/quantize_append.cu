@@ -296,7 +296,7 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
       const size_t row = (size_t)(un.r0 + (first - un.p) + i) * y.Hkv + hk;
       const uint16_t* src = is_v ? v_new + row * y.Dv + 64 * gi : k_new + row * y.D + 64 * gi;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) raw[j] = reinterpret_cast<const uint4*>(src)[j];
+      for (int j = 0; j < 8; ++j) raw[j] = __ldca(reinterpret_cast<const uint4*>(src) + j);
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) raw[j] = make_uint4(0u, 0u, 0u, 0u);
