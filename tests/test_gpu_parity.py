@@ -924,7 +924,7 @@ class QuietStartPair(Pair):
     ((1, 8, 2, 128, 128, False), [3000], [200], 700, 1.0),               # the window starts many 64-key blocks in
     ((1, 8, 2, 128, 128, False), [1500, 64], [129, 64], 0, 2.0),         # the row maximum jumps by more than 2^8, late
     ((1, 8, 2, 128, 128, False), [1500, 64], [129, 64], 0, 8.0),         # a sharp scale is routed to the exact-code kernel
-    ((1, 6, 2, 128, 128, False), [700, 30], [100, 64], 0, 1.0),          # three query heads per KV head: exact-code kernel
+    ((1, 6, 2, 128, 128, False), [700, 30], [100, 64], 0, 1.0),          # three query heads per KV head: tiles of 42 queries
     ((1, 4, 4, 128, 128, False), [0], [257], 0, 1.0),                    # no prefix at all: purely causal
     ((1, 4, 2, 256, 256, False), [900, 5], [140, 70], 0, 1.0),           # d = 256 (one tile per CTA, two score buffers)
     ((1, 8, 2, 256, 256, False), [3000], [200], 700, 1.0),               # d = 256, four heads per KV head, a window
@@ -1092,12 +1092,14 @@ def test_prefill_on_large_magnitude_caches(H, gain, outlier_frac, prefix, chunks
     values, return value rows almost verbatim, so a single binary16 rounding of a dequantized value (half an ulp of
     2^-8 for magnitudes in [8, 16)) is visible.  With exact_products the usual bound holds; without it the
     binary16-tile kernel stays inside the bound the header states for it."""
-    spec_args = (1, 8, 2, d, 128 if d == 192 else d, False)
+    check_large_magnitudes(H, (1, 8, 2, d, 128 if d == 192 else d, False), gain, outlier_frac, prefix, chunks, 1.0 / math.sqrt(d))
+
+
+def check_large_magnitudes(H, spec_args, gain, outlier_frac, prefix, chunks, scale, sb_dtype=0):
     lens = [p0 + c for p0, c in zip(prefix, chunks)]
     q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
-    scale = 1.0 / math.sqrt(d)
     for exact in (True, False):
-        p = Pair(H, spec_args, lens, seed=48, gain=gain, outlier_frac=outlier_frac, exact_products=exact).fill()
+        p = Pair(H, spec_args, lens, seed=48, gain=gain, outlier_frac=outlier_frac, exact_products=exact, sb_dtype=sb_dtype).fill()
         q = p.q(9, int(q_offs[-1]))
         ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, 0, f32(q), scale)
         out, lse = p.dc.prefill(0, lens, q_offs, 0, q, scale)
@@ -1110,6 +1112,37 @@ def test_prefill_on_large_magnitude_caches(H, gain, outlier_frac, prefix, chunks
             assert M >= 8.0
             assert np.abs(got - ref).max() <= bound
         assert p.dc.read_flags() == 0
+
+
+@pytest.mark.parametrize("gain,outlier_frac", [(8.0, 0.0), (1.0, 0.01)])
+@pytest.mark.parametrize("spec_args,scale,sb_dtype", [
+    ((1, 16, 1, 576, 512, True), 1.0 / math.sqrt(192), 0),       # the latent cache: tcgen05, exactly on the shape-agnostic kernel
+    ((1, 5, 1, 576, 512, True), 1.0 / math.sqrt(192), 1),
+    ((1, 16, 2, 128, 128, False), 1.0 / math.sqrt(128), 0),      # eight heads per KV head, likewise
+    ((1, 6, 2, 256, 256, False), 1.0 / 16.0, 1),                 # three: exactly on the kernel that multiplies the codes
+])
+def test_prefill_on_large_magnitude_caches_of_other_routes(H, gain, outlier_frac, spec_args, scale, sb_dtype):
+    check_large_magnitudes(H, spec_args, gain, outlier_frac, [0, 40, 300], [70, 30, 64], scale, sb_dtype)
+
+
+@pytest.mark.parametrize("spec_args,prefix,chunks,window,scale,exact", [
+    ((1, 16, 1, 576, 512, True), [300, 0], [40, 65], 0, 0.1, False),     # scale^2 * d_qk > 4: may not be rounded
+    ((1, 16, 1, 576, 512, True), [300, 0], [40, 65], 90, 1.0 / math.sqrt(192), True),
+    ((1, 16, 2, 128, 128, False), [300, 0], [40, 65], 90, 1.0 / math.sqrt(128), True),
+    ((1, 16, 2, 128, 128, False), [300, 0], [40, 65], 0, 0.5, False),
+    ((1, 7, 1, 192, 128, False), [300, 0], [40, 65], 0, 1.0 / math.sqrt(192), True),
+])
+def test_prefill_on_the_codes_where_only_the_shape_agnostic_kernel_does(H, spec_args, prefix, chunks, window, scale, exact):
+    """Exact products on the latent cache and above four heads per KV head: within the bound of the exact routes (2e-5 * M + 1e-5)."""
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = QuietStartPair(H, spec_args, lens, seed=66, exact_products=exact).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = p.q(9, int(q_offs[-1]))
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, window, f32(q), scale)
+    out, lse = p.dc.prefill(0, lens, q_offs, window, q, scale)
+    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= 2e-5 * max_dequantized_magnitude(p, 0) + 1e-5
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    assert p.dc.read_flags() == 0
 
 
 @pytest.mark.parametrize("d", [128, 256, 192])
