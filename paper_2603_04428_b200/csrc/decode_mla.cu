@@ -32,6 +32,7 @@
 // scales, now 20.6); 32 agents x 8192 tokens 110 us, now 60.
 #include <algorithm>
 
+#include "convert.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
 #include "tcgen05.cuh"
@@ -52,7 +53,6 @@ constexpr int kTileBytes = 8 * kOctetBytes;              // 65536
 constexpr int kGroupStride = (kD / 8) * 128;             // 9216: bytes between 8-row groups of a [rows][576] tile
 constexpr int kStages = 2, kRawSlots = 3;
 constexpr int kRecStride = kDv + 2;                      // acc[512], m, l
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLazy = 8.f;
 
 using MlaParams = MlaDecodeParams;
@@ -74,38 +74,6 @@ struct MlaSmem {
   uint32_t new_words[kD / 8], new_sb[kD / 64];           // the new token's codes and (scale, bias) pairs (update-and-fetch)
 };
 
-// Eight codes of one packed word -> eight binary16 values c * s + b in the order (0,4) (1,5) (2,6) (3,7),
-// one (scale, bias) for all (s2 = (s, s), b2 = (b, b)).  Or-ing a masked nibble into the mantissa of 1024
-// (ulp 1), or of 64 for a nibble four bits up (ulp 1/16), gives 1024 + c or 64 + c exactly.
-__device__ inline uint4 dequant8(uint32_t w, uint32_t s2, uint32_t b2, uint32_t mask_lo, uint32_t mask_hi) {
-  const uint32_t wh = w >> 8;
-  const __half2 k1024 = __half2half2(__ushort_as_half((unsigned short)0x6400));
-  const __half2 k64 = __half2half2(__ushort_as_half((unsigned short)0x5400));
-  auto as_h2 = [](uint32_t u) { return *reinterpret_cast<__half2*>(&u); };
-  auto as_u = [](__half2 h) { return *reinterpret_cast<uint32_t*>(&h); };
-  const __half2 s = as_h2(s2), b = as_h2(b2);
-  const __half2 c04 = __hsub2(as_h2((w & mask_lo) | 0x64006400u), k1024);
-  const __half2 c15 = __hsub2(as_h2((w & mask_hi) | 0x54005400u), k64);
-  const __half2 c26 = __hsub2(as_h2((wh & mask_lo) | 0x64006400u), k1024);
-  const __half2 c37 = __hsub2(as_h2((wh & mask_hi) | 0x54005400u), k64);
-  return make_uint4(as_u(__hfma2(c04, s, b)), as_u(__hfma2(c15, s, b)), as_u(__hfma2(c26, s, b)), as_u(__hfma2(c37, s, b)));
-}
-__device__ inline float fast_exp2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ inline uint32_t f32x2_to_h2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-// A bfloat16 (scale, bias) pair as a binary16 pair: exact while the magnitude is a binary16 normal number (bfloat16
-// has 8 significant bits), within 2^-25 below that; a magnitude beyond binary16's largest number is reported.
-__device__ inline uint32_t bf16_pair_to_h2(uint32_t u, bool& overflow) {
-  const uint32_t h = f32x2_to_h2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
-  overflow |= (((h & 0x7C007C00u) + 0x04000400u) & 0x80008000u) != 0u;     // an exponent field of all ones
-  return h;
-}
 __device__ inline void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // all eight warps
 // the same, and whether the predicate holds for any of the threads
 __device__ inline bool compute_any(bool p) {
@@ -199,8 +167,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the new token was appended by the preceding kernel
   volatile int* abort_flag = &sm.abort_flag;
 
-  // Raw 64-key blocks: one bulk copy each into a two-slot ring, issued by thread 0 -- blocks 0 and 1 here, block
-  // j + 2 once every warp has left block j's raw bytes (the barrier after the dequantize step).
+  // Raw 64-key blocks: one bulk copy each into a three-slot ring, issued by thread 0 -- blocks 0 to 2 here, block
+  // j + 3 once every warp has left block j's raw bytes (the block's CTA-wide barrier).
   auto block_of = [&](int j) { return P.tables[(size_t)a * P.max_blocks + ((2 * (b0 + j)) >> 3)]; };
   auto issue_block = [&](int j, int blk) {
     const int r = j % kRawSlots;
@@ -304,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   const int wr_b = (oct & 1) ? -kOctetBytes : kOctetBytes;
 
   // from memory, so that the compiler does not know them: (w & mask) | magic is one instruction with one immediate
-  const uint32_t mask_lo = sm.masks[0], mask_hi = sm.masks[1];
+  const CodeMasks masks = {sm.masks[0], sm.masks[1]};
 
   // ldmatrix lane addresses (lane l: matrix l / 8, row l % 8)
   const int lm = lane >> 3, lr = lane & 7;
@@ -385,7 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
         if (kBf) sb[i] = bf16_pair_to_h2(sb[i], overflow);
       }
       auto expand = [&](uint32_t w, uint32_t pair) {
-        return dequant8(w, __byte_perm(pair, pair, 0x1010), __byte_perm(pair, pair, 0x3232), mask_lo, mask_hi);
+        return dequant8(w, __byte_perm(pair, pair, 0x1010), __byte_perm(pair, pair, 0x3232), masks);
       };
       float acc[2][4];                                   // [own octet, the other one]
 #pragma unroll

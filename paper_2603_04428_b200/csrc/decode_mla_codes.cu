@@ -36,6 +36,7 @@
 //     probabilities are retaken.  One CTA-wide barrier per block otherwise.
 // The raw blocks arrive on mbarriers with bounded waits (Q4KV_FLAG_INTERNAL when one runs out; the
 // 256 threads then leave together).  Eight warps: the query fragments alone take 144 registers.
+#include "convert.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
 #include "tcgen05.cuh"
@@ -78,15 +79,6 @@ struct MlaSmem {
   uint32_t new_words[kD / 8], new_sb[kD / 64];           // the new token's codes and (scale, bias) pairs (update-and-fetch)
 };
 
-__device__ inline float fast_exp2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ inline uint32_t f32x2_to_h2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 __device__ inline float2 h2_to_f2(uint32_t u) { return __half22float2(*reinterpret_cast<__half2*>(&u)); }
 // two 16-bit numbers of the cache's scale / bias type as binary32
 template <bool kBf>

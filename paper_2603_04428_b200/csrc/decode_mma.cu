@@ -46,8 +46,10 @@
 //     vote says that some score outgrew it; it is then set kMargin above the maximum, so that it moves less often.
 #include <climits>
 
+#include "convert.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
+#include "tcgen05.cuh"
 
 namespace q4kv {
 
@@ -61,38 +63,18 @@ constexpr int kWholeSlack = 12;                        // see find_range
 constexpr float kMargin = 0.35f;                       // see chunk_values
 constexpr int kMaxRecords = 32;                        // a pair is cut over about this many CTAs at most (the merge reads them all)
 constexpr uint32_t kSpinLimit = 1u << 22;              // bounded mbarrier waits (each try blocks a while in hardware)
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kMaskLo = 0x000F000Fu, kMaskHi = 0x00F000F0u;
 
 // ---------------------------------------------------------------------------------------------
 // PTX wrappers
 // ---------------------------------------------------------------------------------------------
-__device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ inline void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ inline void mbar_arrive(uint64_t* bar) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ inline void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
+using tc::bulk_load, tc::mbar_arrive, tc::mbar_arrive_expect_tx, tc::mbar_init, tc::mbar_test_wait, tc::smem_u32;
+// (without the suspension hint of the tcgen05 kernels' waits: every warp here waits for its own next bytes)
 __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ inline bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(smem_u32(bar)), "r"(parity)
       : "memory");
@@ -116,12 +98,6 @@ __device__ inline void prefetch_l2(const void* p) { asm volatile("prefetch.globa
 __device__ inline void prefetch_l2_bulk(const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
-__device__ inline void bulk_load(void* dst_smem, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst_smem)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 __device__ inline void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ inline void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -130,20 +106,11 @@ __device__ inline void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ inline float fast_exp2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 // half2(lo = a, hi = b), both rounded toward zero
 __device__ inline uint32_t f32x2_to_h2_rz(float a, float b) {
   uint32_t r;
   asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
   return r;
-}
-__device__ inline uint32_t f32x2_to_h2_rn(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 constexpr int kMaxLayersPerCall = 64;
@@ -522,8 +489,8 @@ __device__ __forceinline__ void stage_query_row(uint4 (*qfrag)[32], float (*qsum
   if (scale_log2 == 0.f) sf = 0.f;
   const float sl = sf * 0.0625f;
   if (w < D / 8) {
-    const uint4 f = make_uint4(f32x2_to_h2_rn(x[0] * sf, x[4] * sf), f32x2_to_h2_rn(x[1] * sl, x[5] * sl),
-                               f32x2_to_h2_rn(x[2] * sf, x[6] * sf), f32x2_to_h2_rn(x[3] * sl, x[7] * sl));
+    const uint4 f = make_uint4(f32x2_to_h2(x[0] * sf, x[4] * sf), f32x2_to_h2(x[1] * sl, x[5] * sl),
+                               f32x2_to_h2(x[2] * sf, x[6] * sf), f32x2_to_h2(x[3] * sl, x[7] * sl));
     const int gi = w >> 3, i2 = (w >> 2) & 1, t = w & 3;
     qfrag[2 * gi + i2][h * 4 + t] = f;
     if (H == 4) qfrag[2 * gi + i2][(h + 4) * 4 + t] = f;                       // columns 4..7 repeat the heads

@@ -22,8 +22,10 @@
 //     register-resident flash attention, so probabilities never leave their lane.
 // Measured: 146 TFLOP/s on 8 x (8192 + 1024) tokens at d = 128 with 32 / 8 heads; 148 TFLOP/s on 8 x (4096 + 512)
 // tokens at d = 256 with 16 / 8 heads.
+#include "convert.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
+#include "tcgen05.cuh"
 
 namespace q4kv {
 
@@ -33,21 +35,10 @@ constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 constexpr int kSlots = 16;                 // ring depth in chunks
 constexpr uint32_t kSpinLimit = 1u << 22;
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kMaskLo = 0x000F000Fu, kMaskHi = 0x00F000F0u;
 
-__device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ inline void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ inline void mbar_arrive(uint64_t* bar) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ inline void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
+using tc::bulk_load, tc::mbar_arrive, tc::mbar_arrive_expect_tx, tc::mbar_init, tc::smem_u32;
+// (without the suspension hint of the tcgen05 kernels' waits: every warp here waits for its own next bytes)
 __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -65,12 +56,6 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* a
   *abort_flag = 1;
   return false;
 }
-__device__ inline void bulk_load(void* dst_smem, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst_smem)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 __device__ inline void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -81,16 +66,7 @@ __device__ inline void mma_f16(float (&c)[4], const uint4& a, uint32_t b0, uint3
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
-__device__ inline float fast_exp2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 __device__ inline float2 h2_to_f2(uint32_t u) { return __half22float2(*reinterpret_cast<__half2*>(&u)); }
-__device__ inline uint32_t f32x2_to_h2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 struct PrefillParams {
   Layout y;
   const uint8_t* pool;
