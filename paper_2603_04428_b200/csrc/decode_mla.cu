@@ -27,9 +27,9 @@
 // scheduler's two warps alone take 1150), 250 the softmax, 500 the barrier and the wait for the block; and per launch about
 // 6 us of prologue, first block, record and merge.  Eight warps because the queries' fragments, the accumulators and two
 // words in flight need the registers: sixteen warps of 128 registers (four per group of octets) took 22.1 us where this
-// takes 20.2 (4 agents x 16384 tokens with the merge), two groups of four warps with separate chunks 20.9.  The first form,
-// with an expanded key tile read through ldmatrix for the scores and three barriers per block, took 21.3 (23.8 with bfloat16
-// scales, now 20.6); 32 agents x 8192 tokens 110 us, now 60.
+// took 20.2 (4 agents x 16384 tokens with the merge; 19.4 since the merge takes its records by ordinary loads), two groups of
+// four warps with separate chunks 20.9.  The first form, with an expanded key tile read through ldmatrix for the scores and
+// three barriers per block, took 21.3 (23.8 with bfloat16 scales, now 19.9); 32 agents x 8192 tokens 110 us, now 60.
 #include <algorithm>
 
 #include "convert.cuh"
@@ -669,12 +669,12 @@ cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, i
   }
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t mcfg = {};
-  // 4, 8, 16 or 64 groups of threads share the splits, so that a thread's loads are few and all in flight together.  Measured,
-  // merge and kernel: 4 splits x 32 agents 60.1 us on 128 lanes (66.2 on 32), 17 x 8 13.5 on 64 (14.4 on 32), 37 x 4 20.2 on
-  // 32 (21.6 on 64, 21.0 on 16), 148 x 1 22.4 on 8 (24.1 on 32).
-  const int lanes = plan.n_splits <= 8 ? 128 : plan.n_splits <= 24 ? 64 : plan.n_splits <= 64 ? 32 : 8;
+  // 4, 8, 16 or 32 groups of threads share the splits, so that a thread's loads are few and all in flight together.  Measured,
+  // merge and kernel, on 128 / 64 / 32 / 16 / 8 lanes: 4 splits x 32 agents 59.9 / 63.6 / 69.0 / 80 / 90 us, 17 x 8 14.5 / 12.5 /
+  // 14.1 / 17.4 / 19.9, 37 x 4 24.2 / 20.2 / 19.4 / 21.1 / 22.6, 148 x 1 40 / 24.5 / 21.9 / 21.0 / 22.6.
+  const int lanes = plan.n_splits <= 8 ? 128 : plan.n_splits <= 24 ? 64 : plan.n_splits <= 64 ? 32 : 16;
   void (*merge)(int, int, const float*, void*, int, float*) =
-      lanes == 128 ? merge_mla_kernel<128> : lanes == 64 ? merge_mla_kernel<64> : lanes == 32 ? merge_mla_kernel<32> : merge_mla_kernel<8>;
+      lanes == 128 ? merge_mla_kernel<128> : lanes == 64 ? merge_mla_kernel<64> : lanes == 32 ? merge_mla_kernel<32> : merge_mla_kernel<16>;
   mcfg.gridDim = dim3(kHeads, b.n_agents, kDv / 4 / lanes);
   mcfg.blockDim = dim3(kMergeThreads);
   mcfg.stream = st;

@@ -539,6 +539,7 @@ def test_decode_more_than_four_query_heads_per_kv_head(H, spec_args, lens, windo
 @pytest.mark.parametrize("n_heads,lens,sb_dtype", [
     (16, [9000, 70], 0),                                     # 74 key shares per agent
     (16, [4800], 1),                                         # 38, one agent
+    (16, [9300], 0),                                         # one for every SM
     (3, [700 + 9 * i for i in range(8)], 0),                 # twelve; 8 x 19 CTAs would not fit one wave
     (16, [1 + 37 * i for i in range(40)], 1),                # three: 40 x 4 would not either
     (16, [5 + i for i in range(150)], 0),                    # more agents than SMs
