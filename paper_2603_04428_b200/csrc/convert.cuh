@@ -11,7 +11,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 // (3,7) with the scale and bias pair given for each.  Masking a nibble into the mantissa of 1024
 // (ulp 1) or of 64 (ulp 1/16, for a nibble sitting four bits up) gives 1024 + c or 64 + c exactly.  The masks are kernel
 // parameters, so that the compiler does not know them: (w & mask) | magic is then one instruction with one immediate operand,
-// where two immediates take two (d = 256 prefill 391 -> 379 us, 192 / 128 321 -> 303, latent 231 -> 227, d = 128 1310 -> 1290).
+// where two immediates take two (prefill in short runs: d = 256 391 -> 379 us, 192 / 128 321 -> 303, latent 231 -> 227, d = 128 1310 -> 1290).
 struct CodeMasks { uint32_t lo = 0x000F000Fu, hi = 0x00F000F0u; };
 __device__ inline uint4 dequant8(uint32_t w, uint32_t s04, uint32_t b04, uint32_t s15, uint32_t b15, uint32_t s26,
                                  uint32_t b26, uint32_t s37, uint32_t b37, const CodeMasks& m) {

@@ -26,7 +26,7 @@
 //   * With few tiles the keys of a tile are cut over several CTAs as well (plan_prefill_splits); these leave (acc, m, l)
 //     records that merge_prefill_kernel combines.
 // Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads (102 GFLOP): 36 ms on the shape-agnostic kernel,
-// 0.227 ms here = 449 TFLOP/s; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
+// 0.203 ms here = 502 TFLOP/s back to back; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
 // products share the shared-memory bandwidth (256 KB per block: 2000 clocks) and the issue slots.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises Q4KV_FLAG_INTERNAL, drains the tensor
 // pipe and frees the tensor memory before the CTA returns.

@@ -10,7 +10,8 @@
 //     2050, shared memory for 2300 (operands 1570, tiles written 510, raw blocks 150) and the issue slots for 1700, so what
 //     matters is that all of them work at once: few, long hand-offs.  (Steps of 64 keys with the queries in tensor memory and
 //     two threads per row, which exchanged their maxima, took 2 x 3000 clocks.)  Measured on 8 agents x (8192 + 1024 tokens),
-//     32 / 8 heads: 5300 clocks per step, 1616 -> 1290 us per launch = 905 TFLOP/s (723 before).  What is left is the chain of
+//     32 / 8 heads: 5300 clocks per step; 1238 us per launch = 943 TFLOP/s in a run of a few launches, 1357 us = 861 TFLOP/s in a
+//     run of seconds, under the power cap (1616 us = 723 with the 64-key steps).  What is left is the chain of
 //     a tile's step -- scores 330 clocks after their product, exponentials 2 x 1500, value and score products 1700 -- of which
 //     the two tiles overlap a half.  Measured without gain: four softmax warps per row pair (16 in all), score buffers of 64
 //     keys issued two blocks ahead, an issuing warp per tile (the tiles then fall into step), scores fetched ahead.

@@ -33,7 +33,7 @@
 // Bound by the dequantize warps' chain per block (2650 clocks per 64 keys; the two products take 1250, and with the tiles left
 // as they are a block takes 2100).  With one barrier for all eight softmax warps, maxima exchanged in every block and 96
 // registers for every warp (the d = 256 form spilled) it took 3400.  8 agents x (4096 + 512) tokens, 16 query heads, d = 256:
-// 508 -> 379 us (575 -> 771 TFLOP/s); 192 / 128: 350 -> 303 (601).
+// 508 -> 382 us (575 -> 765 TFLOP/s) in a run of seconds, 363 us in one of a few launches; 192 / 128: 350 -> 282 (648), 281.
 #include "prefill_common.cuh"
 
 namespace q4kv {
