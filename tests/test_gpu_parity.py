@@ -501,7 +501,7 @@ def test_update_and_fetch_in_one_launch(H, name, lens, window):
     ((1, 6, 2, 128, 128, False), [700, 33, 1000], 200),
     ((1, 3, 1, 256, 256, False), [1500, 41], 0),
     ((1, 2, 2, 256, 256, False), [1500, 41], 1024),
-    ((1, 16, 2, 128, 128, False), [700, 300], 0),            # eight: beyond the tensor-core kernel, shape-agnostic path
+    ((1, 16, 2, 128, 128, False), [700, 300], 0),            # eight: every score column is a head
     ((1, 16, 2, 128, 128, False), [700, 300], 100),
 ])
 def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
@@ -647,13 +647,14 @@ def test_latent_decode_on_large_magnitude_caches(H, gain, outlier_frac):
 
 
 def test_one_workspace_serves_growing_batches_and_every_kernel(H):
-    """One workspace, allocated once for the largest call and zero-filled once: a latent-cache call, a d = 192 call
-    (shape-agnostic kernel) and GQA calls of 2 agents and then of 10 agents x 8 KV heads (more pairs than arrival
+    """One workspace, allocated once for the largest call and zero-filled once: a latent-cache call, a d_qk 192 call, a d = 64
+    call (shape-agnostic kernel) and GQA calls of 2 agents and then of 10 agents x 8 KV heads (more pairs than arrival
     counters fit in 256 bytes) all run on it, each compared with the oracle, outputs pre-filled with NaN."""
     from paper_2603_04428_b200 import binding as B
     cases = [
         (SPECS["mla"], [600, 70], 1.0 / math.sqrt(192)),
         (SPECS["asym"], [400, 300], 1.0 / math.sqrt(192)),
+        ((1, 4, 2, 64, 64, False), [400, 3000], 0.125),
         ((1, 32, 8, 128, 128, False), [700, 300], 1.0 / math.sqrt(128)),
         ((1, 32, 8, 128, 128, False), [700, 300, 260, 5000, 90, 1200, 64, 33, 2000, 513], 1.0 / math.sqrt(128)),
         ((1, 32, 8, 128, 128, False), [700, 300], 1.0 / math.sqrt(128)),
@@ -722,7 +723,7 @@ def test_one_workspace_serves_prefill_and_decode(H, spec_args, chunks):
     assert p.dc._ws is ws
 
 
-@pytest.mark.parametrize("name", ["gqa128", "mla", "asym"])
+@pytest.mark.parametrize("name", ["gqa128", "mla", "asym", "gqa64"])
 def test_length_beyond_the_stated_maximum_is_flagged_on_every_kernel(H, name):
     """max_kv_len is the caller's bound on every length: an agent above it gets zeros and Q4KV_FLAG_BAD_LENGTH,
     whichever kernel serves the spec; the other agents are unaffected."""

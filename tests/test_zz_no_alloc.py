@@ -79,8 +79,8 @@ def _filled_cache(H, spec_args, lens, seed):
 
 
 def test_static_scratch_entry_across_kernels_and_growing_batches():
-    """Every call shares the one array, whatever kernel serves it: a latent-cache call (its own kernel), a d = 192 call
-    (the shape-agnostic kernel) and a 2-agent call each leave their partial records in it, and the call that follows --
+    """Every call shares the one array, whatever kernel serves it: a latent-cache call (its own kernel), a d_qk 192 call,
+    a d = 64 call (the shape-agnostic kernel) and a 2-agent call each leave their partial records in it, and the call that follows --
     a GQA batch of 10 agents x 8 KV heads, whose arrival counters reach further into the array than any of theirs --
     must still return what q4kv_decode_attention returns on a fresh zero-filled workspace, and what the oracle
     returns.  Outputs start as NaN so that a row nobody wrote is seen."""
@@ -94,6 +94,8 @@ def test_static_scratch_entry_across_kernels_and_growing_batches():
         ((1, 16, 1, 576, 512, True), [600, 70], 1.0 / math.sqrt(192), 21),
         (gqa, big_lens, 1.0 / math.sqrt(128), 22),
         ((1, 4, 4, 192, 128, False), [400, 300], 1.0 / math.sqrt(192), 23),
+        (gqa, big_lens, 1.0 / math.sqrt(128), 22),
+        ((1, 4, 2, 64, 64, False), [400, 3000], 0.125, 25),
         (gqa, big_lens, 1.0 / math.sqrt(128), 22),
         (gqa, [900, 40], 1.0 / math.sqrt(128), 24),
         (gqa, big_lens, 1.0 / math.sqrt(128), 22),
