@@ -10,11 +10,15 @@
 //     2050, shared memory for 2300 (operands 1570, tiles written 510, raw blocks 150) and the issue slots for 1700, so what
 //     matters is that all of them work at once: few, long hand-offs.  (Steps of 64 keys with the queries in tensor memory and
 //     two threads per row, which exchanged their maxima, took 2 x 3000 clocks.)  Measured on 8 agents x (8192 + 1024 tokens),
-//     32 / 8 heads: 5300 clocks per step; 1238 us per launch = 943 TFLOP/s in a run of a few launches, 1357 us = 861 TFLOP/s in a
-//     run of seconds, under the power cap (1616 us = 723 with the 64-key steps).  What is left is the chain of
-//     a tile's step -- scores 330 clocks after their product, exponentials 2 x 1500, value and score products 1700 -- of which
-//     the two tiles overlap a half.  Measured without gain: four softmax warps per row pair (16 in all), score buffers of 64
-//     keys issued two blocks ahead, an issuing warp per tile (the tiles then fall into step), scores fetched ahead.
+//     32 / 8 heads: 4150 clocks per step; 1156 us per launch = 1010 TFLOP/s in a run of a few launches, 1298 us = 900 TFLOP/s in a
+//     run of seconds, under the power cap.  Before, 5000 clocks, 1240 and 1357 us: the issuing warp was the bottleneck, with eight
+//     waits a step of which each cost 140 to 350 clocks although its phase was over; it has five now (see there), and a reference
+//     that moves by the sum of the probabilities instead of their maximum takes 70 of 230 instructions per 64 keys out of the
+//     softmax.  What is left is the chain of a tile's step: scores 250 clocks after their product, exponentials 2 x 1100, value
+//     and score products 1200.  Measured without gain: four softmax warps per row pair (16 in all), score buffers of 64 keys
+//     issued two blocks ahead, an issuing warp per tile (the tiles fall into step: 1399 us), scores fetched ahead (1196 for
+//     1188), the maximum before the exponentials (1351), 1/16, 1/8 or 1/4 of the exponentials as a polynomial on the FMA pipe
+//     (1169, 1182, 1222 for 1168), the issuing warp's group first in the CTA (1188 for 1169).
 //   * Eight "dequantize" warps turn each raw 64-key block into binary16 tiles K^ [64 keys][128 dims] and V^ [128 dims][64
 //     keys] in shared memory (four of each), in the core-matrix order a K-major tcgen05 operand wants: x^ = c * s + b in one
 //     binary16 fma per pair of codes (the code is made a binary16 integer by or-ing the masked nibble into the mantissa of
@@ -26,9 +30,8 @@
 //     memory.  The f32 accumulators fill the tensor memory (O 2 x 128, S 2 x 128); P_t overlays S_t.  At
 //     N = 128 a product whose A operand is in shared memory runs at the full rate (66 clocks per instruction).
 //   * Eight softmax warps, one thread per score row (a tensor-memory lane): mask, online softmax with a lazily updated
-//     reference maximum (the accumulator is rescaled only when the maximum has grown by more than 2^8), P_t as packed
-//     binary16, in halves of 64 keys, so that the first half's value product runs under the second half's exponentials.
-//     The two tiles alternate, so one tile's softmax overlaps the other tile's MMAs.
+//     reference (see kSumLimit), P_t as packed binary16, in halves of 64 keys, so that the first half's value product runs
+//     under the second half's exponentials.  The two tiles alternate, so one tile's softmax overlaps the other tile's MMAs.
 //   * One warp streams the raw blocks through a small ring with bulk asynchronous copies.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises
 // Q4KV_FLAG_INTERNAL, drains the tensor pipe and frees the tensor memory before the CTA returns.
@@ -42,8 +45,8 @@ using namespace tc;
 using namespace prefill;
 
 constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
-constexpr int kMmaWarp = kSoftmaxWarps + kDequantWarps, kLoadWarp = kMmaWarp + 1;
-constexpr int kThreads = (kMmaWarp + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps), ...
+constexpr int kLastGroup = kSoftmaxWarps + kDequantWarps, kLoadWarp = kLastGroup, kMmaWarp = kLastGroup + 3;
+constexpr int kThreads = (kLastGroup + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps), ...
 // ... launched with 96 registers per thread; the softmax warpgroups take 144, the others keep 64 (61440 in all)
 constexpr int kRegsSoftmax = 144, kRegsOther = 64;
 static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * 96, "");
@@ -52,6 +55,10 @@ constexpr int kRawSlots = 3;                             // raw 64-key blocks in
 constexpr int kChunkBytes = 4608;                        // d = 128: [Kc 2048 | Ksb 256 | Vc 2048 | Vsb 256]
 constexpr int kRawBytes = 2 * kChunkBytes;
 constexpr int kTileBytes = 64 * 128 * 2;                 // one binary16 tile
+// The reference of a row's exponentials moves when its probabilities of 64 keys add up to more than this (they are positive, so
+// none is above it, far below binary16's 65504).  The sum is needed anyway, a maximum beside it was 64 comparisons of a warp's
+// 230 instructions: 1233 -> 1188 us on the launch named above.
+constexpr float kSumLimit = 4096.f;
 constexpr uint32_t kColO = 0, kColS = 256;               // tensor-memory columns (+128 t; P inside S)
 
 struct UmmaParams {
@@ -138,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the new tokens were appended by the preceding kernel
   volatile int* abort_flag = &sm.abort_flag;
 
-  if (warp >= kMmaWarp) {
+  if (warp >= kLastGroup) {
     fewer_registers<kRegsOther>();
     if (warp == kLoadWarp) {
     // =============================== raw block loader ==========================================
@@ -175,9 +182,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     // The whole warp runs this code; one elected lane (always the same) issues the MMAs and the commits.
     if (n_step > 0) {
       constexpr uint32_t kIdesc = idesc_f16(128, 128);
+      const uint64_t qd0 = smem_desc(smem_u32(sm.qs[0]), 128, 2048), kd0 = smem_desc(smem_u32(sm.khat[0]), 128, 2048);
+      const uint64_t vd0 = smem_desc(smem_u32(sm.vhat[0]), 128, 1024);
       // one election for a whole product: an election per MMA costs more issue time than the MMA takes
       auto issue_qk = [&](int t, int s) {                // S_t = Q_t K^T over the tiles 2 s, 2 s + 1
-        const uint64_t qd = smem_desc(smem_u32(sm.qs[t]), 128, 2048), kd = smem_desc(smem_u32(sm.khat[2 * s]), 128, 2048);
+        const uint64_t qd = qd0 + (uint64_t)(t * (sizeof(sm.qs[0]) >> 4)), kd = kd0 + (uint64_t)(s * (2 * kTileBytes >> 4));
         if (elect_one()) {
 #pragma unroll                                           // rolled, every MMA waits for its own operand arithmetic: 2x slower
           for (int k = 0; k < 8; ++k) mma_f16_ss(tb + kColS + 128 * t, qd + 16 * k, kd + 16 * k, kIdesc, k > 0);
@@ -187,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         __syncwarp();
       };
       auto issue_pv = [&](int t, int s, int half, bool first) {    // O_t (+)= P_t V^ over half of the step's keys
-        const uint64_t vd = smem_desc(smem_u32(sm.vhat[2 * s + half]), 128, 1024);
+        const uint64_t vd = vd0 + (uint64_t)((2 * s + half) * (kTileBytes >> 4));
         if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
@@ -198,33 +207,31 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         __syncwarp();
       };
       auto wait = [&](uint64_t* bar, int use) {
-        const bool ok = mbar_wait(bar, (uint32_t)use, abort_flag);
+        const bool ok = mbar_spin(bar, (uint32_t)use, abort_flag);
         if (ok) fence_after_sync();
         return ok;
       };
-      auto wait_tiles = [&](uint64_t* bars, int j) {     // both tiles of step j
-        const int s = 2 * (j & 1);
-        return wait(&bars[s], j >> 1) && wait(&bars[s + 1], j >> 1);
-      };
-      bool ok = wait(&sm.q_ready, 0) && wait_tiles(sm.k_full, 0);
+      // A wait costs 150 to 300 clocks here even when its phase is over, and the tensor pipe idles meanwhile, so as few as can be:
+      // a dequantize warp arrives for its tiles in the order K0 V0 K1 V1 of a step's two blocks, so the second key tile of a step
+      // implies the first value tile of the step and everything of the step before it.
+      auto keys_of = [&](int j) { return wait(&sm.k_full[2 * (j & 1) + 1], j >> 1); };
+      bool ok = wait(&sm.q_ready, 0) && keys_of(0);
       if (ok) {
         issue_qk(0, 0);
         issue_qk(1, 0);
       }
       for (int j = 0; ok && j < n_step; ++j) {
+        const int s = j & 1;
 #pragma unroll 1
-        for (int t = 0; t < 2 && ok; ++t) {
-          ok = wait(&sm.p_full[t][0], j) && (t == 1 || wait(&sm.v_full[2 * (j & 1)], j >> 1));
+        for (int t = 0; t < 2; ++t) {
+          ok = wait(&sm.p_full[t][0], j);
           if (!ok) break;
-          issue_pv(t, j & 1, 0, j == 0);
-          ok = wait(&sm.p_full[t][1], j) && (t == 1 || wait(&sm.v_full[2 * (j & 1) + 1], j >> 1));
+          issue_pv(t, s, 0, j == 0);
+          if (t == 0) ok = j + 1 < n_step ? keys_of(j + 1) : wait(&sm.v_full[2 * s + 1], j >> 1);
+          ok = ok && wait(&sm.p_full[t][1], j);
           if (!ok) break;
-          issue_pv(t, j & 1, 1, false);
-          if (j + 1 < n_step) {
-            if (t == 0) ok = wait_tiles(sm.k_full, j + 1);
-            if (!ok) break;
-            issue_qk(t, (j + 1) & 1);
-          }
+          issue_pv(t, s, 1, false);
+          if (j + 1 < n_step) issue_qk(t, s ^ 1);
         }
       }
     }
@@ -337,33 +344,42 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
       fence_async_smem();
       mbar_arrive(&sm.q_ready);
     }
-    float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most kLazy
+    float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most 2^12
     for (int j = 0; j < n_step; ++j) {
       // one warp of the tile polls and the others sleep at a barrier: polling takes issue slots from the other tile's warps
       // (6 % of the kernel's time, like the sleeping waits of the dequantize warps)
-      if ((warp & 3) == 0) mbar_spin(&sm.s_full[t], (uint32_t)j, abort_flag);
+      if ((warp & 3) == 1 + t) mbar_spin(&sm.s_full[t], (uint32_t)j, abort_flag);
       asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
       fence_after_sync();
       const int pos0 = (st0 + j) * 128;
       const bool edge = pos0 + 127 > pq || (W > 0 && pos0 <= pq - W);
+      // column c of x is key pos0 + c0 + (c & ~7) + elem_of(c & 7); causal and window masks on edge steps only
+      auto mask = [&](uint32_t* x, int c0) {
+        const int last = pq - (pos0 + c0), first = W > 0 ? last - W + 1 : -1000;     // columns [first, last] count
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const int k = (c & ~7) + elem_of(c & 7);
+          if (k > last || k < first) x[c] = 0xff800000u;   // -inf
+        }
+      };
+      auto maximum = [&](const uint32_t* x) {
+        float m0 = __uint_as_float(x[0]), m1 = __uint_as_float(x[1]);
+#pragma unroll
+        for (int c = 2; c < 30; c += 4) {
+          m0 = fmaxf(m0, fmaxf(__uint_as_float(x[c]), __uint_as_float(x[c + 1])));
+          m1 = fmaxf(m1, fmaxf(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])));
+        }
+        return fmaxf(fmaxf(m0, __uint_as_float(x[30])), fmaxf(m1, __uint_as_float(x[31])));
+      };
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {             // 64 keys at a time: the first half's value product starts meanwhile
         const uint32_t half_addr = s_addr + 64 * half;
-        // column c is key pos0 + 64 half + (c & ~7) + elem_of(c & 7); causal and window masks on edge steps only
-        auto mask = [&](uint32_t* x, int c0) {
-          const int last = pq - (pos0 + 64 * half + c0), first = W > 0 ? last - W + 1 : -1000;     // columns [first, last] count
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const int k = (c & ~7) + elem_of(c & 7);
-            if (k > last || k < first) x[c] = 0xff800000u;   // -inf
-          }
-        };
-        // Probabilities against the current reference, and the maximum beside them (independent instruction streams); only
-        // when some row's maximum has outgrown its reference is the reference moved, the accumulator rescaled and the
-        // probabilities taken again.
+        const uint64_t kk = pair64(kappa, kappa);
+        float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+        uint64_t nn = pair64(neg_m, neg_m);
         uint32_t pr[32];
-        uint64_t sum0, sum1;
-        auto probabilities = [&](const uint32_t* x, uint32_t* p, uint64_t kk, uint64_t nn) {
+        uint64_t sum0 = 0ull, sum1 = 0ull;
+        auto probabilities = [&](const uint32_t* x, uint32_t* p) {
 #pragma unroll
           for (int c = 0; c < 16; c += 2) {
             const float2 a = unpair64(fma2(pair64(__uint_as_float(x[2 * c]), __uint_as_float(x[2 * c + 1])), kk, nn));
@@ -375,35 +391,28 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             p[c + 1] = f32x2_to_h2(b0, b1);
           }
         };
-        float cm0 = -INFINITY, cm1 = -INFINITY;
-        auto maximum = [&](const uint32_t* x) {
-#pragma unroll
-          for (int c = 0; c < 32; c += 4) {
-            cm0 = fmaxf(cm0, fmaxf(__uint_as_float(x[c]), __uint_as_float(x[c + 1])));
-            cm1 = fmaxf(cm1, fmaxf(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])));
-          }
-        };
-        uint32_t x[64];
-        float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
-        sum0 = sum1 = 0ull;
-        const uint64_t kk = pair64(kappa, kappa);
-        uint64_t nn = pair64(neg_m, neg_m);
-        tmem_ld32(half_addr, x);
-        wait_ld32(x);
-        tmem_ld32(half_addr + 32, x + 32);
-        if (edge) mask(x, 0);
-        probabilities(x, pr, kk, nn);
-        maximum(x);
-        wait_ld32(x + 32);
-        if (edge) mask(x + 32, 32);
-        probabilities(x + 32, pr + 16, kk, nn);
-        maximum(x + 32);
-        float cm = fmaxf(cm0, cm1);
-        if (cm != -INFINITY) cm *= kappa;                // kappa > 0
-        const float m_new = fmaxf(m_ref, cm);
-        const bool grow = m_new > m_ref + kLazy || (m_ref == -INFINITY && m_new != -INFINITY);
-        if (__any_sync(0xffffffffu, grow)) {
-          if (j + half > 0) {
+        // P overlays the half's first 32 columns of S, each part stored as soon as it is there (1168 -> 1156 us); the scores stay
+        // in registers until the half is final
+        uint32_t xa[32], xb[32];
+        tmem_ld32(half_addr, xa);
+        wait_ld32(xa);
+        tmem_ld32(half_addr + 32, xb);
+        if (edge) mask(xa, 64 * half);
+        probabilities(xa, pr);
+        wait_ld32(xb);
+        tmem_st16(half_addr, pr);
+        if (edge) mask(xb, 64 * half + 32);
+        probabilities(xb, pr + 16);
+        tmem_st16(half_addr + 16, pr + 16);
+        float2 u = unpair64(add2(sum0, sum1));
+        float s_half = u.x + u.y;
+        const bool outgrown = !(s_half <= kSumLimit) || m_ref == -INFINITY;
+        if (__any_sync(0xffffffffu, outgrown)) {         // rare: the row's reference moves and the half is taken again
+          float cm = fmaxf(maximum(xa), maximum(xb));
+          if (cm != -INFINITY) cm *= kappa;              // kappa > 0
+          const float m_new = fmaxf(m_ref, cm);
+          const bool grow = outgrown && m_new > m_ref;
+          if (j + half > 0 && __any_sync(0xffffffffu, grow)) {
             // rescale the accumulator row once the value products issued so far have landed (those of earlier steps have: the
             // scores were issued behind them)
             if (half == 1 && !__all_sync(0xffffffffu, mbar_wait(&sm.o_half[t], (uint32_t)j, abort_flag))) break;
@@ -424,12 +433,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
           neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
           nn = pair64(neg_m, neg_m);
           sum0 = sum1 = 0ull;
-          probabilities(x, pr, kk, nn);
-          probabilities(x + 32, pr + 16, kk, nn);
+          probabilities(xa, pr);
+          probabilities(xb, pr + 16);
+          tmem_st32(half_addr, pr);
+          u = unpair64(add2(sum0, sum1));
+          s_half = u.x + u.y;
         }
-        tmem_st32(half_addr, pr);                        // P overlays the half's first 32 columns of S
-        const float2 u = unpair64(add2(sum0, sum1));
-        l += u.x + u.y;
+        l += s_half;
         wait_st();
         fence_before_sync();
         __syncwarp();

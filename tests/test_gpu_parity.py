@@ -1086,6 +1086,45 @@ def test_append_on_both_sides_of_the_unit_split(H, spec_args, lens, sb_dtype):
     Pair(H, spec_args, lens, seed=61, sb_dtype=sb_dtype).fill().check_packed_equal()
 
 
+class SteepPair(Pair):
+    """Keys that quantize and round to binary16 without error (a code times a power of two that grows along the positions)."""
+
+    def kv(self, layer, agent, n):
+        k, v = super().kv(layer, agent, n)
+        c = synth.rng(self.seed, 500 + agent).integers(0, 16, k.shape).astype(np.float32)
+        c[..., 0::64], c[..., 1::64] = 0.0, 15.0             # every group spans its codes: scale 2^e, bias 0
+        e = np.arange(n) * 7 // max(n, 1) - 5
+        return synth.f32_to_bf16_bits(c * np.exp2(e).astype(np.float32)[:, None, None]), v
+
+
+@pytest.mark.parametrize("spec_args,prefix,chunks,window", [
+    ((1, 8, 2, 128, 128, False), [900, 0, 70], [100, 300, 1], 0),
+    ((1, 8, 2, 128, 128, False), [1500], [200], 300),
+    ((1, 4, 4, 128, 128, False), [6000], [40], 0),           # few tiles: the keys are split
+    ((1, 4, 2, 256, 256, False), [900, 0], [100, 300], 0),
+    ((1, 4, 4, 192, 128, False), [900, 0], [100, 300], 200),
+    ((1, 16, 1, 576, 512, True), [900, 0], [10, 300], 0),
+])
+def test_prefill_reference_moves_within_and_between_steps(H, spec_args, prefix, chunks, window):
+    """Scores whose spread grows to hundreds of binary orders along the keys, so that the reference of the exponentials has to
+    move by far more than its slack again and again.  The keys carry no rounding error, so what is left is one binary16
+    rounding of the probabilities and one of the values (2^-11 of the largest value each) and binary32 sums of scores below
+    2^9 binary orders (2^9 * 2^-22 of a probability)."""
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = SteepPair(H, spec_args, lens, seed=71).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = p.q(9, int(q_offs[-1]))
+    scale = 1.0 / math.sqrt(192 if spec_args[5] else spec_args[3])
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, window, f32(q), scale)
+    assert np.abs(lse_ref).max() > 60.0
+    out, lse = p.dc.prefill(0, lens, q_offs, window, q, scale)
+    m = max(float(np.abs(O.gather_dequant(p.opool, 0, p.tabs[a], 0, n, h)[1]).max())
+            for a, n in enumerate(lens) for h in range(spec_args[2]))
+    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= m * (2.0 ** -10 + 2.0 ** -12)
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("gain,outlier_frac", [(8.0, 0.0), (1.0, 0.01)])
 @pytest.mark.parametrize("prefix,chunks", [([0, 40], [70, 30]), ([300], [64])])
 @pytest.mark.parametrize("d", [128, 256, 192])
