@@ -25,10 +25,10 @@
 //
 // What bounds it: 2800 clocks per block, of which 2050 are the expansion with both products (the tensor instructions of a
 // scheduler's two warps alone take 1150), 250 the softmax, 500 the barrier and the wait for the block; and per launch about
-// 6 us of prologue, first block, record and merge.  Eight warps because the queries' fragments, the accumulators and two
+// 5 us of prologue, first block, record and merge.  Eight warps because the queries' fragments, the accumulators and two
 // words in flight need the registers: sixteen warps of 128 registers (four per group of octets) took 22.1 us where this
-// took 20.2 (4 agents x 16384 tokens with the merge; 19.4 since the merge takes its records by ordinary loads), two groups of
-// four warps with separate chunks 20.9.  The first form, with an expanded key tile read through ldmatrix for the scores and
+// took 20.2 (4 agents x 16384 tokens with the merge; 18.3 with the present merge), two groups of four warps with separate
+// chunks 20.9.  The first form, with an expanded key tile read through ldmatrix for the scores and
 // three barriers per block, took 21.3 (23.8 with bfloat16 scales, now 19.9); 32 agents x 8192 tokens 110 us, now 60.
 #include <algorithm>
 
@@ -52,7 +52,6 @@ constexpr int kOctetBytes = (kDv / 8) * 128;             // 8192: one key octet 
 constexpr int kTileBytes = 8 * kOctetBytes;              // 65536
 constexpr int kGroupStride = (kD / 8) * 128;             // 9216: bytes between 8-row groups of a [rows][576] tile
 constexpr int kStages = 2, kRawSlots = 3;
-constexpr int kRecStride = kDv + 2;                      // acc[512], m, l
 constexpr float kLazy = 8.f;
 
 using MlaParams = MlaDecodeParams;
@@ -138,11 +137,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   const int b_lo = lo >> 6, b_hi = (n + 63) >> 6;        // 64-key blocks of the attended range
   const int b0 = min(b_hi, b_lo + split * P.blocks_per_split);
   const int n_iter = min(b_hi, b0 + P.blocks_per_split) - b0;
-  float* rec = P.records + ((size_t)a * P.n_splits + split) * kHeads * kRecStride;
+  float* rec = P.records + ((size_t)a * P.n_splits + split) * kHeads * kDv;
+  float2* rec_ml = mla_record_pairs(P.records, P.n_agents, P.n_splits) + (size_t)a * kHeads * P.n_splits + split;   // + head * n_splits
   if (n_iter <= 0) {
     // nothing to attend in this share: an empty record (the preceding kernels may still be reading the records)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (threadIdx.x < kHeads) { rec[threadIdx.x * kRecStride + kDv] = -INFINITY; rec[threadIdx.x * kRecStride + kDv + 1] = 0.f; }
+    if (threadIdx.x < kHeads) rec_ml[threadIdx.x * P.n_splits] = make_float2(-INFINITY, 0.f);
     if (bad_len && split == 0 && threadIdx.x == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
     return;
   }
@@ -155,10 +155,14 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
     fence_async_smem();
   }
   __syncthreads();
-  if (threadIdx.x < 2 && threadIdx.x < n_iter)           // the first two block-table entries, fetched towards the SM meanwhile
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(P.tables + (size_t)a * P.max_blocks + ((2 * (b0 + (int)threadIdx.x)) >> 3)) : "memory");
-  // While the preceding kernel drains, L2 is asked for the agent's query rows (a prefetch returns nothing to the kernel,
-  // so it may precede the wait; in a decode step they are what the preceding kernels have just written).
+  // While the preceding kernel drains, L2 is asked for the first raw blocks (block tables are inputs) and the agent's query rows (a
+  // prefetch returns nothing to the kernel, so it may precede the wait, and L2 is where the preceding kernels' writes land).
+  if (threadIdx.x < kRawSlots && threadIdx.x < n_iter) {
+    const int c = 2 * (b0 + (int)threadIdx.x), blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
+    if (blk >= 0 && blk < P.n_blocks)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(head_block(P.pool, y, P.layer, blk, 0) + (size_t)(c & 7) * kChunkBytes),
+                   "r"((uint32_t)kRawBytes) : "memory");
+  }
   {
     const int lines = n_rep * kD * 2 / 128;                // 128-byte lines of the agent's n_rep query rows
     const uint16_t* qrows = P.q + (size_t)a * y.Hq * kD;
@@ -192,26 +196,13 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
   }
 
   // Update-and-fetch: the CTA whose share ends with the agent's last block quantizes the row of position n - 1
-  // (one warp, while the first copies are in flight) and, once that block has landed, patches it in shared memory
-  // and stores the same words to the pool.  No other CTA reads that block.
+  // (a warp per group, while the first copies are in flight; one warp for all of it was 3.4 us on this CTA's path) and, once
+  // that block has landed, patches it in shared memory and stores the same words to the pool.  No other CTA reads that block.
   const bool has_new = P.k_new != nullptr && b0 + n_iter == b_hi;
-  if (has_new && warp == 0) {
-#pragma unroll 1
-    for (int base = 0; base < kD / 8; base += 32) {
-      const int w = base + lane;
-      float x[8];
-      if (w < kD / 8) {
-        load_eight_bf16(P.k_new, (size_t)a * kD + 8 * w, x);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = 0.f;
-      }
-      const QuantOut qo = quantize_eight(x, kBf);             // eight lanes per group of 64; 72 words = 9 whole groups
-      if (w < kD / 8) {
-        sm.new_words[w] = qo.word;
-        if ((w & 7) == 0) sm.new_sb[w >> 3] = *reinterpret_cast<const uint32_t*>(&qo.sb);
-      }
-    }
+  if (has_new) {
+    for (int grp = warp; grp < kD / 64; grp += kComputeWarps)
+      quantize_row_group(*reinterpret_cast<const uint32_t*>(P.k_new + (size_t)a * kD + 64 * grp + 2 * lane), kBf, lane, sm.new_words + 8 * grp,
+                         sm.new_sb + grp);
   }
 
   // =============================== compute warps ================================================
@@ -471,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
       const float got = __shfl_xor_sync(0xffffffffu, (tid & 1) ? o[c][2 * e] : o[c][2 * e + 1], 1);
       float2 v = (tid & 1) ? make_float2(got, o[c][2 * e + 1]) : make_float2(o[c][2 * e], got);
       if (spoiled) v = make_float2(0.f, 0.f);
-      *reinterpret_cast<float2*>(rec + (g + 8 * e) * kRecStride + d_lane + 8 * c) = v;      // 514 floats a head: 8-byte aligned
+      *reinterpret_cast<float2*>(rec + (g + 8 * e) * kDv + d_lane + 8 * c) = v;
     }
   }
   if (warp == 0 && tid == 0) {
@@ -481,93 +472,80 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_kernel(const __grid_co
       float lsum = 0.f;
 #pragma unroll
       for (int w = 0; w < kComputeWarps; ++w) lsum += sm.wsum[w][h];
-      rec[h * kRecStride + kDv] = spoiled ? -INFINITY : m_ref[e];
-      rec[h * kRecStride + kDv + 1] = spoiled ? -1.f : lsum;               // negative: poisoned
+      rec_ml[h * P.n_splits] = make_float2(spoiled ? -INFINITY : m_ref[e], spoiled ? -1.f : lsum);         // negative: poisoned
     }
   }
 }
 
 // grid: (16 heads, n_agents, 128 / kLanes slices of the value dims), 512 threads; combines the records of one (agent, head)
-// for 4 kLanes output dims.  The records sit in L2 a microsecond away, so nothing here is a chain of dependent loads: thread
-// s fetches (m, l) of split s, the block agrees on the weights, while the 512 / kLanes groups of threads each take every
-// so-many-th split with their loads issued together before the weights are known, and the groups' sums meet in registers
-// (groups of one warp) and shared memory.  How narrow the slices are depends on the count of splits: with four of them
-// sixteen groups would leave most threads idle (and make four times the CTAs), with 148 each group would walk nine.
+// for 4 kLanes output dims.  The records sit in L2 a microsecond away, so nothing here is a chain of dependent loads: the
+// 512 / kLanes groups of threads each take every so-many-th split, with its m, while every warp fetches all (m, l) pairs for
+// itself -- one round trip --, works out the maximum and the sum without the others, and the groups' sums meet in registers
+// (groups of one warp) and shared memory, at the kernel's only barrier.  (With the weights agreed on by the block, behind four
+// barriers, and the pairs beside the records, 32 KB apart: 4 agents x 16384 tokens 19.2 us for kernel and merge, now 18.3;
+// 3 x 700 10.8, now 8.7.  Every warp for itself with the pairs beside the records: 20.0.)  How narrow the slices are depends on the count of
+// splits: with four of them sixteen groups would leave most threads idle (and make four times the CTAs), with 148 each group
+// would walk nine.
 // The pointers carry no __restrict__: the records are written by the preceding kernel while this one is already resident, and
 // read-only loads are not defined for such data.
 constexpr int kMergeThreads = 512, kMaxSplits = 512;
 template <int kLanes>
 __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_splits, const float* records, void* out, int out_dtype,
                                                                   float* lse) {
-  __shared__ float s_w[kMaxSplits];                      // weight of each split (0: empty)
-  __shared__ float s_red[kMergeThreads / 32][2];
   constexpr int kGroups = kMergeThreads / kLanes;
   constexpr int kRows = kLanes < 32 ? kMergeThreads / 32 : kGroups;         // sums that meet in shared memory
   __shared__ float4 s_acc[kRows - 1][kLanes];
-  __shared__ float s_ml[2];
   const int h = blockIdx.x, a = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the records come from the preceding kernel
   if (h >= Hq) return;
-  const float* rec = records + ((size_t)a * n_splits * kHeads + h) * kRecStride;
-  const size_t step = (size_t)kHeads * kRecStride;       // between the splits of one head
-  // The record loads of the first kGroups * kPre splits do not wait for the weights: they are issued first and overlap the
-  // round trip of the (m, l) loads (an empty split's data is whatever an earlier call left there; it is dropped below).
+  const float* rec = records + ((size_t)a * n_splits * kHeads + h) * kDv;
+  const float2* pairs = mla_record_pairs(const_cast<float*>(records), gridDim.y, n_splits) + ((size_t)a * kHeads + h) * n_splits;
+  const size_t step = (size_t)kHeads * kDv;              // between the splits of one head
+  // The loads of the first kGroups * kPre splits are issued before anything is known (an empty split's data is whatever an
+  // earlier call left there; it is dropped below).
   constexpr int kPre = 4;
   const int grp = tid / kLanes, gl = tid % kLanes, d = 4 * (kLanes * blockIdx.z + gl);   // 4 consecutive dims per thread
+  auto fetch = [&](int sp) { return *reinterpret_cast<const float4*>(rec + sp * step + d); };
   float4 pre[kPre];
+  float pre_m[kPre];
 #pragma unroll
   for (int u = 0; u < kPre; ++u) {
     const int sp = grp + kGroups * u;
     pre[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (sp < n_splits) {
-      const float2 lo2 = *reinterpret_cast<const float2*>(rec + sp * step + d);       // records are 8-byte aligned
-      const float2 hi2 = *reinterpret_cast<const float2*>(rec + sp * step + d + 2);
-      pre[u] = make_float4(lo2.x, lo2.y, hi2.x, hi2.y);
+    pre_m[u] = -INFINITY;
+    if (sp < n_splits) { pre[u] = fetch(sp); pre_m[u] = pairs[sp].x; }
+  }
+  float M = -INFINITY, L = 0.f;
+  bool bad = false;
+  for (int base = 0; base < n_splits; base += 64) {      // two pairs per lane at a time
+    float2 ml[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int sp = base + 32 * k + lane;
+      ml[k] = sp < n_splits ? pairs[sp] : make_float2(-INFINITY, 0.f);
     }
+    float m = fmaxf(ml[0].x, ml[1].x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    m = fmaxf(m, M);
+    float s = (ml[0].x == -INFINITY ? 0.f : fast_exp2(ml[0].x - m) * ml[0].y) + (ml[1].x == -INFINITY ? 0.f : fast_exp2(ml[1].x - m) * ml[1].y);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    L = (M == -INFINITY ? 0.f : L * fast_exp2(M - m)) + s;
+    M = m;
+    bad |= ml[0].y < 0.f || ml[1].y < 0.f;
   }
-  float ms = -INFINITY, ls = 0.f;
-  if (tid < n_splits) { ms = rec[tid * step + kDv]; ls = rec[tid * step + kDv + 1]; }
-  float M = ms, bad = ls < 0.f ? 1.f : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o)); bad = fmaxf(bad, __shfl_xor_sync(0xffffffffu, bad, o)); }
-  if (lane == 0) { s_red[warp][0] = M; s_red[warp][1] = bad; }
-  __syncthreads();
-  M = s_red[0][0]; bad = s_red[0][1];
-#pragma unroll
-  for (int w = 1; w < kMergeThreads / 32; ++w) { M = fmaxf(M, s_red[w][0]); bad = fmaxf(bad, s_red[w][1]); }
-  const float wgt = ms == -INFINITY ? 0.f : exp2f(ms - M);
-  if (tid < n_splits) s_w[tid] = wgt;
-  float L = wgt * ls;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-  __syncthreads();                                       // s_red is read by everyone before it is reused
-  if (lane == 0) s_red[warp][0] = L;
-  __syncthreads();
-  if (tid == 0) {
-    float t = 0.f;
-    for (int w = 0; w < kMergeThreads / 32; ++w) t += s_red[w][0];
-    s_ml[0] = M; s_ml[1] = bad > 0.f ? 0.f : t;          // a poisoned split zeroes the row
-  }
+  if (__any_sync(0xffffffffu, bad)) L = 0.f;             // a poisoned split zeroes the row
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](float m, const float4& v) {
+    if (m == -INFINITY) return;                          // an empty split's record holds no data
+    const float w = fast_exp2(m - M);
+    acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y); acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
+  };
 #pragma unroll
-  for (int u = 0; u < kPre; ++u) {
-    const int sp = grp + kGroups * u;
-    const float wu = sp < n_splits ? s_w[sp] : 0.f;
-    if (wu > 0.f) {                                      // an empty split's record holds no data
-      acc.x = fmaf(wu, pre[u].x, acc.x); acc.y = fmaf(wu, pre[u].y, acc.y);
-      acc.z = fmaf(wu, pre[u].z, acc.z); acc.w = fmaf(wu, pre[u].w, acc.w);
-    }
-  }
-  for (int sp = grp + kGroups * kPre; sp < n_splits; sp += kGroups) {
-    const float wu = s_w[sp];
-    if (wu > 0.f) {
-      const float2 lo2 = *reinterpret_cast<const float2*>(rec + sp * step + d);
-      const float2 hi2 = *reinterpret_cast<const float2*>(rec + sp * step + d + 2);
-      acc.x = fmaf(wu, lo2.x, acc.x); acc.y = fmaf(wu, lo2.y, acc.y);
-      acc.z = fmaf(wu, hi2.x, acc.z); acc.w = fmaf(wu, hi2.y, acc.w);
-    }
-  }
+  for (int u = 0; u < kPre; ++u) add(pre_m[u], pre[u]);
+  for (int sp = grp + kGroups * kPre; sp < n_splits; sp += kGroups) add(pairs[sp].x, fetch(sp));
   if (kLanes < 32) {
 #pragma unroll
     for (int o = kLanes; o < 32; o *= 2) {
@@ -579,8 +557,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
   if (row > 0 && (kLanes >= 32 || lane < kLanes)) s_acc[row - 1][gl] = acc;
   __syncthreads();
   if (tid >= kLanes) return;
-  const float Lsum = s_ml[1];
-  const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
+  const float inv = L > 0.f ? 1.f / L : 0.f;
 #pragma unroll
   for (int g = 0; g < kRows - 1; ++g) { const float4 o = s_acc[g][gl]; acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w; }
   acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
@@ -594,7 +571,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
   } else {
     *reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + out_index + d) = acc;
   }
-  if (tid == 0 && blockIdx.z == 0 && lse) lse[(size_t)a * Hq + h] = Lsum > 0.f ? (s_ml[0] + log2f(Lsum)) / kLog2e : -INFINITY;
+  if (tid == 0 && blockIdx.z == 0 && lse) lse[(size_t)a * Hq + h] = L > 0.f ? (M + log2f(L)) / kLog2e : -INFINITY;
 }
 
 struct MlaPlan { int n_splits, blocks_per_split; };
@@ -625,7 +602,7 @@ size_t decode_mla_workspace_bytes(const Layout& y, int n_agents, int max_kv_len)
   (void)y;
   // the split count depends on the window through the span: room for the most that any span gets
   const int blocks = (max_kv_len + 63) / 64 + 1, most = (sm_count() + n_agents - 1) / n_agents;
-  return (size_t)n_agents * std::min(std::min(blocks, most), kMaxSplits) * kHeads * kRecStride * sizeof(float);
+  return (size_t)n_agents * std::min(std::min(blocks, most), kMaxSplits) * kHeads * (kDv + 2) * sizeof(float);
 }
 
 cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, int layer, const q4kv_batch& b,
@@ -669,10 +646,11 @@ cudaError_t launch_decode_mla(const Layout& y, const void* pool, int n_blocks, i
   }
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t mcfg = {};
-  // 4, 8, 16 or 32 groups of threads share the splits, so that a thread's loads are few and all in flight together.  Measured,
-  // merge and kernel, on 128 / 64 / 32 / 16 / 8 lanes: 4 splits x 32 agents 59.9 / 63.6 / 69.0 / 80 / 90 us, 17 x 8 14.5 / 12.5 /
-  // 14.1 / 17.4 / 19.9, 37 x 4 24.2 / 20.2 / 19.4 / 21.1 / 22.6, 148 x 1 40 / 24.5 / 21.9 / 21.0 / 22.6.
-  const int lanes = plan.n_splits <= 8 ? 128 : plan.n_splits <= 24 ? 64 : plan.n_splits <= 64 ? 32 : 16;
+  // 4, 8, 16 or 32 groups of threads share the splits, so that a thread's loads are few and all in flight together, but no more
+  // CTAs than needed.  Measured, merge and kernel, on 128 / 64 / 32 / 16 lanes: 4 splits x 32 agents 58.9 / 61.3 / 64.0 / 74.0 us,
+  // 9 x 16 19.7 / 20.7 / 22.2 / 27.2, 14 x 10 23.1 / 23.6 / 24.4 / 27.7, 18 x 8 20.5 / 19.6 / 20.7 / 23.1, 24 x 6 25.2 / 24.6 / 25.0 / 27.1,
+  // 37 x 4 20.2 / 19.1 / 18.8 / 19.5, 49 x 3 18.1 / 17.4 / 16.9 / 17.5, 74 x 2 16.4 / 16.4 / 15.9 / 14.9, 148 x 1 26.1 / 23.0 / 22.0 / 20.0.
+  const int lanes = plan.n_splits <= 14 ? 128 : plan.n_splits <= 30 ? 64 : plan.n_splits <= 64 ? 32 : 16;
   void (*merge)(int, int, const float*, void*, int, float*) =
       lanes == 128 ? merge_mla_kernel<128> : lanes == 64 ? merge_mla_kernel<64> : lanes == 32 ? merge_mla_kernel<32> : merge_mla_kernel<16>;
   mcfg.gridDim = dim3(kHeads, b.n_agents, kDv / 4 / lanes);

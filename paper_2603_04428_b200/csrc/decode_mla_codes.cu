@@ -53,7 +53,6 @@ constexpr int kThreads = kComputeWarps * 32;            // 256
 constexpr int kChunkBytes = 32 * (kD / 2 + 4 * kG);      // 10368: [Kc 9216 | Ksb 1152]
 constexpr int kRawBytes = 2 * kChunkBytes;               // one 64-key block
 constexpr int kRawSlots = 4;
-constexpr int kRecStride = kDv + 2;                      // acc[512], m, l
 constexpr float kLazy = 3.f;                             // probabilities stay below 2^3: p * scale fits binary16 for any binary16 scale
 constexpr uint32_t kMaskLo = 0x000F000Fu, kMaskHi = 0x00F000F0u;
 
@@ -118,11 +117,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_codes_kernel(const __g
   const int b_lo = lo >> 6, b_hi = (n + 63) >> 6;        // 64-key blocks of the attended range
   const int b0 = min(b_hi, b_lo + split * P.blocks_per_split);
   const int n_iter = min(b_hi, b0 + P.blocks_per_split) - b0;
-  float* rec = P.records + ((size_t)a * P.n_splits + split) * kHeads * kRecStride;
+  float* rec = P.records + ((size_t)a * P.n_splits + split) * kHeads * kDv;
+  float2* rec_ml = mla_record_pairs(P.records, P.n_agents, P.n_splits) + (size_t)a * kHeads * P.n_splits + split;   // + head * n_splits
   if (n_iter <= 0) {
     // nothing to attend in this share: an empty record (the preceding kernels may still be reading the records)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (threadIdx.x < kHeads) { rec[threadIdx.x * kRecStride + kDv] = -INFINITY; rec[threadIdx.x * kRecStride + kDv + 1] = 0.f; }
+    if (threadIdx.x < kHeads) rec_ml[threadIdx.x * P.n_splits] = make_float2(-INFINITY, 0.f);
     if (bad_len && split == 0 && threadIdx.x == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
     return;
   }
@@ -164,26 +164,13 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_codes_kernel(const __g
   }
 
   // Update-and-fetch: the CTA whose share ends with the agent's last block quantizes the row of position n - 1
-  // (one warp, while the first copies are in flight) and, once that block has landed, patches it in shared memory
+  // (a warp per group, while the first copies are in flight) and, once that block has landed, patches it in shared memory
   // and stores the same words to the pool.  No other CTA reads that block.
   const bool has_new = P.k_new != nullptr && b0 + n_iter == b_hi;
-  if (has_new && warp == 0) {
-#pragma unroll 1
-    for (int base = 0; base < kD / 8; base += 32) {
-      const int w = base + lane;
-      float x[8];
-      if (w < kD / 8) {
-        load_eight_bf16(P.k_new, (size_t)a * kD + 8 * w, x);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = 0.f;
-      }
-      const QuantOut qo = quantize_eight(x, kBf);        // eight lanes per group of 64; 72 words = 9 whole groups
-      if (w < kD / 8) {
-        sm.new_words[w] = qo.word;
-        if ((w & 7) == 0) sm.new_sb[w >> 3] = qo.sb;
-      }
-    }
+  if (has_new) {
+    for (int grp = warp; grp < kD / 64; grp += kThreads / 32)
+      quantize_row_group(*reinterpret_cast<const uint32_t*>(P.k_new + (size_t)a * kD + 64 * grp + 2 * lane), kBf, lane, sm.new_words + 8 * grp,
+                         sm.new_sb + grp);
   }
 
   const int tq = threadIdx.x;                            // 0..255
@@ -467,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_codes_kernel(const __g
       v.x = fmaf(o[0][nt][cr], 16777216.f, bias); v.y = fmaf(o[1][nt][cr], 1048576.f, bias);   // 2^24; 2^24 / 16
       v.z = fmaf(o[2][nt][cr], 16777216.f, bias); v.w = fmaf(o[3][nt][cr], 1048576.f, bias);
       if (spoiled) v = make_float4(0.f, 0.f, 0.f, 0.f);
-      float* at = rec + head * kRecStride + d_base;      // records are 8-byte aligned (514 floats per head)
+      float* at = rec + head * kDv + d_base;
       *reinterpret_cast<float2*>(at) = make_float2(v.x, v.y);
       *reinterpret_cast<float2*>(at + 2) = make_float2(v.z, v.w);
     }
@@ -478,8 +465,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_mla_codes_kernel(const __g
       float lsum = 0.f;
 #pragma unroll
       for (int w = 0; w < kComputeWarps; ++w) lsum += sm.wsum[w][h];
-      rec[h * kRecStride + kDv] = spoiled ? -INFINITY : m_ref[e];
-      rec[h * kRecStride + kDv + 1] = spoiled ? -1.f : lsum;               // negative: poisoned
+      rec_ml[h * P.n_splits] = make_float2(spoiled ? -INFINITY : m_ref[e], spoiled ? -1.f : lsum);         // negative: poisoned
     }
   }
 }

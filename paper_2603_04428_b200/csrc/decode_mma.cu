@@ -509,23 +509,6 @@ __device__ __forceinline__ void stage_query_row(uint4 (*qfrag)[32], float (*qsum
 // launch, in the pool for the following ones.  Every chunk is held by exactly one warp of the grid, so nobody else reads
 // or writes these words during the launch.  (One warp doing all of it, eight elements per lane, was 3.5 us on the
 // critical path of every launch: 500 instructions that run once per launch and come from far away.)
-template <int G, int H>
-__device__ __forceinline__ void quantize_new_group(Smem<G, H>& sm, uint32_t two, int grp, bool bf16, int lane) {
-  const float x0 = __uint_as_float(two << 16), x1 = __uint_as_float(two & 0xffff0000u);
-  float mn = fminf(x0, x1), mx = fmaxf(x0, x1);
-  asm("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(mn));
-  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(mx));
-  const GroupScale gs = group_scale(mn, mx, bf16);
-  uint32_t w = 0u;
-  if (gs.sf != 0.f) {
-    const float inv = __frcp_rn(gs.sf);
-    w = (quantize_code(x0, gs, inv) | (quantize_code(x1, gs, inv) << 4)) << (8 * (lane & 3));
-  }
-  w |= __shfl_xor_sync(0xffffffffu, w, 1);
-  w |= __shfl_xor_sync(0xffffffffu, w, 2);
-  if ((lane & 3) == 0) sm.new_words[8 * grp + (lane >> 2)] = w;
-  if (lane == 0) sm.new_sb[grp] = gs.hs | (gs.hb << 16);
-}
 // The value codes are token-packed: one nibble of each of the row's d_v words is replaced.
 template <int G, int H>
 __device__ __noinline__ void patch_new_row(const Smem<G, H>& sm, uint8_t* keys, uint8_t* values, uint8_t* gchunk, int tau, int lane) {
@@ -1132,7 +1115,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
     if (warp >= 4 && newest) {
 #pragma unroll
       for (int r = 0; r < kNewRounds; ++r)
-        if (warp - 4 + kNewWarps * r < G + Gv) quantize_new_group<G, H>(sm, nv[r], warp - 4 + kNewWarps * r, kBf, lane);
+        if (const int grp = warp - 4 + kNewWarps * r; grp < G + Gv) quantize_row_group(nv[r], kBf, lane, sm.new_words + 8 * grp, sm.new_sb + grp);
     }
     __syncthreads();
     const float* const qs0 = sm.qsum[hcol[0]];

@@ -218,9 +218,13 @@ struct MlaDecodeParams {
   const uint16_t* k_new;      // bf16 [n_agents][576]: the row at position kv_len - 1, quantized and stored by this launch; or null
   float scale_log2;
   int n_splits, blocks_per_split;
-  float* records;             // [n_agents][n_splits][16][514]: acc[512] (unnormalised, relative to m), m, l
+  float* records;             // acc [n_agents][n_splits][16][512] (unnormalised, relative to m), then the pairs (m, l)
   int32_t* flags;
 };
+// The pairs (m, l) of the records, [n_agents][16][n_splits]: the merge reads all of a head at once.
+__host__ __device__ inline float2* mla_record_pairs(float* records, int n_agents, int n_splits) {
+  return reinterpret_cast<float2*>(records + (size_t)n_agents * n_splits * 16 * 512);
+}
 cudaError_t launch_mla_codes_kernel(const MlaDecodeParams& P, cudaStream_t st);   // grid (n_splits, n_agents)
 
 }  // namespace q4kv

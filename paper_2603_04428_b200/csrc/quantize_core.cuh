@@ -60,6 +60,24 @@ __device__ inline uint32_t quantize_code(float x, const GroupScale& gs, float in
   return (uint32_t)min(max(__float2int_rn(q), 0), 15);
 }
 
+// One group of 64 elements by one warp, two elements per lane (`two`: their bf16 bits): eight words of codes and the pair.
+__device__ __forceinline__ void quantize_row_group(uint32_t two, bool bf16, int lane, uint32_t* words, uint32_t* sb) {
+  const float x0 = __uint_as_float(two << 16), x1 = __uint_as_float(two & 0xffff0000u);
+  float mn = fminf(x0, x1), mx = fmaxf(x0, x1);
+  asm("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(mn));
+  asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(mx));
+  const GroupScale gs = group_scale(mn, mx, bf16);
+  uint32_t w = 0u;
+  if (gs.sf != 0.f) {
+    const float inv = __frcp_rn(gs.sf);
+    w = (quantize_code(x0, gs, inv) | (quantize_code(x1, gs, inv) << 4)) << (8 * (lane & 3));
+  }
+  w |= __shfl_xor_sync(0xffffffffu, w, 1);
+  w |= __shfl_xor_sync(0xffffffffu, w, 2);
+  if ((lane & 3) == 0) words[lane >> 2] = w;
+  if (lane == 0) *sb = gs.hs | (gs.hb << 16);
+}
+
 // A (scale, bias) pair of the cache as two binary32 numbers.
 template <bool kBf16>
 __device__ __forceinline__ float2 sb_to_f2(uint32_t u) {

@@ -555,6 +555,11 @@ def test_latent_decode_shares_and_merges(H, n_heads, lens, sb_dtype):
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("length", [750, 1000, 1800, 2000, 3800, 4090])     # 13, 17, 29, 33, 61 and 65 shares
+def test_latent_merge_on_both_sides_of_its_widths(H, length):
+    test_latent_decode_shares_and_merges(H, 16, [length], 0)
+
+
 @pytest.mark.parametrize("window", [0, 150])
 def test_decode_latent_cache_at_a_sharp_scale_takes_the_exact_kernel(H, window):
     """scale^2 * d_qk > 4 on the V-aliasing cache: routed to the kernel that keeps the values exact."""
