@@ -60,6 +60,7 @@ constexpr int kCtasPerSm = 2;
 // warps per CTA: eight of 128 registers, or at d = 256, where the accumulators alone are 64, six of 168
 __host__ __device__ constexpr int warps_of(int G) { return G == 4 ? 6 : 8; }
 constexpr int kWholeSlack = 12;                        // see find_range
+constexpr int kOnePerSm = 21;                          // see launch_decode_mma
 constexpr float kMargin = 0.35f;                       // see chunk_values
 constexpr int kMaxRecords = 32;                        // a pair is cut over about this many CTAs at most (the merge reads them all)
 constexpr uint32_t kSpinLimit = 1u << 22;              // bounded mbarrier waits (each try blocks a while in hardware)
@@ -222,8 +223,9 @@ __device__ __noinline__ void find_agent(const Par& P, RangeStart& rs) {
   }
 }
 
+// more_rounds: 0, 1, or 2 for 1 where the pairs are few (see below)
 template <class Par>
-__device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_t nw) {
+__device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_t nw, int more_rounds) {
   const int lane = threadIdx.x & 31;
   const int n_agents = P.n_agents, Hkv = P.Hkv;
   RangeStart rs;
@@ -280,12 +282,19 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
 #pragma unroll 1
     for (int a = 0; a < n_agents; ++a) total += parts_of(__shfl_sync(0xffffffffu, nc, a), size, inv);
     const unsigned fits = __ballot_sync(0xffffffffu, total * Hkv <= (int)most && lane <= kWholeSlack);
-    if (fits) {
-      const int l = __ffs(fits) - 1;
-      const int best = size0 + l;
-      rs.n_ctas = __shfl_sync(0xffffffffu, total, l) * Hkv;
+    // A pair whole in one CTA needs no records and no ticket (2 us).  That is worth a round of chunks, one per warp (0.9 us at d = 128;
+    // not where a round is two chunks' work: d = 256, and eight heads but for few pairs), and more where there are many.  Measured, us a
+    // launch, cut and whole: 8 KV heads, one agent x 350 tokens 6.4 / 5.6, x 480 6.5 / 5.8, x 600 (two rounds more) 6.4 / 7.2; 32 agents x
+    // 4096 41.3 / 38.3; d = 256, one x 350 9.0 / 9.9, 20 agents in a window of 1024 27.0 / 26.2; eight heads, 16 x 700 15.0 / 15.9.
+    const int l = fits ? __ffs(fits) - 1 : 0, pairs = n_agents * Hkv;
+    const int rounds = (size0 + l + (int)nw - 1) / (int)nw;
+    const int extra = more_rounds == 1 || 4 * pairs <= (int)most ? min(more_rounds, 1) : 0;
+    const bool uncut = pairs <= (int)most && (nc_max + (int)nw - 1) / (int)nw <= rounds + extra + ((rounds * 37) >> 8);
+    if (fits || uncut) {
+      const int best = uncut ? nc_max : size0 + l;
+      rs.n_ctas = uncut ? pairs : __shfl_sync(0xffffffffu, total, l) * Hkv;
       if (cta >= rs.n_ctas) return rs;
-      const int m = parts_of(nc, best, __shfl_sync(0xffffffffu, inv, l));
+      const int m = uncut ? (lane < n_agents ? 1 : 0) : parts_of(nc, best, __shfl_sync(0xffffffffu, inv, l));
       int inc = m * Hkv;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -998,7 +1007,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   // ---- this CTA's unit range and its first two segments: one warp, the others set up shared memory (lengths and block
   // tables are inputs that no kernel writes) ----
   if (warp == 0) {
-    const RangeStart rs = find_range(P, cta, gridDim.x, NW);
+    const RangeStart rs = find_range(P, cta, gridDim.x, NW, G == 4 ? 0 : H == 8 ? 2 : 1);
     if (lane == 0) {
       if (rs.any_bad && cta == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
       sm.range = rs;
@@ -1115,7 +1124,8 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
     if (warp >= 4 && newest) {
 #pragma unroll
       for (int r = 0; r < kNewRounds; ++r)
-        if (const int grp = warp - 4 + kNewWarps * r; grp < G + Gv) quantize_row_group(nv[r], kBf, lane, sm.new_words + 8 * grp, sm.new_sb + grp);
+        if (warp - 4 + kNewWarps * r < G + Gv)
+          quantize_row_group(nv[r], kBf, lane, sm.new_words + 8 * (warp - 4 + kNewWarps * r), sm.new_sb + warp - 4 + kNewWarps * r);
     }
     __syncthreads();
     const float* const qs0 = sm.qsum[hcol[0]];
@@ -1344,12 +1354,14 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents * layer_count;
   P.n_real = b.n_agents; P.layer_count = layer_count;
   P.sets = head_sets(y); P.Hkv = y.Hkv * P.sets; P.n_rep = y.n_rep / P.sets;
-  long long units = 0;
+  long long units = 0, wanted = 0;
   for (int i = 0; i < kMaxLayersPerCall; ++i) {
     P.windows[i] = i < layer_count ? windows[i] : 0;
     if (i < layer_count) {
       const int span = (windows[i] > 0 && windows[i] + 32 < max_kv_len) ? windows[i] + 32 : max_kv_len;
-      units += (long long)b.n_agents * P.Hkv * ((span + 31) / 32 + 1);
+      const int chunks = (span + 31) / 32, nw = warps_of(y.G);
+      units += (long long)b.n_agents * P.Hkv * chunks;
+      wanted += (long long)b.n_agents * P.Hkv * ((chunks + nw - 1) / nw);       // a chunk per warp, and no CTA with two pairs
     }
   }
   P.max_blocks = b.max_blocks; P.len_cap = max_kv_len; P.tables = b.block_tables; P.kv_lens = kv_lens;
@@ -1358,9 +1370,15 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   P.out = out; P.out_dtype = out_dtype; P.lse = lse; P.flags = flags;
   P.k_new = (const uint16_t*)k_new; P.v_new = (const uint16_t*)v_new;
   P.q_offs = q_offs;
-  const long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
-  const int nw = warps_of(y.G);
-  const long long wanted = (units + nw - 1) / nw;        // a chunk per warp at least
+  // No more CTAs than can be of use: one that finds nothing to do costs the next launch a microsecond, because its CTAs come in as
+  // this one's leave.  No fewer than pairs, which one CTA would take in turn: a launch on contexts of 30 tokens took 25.5 us with
+  // a CTA per eight chunks, 4.3 with one per pair, on 100 tokens 7.2 and 4.3, at d = 256 13.8 and 6.7.
+  // One CTA per SM where that leaves a warp at most 2.6 chunks: the next launch's CTAs then sit beside this one's with their work
+  // laid out and their first chunks in L2.  Us a launch with two and with one: 2 agents x 4096 tokens 9.8 / 9.2, 3 x 4096 11.0 /
+  // 10.3, 6 x 1500 9.7 / 8.8, 13 x 600 9.8 / 8.2; 5 x 4096 (4.4 chunks) 11.7 / 12.4; not at d = 256 (10 in a window of 1024: 15.9 /
+  // 20.9) and with eight heads (6 x 1000: 11.8 / 12.8), whose chunks are twice the work.
+  long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
+  if (y.G == 2 && P.n_rep <= 4 && (long long)P.n_agents * P.Hkv <= sm_count() && units <= (long long)kOnePerSm * sm_count()) slots = sm_count();
   const int grid = (int)(wanted < slots ? (wanted < 1 ? 1 : wanted) : slots);
   if (y.G == 2) return P.n_rep > 4 ? launch_gh<2, 8>(P, grid, st) : launch_gh<2, 4>(P, grid, st);
   return y.G == 3 ? launch_gh<3, 4>(P, grid, st) : launch_gh<4, 4>(P, grid, st);

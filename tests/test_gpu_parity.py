@@ -517,6 +517,38 @@ def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
 
 
 @pytest.mark.parametrize("spec_args,lens,window", [
+    ((1, 8, 2, 128, 128, False), [1], 0),                    # one chunk per pair, a CTA each
+    ((1, 8, 2, 128, 128, False), [32, 33, 0, 7], 0),
+    ((1, 8, 2, 128, 128, False), [255], 0),                  # eight chunks: a round of one CTA
+    ((1, 8, 2, 128, 128, False), [257, 1], 0),               # nine to sixteen: two rounds, whole
+    ((1, 8, 2, 128, 128, False), [512, 100], 0),
+    ((1, 8, 2, 128, 128, False), [513, 769], 0),             # three rounds: cut
+    ((1, 32, 8, 128, 128, False), [3000, 2900], 0),          # one CTA per SM
+    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(18)], 0),       # 144 pairs: whole, one per SM
+    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(20)], 0),       # 160: two per SM
+    ((1, 4, 2, 128, 128, False), [100 + 7 * i for i in range(34)], 0),         # more agents than lanes: equal ranges
+    ((1, 8, 2, 128, 128, False), [900, 300, 64], 200),       # a window
+    ((1, 16, 2, 128, 128, False), [256, 257, 480], 0),       # eight heads, few pairs
+    ((1, 64, 8, 128, 128, False), [300 + 9 * i for i in range(12)], 0),        # many
+    ((1, 4, 2, 256, 256, False), [31], 0),
+    ((1, 4, 2, 256, 256, False), [192, 193, 350], 0),        # six warps: one round and two
+    ((1, 2, 2, 256, 256, False), [3000, 70], 1024),
+    ((1, 4, 4, 192, 128, False), [1, 255, 257, 520], 0),
+])
+def test_decode_launch_sizes(H, spec_args, lens, window):
+    """Sizes at which the launch chooses its CTAs: a pair whole in one, cut, one or two CTAs per SM."""
+    p = Pair(H, spec_args, lens, seed=43).fill()
+    q = p.q(7, len(lens))
+    scale = 1.0 / math.sqrt(spec_args[3])
+    ref, lse_ref = O.decode_attention(p.opool, 0, p.tabs, lens, window, f32(q), scale)
+    for _ in range(2):                                       # the arrival counters are left as they were found
+        out, lse = p.dc.decode(0, lens, window, q, scale, max_kv_len=max(lens))
+        assert_attention_close(out.cpu().numpy(), ref)
+        assert_lse_close(lse.cpu().numpy(), lse_ref)
+    assert p.dc.read_flags() == 0
+
+
+@pytest.mark.parametrize("spec_args,lens,window", [
     ((1, 10, 2, 128, 128, False), [700, 0, 33], 0),          # five query heads per KV head: three columns stay empty
     ((1, 16, 2, 128, 128, False), [1, 31, 32, 257, 3000], 0),
     ((1, 16, 2, 128, 128, False), [1, 31, 32, 257, 3000], 100),
