@@ -232,7 +232,7 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
   rs.any_bad = false;
   rs.agent = -1;
   rs.agent_start = 0;
-  uint32_t cum = 0, inc0 = 0, cnt0 = 0;
+  uint32_t cum = 0, cnt0 = 0;
   rs.r.n = 0; rs.r.lo = 0; rs.r.cf = 0; rs.r.nc = 0;
 #pragma unroll 1
   for (int base = 0; base < n_agents; base += 32) {
@@ -241,14 +241,8 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
     bool bad = false;
     if (a < n_agents) { rs.r = agent_range(P, a, bad); cnt = (uint32_t)(rs.r.nc * Hkv); }
     rs.any_bad |= __any_sync(0xffffffffu, bad);
-    uint32_t inc = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += v;
-    }
-    if (base == 0) { inc0 = inc; cnt0 = cnt; }
-    cum += __shfl_sync(0xffffffffu, inc, 31);
+    cum += __reduce_add_sync(0xffffffffu, cnt);
+    cnt0 = cnt;
   }
   rs.U = cum;
   // at least a chunk for every warp of a CTA, and not more CTAs on a pair than the merge takes quickly
@@ -266,12 +260,12 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
     // 14.4 / 11.8 / 11.8 / 11.8 / 11.8; 13 agents x 1024..16384 23.6 / 23.6 / 21.0 / 21.0 / 21.0; 13 x 4096 23.7 / 23.7 / 23.7 /
     // 24.1 / 24.1; 32 x 4096 41.4 / 41.4 / 41.4 / 38.4 / 38.4; d = 256, 10 x 1024..16384 39.3 / 39.3 / 35.8 / 35.9 / 35.8.
     const int nc = lane < n_agents ? rs.r.nc : 0;
-    int nc_max = nc;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nc_max = max(nc_max, __shfl_xor_sync(0xffffffffu, nc_max, o));
-    const int size0 = max(max((int)nw, (int)((cum + most - 1) / most)), (nc_max + kMaxRecords - 1) / kMaxRecords);
+    // (No integer divisions: they and their like were 1.2 us of every CTA's start, which the late ones of a launch pay.  The
+    // quotients of floats that size0 starts from may be off by one; every CTA finds the same.)
+    const int nc_max = __reduce_max_sync(0xffffffffu, nc);
+    const int size0 = max(max((int)nw, (int)ceilf(__fdividef((float)cum, (float)most))), (nc_max + kMaxRecords - 1) / kMaxRecords);
     const int size = size0 + lane;
-    const float inv = 1.f / (float)size;
+    const float inv = __fdividef(1.f, (float)size);
     auto parts_of = [](int n, int sz, float rcp) {       // ceil(n / sz)
       int q = (int)((float)n * rcp);
       q += q * sz < n;
@@ -279,7 +273,7 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
       return q;
     };
     int total = 0;
-#pragma unroll 1
+#pragma unroll 4
     for (int a = 0; a < n_agents; ++a) total += parts_of(__shfl_sync(0xffffffffu, nc, a), size, inv);
     const unsigned fits = __ballot_sync(0xffffffffu, total * Hkv <= (int)most && lane <= kWholeSlack);
     // A pair whole in one CTA needs no records and no ticket (2 us).  That is worth a round of chunks, one per warp (0.9 us at d = 128;
@@ -305,13 +299,21 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
       rs.agent = a;
       rs.splits = __shfl_sync(0xffffffffu, m, a);
       const int at = cta - (__shfl_sync(0xffffffffu, inc, a) - rs.splits * Hkv), n = __shfl_sync(0xffffffffu, nc, a);
-      rs.pair = at / rs.splits;
+      const float per = __fdividef(1.f, (float)rs.splits);
+      auto quotient = [&](int x) {                       // below 2^24 the float quotient is off by one at most
+        if (x >= 1 << 24) return x / rs.splits;
+        int q = (int)((float)x * per);
+        q -= q * rs.splits > x;
+        return q + ((q + 1) * rs.splits <= x);
+      };
+      rs.pair = quotient(at);
       rs.split = at - rs.pair * rs.splits;
       rs.agent_start = 0;                                // units count from the pair's first chunk here
       rs.r.n = __shfl_sync(0xffffffffu, rs.r.n, a); rs.r.lo = __shfl_sync(0xffffffffu, rs.r.lo, a);
       rs.r.cf = __shfl_sync(0xffffffffu, rs.r.cf, a); rs.r.nc = n;
-      rs.u_begin = (uint32_t)n * (uint32_t)rs.split / (uint32_t)rs.splits;
-      rs.u_end = (uint32_t)n * (uint32_t)(rs.split + 1) / (uint32_t)rs.splits;
+      const int each = quotient(n), more = n - each * rs.splits;         // the first `more` parts hold a chunk more
+      rs.u_begin = (uint32_t)(rs.split * each + min(rs.split, more));
+      rs.u_end = (uint32_t)(rs.u_begin + each + (rs.split < more ? 1 : 0));
       return rs;
     }
   }
@@ -321,6 +323,12 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
   rs.u_end = rs.part.begin(cta + 1);
   const uint32_t want = rs.u_begin;
   if (n_agents <= 32) {
+    uint32_t inc0 = cnt0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc0, o);
+      if (lane >= o) inc0 += v;
+    }
     const unsigned bal = __ballot_sync(0xffffffffu, inc0 > want);
     const int l = __ffs(bal) - 1;
     rs.agent = l;
@@ -960,7 +968,7 @@ __device__ __forceinline__ uint32_t chunk_offset(const DecodeParams& P, const Se
   const int blk = P.tables[(size_t)s.ar * P.max_blocks + (c >> 3)];
   if (blk < 0 || blk >= P.n_blocks) { raise_flag(P.flags, Q4KV_FLAG_BAD_BLOCK); return kOffBad; }
   return (uint32_t)(((uint64_t)s.li * P.y.layer_bytes + (uint64_t)blk * P.y.block_bytes +
-                     (uint64_t)(s.hk / P.sets) * P.y.head_block_bytes + (uint64_t)(c & 7) * chunk_bytes) >> 4);
+                     (uint64_t)(P.sets == 1 ? s.hk : s.hk / P.sets) * P.y.head_block_bytes + (uint64_t)(c & 7) * chunk_bytes) >> 4);
 }
 template <class Par>
 __device__ __noinline__ uint32_t batch_offsets(const Par& P, const RangeStart& rs, int nw, int warp, int b, uint32_t chunk_bytes) {
