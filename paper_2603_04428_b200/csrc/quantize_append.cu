@@ -16,6 +16,7 @@ namespace q4kv {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kItemBytes = 8 * 4 * 128;                  // eight positions, four groups (see the bulk kernel)
 
 struct UnitInfo { int agent, first, cnt, row0, block; };
 
@@ -157,19 +158,21 @@ quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_a
 
 // ---------------------------------------------------------------------------------------------
 // Bulk form (a prefill phase: many new tokens per agent).  kWpc warps own one (32-token chunk, KV head) unit and walk its
-// items -- (octet of eight positions, pass of four groups: K groups first, then V groups) -- with the loads of the
-// next item in flight while the current one is quantized.  Within an item a lane owns one of the eight positions and
-// one 64-element group: it loads its 64 elements as eight 16-byte words, takes minimum and maximum with packed bf16
+// items -- four (octet of eight positions, group) pairs, K groups first, then V groups -- with the next item's rows on their way
+// into shared memory while the current one is quantized.  Within an item a lane owns one of the eight positions and
+// one 64-element group: it reads its 64 elements as eight 16-byte words, takes minimum and maximum with packed bf16
 // instructions (no cross-lane step at all), and quantizes them two at a time (packed binary32; see quantize_code for why the
 // codes equal those of the fixed sequence bit for bit).  V words
 // are first exchanged between the eight lanes of a group (an 8 x 8 transposition of words by twelve shuffles), which leaves
 // in each lane the 8 positions x 8 elements block of nibbles that an in-register transposition turns into eight token-packed
 // words.  The chunk is assembled in shared memory and stored as whole 16-byte pieces; a chunk that the phase fills only in
 // part (an unaligned start or end) starts from its present bytes.
-// Bound by instruction issue and, with the sixteen warps an SM has room for, by the latency of the loads: 14.4 instructions an
-// element (18.7 before ties were left to the corrected quotient), issued at 0.46 a clock.  Measured at d = 128, 8 KV heads:
-// 8 x 1024 tokens 20.4 -> 16.3 us, 8 x 4096 69 -> 56 us.  kWpc = 1 where the units fill the GPU; 4 for smaller phases, whose
-// time is one unit's chain of items: 5 x 64 tokens 12.8 -> 4.4 us, latent cache 8 x 1024 tokens 29 -> 10 us.
+// Bound by instruction issue (about 14 instructions an element) with the sixteen warps an SM has room for.  Measured, each lane
+// loading its own rows (32 lines per load) -> rows copied whole lines at a time: d = 128, 8 KV heads, 8 x 1024 tokens 16.6 -> 15.8 us,
+// 8 x 4096 55.8 -> 48.7; d = 256 97.7 -> 84.4; 192 / 128, where an item was four groups of one octet, 16 KV heads, 8 x 1024 53.1 ->
+// 37.4; latent cache 8 x 4096 21.2 -> 18.3.  Three CTAs per SM of 80 registers: 21.8 us on the first.  kWpc = 1 where the units fill the
+// GPU and two CTAs' chunks fit an SM; 4 otherwise and for smaller phases, whose time is one unit's chain of items: 5 x 64 tokens 12.8 ->
+// 4.7 us.
 // ---------------------------------------------------------------------------------------------
 __device__ inline void transpose_nibbles_8x8_regs(uint32_t (&r)[8]) {
   // rows = registers, columns = nibbles: three rounds of block swaps
@@ -241,7 +244,8 @@ __device__ inline void find_chunk_unit(int u, int n_agents, int max_blocks, int 
   if (!found && lane == 0) out->agent = -1;
 }
 
-template <int kWpc>
+// kFour: four groups per token, so that an item is one octet (fewer instructions for the common shape)
+template <int kWpc, bool kFour>
 __global__ void __launch_bounds__(kThreads, 2)
 quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                             const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
@@ -279,43 +283,60 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
     unit_sync();
   }
   const int n_groups = y.G + (y.alias ? 0 : y.Gv);
-  const int n_pass = (n_groups + 3) >> 2;
-  const int n_items = (o_last - o_first + 1) * n_pass;
+  const int n_items = ((o_last - o_first + 1) * n_groups + 3) >> 2;
   constexpr float kMagic = 12582912.0f;                  // 1.5 * 2^23: q + kMagic holds q rounded to nearest even in its low bits
   constexpr uint32_t kMagicSum = 0x4B400000u * (1u + 16u + 256u);           // what eight of them add to a word (e > 2: shifted out)
 
-  // item t: octet o_first + t / n_pass of the chunk, groups 4 * (t % n_pass) .. + 3
-  auto load_item = [&](int t, uint4 (&raw)[8]) {
-    const int o = o_first + t / n_pass, pass = t - (t / n_pass) * n_pass;
-    const int first = max(lo, c0 + 8 * o), cnt = min(hi, c0 + 8 * o + 8) - first;
-    const int i = s - (first & 7);
-    const int gq = pass * 4 + gq0;
-    const bool is_v = gq >= y.G;
-    const int gi = is_v ? gq - y.G : gq;
-    if (gq < n_groups && i >= 0 && i < cnt) {
-      const size_t row = (size_t)(un.r0 + (first - un.p) + i) * y.Hkv + hk;
-      const uint16_t* src = is_v ? v_new + row * y.Dv + 64 * gi : k_new + row * y.D + 64 * gi;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) raw[j] = __ldca(reinterpret_cast<const uint4*>(src) + j);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) raw[j] = make_uint4(0u, 0u, 0u, 0u);
-    }
+  // Item t: the (octet, group) pairs 4 t .. 4 t + 3 of the chunk, groups fastest, K before V; lanes 8 i .. 8 i + 7 have pair 4 t + i.  (A
+  // pass of four groups per octet left three quarters of every second item of the five groups at 192 / 128 without work, and of every
+  // third of the latent cache's nine.)  The 32 rows of 128 bytes (pair, position) come by asynchronous copies, a position at a time --
+  // the lanes of a copy then cover whole lines, where a lane that loads its own row asks for a piece of 32 lines --, while the item
+  // before is quantized; 16-byte piece j of a row of position s lies at j ^ s, so that neither the copies nor the reads of a row
+  // per lane conflict.  Rows that do not exist are zeros.
+  uint8_t* const ring = stage_all + (size_t)(kThreads / 32 / kWpc) * y.chunk_bytes + (size_t)warp * kItemBytes;
+  const float per_group = __fdividef(1.f, (float)n_groups);
+  struct Pair { int o, gq; bool has; };
+  auto pair_of = [&](int t) {                            // at most 4 x 24 pairs: the float quotient is exact
+    if (kFour) return Pair{o_first + t, gq0, true};
+    const int v = 4 * t + gq0, oo = (int)(((float)v + 0.5f) * per_group);
+    return Pair{o_first + oo, v - oo * n_groups, o_first + oo <= o_last};
   };
-
-  uint4 raw[8], nxt[8];
-  if (sub < n_items) load_item(sub, raw);
+  auto copy_item = [&](int t) {
+    const Pair pr = pair_of(t);
+    const int first = max(lo, c0 + 8 * pr.o), cnt = min(hi, c0 + 8 * pr.o + 8) - first, k0 = first & 7;
+    const int gq = pr.gq;
+    const bool is_v = gq >= y.G, has = pr.has;
+    const uint16_t* const rows = is_v ? v_new + 64 * (gq - y.G) : k_new + 64 * gq;
+    const size_t width = is_v ? y.Dv : y.D;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(ring + gq0 * 128);
+    const size_t row0 = (size_t)(un.r0 + (first - un.p)) * y.Hkv + hk;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {                        // position k, piece s of this lane's group
+      const bool real = has && k >= k0 && k < k0 + cnt;
+      const uint16_t* src = real ? rows + (row0 + (size_t)(k - k0) * y.Hkv) * width + 8 * s : k_new;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)(k * 512 + ((s ^ k) << 4))), "l"(src), "r"(real ? 16 : 0)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (sub < n_items) copy_item(sub);
   for (int t = sub; t < n_items; t += kWpc) {
-    if (t + kWpc < n_items) load_item(t + kWpc, nxt);
-    const int o = o_first + t / n_pass, pass = t - (t / n_pass) * n_pass;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    uint4 raw[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) raw[j] = *reinterpret_cast<const uint4*>(ring + s * 512 + gq0 * 128 + ((j ^ s) << 4));
+    __syncwarp();                                        // the whole warp has its rows: the next item's may come
+    if (t + kWpc < n_items) copy_item(t + kWpc);
+    const Pair pr = pair_of(t);
+    const int o = pr.o, gq = pr.gq;
     const int first = max(lo, c0 + 8 * o), cnt = min(hi, c0 + 8 * o + 8) - first;
     const int k0 = first & 7;
     const int i = s - k0;                                // this lane's token of the octet
     const bool tok = i >= 0 && i < cnt;
     const int tau = 8 * o + s;                           // chunk token of this lane's position
     const uint32_t nib_mask = cnt == 8 ? 0xFFFFFFFFu : (((1u << (4 * cnt)) - 1u) << (4 * k0));
-    const int gq = pass * 4 + gq0;
-    const bool has = gq < n_groups;
+    const bool has = pr.has;
     const bool is_v = has && gq >= y.G;
     const int gi = is_v ? gq - y.G : gq;
     const bool active = has && tok;
@@ -372,7 +393,7 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
         *reinterpret_cast<uint2*>(kc + k_word_offset(tau, 8 * gi + w, y.G)) = make_uint2(cw[w], cw[4 + w]);
       reinterpret_cast<uint32_t*>(chunk + y.off_ksb)[sb_offset(tau, gi, y.G)] = sb;
     }
-    if (pass * 4 + 3 >= y.G) {                           // not a pass of K groups only (warp-uniform)
+    if (kFour ? !y.alias : __any_sync(0xffffffffu, is_v)) {             // not K groups only
       if (active && is_v) reinterpret_cast<uint32_t*>(chunk + y.off_vsb)[sb_offset(tau, gi, y.Gv)] = sb;
       // 8 x 8 transposition of words between the eight lanes of a group: afterwards lane s holds, in cw[w], word s
       // (elements 8s .. 8s+7 of the group) of position w
@@ -396,14 +417,15 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
         }
       }
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) raw[j] = nxt[j];
   }
   unit_sync();
   for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(gchunk)[q] = reinterpret_cast<const uint4*>(chunk)[q];
 }
 
-template <int kWpc>
+constexpr size_t kBulkSmem = 112 * 1024;                 // two CTAs per SM
+size_t bulk_smem(const Layout& y, int wpc) { return (size_t)(kThreads / 32 / wpc) * y.chunk_bytes + (size_t)(kThreads / 32) * kItemBytes; }
+
+template <int kWpc, bool kFour>
 cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer, const q4kv_batch& b, const int32_t* pos,
                         const int32_t* new_offs, int chunk_units, const void* k_new, const void* v_new, int32_t* flags,
                         cudaStream_t st) {
@@ -411,14 +433,14 @@ cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((warps + kThreads / 32 - 1) / (kThreads / 32)));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = (size_t)(kThreads / 32 / kWpc) * y.chunk_bytes;
+  cfg.dynamicSmemBytes = bulk_smem(y, kWpc);
   cfg.stream = st;
   static bool configured[64] = {};     // the attribute is per function and device: set it once for each
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(quantize_append_bulk_kernel<kWpc>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+    e = cudaFuncSetAttribute(quantize_append_bulk_kernel<kWpc, kFour>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
@@ -427,7 +449,7 @@ cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel<kWpc>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
+  return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel<kWpc, kFour>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
                             b.block_tables, pos, new_offs, (const uint16_t*)k_new, (const uint16_t*)v_new, flags, chunk_units);
 }
 
@@ -456,13 +478,14 @@ cudaError_t launch_quantize_append(const Layout& y, void* pool, int n_blocks, in
                                    const void* k_new, const void* v_new, int32_t* flags, cudaStream_t st) {
   if (total_new <= 0 || b.n_agents <= 0) return cudaSuccess;
   const int units = total_new / 8 + 2 * b.n_agents;        // >= sum over agents of ceil((pos%8+n)/8)
-  if (total_new >= 8 * b.n_agents && (size_t)(kThreads / 32) * y.chunk_bytes <= 112 * 1024) {
+  if (total_new >= 8 * b.n_agents && (size_t)(kThreads / 32) * y.chunk_bytes <= kBulkSmem) {
     // a phase of many tokens per agent: one warp per (32-token chunk, KV head)
     const int chunk_units = total_new / 32 + 2 * b.n_agents;   // >= sum over agents of the chunks their new range touches
     // four warps per unit while one warp each would leave half of the resident warps (sixteen per SM) without work
-    if ((long long)chunk_units * y.Hkv < 8ll * sm_count())
-      return launch_bulk<4>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
-    return launch_bulk<1>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
+    const bool four = (long long)chunk_units * y.Hkv < 8ll * sm_count() || bulk_smem(y, 1) > kBulkSmem;
+    const auto launch = y.G + (y.alias ? 0 : y.Gv) == 4 ? (four ? launch_bulk<4, true> : launch_bulk<1, true>)
+                                                        : (four ? launch_bulk<4, false> : launch_bulk<1, false>);
+    return launch(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
   }
   return launch_m<1>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, units, k_new, v_new, flags, st);
 }

@@ -1162,6 +1162,13 @@ def test_prefill_reference_moves_within_and_between_steps(H, spec_args, prefix, 
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("name", list(SPECS))                # 2, 4, 5, 8 and 9 groups per token
+@pytest.mark.parametrize("chunks", [[13, 40, 9, 100], [8, 33, 31, 65, 300], [256]])
+def test_bulk_append_of_unaligned_phases(H, name, chunks):
+    """Phases that start and end inside an octet and inside a chunk, whatever the count of groups an item packs."""
+    Pair(H, SPECS[name], [sum(chunks), sum(chunks) - 3], seed=73).fill(chunks).check_packed_equal()
+
+
 @pytest.mark.parametrize("gain,outlier_frac", [(8.0, 0.0), (1.0, 0.01)])
 @pytest.mark.parametrize("prefix,chunks", [([0, 40], [70, 30]), ([300], [64])])
 @pytest.mark.parametrize("d", [128, 256, 192])
