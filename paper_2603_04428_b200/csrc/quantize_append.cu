@@ -7,6 +7,8 @@
 // Eight consecutive lanes own one 64-element group (eight elements each) and reduce
 // min/max with three shuffles.  Every arithmetic step is a single rounded binary32
 // operation in the documented order so that codes/scales/biases are reproducible.
+#include <algorithm>
+
 #include "f32x2.cuh"
 #include "q4kv_layout.cuh"
 #include "quantize_core.cuh"
@@ -65,94 +67,97 @@ __device__ inline void find_unit(int u, int n_agents, int max_blocks, int n_bloc
   if (!found && lane == 0) out->agent = -1;
 }
 
-// grid: (ceil(unit upper bound / M), Hkv); a CTA handles M consecutive octets.  Dynamic smem: M * 8 * Dv bytes of V
-// codes (one byte per code).  M = 1 is what is launched: several octets per CTA, and one octet for all KV heads per
-// CTA, both measured slower on a 8 x 1024-token phase (37 us -> 63 us for the latter): more registers per thread and
-// less parallelism cost more than the shared prologue saves.  Phases of many tokens per agent take the bulk kernel
-// further down; this kernel serves the appends of a few tokens per agent (3.4 us for one token of each of 5 agents).
-template <int M>
+// grid: (unit upper bound, Hkv); a CTA handles one octet.  Dynamic smem: 8 * Dv bytes of V codes (one byte per code).  Phases of
+// many tokens per agent take the bulk kernel further down; this kernel serves the appends of a few tokens per agent.  Its time is a
+// chain of latencies -- the predecessor's end, the rows, the quantizer, the value words --, so the value words that are patched are
+// fetched beside the rows, and only the tokens there are get threads.  One token of each of 12 agents, us a launch: 8 KV heads
+// 2.9 -> 2.2, d = 256 3.7 -> 2.0, 16 heads at 192 / 128 4.6 -> 2.3, latent cache 2.7 -> 1.8 (before: a thread for every word that eight tokens
+// would have, two divisions each, the value words fetched at the end, a grid for two octets more per agent).  Several octets per CTA, and
+// one octet for all KV heads per CTA, were slower on phases: 37 -> 63 us for the latter on 8 x 1024 tokens.
+constexpr int kMaxDv = 512;
 __global__ void __launch_bounds__(kThreads)
 quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                        const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
                        const int32_t* __restrict__ new_offs, const void* k_new, const void* v_new, int32_t* flags) {
-  extern __shared__ uint8_t vcodes_all[];   // [M][8][Dv]
-  __shared__ UnitInfo s_unit[M];
+  extern __shared__ uint8_t vcodes[];       // [8][Dv]
+  __shared__ UnitInfo s_unit;
   // (k_new, v_new carry no __restrict__: the preceding kernel may write them while this one is resident, and read-only loads are
   // not defined for such data.)
   // let the next kernel of the stream start its prologue; the unit is found from the lengths and block tables (inputs
   // that no kernel writes) while the preceding kernels drain, and the wait comes before the new rows and the pool
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x < 32) {
-    for (int r = 0; r < M; ++r)
-      find_unit(blockIdx.x * M + r, n_agents, max_blocks, n_blocks, tables, pos, new_offs, flags,
-                blockIdx.x == 0 && blockIdx.y == 0 && r == 0, &s_unit[r]);
-  }
+  if (threadIdx.x < 32)
+    find_unit(blockIdx.x, n_agents, max_blocks, n_blocks, tables, pos, new_offs, flags, blockIdx.x == 0 && blockIdx.y == 0, &s_unit);
   __syncthreads();
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const UnitInfo un = s_unit;
   const int hk = blockIdx.y;
-  const int kw = y.D / 8, vw = y.alias ? 0 : y.Dv / 8;
-  const int n_items = 8 * (kw + vw);
-
-  // ---- K and V rows in one sweep: items (tensor, token i, word w), eight lanes per group.  K words and
+  const int kw = y.D / 8, per = kw + (y.alias ? 0 : y.Dv / 8);           // words of a token: K, then V
+  const int slot0 = un.first & 255;                     // the octet lies inside one 32-token chunk
+  uint8_t* const chunk = head_block(pool, y, layer, un.agent < 0 ? 0 : un.block, hk) + (size_t)(slot0 >> 5) * y.chunk_bytes;
+  uint32_t* const vc = reinterpret_cast<uint32_t*>(chunk + y.off_vc);
+  // while the preceding kernel drains, L2 is asked for the first token's rows and the value words (a prefetch returns nothing)
+  if (un.agent >= 0) {
+    const size_t row = (size_t)un.row0 * y.Hkv + hk;
+    const int lines_k = y.D / 64, lines = y.alias ? lines_k : lines_k + y.Dv / 64 + y.Dv / 8;
+    for (int i = threadIdx.x; i < lines; i += kThreads) {
+      const void* at = i < lines_k ? (const void*)((const uint16_t*)k_new + row * y.D + 64 * i)
+                     : i < lines_k + y.Dv / 64 ? (const void*)((const uint16_t*)v_new + row * y.Dv + 64 * (i - lines_k))
+                                               : (const void*)(vc + 32 * (i - lines_k - y.Dv / 64));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(at));
+    }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (un.agent < 0) return;                             // uniform over the CTA
+  uint32_t old[kMaxDv / kThreads] = {};
+  if (!y.alias && un.cnt < 8) {
+#pragma unroll
+    for (int r = 0; r < kMaxDv / kThreads; ++r) {
+      const int d = threadIdx.x + kThreads * r;
+      if (d < y.Dv) old[r] = vc[v_word_offset((slot0 & 31) >> 3, d)];
+    }
+  }
+  // ---- K and V rows in one sweep: items (token i, word w), eight lanes per group.  K words and
   // scale/bias pairs go straight to the pool; V codes go to shared memory as bytes for the transposition. ----
+  const int n_items = un.cnt * per;
   for (int base = 0; base < n_items; base += kThreads) {
     const int idx = base + threadIdx.x;
-    const bool is_v = idx >= 8 * kw;
-    const int j = is_v ? idx - 8 * kw : idx, ww = is_v ? vw : kw;
-    const int i = j / (ww > 0 ? ww : 1), w = j % (ww > 0 ? ww : 1);
-    float x[M][8];
-    bool live[M];
+    const bool live = idx < n_items;
+    const int i = un.cnt == 1 ? 0 : idx / per, ww = idx - i * per;       // (eight lanes of a group: per is a multiple of eight)
+    const bool is_v = ww >= kw;
+    const int w = is_v ? ww - kw : ww;
+    float x[8];
+    if (live) {
+      const size_t row = (size_t)(un.row0 + i) * y.Hkv + hk;
+      if (is_v) load_eight_bf16(v_new, row * y.Dv + 8 * w, x);
+      else load_eight_bf16(k_new, row * y.D + 8 * w, x);
+    } else {
 #pragma unroll
-    for (int r = 0; r < M; ++r) {
-      const UnitInfo un = s_unit[r];
-      live[r] = un.agent >= 0 && idx < n_items && i < un.cnt;
-      if (live[r]) {
-        if (is_v) load_eight_bf16(v_new, ((size_t)(un.row0 + i) * y.Hkv + hk) * y.Dv + 8 * w, x[r]);
-        else load_eight_bf16(k_new, ((size_t)(un.row0 + i) * y.Hkv + hk) * y.D + 8 * w, x[r]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[r][e] = 0.f;
-      }
+      for (int e = 0; e < 8; ++e) x[e] = 0.f;
     }
+    const QuantOut o = quantize_eight(x, y.sb_bf16 != 0);
+    if (!live) continue;
+    const int tau = (slot0 & 31) + i;
+    if (is_v) {
 #pragma unroll
-    for (int r = 0; r < M; ++r) {
-      const QuantOut o = quantize_eight(x[r], y.sb_bf16 != 0);
-      if (!live[r]) continue;
-      const UnitInfo un = s_unit[r];
-      const int slot0 = un.first & 255;                 // the octet lies inside one 32-token chunk
-      uint8_t* chunk = head_block(pool, y, layer, un.block, hk) + (size_t)(slot0 >> 5) * y.chunk_bytes;
-      const int tau = (slot0 & 31) + i;
-      if (is_v) {
-        uint8_t* vcodes = vcodes_all + (size_t)r * 8 * y.Dv;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) vcodes[i * y.Dv + 8 * w + e] = (o.word >> (4 * e)) & 15u;
-        if ((w & 7) == 0) reinterpret_cast<uint32_t*>(chunk + y.off_vsb)[sb_offset(tau, w >> 3, y.Gv)] = o.sb;
-      } else {
-        reinterpret_cast<uint32_t*>(chunk + y.off_kc)[k_word_offset(tau, w, y.G)] = o.word;
-        if ((w & 7) == 0) reinterpret_cast<uint32_t*>(chunk + y.off_ksb)[sb_offset(tau, w >> 3, y.G)] = o.sb;
-      }
+      for (int e = 0; e < 8; ++e) vcodes[i * y.Dv + 8 * w + e] = (o.word >> (4 * e)) & 15u;
+      if ((w & 7) == 0) reinterpret_cast<uint32_t*>(chunk + y.off_vsb)[sb_offset(tau, w >> 3, y.Gv)] = o.sb;
+    } else {
+      reinterpret_cast<uint32_t*>(chunk + y.off_kc)[k_word_offset(tau, w, y.G)] = o.word;
+      if ((w & 7) == 0) reinterpret_cast<uint32_t*>(chunk + y.off_ksb)[sb_offset(tau, w >> 3, y.G)] = o.sb;
     }
   }
   if (y.alias) return;
   __syncthreads();
   // ---- token-packed V words: one word = one head-dim element of the octet's 8 positions ----
+  const int k0 = un.first & 7;                           // nibble of the first new token inside the word
+  const uint32_t mask = un.cnt == 8 ? 0xffffffffu : ((1u << (4 * un.cnt)) - 1u) << (4 * k0);
 #pragma unroll
-  for (int r = 0; r < M; ++r) {
-    const UnitInfo un = s_unit[r];
-    if (un.agent < 0) continue;
-    const uint8_t* vcodes = vcodes_all + (size_t)r * 8 * y.Dv;
-    const int slot0 = un.first & 255, tau0 = slot0 & 31;
-    uint8_t* chunk = head_block(pool, y, layer, un.block, hk) + (size_t)(slot0 >> 5) * y.chunk_bytes;
-    const int k0 = un.first & 7;              // nibble of the first new token inside the word
-    uint32_t mask = 0;
-    for (int i = 0; i < un.cnt; ++i) mask |= 15u << (4 * (k0 + i));
-    uint32_t* vc = reinterpret_cast<uint32_t*>(chunk + y.off_vc);
-    for (int d = threadIdx.x; d < y.Dv; d += kThreads) {
-      uint32_t bits = 0;
-      for (int i = 0; i < un.cnt; ++i) bits |= (uint32_t)vcodes[i * y.Dv + d] << (4 * (k0 + i));
-      const int wi = v_word_offset(tau0 >> 3, d);
-      vc[wi] = (mask == 0xffffffffu) ? bits : ((vc[wi] & ~mask) | bits);
-    }
+  for (int r = 0; r < kMaxDv / kThreads; ++r) {
+    const int d = threadIdx.x + kThreads * r;
+    if (d >= y.Dv) break;
+    uint32_t bits = 0;
+    for (int i = 0; i < un.cnt; ++i) bits |= (uint32_t)vcodes[i * y.Dv + d] << (4 * (k0 + i));
+    vc[v_word_offset((slot0 & 31) >> 3, d)] = (old[r] & ~mask) | bits;
   }
 }
 
@@ -453,21 +458,20 @@ cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer,
                             b.block_tables, pos, new_offs, (const uint16_t*)k_new, (const uint16_t*)v_new, flags, chunk_units);
 }
 
-template <int M>
-cudaError_t launch_m(const Layout& y, uint8_t* pool, int n_blocks, int layer, const q4kv_batch& b, const int32_t* pos,
-                     const int32_t* new_offs, int units, const void* k_new, const void* v_new, int32_t* flags,
-                     cudaStream_t st) {
+cudaError_t launch_octets(const Layout& y, uint8_t* pool, int n_blocks, int layer, const q4kv_batch& b, const int32_t* pos,
+                          const int32_t* new_offs, int units, const void* k_new, const void* v_new, int32_t* flags,
+                          cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((units + M - 1) / M, y.Hkv);
+  cfg.gridDim = dim3(units, y.Hkv);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = y.alias ? 0 : (size_t)M * 8 * y.Dv;
+  cfg.dynamicSmemBytes = y.alias ? 0 : (size_t)8 * y.Dv;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, quantize_append_kernel<M>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
+  return cudaLaunchKernelEx(&cfg, quantize_append_kernel, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
                             b.block_tables, pos, new_offs, k_new, v_new, flags);
 }
 
@@ -477,7 +481,8 @@ cudaError_t launch_quantize_append(const Layout& y, void* pool, int n_blocks, in
                                    const int32_t* pos, const int32_t* new_offs, int total_new,
                                    const void* k_new, const void* v_new, int32_t* flags, cudaStream_t st) {
   if (total_new <= 0 || b.n_agents <= 0) return cudaSuccess;
-  const int units = total_new / 8 + 2 * b.n_agents;        // >= sum over agents of ceil((pos%8+n)/8)
+  // >= sum over agents of ceil((pos%8+n)/8): n tokens touch at most n octets, and at most n / 8 + 2
+  const int units = std::min(total_new, total_new / 8 + 2 * b.n_agents);
   if (total_new >= 8 * b.n_agents && (size_t)(kThreads / 32) * y.chunk_bytes <= kBulkSmem) {
     // a phase of many tokens per agent: one warp per (32-token chunk, KV head)
     const int chunk_units = total_new / 32 + 2 * b.n_agents;   // >= sum over agents of the chunks their new range touches
@@ -487,7 +492,7 @@ cudaError_t launch_quantize_append(const Layout& y, void* pool, int n_blocks, in
                                                         : (four ? launch_bulk<4, false> : launch_bulk<1, false>);
     return launch(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
   }
-  return launch_m<1>(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, units, k_new, v_new, flags, st);
+  return launch_octets(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, units, k_new, v_new, flags, st);
 }
 
 }  // namespace q4kv
