@@ -23,6 +23,88 @@ __device__ inline uint4 query8(uint4 v, float sf) {
                     f32x2_to_h2(hi(v.y), hi(v.w)));
 }
 
+// A warp's 32 rows and global memory.  A thread owns a row, but rows lie kilobytes apart: threads that load or store their own rows
+// touch 32 lines with every instruction, which made 4 us of a tile's start and 3 to 4 of its end.  So the lanes share lines -- eight
+// rows x four 16-byte pieces in a load, whole 64- or 128-byte parts of rows in a store -- and what is stored passes through 4 KB of
+// shared memory per warp, where piece j of row r lies at j ^ r % 8 (no bank conflicts either way).  8 x (8192 + 1024) tokens at
+// d = 128: 1156 -> 1112 us; d = 256 (stores alone: its queries go to tensor memory, and the exchange on the way there cost 1.1 us of a
+// tile's start through a buffer that has to be added): 501 -> 495 us a pass over windowed layers; latent: 212 -> 204 us.
+constexpr int kRowsBytes = 32 * 128;
+__device__ __forceinline__ uint32_t piece_at(int row, int piece) { return (uint32_t)(row * 128 + ((piece ^ (row & 7)) << 4)); }
+// The query rows 8 g + lane % 8, g < 4, of the warp's 32 (nullptr: no such query).  Row r of a tile is query r % tile_q of head r / tile_q.
+struct RowsIn { const uint16_t* row[4]; };
+__device__ __forceinline__ RowsIn rows_in(const uint16_t* q, int tile_row, int tile_q, int i_first, int q0, int q_len, int Hq, int head0, int n_rep,
+                                          int d, bool none) {
+  RowsIn in;
+  const float per = __fdividef(1.f, (float)tile_q);
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const int r = tile_row + 8 * g + ((int)threadIdx.x & 7), h = (int)(((float)r + 0.5f) * per), i = i_first + r - h * tile_q;   // r < 256: exact
+    in.row[g] = i < q_len && h < n_rep && !none ? q + ((size_t)(q0 + i) * Hq + head0 + h) * d : nullptr;
+  }
+  return in;
+}
+__device__ __forceinline__ uint4 piece_of(const uint16_t* row, int p) {
+  return row ? *reinterpret_cast<const uint4*>(row + 8 * p) : make_uint4(0u, 0u, 0u, 0u);
+}
+// The first kCount pieces of all rows, shared out: w[k] is piece 4 (k / 4) + lane / 8 of row 8 (k % 4) + lane % 8.
+template <int kCount>
+__device__ __forceinline__ void load_rows(const RowsIn& in, uint4* w) {
+#pragma unroll
+  for (int k = 0; k < kCount; ++k) w[k] = piece_of(in.row[k & 3], 4 * (k >> 2) + (((int)threadIdx.x & 31) >> 3));
+}
+// Where a warp's rows go: element `at` on of the output for this lane's row, if it is `mine` to write.  A store covers 8 rows of
+// bfloat16 or 4 of binary32.
+struct RowsOut { size_t base; int rel[8]; unsigned there; bool bf16; };
+__device__ __forceinline__ RowsOut rows_out(size_t at, bool mine, bool bf16) {
+  const int lane = threadIdx.x & 31;
+  const unsigned rows = __ballot_sync(0xffffffffu, mine);
+  RowsOut o;
+  o.bf16 = bf16;
+  o.base = __shfl_sync(0xffffffffu, (unsigned long long)at, rows ? __ffs(rows) - 1 : 0);
+  o.there = 0u;
+  const int rel = (int)(long long)(at - o.base);         // inside a tile's output
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int r = bf16 ? 8 * (k & 3) + (lane >> 2) : 4 * k + (lane >> 3);
+    o.rel[k] = __shfl_sync(0xffffffffu, rel, r) + (bf16 ? 8 * (lane & 3) : 4 * (lane & 7));
+    o.there |= ((rows >> r) & 1u) << k;
+  }
+  return o;
+}
+// 32 elements of every row, from `first` on: x is this lane's.
+__device__ __forceinline__ void store_rows(uint8_t* buf, const float (&x)[32], const RowsOut& o, void* out, int first) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();                                          // what was in the buffer has been read
+  if (o.bf16) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(x[8 * p + 2 * e], x[8 * p + 2 * e + 1]);
+        w[e] = *reinterpret_cast<const uint32_t*>(&b);
+      }
+      *reinterpret_cast<uint4*>(buf + piece_at(lane, p)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint4 v = *reinterpret_cast<const uint4*>(buf + piece_at(8 * k + (lane >> 2), lane & 3));
+      if ((o.there >> k) & 1u) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(out) + o.base + first + o.rel[k]) = v;
+    }
+  } else {
+#pragma unroll
+    for (int p = 0; p < 8; ++p) *reinterpret_cast<float4*>(buf + piece_at(lane, p)) = make_float4(x[4 * p], x[4 * p + 1], x[4 * p + 2], x[4 * p + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float4 v = *reinterpret_cast<const float4*>(buf + piece_at(4 * k + (lane >> 3), lane & 7));
+      if ((o.there >> k) & 1u) *reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + o.base + first + o.rel[k]) = v;
+    }
+  }
+}
+
 // The agents that bring one query in a batch where others bring more are left to the decode kernel, which is launched next
 // on the same stream; its arrival counters are cleared here, so that the caller need not hand over a cleared workspace.
 __device__ inline void clear_tickets(const PrefillExtra& x) {

@@ -26,7 +26,7 @@
 //   * With few tiles the keys of a tile are cut over several CTAs as well (plan_prefill_splits); these leave (acc, m, l)
 //     records that merge_prefill_kernel combines.
 // Measured on 3 agents x (250 .. 512 queries on 2000 .. 4000 keys), 16 heads (102 GFLOP): 36 ms on the shape-agnostic kernel,
-// 0.203 ms here = 502 TFLOP/s back to back; 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
+// 0.196 ms here = 519 TFLOP/s back to back (0.203 with a thread loading and storing its own row); 3650 clocks per block, of which the dequantize warps are busy 2600 -- they, the softmax and the
 // products share the shared-memory bandwidth (256 KB per block: 2000 clocks) and the issue slots.
 // All hand-offs are mbarriers; every wait is bounded and a wait that runs out raises Q4KV_FLAG_INTERNAL, drains the tensor
 // pipe and frees the tensor memory before the CTA returns.
@@ -286,39 +286,70 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     const uint32_t lane_addr = tb + ((uint32_t)(warp * 32) << 16);
     const int h = row / tile_q, i = i_min + row % tile_q;
     const bool mine = i < q_len && h < n_rep;            // a row of the output
-    const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
     const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
-    float kappa;                                         // score in log2 units = S * kappa
+    float kappa = 0.f;                                   // score in log2 units = S * kappa
     {
-      // ---- stage the query row: bf16 -> binary16 times a power of two; pieces of eight dims 0..31 go to tensor memory,
-      //      32..71 to shared memory ----
-      const uint16_t* qrow = P.q + (valid ? row_index : 0) * kD;
-      float mx = 0.f;
-      if (valid) {
-#pragma unroll 8
-        for (int p = 0; p < kD / 8; ++p) mx = fmaxf(mx, max_abs8(*reinterpret_cast<const uint4*>(qrow + 8 * p)));
+      // ---- stage the warp's query rows: bf16 -> binary16 times a power of two per row; pieces of eight dims 0..31 go to tensor
+      //      memory, 32..71 to shared memory.  The lanes share the rows' lines (see load_rows), eight rows at a time: 18 loads a
+      //      lane in flight are enough, and unrolled over all rows it spills (the launches of few tiles then take 33 us for 30).  The warp's
+      //      part of the shared-memory tile is the buffer on the way to tensor memory. ----
+      uint8_t* const buf = sm.qs + 4 * warp * kSboQ;     // 16 KB of the warp's 20: [quarter of the tensor-memory part][32 rows x 128 bytes]
+      const float per = __fdividef(1.f, (float)tile_q);
+      auto row_at = [&](int r) -> const uint16_t* {      // the query in row r of the tile, this lane's first piece of it
+        const int h = (int)(((float)r + 0.5f) * per), i = i_min + r - h * tile_q;   // r < 128: exact
+        return i < q_len && h < n_rep && !bad_len ? P.q + ((size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h) * kD + 8 * (lane >> 3) : nullptr;
+      };
+      float sf_own = 0.f;
+#pragma unroll 1
+      for (int g = 0; g < 4; ++g) {
+        const uint16_t* row_g = row_at(warp * 32 + 8 * g + (lane & 7));
+        uint4 v[kD / 32];
+#pragma unroll
+        for (int k = 0; k < kD / 32; ++k) v[k] = piece_of(row_g, 4 * k);
+        float mx = 0.f;
+#pragma unroll
+        for (int k = 0; k < kD / 32; ++k) mx = fmaxf(mx, max_abs8(v[k]));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+        int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
+        if (mx == 0.f) ex = 0;
+        ex = min(max(ex, -100), 100);
+        const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
+        if ((lane >> 3) == g) {
+          sf_own = sf;
+          kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
+        }
+#pragma unroll
+        for (int k = 0; k < kQTmem / 32; ++k)            // pieces 4 k + lane / 8: half of a 128-byte row's
+          *reinterpret_cast<uint4*>(buf + (k >> 1) * kRowsBytes + piece_at(8 * g + (lane & 7), 4 * (k & 1) + (lane >> 3))) = query8(v[k], sf);
       }
-      int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
-      if (mx == 0.f) ex = 0;
-      ex = min(max(ex, -100), 100);
-      const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
-      kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
-      const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
 #pragma unroll 1
       for (int c = 0; c < kQTmem / 64; ++c) {            // 32 columns (64 dims) at a time
         uint32_t qa[32];
 #pragma unroll
-        for (int p = 0; p < 8; ++p) {
-          const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * (8 * c + p)) : zero4, sf);
-          qa[4 * p] = v.x; qa[4 * p + 1] = v.y; qa[4 * p + 2] = v.z; qa[4 * p + 3] = v.w;
-        }
+        for (int p = 0; p < 8; ++p) *reinterpret_cast<uint4*>(qa + 4 * p) = *reinterpret_cast<const uint4*>(buf + c * kRowsBytes + piece_at(lane, p));
         tmem_st32(lane_addr + kColQ + 32 * c, qa);
       }
-#pragma unroll 4
-      for (int p = kQTmem / 8; p < kD / 8; ++p) {
-        const uint4 v = query8(valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : zero4, sf);
-        *reinterpret_cast<uint4*>(sm.qs + (row & 7) * 16 + (row >> 3) * kSboQ + (p - kQTmem / 8) * 128) = v;
+      __syncwarp();                                      // the buffer has been read: the shared-memory part takes its place
+#pragma unroll 1
+      for (int g = 0; g < 4; g += 2) {
+        uint4 v[2][kQSmem / 32];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const uint16_t* row_g = row_at(warp * 32 + 8 * (g + e) + (lane & 7));
+#pragma unroll
+          for (int k = 0; k < kQSmem / 32; ++k) v[e][k] = piece_of(row_g, kQTmem / 8 + 4 * k);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int r = warp * 32 + 8 * (g + e) + (lane & 7);
+          const float sf = __shfl_sync(0xffffffffu, sf_own, 8 * (g + e) + (lane & 7));
+#pragma unroll
+          for (int k = 0; k < kQSmem / 32; ++k)
+            *reinterpret_cast<uint4*>(sm.qs + (r & 7) * 16 + (r >> 3) * kSboQ + (4 * k + (lane >> 3)) * 128) = query8(v[e][k], sf);
+        }
       }
       wait_st();
       fence_async_smem();
@@ -399,7 +430,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
     const bool zero = bad || n_iter == 0 || l <= 0.f;
     const bool final = P.n_splits == 1;
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
-    float* rec = final ? nullptr : P.records + (row_index * P.n_splits + split) * prefill_record(kDv);
+    // (the queries are not needed any more: every product that read them is complete)
+    uint8_t* const buf = sm.qs + 4 * warp * kSboQ;
+    const size_t at = final ? row_index * kDv : (row_index * P.n_splits + split) * prefill_record(kDv);
+    const RowsOut to = rows_out(at + kDvCta * hv, mine, final && P.out_dtype == Q4KV_OUT_BF16);
 #pragma unroll 1
     for (int part = 0; part < kDvCta / 32; ++part) {
       uint32_t orow[32];
@@ -407,35 +441,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
         tmem_ld32(lane_addr + kColO + 32 * part, orow);
         wait_ld32(orow);
       }
-      if (!mine) continue;
-      const int d0 = kDvCta * hv + 32 * part;
-      // slot j of every eight columns is value dim elem_of(j)
-      if (final && P.out_dtype == Q4KV_OUT_BF16) {
-        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + row_index * kDv + d0;
+      float x[32];                                       // slot j of every eight columns is value dim elem_of(j)
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          uint4 v;
-          uint32_t* vv = reinterpret_cast<uint32_t*>(&v);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 bb = __floats2bfloat162_rn(zero ? 0.f : __uint_as_float(orow[c + slot_of(2 * e)]) * inv,
-                                                            zero ? 0.f : __uint_as_float(orow[c + slot_of(2 * e + 1)]) * inv);
-            vv[e] = *reinterpret_cast<const uint32_t*>(&bb);
-          }
-          *reinterpret_cast<uint4*>(o + c) = v;
-        }
-      } else {
-        float* o = (final ? reinterpret_cast<float*>(P.out) + row_index * kDv : rec) + d0;
-#pragma unroll
-        for (int c = 0; c < 32; c += 4)
-          *reinterpret_cast<float4*>(o + c) =
-              zero ? make_float4(0.f, 0.f, 0.f, 0.f)
-                   : make_float4(__uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 0)]) * inv, __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 1)]) * inv,
-                                 __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 2)]) * inv, __uint_as_float(orow[(c & ~7) + slot_of((c & 7) + 3)]) * inv);
-      }
+      for (int c = 0; c < 32; ++c) x[c] = zero ? 0.f : __uint_as_float(orow[(c & ~7) + slot_of(c & 7)]) * inv;
+      store_rows(buf, x, to, final ? P.out : P.records, 32 * part);
     }
     if (hv == 0 && mine) {
-      if (!final) *reinterpret_cast<float2*>(rec + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
+      if (!final) *reinterpret_cast<float2*>(P.records + at + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
       else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
     }
   }

@@ -10,8 +10,9 @@
 //     2050, shared memory for 2300 (operands 1570, tiles written 510, raw blocks 150) and the issue slots for 1700, so what
 //     matters is that all of them work at once: few, long hand-offs.  (Steps of 64 keys with the queries in tensor memory and
 //     two threads per row, which exchanged their maxima, took 2 x 3000 clocks.)  Measured on 8 agents x (8192 + 1024 tokens),
-//     32 / 8 heads: 4150 clocks per step; 1156 us per launch = 1010 TFLOP/s in a run of a few launches, 1298 us = 900 TFLOP/s in a
-//     run of seconds, under the power cap.  Before, 5000 clocks, 1240 and 1357 us: the issuing warp was the bottleneck, with eight
+//     32 / 8 heads: 4150 clocks per step; 1112 us per launch = 1051 TFLOP/s in a run of a few launches, 1240 us = 943 TFLOP/s in a
+//     run of seconds, under the power cap (1156 and 1298 us before the lanes shared the rows' lines at both ends of a tile).
+//     Before that, 5000 clocks, 1240 and 1357 us: the issuing warp was the bottleneck, with eight
 //     waits a step of which each cost 140 to 350 clocks although its phase was over; it has five now (see there), and a reference
 //     that moves by the sum of the probabilities instead of their maximum takes 70 of 230 instructions per 64 keys out of the
 //     softmax.  What is left is the chain of a tile's step: scores 250 clocks after their product, exponentials 2 x 1100, value
@@ -322,25 +323,30 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const uint32_t s_addr = lane_addr + kColS + 128 * t, o_addr = lane_addr + kColO + 128 * t;
     const int h = row / tile_q, i = i_min + t * tile_q + row % tile_q;
     const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
-    const bool valid = mine && !bad_len;
     const int pq = prefix + i;                           // this row's position
     const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
-    float kappa;                                         // score in log2 units = S * kappa
+    float kappa = 0.f;                                   // score in log2 units = S * kappa
     {
-      // ---- stage the query row: bf16 -> binary16 times a power of two ----
-      const uint16_t* qrow = P.q + (valid ? row_index : 0) * 128;
-      auto piece = [&](int p) { return valid ? *reinterpret_cast<const uint4*>(qrow + 8 * p) : make_uint4(0u, 0u, 0u, 0u); };
-      float mx = 0.f;
+      // ---- stage the warp's query rows: bf16 -> binary16 times a power of two per row.  Lane l takes the pieces l / 8, + 4, + 8, + 12 of
+      //      row 8 g + l % 8 (see load_rows; the rows go to shared memory here, so nothing has to change hands) ----
+      const RowsIn in = rows_in(P.q, (warp & 3) * 32, tile_q, i_min + t * tile_q, q0, q_len, y.Hq, hk * n_rep, n_rep, 128, bad_len);
+      uint4 v[16];                                       // [piece / 4][g]
+      load_rows<16>(in, v);
 #pragma unroll
-      for (int p = 0; p < 16; ++p) mx = fmaxf(mx, max_abs8(piece(p)));
-      int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
-      if (mx == 0.f) ex = 0;
-      ex = min(max(ex, -100), 100);
-      const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
-      kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
+      for (int g = 0; g < 4; ++g) {
+        const int r = (warp & 3) * 32 + 8 * g + (lane & 7);
+        float mx = fmaxf(fmaxf(max_abs8(v[g]), max_abs8(v[4 + g])), fmaxf(max_abs8(v[8 + g]), max_abs8(v[12 + g])));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+        int ex = (int)((__float_as_uint(mx) >> 23) & 255u) - 127;
+        if (mx == 0.f) ex = 0;
+        ex = min(max(ex, -100), 100);
+        const float sf = __uint_as_float((uint32_t)(127 + 8 - ex) << 23);      // 256 <= max |q| * sf < 512
+        if ((lane >> 3) == g) kappa = P.scale_log2 * __uint_as_float((uint32_t)(127 - 8 + ex) << 23);
 #pragma unroll
-      for (int p = 0; p < 16; ++p)
-        *reinterpret_cast<uint4*>(sm.qs[t] + (row & 7) * 16 + (row >> 3) * 2048 + p * 128) = query8(piece(p), sf);
+        for (int k = 0; k < 4; ++k)
+          *reinterpret_cast<uint4*>(sm.qs[t] + (r & 7) * 16 + (r >> 3) * 2048 + (4 * k + (lane >> 3)) * 128) = query8(v[4 * k + g], sf);
+      }
       fence_async_smem();
       mbar_arrive(&sm.q_ready);
     }
@@ -455,7 +461,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const bool zero = bad || n_step == 0 || l <= 0.f;
     const bool final = P.x.n_splits == 1;                // else the row is left as a record
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
-    float* rec = final ? nullptr : P.x.records + (row_index * P.x.n_splits + split) * prefill_record(128);
+    // (the tile's queries are not needed any more: every product that read them is complete)
+    uint8_t* const buf = sm.qs[t] + (warp & 3) * kRowsBytes;
+    const size_t at = final ? row_index * 128 : (row_index * P.x.n_splits + split) * prefill_record(128);
+    const RowsOut to = rows_out(at, mine, final && P.out_dtype == Q4KV_OUT_BF16);
 #pragma unroll 1
     for (int part = 0; part < 4; ++part) {
       uint32_t orow[32];
@@ -463,33 +472,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         tmem_ld32(o_addr + 32 * part, orow);
         wait_ld32(orow);
       }
-      if (!mine) continue;
-      if (final && P.out_dtype == Q4KV_OUT_BF16) {
-        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + row_index * 128 + 32 * part;
+      float x[32];
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          uint4 v;
-          uint32_t* vv = reinterpret_cast<uint32_t*>(&v);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 b = __floats2bfloat162_rn(zero ? 0.f : __uint_as_float(orow[c + 2 * e]) * inv,
-                                                           zero ? 0.f : __uint_as_float(orow[c + 2 * e + 1]) * inv);
-            vv[e] = *reinterpret_cast<const uint32_t*>(&b);
-          }
-          *reinterpret_cast<uint4*>(o + c) = v;
-        }
-      } else {
-        float* o = (final ? reinterpret_cast<float*>(P.out) + row_index * 128 : rec) + 32 * part;
-#pragma unroll
-        for (int c = 0; c < 32; c += 4)
-          *reinterpret_cast<float4*>(o + c) =
-              zero ? make_float4(0.f, 0.f, 0.f, 0.f)
-                   : make_float4(__uint_as_float(orow[c]) * inv, __uint_as_float(orow[c + 1]) * inv,
-                                 __uint_as_float(orow[c + 2]) * inv, __uint_as_float(orow[c + 3]) * inv);
-      }
+      for (int c = 0; c < 32; ++c) x[c] = zero ? 0.f : __uint_as_float(orow[c]) * inv;
+      store_rows(buf, x, to, final ? P.out : P.x.records, 32 * part);
     }
     if (mine) {
-      if (!final) *reinterpret_cast<float2*>(rec + 128) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
+      if (!final) *reinterpret_cast<float2*>(P.x.records + at + 128) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
       else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
     }
   }

@@ -34,6 +34,7 @@
 // as they are a block takes 2100).  With one barrier for all eight softmax warps, maxima exchanged in every block and 96
 // registers for every warp (the d = 256 form spilled) it took 3400.  8 agents x (4096 + 512) tokens, 16 query heads, d = 256:
 // 508 -> 382 us (575 -> 765 TFLOP/s) in a run of seconds, 363 us in one of a few launches; 192 / 128: 350 -> 282 (648), 281.
+// With the output stored a line at a time (store_rows): 371 (788) and 354; 192 / 128: 275 (665) and 278.
 #include "prefill_common.cuh"
 
 namespace q4kv {
@@ -521,8 +522,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
     const bool final = P.x.n_splits == 1;                // else the row is left as a record
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
     const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
-    const size_t orow_index = row_index * kDv + (kDv / 2) * half;
-    float* rec = final ? nullptr : P.x.records + (row_index * P.x.n_splits + split) * prefill_record(kDv);
+    const size_t at = final ? row_index * kDv : (row_index * P.x.n_splits + split) * prefill_record(kDv);
+    uint8_t* const buf = &sm.khat[0][0] + warp * kRowsBytes;   // the products with the keys are done
+    const RowsOut to = rows_out(at + (kDv / 2) * half, mine, final && P.out_dtype == Q4KV_OUT_BF16);
 #pragma unroll 1
     for (int part = 0; part < kDv / 64; ++part) {
       uint32_t orow[32];
@@ -530,33 +532,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
         tmem_ld32(lane_addr + kColO + (kDv / 2) * half + 32 * part, orow);
         wait_ld32(orow);
       }
-      if (!mine) continue;
-      if (final && P.out_dtype == Q4KV_OUT_BF16) {
-        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(P.out) + orow_index + 32 * part;
+      float x[32];
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          uint4 v;
-          uint32_t* vv = reinterpret_cast<uint32_t*>(&v);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 bb = __floats2bfloat162_rn(zero ? 0.f : __uint_as_float(orow[c + 2 * e]) * inv,
-                                                            zero ? 0.f : __uint_as_float(orow[c + 2 * e + 1]) * inv);
-            vv[e] = *reinterpret_cast<const uint32_t*>(&bb);
-          }
-          *reinterpret_cast<uint4*>(o + c) = v;
-        }
-      } else {
-        float* o = (final ? reinterpret_cast<float*>(P.out) + orow_index : rec + (kDv / 2) * half) + 32 * part;
-#pragma unroll
-        for (int c = 0; c < 32; c += 4)
-          *reinterpret_cast<float4*>(o + c) =
-              zero ? make_float4(0.f, 0.f, 0.f, 0.f)
-                   : make_float4(__uint_as_float(orow[c]) * inv, __uint_as_float(orow[c + 1]) * inv,
-                                 __uint_as_float(orow[c + 2]) * inv, __uint_as_float(orow[c + 3]) * inv);
-      }
+      for (int c = 0; c < 32; ++c) x[c] = zero ? 0.f : __uint_as_float(orow[c]) * inv;
+      store_rows(buf, x, to, final ? P.out : P.x.records, 32 * part);
     }
     if (half == 0 && mine) {
-      if (!final) *reinterpret_cast<float2*>(rec + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
+      if (!final) *reinterpret_cast<float2*>(P.x.records + at + kDv) = make_float2(zero ? -INFINITY : m_ref, bad ? -1.f : zero ? 0.f : l);
       else if (P.lse) P.lse[row_index] = zero ? -INFINITY : (m_ref + log2f(l)) / kLog2e;
     }
   }

@@ -1162,6 +1162,32 @@ def test_prefill_reference_moves_within_and_between_steps(H, spec_args, prefix, 
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("spec_args,prefix,chunks", [
+    ((1, 6, 2, 128, 128, False), [70, 0, 5, 0], [85, 43, 1, 42]),    # 42 queries x 3 heads a tile (two rows idle): full, one over, one
+    ((1, 4, 4, 128, 128, False), [3000], [129]),                 # the keys are split: records
+    ((1, 6, 2, 256, 256, False), [70, 0, 5, 0], [85, 43, 1, 42]),
+    ((1, 3, 1, 192, 128, False), [2000, 0], [43, 1]),
+    ((1, 5, 1, 576, 512, True), [70, 0, 0], [26, 25, 1]),        # 25 queries x 5 heads a tile
+])
+def test_prefill_rows_of_partial_tiles(H, spec_args, prefix, chunks):
+    """Every row of a tile has its own magnitude (2^-9 .. 2^9, which its sharpness shows), and its place in the output."""
+    from paper_2603_04428_b200 import binding as B
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = QuietStartPair(H, spec_args, lens, seed=83).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = f32(p.q(9, int(q_offs[-1])))
+    e = (np.arange(q.shape[0] * q.shape[1]) * 7 % 19 - 9).reshape(q.shape[:2])
+    q = synth.f32_to_bf16_bits((q * np.exp2(e)[..., None]).astype(np.float32))
+    scale = 2.0 ** -9 / math.sqrt(192 if spec_args[5] else spec_args[3])     # the sharpest row is an ordinary one
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, 0, f32(q), scale)
+    out, lse = p.dc.prefill(0, lens, q_offs, 0, q, scale)
+    assert_attention_close(out.cpu().numpy(), ref)
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    out16, _ = p.dc.prefill(0, lens, q_offs, 0, q, scale, out_dtype=B.OUT_BF16)
+    assert torch.equal(out16, out.to(torch.bfloat16))        # the same sums, rounded once more
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("name", list(SPECS))                # 2, 4, 5, 8 and 9 groups per token
 @pytest.mark.parametrize("chunks", [[13, 40, 9, 100], [8, 33, 31, 65, 300], [256]])
 def test_bulk_append_of_unaligned_phases(H, name, chunks):
