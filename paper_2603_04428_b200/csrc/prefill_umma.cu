@@ -47,7 +47,7 @@ using namespace prefill;
 
 constexpr int kSoftmaxWarps = 8, kDequantWarps = 8;
 constexpr int kLastGroup = kSoftmaxWarps + kDequantWarps, kLoadWarp = kLastGroup, kMmaWarp = kLastGroup + 3;
-constexpr int kThreads = (kLastGroup + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two idle warps), ...
+constexpr int kThreads = (kLastGroup + 4) * 32;            // 640: five warpgroups (the last: MMA, load, two that only bfloat16 caches need), ...
 // ... launched with 96 registers per thread; the softmax warpgroups take 144, the others keep 64 (61440 in all)
 constexpr int kRegsSoftmax = 144, kRegsOther = 64;
 static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * 96, "");
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
 
   if (threadIdx.x == 0) {
     if (bad_len) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
-    for (int s = 0; s < kRawSlots; ++s) { mbar_init(&sm.raw_full[s], 1); mbar_init(&sm.raw_free[s], kDequantWarps); mbar_init(&sm.sb_done[s], kDequantWarps); sm.bad[s] = 0; }
+    for (int s = 0; s < kRawSlots; ++s) { mbar_init(&sm.raw_full[s], 1); mbar_init(&sm.raw_free[s], kDequantWarps); mbar_init(&sm.sb_done[s], 2); sm.bad[s] = 0; }
     for (int s = 0; s < kStages; ++s) { mbar_init(&sm.k_full[s], kDequantWarps); mbar_init(&sm.v_full[s], kDequantWarps); }
     for (int s = 0; s < kStages / 2; ++s) { mbar_init(&sm.k_free[s], 1); mbar_init(&sm.v_free[s], 1); }
     for (int t = 0; t < 2; ++t) {
@@ -236,6 +236,28 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         }
       }
     }
+    } else if (kBf) {
+    // =============================== bfloat16 scales and biases ==================================
+    // They become binary16 in place (the tiles are binary16), by a warp for each chunk of a block, ahead of the dequantize warps (which
+    // did it themselves, behind a barrier of their own, one more wait in their chain: 1350 us on 8 x (8192 + 1024) tokens, 1227 this way).
+    // Only tokens below the agent's length count for the range report (bytes past the end are whatever was there).
+    const int ci = warp - (kLoadWarp + 1);
+    const int tau = 8 * ((lane >> 1) & 3) + 4 * (lane & 1) + (lane >> 3);        // row (i * 4 + tid) * 2 + e: token 8 tid + 4 e + i
+    for (int j = 0; j < n_iter; ++j) {
+      const int r = j % kRawSlots;
+      if (!mbar_wait(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
+      uint2* at = reinterpret_cast<uint2*>(sm.raw[r] + ci * kChunkBytes + 2048) + lane;      // both groups of the row's token: Ksb, Vsb
+      uint2 k = at[0], v = at[(4352 - 2048) / 8];
+      bool over = false;
+      k.x = bf16_pair_to_h2(k.x, over); k.y = bf16_pair_to_h2(k.y, over);
+      v.x = bf16_pair_to_h2(v.x, over); v.y = bf16_pair_to_h2(v.y, over);
+      at[0] = k;
+      at[(4352 - 2048) / 8] = v;
+      if (over && !sm.bad[r] && (it0 + j) * 64 + ci * 32 + tau < kv_len) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.sb_done[r]);
+    }
     }
   } else if (warp >= kSoftmaxWarps) {
     fewer_registers<kRegsOther>();
@@ -257,24 +279,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     for (int j = 0; j < n_iter; ++j) {
       const int s = j % kStages, r = j % kRawSlots;
       if (j >= kStages && !mbar_doze(&sm.k_free[s >> 1], (uint32_t)(j / kStages - 1), abort_flag)) break;
-      if (!mbar_doze(&sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
+      if (!mbar_doze(kBf ? &sm.sb_done[r] : &sm.raw_full[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
       const bool bad = sm.bad[r] != 0;
       const int pos_base = (it0 + j) * 64 + ci * 32;
       const uint8_t* raw = sm.raw[r];
-      if (kBf) {
-        // bfloat16 scales and biases become binary16 in place, once per block (the tiles are binary16), one word per thread;
-        // only the tokens below the agent's length count for the range report (bytes past the end are whatever was there)
-        const int o = x7;                                // 64 words of Ksb, 64 of Vsb
-        const int row = (o & 63) >> 1;                   // (i * 4 + tid) * 2 + e: token 8 tid + 4 e + i
-        const int tau = 8 * ((row >> 1) & 3) + 4 * (row & 1) + (row >> 3);
-        uint32_t* at = reinterpret_cast<uint32_t*>(sm.raw[r] + ci * kChunkBytes + (o < 64 ? 2048 + 4 * o : 4352 + 4 * (o - 64)));
-        bool over = false;
-        *at = bf16_pair_to_h2(*at, over);
-        if (over && !bad && pos_base + tau < kv_len) raise_flag(P.flags, Q4KV_FLAG_SB_RANGE);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.sb_done[r]);
-        if (!mbar_wait(&sm.sb_done[r], (uint32_t)(j / kRawSlots), abort_flag)) break;
-      }
       {
         const uint4 kw = *reinterpret_cast<const uint4*>(raw + k_read);
         uint2 sb = *reinterpret_cast<const uint2*>(raw + k_sb);            // (scale, bias) of groups 0 and 1

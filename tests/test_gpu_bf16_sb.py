@@ -266,3 +266,29 @@ def test_a_scale_beyond_binary16_is_reported_by_the_tile_kernels(H, name):
         if not expect:
             assert torch.equal(out, good)
         p.dc.flags.zero_()
+
+
+@pytest.mark.parametrize("name", ["gqa128", "gqa256", "asym"])
+def test_prefill_looks_at_the_scales_of_every_token_below_the_length(H, name):
+    """The report of a scale or bias beyond binary16, at the ends of both chunks of a 64-key block, for keys and values, first and last
+    group, and lengths that end inside either chunk."""
+    from paper_2603_04428_b200 import binding as B
+    n, q_len = 85, 21                                  # blocks of 64 and 21 keys
+    p = Pair(H, SPECS[name], [n, 40], seed=157, sb_dtype=1).fill()
+    s = p.ospec
+    q = p.q(7, 2 * q_len)
+    scale = 1.0 / math.sqrt(s.d_qk)
+    blk = int(p.tabs[0][0])
+    image = O.pack(p.opool, p.tabs[0], n)
+    for which, groups in (("K", s.d_qk // 64), ("V", s.d_v // 64)):
+        for sb in ("s", "b"):
+            plane = getattr(p.opool, which + sb)
+            for tok, g, length in ((0, 0, n), (31, groups - 1, n), (32, groups - 1, n), (63, 0, n), (n - 1, groups - 1, n),
+                                   (n - 1, 0, n - 1), (63, groups - 1, 63), (31, 0, 31), (40, 0, 40)):
+                plane[0, blk, :, tok, g] = 0x4980      # 2^20 as bfloat16
+                p.dc.unpack(0, n, O.pack(p.opool, p.tabs[0], n))
+                p.dc.prefill(0, [length, 40], [0, q_len, 2 * q_len], 0, q, scale)
+                assert p.dc.read_flags() == (B.FLAG_SB_RANGE if tok < length else 0), (which, sb, tok, g, length)
+                p.dc.flags.zero_()
+                p.dc.unpack(0, n, image)
+                O.unpack(p.opool, p.tabs[0], n, image)
