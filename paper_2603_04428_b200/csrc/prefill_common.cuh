@@ -23,6 +23,25 @@ __device__ inline uint4 query8(uint4 v, float sf) {
                     f32x2_to_h2(hi(v.y), hi(v.w)));
 }
 
+// What a CTA reads first, asked of L2 while the preceding kernel drains: a prefetch returns nothing, and L2 is where the writes of the
+// preceding kernels land, so it may come before the wait for them.  Lane l of one warp asks for the 64-key block it0 + l (block tables are
+// inputs that no kernel writes; the table entries are then in L1 for the loader), the threads of the tile's rows for their query row.
+// Latent cache, 3 agents of 250 to 512 on 2000 to 4000 tokens, with the append: 210.3 -> 206.3 us a layer; d = 256, six windowed layers
+// 496.8 -> 494.9.  Not at d = 128, whose tiles' steps are long beside it: one agent 1377.0 / 1375.6, injection pass 5135 / 5145.
+template <class Par>
+__device__ __forceinline__ void ask_for_blocks(const Par& P, int a, int hk, int it0, int count, uint32_t chunk_bytes) {
+  const int l = threadIdx.x & 31;
+  if (l >= count) return;
+  const int c = 2 * (it0 + l), blk = P.tables[(size_t)a * P.max_blocks + (c >> 3)];
+  if (blk >= 0 && blk < P.n_blocks)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(head_block(P.pool, P.y, P.layer, blk, hk) + (size_t)(c & 7) * chunk_bytes),
+                 "r"(2 * chunk_bytes) : "memory");
+}
+template <int kElements>
+__device__ __forceinline__ void ask_for_row(const uint16_t* row) {
+#pragma unroll
+  for (int e = 0; e < kElements; e += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + e) : "memory");
+}
 // A warp's 32 rows and global memory.  A thread owns a row, but rows lie kilobytes apart: threads that load or store their own rows
 // touch 32 lines with every instruction, which made 4 us of a tile's start and 3 to 4 of its end.  So the lanes share lines -- eight
 // rows x four 16-byte pieces in a load, whole 64- or 128-byte parts of rows in a store -- and what is stored passes through 4 KB of

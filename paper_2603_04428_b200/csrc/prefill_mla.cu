@@ -126,6 +126,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_mla_kernel(const __grid_c
   __syncthreads();
   fence_after_sync();
   const uint32_t tb = sm.tmem_base;
+  if (warp == kSoftmaxWarps) ask_for_blocks(P, a, hk, it0, min(n_iter, 2), kChunkBytes);
+  if (warp < kSoftmaxWarps && !bad_len) {
+    const int h = (int)threadIdx.x / tile_q, i = i_min + (int)threadIdx.x % tile_q;
+    if (i < q_len && h < n_rep) ask_for_row<kD>(P.q + ((size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h) * kD);
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the new tokens were appended by the preceding kernel
   volatile int* abort_flag = &sm.abort_flag;
 
