@@ -60,7 +60,6 @@ constexpr int kCtasPerSm = 2;
 // warps per CTA: eight of 128 registers, or at d = 256, where the accumulators alone are 64, six of 168
 __host__ __device__ constexpr int warps_of(int G) { return G == 4 ? 6 : 8; }
 constexpr int kWholeSlack = 12;                        // see find_range
-constexpr int kOnePerSm = 21;                          // see launch_decode_mma
 constexpr float kMargin = 0.35f;                       // see chunk_values
 constexpr int kMaxRecords = 32;                        // a pair is cut over about this many CTAs at most (the merge reads them all)
 constexpr uint32_t kSpinLimit = 1u << 22;              // bounded mbarrier waits (each try blocks a while in hardware)
@@ -1362,13 +1361,12 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   P.y = y; P.pool = (const uint8_t*)pool; P.n_blocks = n_blocks; P.layer = layer; P.n_agents = b.n_agents * layer_count;
   P.n_real = b.n_agents; P.layer_count = layer_count;
   P.sets = head_sets(y); P.Hkv = y.Hkv * P.sets; P.n_rep = y.n_rep / P.sets;
-  long long units = 0, wanted = 0;
+  long long wanted = 0;
   for (int i = 0; i < kMaxLayersPerCall; ++i) {
     P.windows[i] = i < layer_count ? windows[i] : 0;
     if (i < layer_count) {
       const int span = (windows[i] > 0 && windows[i] + 32 < max_kv_len) ? windows[i] + 32 : max_kv_len;
       const int chunks = (span + 31) / 32, nw = warps_of(y.G);
-      units += (long long)b.n_agents * P.Hkv * chunks;
       wanted += (long long)b.n_agents * P.Hkv * ((chunks + nw - 1) / nw);       // a chunk per warp, and no CTA with two pairs
     }
   }
@@ -1381,12 +1379,11 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   // No more CTAs than can be of use: one that finds nothing to do costs the next launch a microsecond, because its CTAs come in as
   // this one's leave.  No fewer than pairs, which one CTA would take in turn: a launch on contexts of 30 tokens took 25.5 us with
   // a CTA per eight chunks, 4.3 with one per pair, on 100 tokens 7.2 and 4.3, at d = 256 13.8 and 6.7.
-  // One CTA per SM where that leaves a warp at most 2.6 chunks: the next launch's CTAs then sit beside this one's with their work
-  // laid out and their first chunks in L2.  Us a launch with two and with one: 2 agents x 4096 tokens 9.8 / 9.2, 3 x 4096 11.0 /
-  // 10.3, 6 x 1500 9.7 / 8.8, 13 x 600 9.8 / 8.2; 5 x 4096 (4.4 chunks) 11.7 / 12.4; not at d = 256 (10 in a window of 1024: 15.9 /
-  // 20.9) and with eight heads (6 x 1000: 11.8 / 12.8), whose chunks are twice the work.
-  long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
-  if (y.G == 2 && P.n_rep <= 4 && (long long)P.n_agents * P.Hkv <= sm_count() && units <= (long long)kOnePerSm * sm_count()) slots = sm_count();
+  // Two CTAs per SM for small batches too.  One, so that the next launch's CTAs sit beside this one's: us a launch with one and with two,
+  // 8 KV heads: 2 x 4096 9.8 / 9.2, 6 x 1500 9.4 / 8.8, 8 x 1000 9.8 / 8.6, 10 x 1000 12.0 / 9.6, 5 x 1100 9.1 / 7.9, 3 x 4096 11.1 / 10.4;
+  // the other way round 16 agents x 300..700, 9.3 / 9.7.  It also doubles the chunks that a warp adds up, and the tensor cores truncate
+  // their sums: against 64 bits, one agent x 4264 at 16 KV heads was off by 5.2e-4 instead of 4.1e-4.
+  const long long slots = sm_count() * kCtasPerSm < kMaxGrid ? sm_count() * kCtasPerSm : kMaxGrid;
   const int grid = (int)(wanted < slots ? (wanted < 1 ? 1 : wanted) : slots);
   if (y.G == 2) return P.n_rep > 4 ? launch_gh<2, 8>(P, grid, st) : launch_gh<2, 4>(P, grid, st);
   return y.G == 3 ? launch_gh<3, 4>(P, grid, st) : launch_gh<4, 4>(P, grid, st);

@@ -523,7 +523,7 @@ def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
     ((1, 8, 2, 128, 128, False), [257, 1], 0),               # nine to sixteen: two rounds, whole
     ((1, 8, 2, 128, 128, False), [512, 100], 0),
     ((1, 8, 2, 128, 128, False), [513, 769], 0),             # three rounds: cut
-    ((1, 32, 8, 128, 128, False), [3000, 2900], 0),          # one CTA per SM
+    ((1, 32, 8, 128, 128, False), [3000, 2900], 0),          # two rounds of chunks
     ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(18)], 0),       # 144 pairs: whole, one per SM
     ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(20)], 0),       # 160: two per SM
     ((1, 4, 2, 128, 128, False), [100 + 7 * i for i in range(34)], 0),         # more agents than lanes: equal ranges
