@@ -449,6 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
           sum0 = sum1 = 0ull;
           probabilities(xa, pr);
           probabilities(xb, pr + 16);
+          wait_st();                                     // the stores above go to the same columns, and only this orders two stores
           tmem_st32(half_addr, pr);
           u = unpair64(add2(sum0, sum1));
           s_half = u.x + u.y;

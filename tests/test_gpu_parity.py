@@ -1162,6 +1162,48 @@ def test_prefill_reference_moves_within_and_between_steps(H, spec_args, prefix, 
     assert p.dc.read_flags() == 0
 
 
+class HighPair(SteepPair):
+    """SteepPair's keys, whose first element of every group is the same large one at every position."""
+
+    def kv(self, layer, agent, n):
+        k, v = super().kv(layer, agent, n)
+        c = synth.rng(self.seed, 600 + agent).integers(0, 16, k.shape).astype(np.float32)
+        c[..., 0::64], c[..., 1::64] = 15.0, 0.0
+        return synth.f32_to_bf16_bits(c * np.float32(2.0 ** -4)), v
+
+
+@pytest.mark.parametrize("spec_args,prefix,chunks,window", [
+    ((1, 8, 2, 128, 128, False), [300, 0, 70], [100, 300, 1], 0),
+    ((1, 8, 2, 128, 128, False), [700], [200], 300),
+    ((1, 4, 4, 128, 128, False), [3000], [40], 0),           # few tiles: the keys are split
+    ((1, 4, 2, 256, 256, False), [300, 0], [100, 300], 0),
+    ((1, 4, 4, 192, 128, False), [300, 0], [100, 300], 200),
+    ((1, 16, 1, 576, 512, True), [300, 0], [10, 300], 0),
+])
+def test_prefill_probabilities_taken_again_replace_the_first_ones(H, spec_args, prefix, chunks, window):
+    """Every score lies hundreds of binary orders above a row's first reference (0), so all probabilities that are taken against
+    it are infinite, in every row and column; what the value product reads has to be those taken after the reference has moved,
+    in every launch.  The bound is that of the keys without rounding error above."""
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = HighPair(H, spec_args, lens, seed=79).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = f32(p.q(9, int(q_offs[-1])))
+    scale = 1.0 / math.sqrt(192 if spec_args[5] else spec_args[3])
+    q[..., 0::64] = 256.0 / scale / (spec_args[3] // 64)     # 15 / 16 of 256 from the groups' first elements, the others add a few
+    q = synth.f32_to_bf16_bits(q.astype(np.float32))
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, window, f32(q), scale)
+    assert lse_ref.min() > 200.0
+    m = max(float(np.abs(O.gather_dequant(p.opool, 0, p.tabs[a], 0, n, h)[1]).max())
+            for a, n in enumerate(lens) for h in range(spec_args[2]))
+    out, lse = p.dc.prefill(0, lens, q_offs, window, q, scale)
+    assert np.abs(out.cpu().numpy().astype(np.float64) - ref).max() <= m * (2.0 ** -10 + 2.0 ** -12)
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    for _ in range(3):
+        again, lse_again = p.dc.prefill(0, lens, q_offs, window, q, scale)
+        assert torch.equal(again, out) and torch.equal(lse_again, lse)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("spec_args,prefix,chunks", [
     ((1, 6, 2, 128, 128, False), [70, 0, 5, 0], [85, 43, 1, 42]),    # 42 queries x 3 heads a tile (two rows idle): full, one over, one
     ((1, 4, 4, 128, 128, False), [3000], [129]),                 # the keys are split: records
