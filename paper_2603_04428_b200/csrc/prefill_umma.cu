@@ -470,8 +470,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const bool zero = bad || n_step == 0 || l <= 0.f;
     const bool final = P.x.n_splits == 1;                // else the row is left as a record
     const float inv = zero ? 0.f : final ? 1.f / l : 1.f;
-    // (the tile's queries are not needed any more: every product that read them is complete)
-    uint8_t* const buf = sm.qs[t] + (warp & 3) * kRowsBytes;
+    // the warp's own query rows, which no product needs any more (another warp's may still be on their way here where the CTA has no keys)
+    uint8_t* const buf = sm.qs[t] + (warp & 3) * 4 * 2048;
+    static_assert(kRowsBytes <= 4 * 2048, "");
     const size_t at = final ? row_index * 128 : (row_index * P.x.n_splits + split) * prefill_record(128);
     const RowsOut to = rows_out(at, mine, final && P.out_dtype == Q4KV_OUT_BF16);
 #pragma unroll 1

@@ -1074,6 +1074,34 @@ def test_prefill_key_splits_and_head_counts(H, spec_args, prefix, chunks, window
     check_prefill(H, spec_args, prefix, chunks, window, sb_dtype)
 
 
+@pytest.mark.parametrize("spec_args", [(1, 4, 4, 128, 128, False), (1, 8, 2, 128, 128, False), (1, 4, 2, 256, 256, False),
+                                       (1, 4, 4, 192, 128, False), (1, 16, 1, 576, 512, True)])
+def test_parts_without_keys_leave_empty_records(H, spec_args):
+    """A part of the keys that holds none of a row's leaves an accumulator of zeros and weight zero: nothing that a warp keeps in
+    shared memory meanwhile (its query rows, or its neighbour's) gets into the record."""
+    from paper_2603_04428_b200 import binding as B
+    prefix, chunks = [6000, 3], [40, 40]                     # the second agent's keys lie in the first part
+    lens = [p0 + c for p0, c in zip(prefix, chunks)]
+    p = Pair(H, spec_args, lens, seed=97).fill()
+    q_offs = np.concatenate([[0], np.cumsum(chunks)]).astype(np.int32)
+    q = p.q(9, int(q_offs[-1]))
+    scale = 1.0 / math.sqrt(192 if spec_args[5] else spec_args[3])
+    ref, lse_ref = O.prefill_attention(p.opool, 0, p.tabs, lens, q_offs, 0, f32(q), scale)
+    stride, rows = spec_args[4] + 4, int(q_offs[-1]) * spec_args[1]
+    need = B.q4kv_workspace_bytes(p.dc.spec, 2, max(lens), int(q_offs[-1]))
+    p.dc._ws = torch.zeros(need + 16 * rows * stride * 4, dtype=torch.uint8, device="cuda")
+    rec = p.dc._ws[B.WORKSPACE_HEADER_BYTES:][:16 * rows * stride * 4].view(torch.float32).view(-1, stride)
+    for _ in range(5):
+        rec.fill_(7.0)
+        out, lse = p.dc.prefill(0, lens, q_offs, 0, q, scale, max_kv_len=max(lens))
+        empty = torch.isneginf(rec[:, spec_args[4]])
+        assert int(empty.sum()) >= 40 * spec_args[1]         # the launch was cut, and the second agent's later parts are empty
+        assert not rec[empty][:, :spec_args[4]].any() and not rec[empty][:, spec_args[4] + 1].any()
+    assert_attention_close(out.cpu().numpy(), ref)
+    assert_lse_close(lse.cpu().numpy(), lse_ref)
+    assert p.dc.read_flags() == 0
+
+
 @pytest.mark.parametrize("spec_args,window", [
     ((1, 8, 2, 128, 128, False), 0),
     ((1, 8, 2, 128, 128, False), 90),
