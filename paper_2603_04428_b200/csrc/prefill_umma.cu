@@ -421,38 +421,41 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         float2 u = unpair64(add2(sum0, sum1));
         float s_half = u.x + u.y;
         const bool outgrown = !(s_half <= kSumLimit) || m_ref == -INFINITY;
-        if (__any_sync(0xffffffffu, outgrown)) {         // rare: the row's reference moves and the half is taken again
+        if (__any_sync(0xffffffffu, outgrown)) {         // rare: a row's reference may have to move
           float cm = fmaxf(maximum(xa), maximum(xb));
           if (cm != -INFINITY) cm *= kappa;              // kappa > 0
           const float m_new = fmaxf(m_ref, cm);
           const bool grow = outgrown && m_new > m_ref;
-          if (j + half > 0 && __any_sync(0xffffffffu, grow)) {
-            // rescale the accumulator row once the value products issued so far have landed (those of earlier steps have: the
-            // scores were issued behind them)
-            if (half == 1 && !__all_sync(0xffffffffu, mbar_wait(&sm.o_half[t], (uint32_t)j, abort_flag))) break;
-            fence_after_sync();
-            const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;         // m_ref = -inf: 0
+          // (no row's moves where the rows without a reference have no key here either: a window's or a part's first steps)
+          if (__any_sync(0xffffffffu, grow)) {
+            if (j + half > 0) {
+              // rescale the accumulator row once the value products issued so far have landed (those of earlier steps have:
+              // the scores were issued behind them)
+              if (half == 1 && !__all_sync(0xffffffffu, mbar_wait(&sm.o_half[t], (uint32_t)j, abort_flag))) break;
+              fence_after_sync();
+              const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;       // m_ref = -inf: 0
 #pragma unroll 1
-            for (int part = 0; part < 8; ++part) {
-              uint32_t orow[16];
-              tmem_ld16(o_addr + 16 * part, orow);
-              wait_ld16(orow);
+              for (int part = 0; part < 8; ++part) {
+                uint32_t orow[16];
+                tmem_ld16(o_addr + 16 * part, orow);
+                wait_ld16(orow);
 #pragma unroll
-              for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
-              tmem_st16(o_addr + 16 * part, orow);
+                for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * f);
+                tmem_st16(o_addr + 16 * part, orow);
+              }
+              if (grow) l *= f;
             }
-            if (grow) l *= f;
+            if (grow) m_ref = m_new;
+            neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+            nn = pair64(neg_m, neg_m);
+            sum0 = sum1 = 0ull;
+            probabilities(xa, pr);
+            probabilities(xb, pr + 16);
+            wait_st();                                   // the stores above go to the same columns, and only this orders two stores
+            tmem_st32(half_addr, pr);
+            u = unpair64(add2(sum0, sum1));
+            s_half = u.x + u.y;
           }
-          if (grow) m_ref = m_new;
-          neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
-          nn = pair64(neg_m, neg_m);
-          sum0 = sum1 = 0ull;
-          probabilities(xa, pr);
-          probabilities(xb, pr + 16);
-          wait_st();                                     // the stores above go to the same columns, and only this orders two stores
-          tmem_st32(half_addr, pr);
-          u = unpair64(add2(sum0, sum1));
-          s_half = u.x + u.y;
         }
         l += s_half;
         wait_st();
