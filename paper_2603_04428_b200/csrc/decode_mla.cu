@@ -539,8 +539,8 @@ __global__ void __launch_bounds__(kMergeThreads) merge_mla_kernel(int Hq, int n_
   if (__any_sync(0xffffffffu, bad)) L = 0.f;             // a poisoned split zeroes the row
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   auto add = [&](float m, const float4& v) {
-    if (m == -INFINITY) return;                          // an empty split's record holds no data
     const float w = fast_exp2(m - M);
+    if (!(w > 0.f)) return;                              // an empty split's record holds no data; no weight (NaN) where M is infinite
     acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y); acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
   };
 #pragma unroll

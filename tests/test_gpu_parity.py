@@ -1232,6 +1232,24 @@ def test_prefill_probabilities_taken_again_replace_the_first_ones(H, spec_args, 
     assert p.dc.read_flags() == 0
 
 
+@pytest.mark.parametrize("exact", [False, True])
+def test_latent_decode_of_an_infinite_score_is_an_empty_row(H, exact):
+    """Scores that overflow binary32 leave no weights: the row is zeros with lse -inf, and the other rows are what they were."""
+    lens = [300, 2000]
+    p = HighPair(H, (1, 16, 1, 576, 512, True), lens, seed=89, exact_products=exact).fill()
+    q = f32(p.q(9, 2))
+    scale = 1.0 / math.sqrt(192)
+    good, lse_good = p.dc.decode(0, lens, 0, synth.f32_to_bf16_bits(q), scale)
+    for a, h in ((0, 3), (1, 15)):
+        q[a, h] = 0.0
+        q[a, h, 0] = 3.0e38
+    out, lse = p.dc.decode(0, lens, 0, synth.f32_to_bf16_bits(q), scale)
+    hit = torch.zeros((2, 16), dtype=torch.bool, device="cuda")
+    hit[0, 3] = hit[1, 15] = True
+    assert not out[hit].any() and torch.isneginf(lse[hit]).all()
+    assert torch.isfinite(out[~hit]).all() and torch.allclose(out[~hit], good[~hit], atol=1e-3) and torch.allclose(lse[~hit], lse_good[~hit], atol=1e-3)
+
+
 @pytest.mark.parametrize("spec_args,prefix,chunks", [
     ((1, 6, 2, 128, 128, False), [70, 0, 5, 0], [85, 43, 1, 42]),    # 42 queries x 3 heads a tile (two rows idle): full, one over, one
     ((1, 4, 4, 128, 128, False), [3000], [129]),                 # the keys are split: records
