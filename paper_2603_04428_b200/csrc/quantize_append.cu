@@ -172,7 +172,7 @@ quantize_append_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_a
 // in each lane the 8 positions x 8 elements block of nibbles that an in-register transposition turns into eight token-packed
 // words.  The chunk is assembled in shared memory and stored as whole 16-byte pieces; a chunk that the phase fills only in
 // part (an unaligned start or end) starts from its present bytes.
-// Bound by instruction issue (about 14 instructions an element) with the sixteen warps an SM has room for.  Measured, each lane
+// Bound by instruction issue (about 16 instructions an element) with the sixteen warps an SM has room for.  Measured, each lane
 // loading its own rows (32 lines per load) -> rows copied whole lines at a time: d = 128, 8 KV heads, 8 x 1024 tokens 16.6 -> 15.8 us,
 // 8 x 4096 55.8 -> 48.7; d = 256 97.7 -> 84.4; 192 / 128, where an item was four groups of one octet, 16 KV heads, 8 x 1024 53.1 ->
 // 37.4; latent cache 8 x 4096 21.2 -> 18.3.  Three CTAs per SM of 80 registers: 21.8 us on the first.  kWpc = 1 where the units fill the
@@ -283,10 +283,6 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
   uint8_t* gchunk = head_block(pool, y, layer, un.block, hk) + (size_t)(un.chunk & 7) * y.chunk_bytes;
   uint8_t* chunk = stage_all + (size_t)(warp / kWpc) * y.chunk_bytes;
   const int n16 = y.chunk_bytes / 16;
-  if (lo != c0 || hi != c0 + 32) {
-    for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(chunk)[q] = reinterpret_cast<const uint4*>(gchunk)[q];
-    unit_sync();
-  }
   const int n_groups = y.G + (y.alias ? 0 : y.Gv);
   const int n_items = ((o_last - o_first + 1) * n_groups + 3) >> 2;
   constexpr float kMagic = 12582912.0f;                  // 1.5 * 2^23: q + kMagic holds q rounded to nearest even in its low bits
@@ -324,7 +320,13 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  // On its way while the chunk's present bytes are fetched (behind them: 3 x 300 tokens at 8 KV heads 6.3 us a launch, now 5.8; 5 x 64 on
+  // 1003 cached ones 6.1, now 5.8; and the registers did not suffice by three words)
   if (sub < n_items) copy_item(sub);
+  if (lo != c0 || hi != c0 + 32) {
+    for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(chunk)[q] = reinterpret_cast<const uint4*>(gchunk)[q];
+    unit_sync();
+  }
   for (int t = sub; t < n_items; t += kWpc) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
