@@ -249,8 +249,9 @@ __device__ inline void find_chunk_unit(int u, int n_agents, int max_blocks, int 
   if (!found && lane == 0) out->agent = -1;
 }
 
-// kFour: four groups per token, so that an item is one octet (fewer instructions for the common shape)
-template <int kWpc, bool kFour>
+// kFour: four groups per token, so that an item is one octet (fewer instructions for the common shape).  kRing: the rows come through
+// shared memory; else (few units) a lane loads its own.
+template <int kWpc, bool kFour, bool kRing>
 __global__ void __launch_bounds__(kThreads, 2)
 quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, int n_agents, int max_blocks,
                             const int32_t* __restrict__ tables, const int32_t* __restrict__ pos,
@@ -320,21 +321,36 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  auto load_item = [&](int t, uint4 (&raw)[8]) {
+    const Pair pr = pair_of(t);
+    const int first = max(lo, c0 + 8 * pr.o), cnt = min(hi, c0 + 8 * pr.o + 8) - first, i = s - (first & 7);
+    const bool is_v = pr.gq >= y.G, real = pr.has && i >= 0 && i < cnt;
+    const size_t row = (size_t)(un.r0 + (first - un.p) + i) * y.Hkv + hk;
+    const uint4* const src = reinterpret_cast<const uint4*>(is_v ? v_new + row * y.Dv + 64 * (pr.gq - y.G) : k_new + row * y.D + 64 * pr.gq);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) raw[j] = real ? __ldca(src + j) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  uint4 raw[8];
   // On its way while the chunk's present bytes are fetched (behind them: 3 x 300 tokens at 8 KV heads 6.3 us a launch, now 5.8; 5 x 64 on
   // 1003 cached ones 6.1, now 5.8; and the registers did not suffice by three words)
-  if (sub < n_items) copy_item(sub);
+  if (kRing && sub < n_items) copy_item(sub);
   if (lo != c0 || hi != c0 + 32) {
     for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(chunk)[q] = reinterpret_cast<const uint4*>(gchunk)[q];
     unit_sync();
   }
+  if (!kRing && sub < n_items) load_item(sub, raw);
   for (int t = sub; t < n_items; t += kWpc) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-    uint4 raw[8];
+    uint4 nxt[kRing ? 1 : 8];
+    if constexpr (kRing) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 8; ++j) raw[j] = *reinterpret_cast<const uint4*>(ring + s * 512 + gq0 * 128 + ((j ^ s) << 4));
-    __syncwarp();                                        // the whole warp has its rows: the next item's may come
-    if (t + kWpc < n_items) copy_item(t + kWpc);
+      for (int j = 0; j < 8; ++j) raw[j] = *reinterpret_cast<const uint4*>(ring + s * 512 + gq0 * 128 + ((j ^ s) << 4));
+      __syncwarp();                                      // the whole warp has its rows: the next item's may come
+      if (t + kWpc < n_items) copy_item(t + kWpc);
+    } else if (t + kWpc < n_items) {
+      load_item(t + kWpc, nxt);
+    }
     const Pair pr = pair_of(t);
     const int o = pr.o, gq = pr.gq;
     const int first = max(lo, c0 + 8 * o), cnt = min(hi, c0 + 8 * o + 8) - first;
@@ -424,15 +440,21 @@ quantize_append_bulk_kernel(Layout y, uint8_t* pool, int n_blocks, int layer, in
         }
       }
     }
+    if constexpr (!kRing) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) raw[j] = nxt[j];
+    }
   }
   unit_sync();
   for (int q = lane + 32 * sub; q < n16; q += 32 * kWpc) reinterpret_cast<uint4*>(gchunk)[q] = reinterpret_cast<const uint4*>(chunk)[q];
 }
 
 constexpr size_t kBulkSmem = 112 * 1024;                 // two CTAs per SM
-size_t bulk_smem(const Layout& y, int wpc) { return (size_t)(kThreads / 32 / wpc) * y.chunk_bytes + (size_t)(kThreads / 32) * kItemBytes; }
+size_t bulk_smem(const Layout& y, int wpc, bool ring = true) {
+  return (size_t)(kThreads / 32 / wpc) * y.chunk_bytes + (ring ? (size_t)(kThreads / 32) * kItemBytes : 0);
+}
 
-template <int kWpc, bool kFour>
+template <int kWpc, bool kFour, bool kRing = true>
 cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer, const q4kv_batch& b, const int32_t* pos,
                         const int32_t* new_offs, int chunk_units, const void* k_new, const void* v_new, int32_t* flags,
                         cudaStream_t st) {
@@ -440,14 +462,14 @@ cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((warps + kThreads / 32 - 1) / (kThreads / 32)));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = bulk_smem(y, kWpc);
+  cfg.dynamicSmemBytes = bulk_smem(y, kWpc, kRing);
   cfg.stream = st;
   static bool configured[64] = {};     // the attribute is per function and device: set it once for each
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(quantize_append_bulk_kernel<kWpc, kFour>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmem);
+    e = cudaFuncSetAttribute(quantize_append_bulk_kernel<kWpc, kFour, kRing>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
@@ -456,7 +478,7 @@ cudaError_t launch_bulk(const Layout& y, uint8_t* pool, int n_blocks, int layer,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel<kWpc, kFour>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
+  return cudaLaunchKernelEx(&cfg, quantize_append_bulk_kernel<kWpc, kFour, kRing>, y, pool, n_blocks, layer, b.n_agents, b.max_blocks,
                             b.block_tables, pos, new_offs, (const uint16_t*)k_new, (const uint16_t*)v_new, flags, chunk_units);
 }
 
@@ -489,9 +511,16 @@ cudaError_t launch_quantize_append(const Layout& y, void* pool, int n_blocks, in
     // a phase of many tokens per agent: one warp per (32-token chunk, KV head)
     const int chunk_units = total_new / 32 + 2 * b.n_agents;   // >= sum over agents of the chunks their new range touches
     // four warps per unit while one warp each would leave half of the resident warps (sixteen per SM) without work
-    const bool four = (long long)chunk_units * y.Hkv < 8ll * sm_count() || bulk_smem(y, 1) > kBulkSmem;
+    const long long all_units = (long long)chunk_units * y.Hkv;
+    const bool four = all_units < 8ll * sm_count() || bulk_smem(y, 1) > kBulkSmem;
+    // One unit or less for every two SMs, and not four groups a token: lanes load their own rows, which takes fewer steps and leaves
+    // the next launch's CTAs their shared memory.  16 layers, us, through shared memory and without: latent cache 1 x 64 tokens (4 units)
+    // 101.6 / 89.3, 4 x 500 (70) 120.6 / 118.4, 6 x 500 (105) 145.1 / 145.0, 6 x 1000 135.3 / 137.4; d = 256 1 x 44 (24) 104.2 / 99.9, 2 x 128
+    // (96) 131.8 / 137.1; 192 / 128 2 x 64 (128) 109.2 / 112.0.  Before attention, four layers: d = 256, 44 tokens 81.3 / 75.7, 192 / 128, 56
+    // tokens (48) 92.3 / 90.1.  Four groups a token (an item is an octet, a warp has one): 5 x 64 tokens 75.7 / 86.9, 2 x 100 79.5 / 84.6.
+    const bool few = 2 * all_units <= sm_count();
     const auto launch = y.G + (y.alias ? 0 : y.Gv) == 4 ? (four ? launch_bulk<4, true> : launch_bulk<1, true>)
-                                                        : (four ? launch_bulk<4, false> : launch_bulk<1, false>);
+                        : few ? launch_bulk<4, false, false> : (four ? launch_bulk<4, false> : launch_bulk<1, false>);
     return launch(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, chunk_units, k_new, v_new, flags, st);
   }
   return launch_octets(y, (uint8_t*)pool, n_blocks, layer, b, pos, new_offs, units, k_new, v_new, flags, st);

@@ -1145,7 +1145,7 @@ def test_one_wave_of_tiles_beside_single_queries_is_not_cut(H):
 @pytest.mark.parametrize("spec_args,lens,sb_dtype", [
     ((1, 16, 16, 192, 128, False), [2200, 31], 0),           # 16 x (69 + 4) units: four warps each
     ((1, 16, 16, 192, 128, False), [2290, 31], 1),           # 16 x (72 + 4) units: one warp each
-    ((1, 16, 1, 576, 512, True), [38000], 0),                # latent rows, one warp per unit
+    ((1, 16, 1, 576, 512, True), [38000], 0),                # latent rows: four (eight chunks and their rows are more than an SM's half)
 ])
 def test_append_on_both_sides_of_the_unit_split(H, spec_args, lens, sb_dtype):
     Pair(H, spec_args, lens, seed=61, sb_dtype=sb_dtype).fill().check_packed_equal()
@@ -1274,6 +1274,20 @@ def test_prefill_rows_of_partial_tiles(H, spec_args, prefix, chunks):
     out16, _ = p.dc.prefill(0, lens, q_offs, 0, q, scale, out_dtype=B.OUT_BF16)
     assert torch.equal(out16, out.to(torch.bfloat16))        # the same sums, rounded once more
     assert p.dc.read_flags() == 0
+
+
+@pytest.mark.parametrize("spec_args,chunks", [               # units of 32 tokens and a KV head, two more per agent than whole ones
+    ((1, 16, 1, 576, 512, True), [13, 2335]),                # 74: lanes load their own rows
+    ((1, 16, 1, 576, 512, True), [13, 2336]),                # 75: through shared memory
+    ((1, 16, 8, 256, 256, False), [107, 44, 255]),           # 24 and 72
+    ((1, 16, 8, 256, 256, False), [8, 256]),                 # 80
+    ((1, 16, 16, 192, 128, False), [13, 95, 8]),             # 64 and 32
+    ((1, 16, 16, 192, 128, False), [13, 96]),                # 80
+    ((1, 8, 2, 64, 64, False), [13, 70, 1100]),              # 8 and 72; two groups a token
+])
+@pytest.mark.parametrize("sb_dtype", [0, 1])
+def test_append_on_both_sides_of_the_few_unit_form(H, spec_args, chunks, sb_dtype):
+    Pair(H, spec_args, [sum(chunks)], seed=67, sb_dtype=sb_dtype).fill(chunks).check_packed_equal()
 
 
 @pytest.mark.parametrize("name", list(SPECS))                # 2, 4, 5, 8 and 9 groups per token
