@@ -329,10 +329,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const int row = (warp & 3) * 32 + lane;              // tensor-memory lane
     const uint32_t lane_addr = tb + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_addr = lane_addr + kColS + 128 * t, o_addr = lane_addr + kColO + 128 * t;
-    const int h = row / tile_q, i = i_min + t * tile_q + row % tile_q;
-    const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
-    const int pq = prefix + i;                           // this row's position
-    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
     float kappa = 0.f;                                   // score in log2 units = S * kappa
     {
       // ---- stage the warp's query rows: bf16 -> binary16 times a power of two per row.  Lane l takes the pieces l / 8, + 4, + 8, + 12 of
@@ -358,6 +354,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
       fence_async_smem();
       mbar_arrive(&sm.q_ready);
     }
+    const int h = row / tile_q, i = i_min + t * tile_q + row % tile_q;
+    const bool mine = i < q_len && h < n_rep;            // (128 need not be a multiple of n_rep: the last rows are idle)
+    const int pq = prefix + i;                           // this row's position
+    const size_t row_index = (size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h;
     float m_ref = -INFINITY, l = 0.f;                    // p = 2^(s - m_ref); m_ref trails the true maximum by at most 2^12
     for (int j = 0; j < n_step; ++j) {
       // one warp of the tile polls and the others sleep at a barrier: polling takes issue slots from the other tile's warps
