@@ -26,8 +26,10 @@ __device__ inline uint4 query8(uint4 v, float sf) {
 // What a CTA reads first, asked of L2 while the preceding kernel drains: a prefetch returns nothing, and L2 is where the writes of the
 // preceding kernels land, so it may come before the wait for them.  Lane l of one warp asks for the 64-key block it0 + l (block tables are
 // inputs that no kernel writes; the table entries are then in L1 for the loader), the threads of the tile's rows for their query row.
-// Latent cache, 3 agents of 250 to 512 on 2000 to 4000 tokens, with the append: 210.3 -> 206.3 us a layer; d = 256, six windowed layers
-// 496.8 -> 494.9.  Not at d = 128, whose tiles' steps are long beside it: one agent 1377.0 / 1375.6, injection pass 5135 / 5145.
+// Latent cache, 3 agents of 250 to 512 on 2000 to 4000 tokens, with the append: 210.3 -> 206.3 us a layer, blocks and rows.  d = 256 and
+// 192 / 128: rows only.  Their blocks come by bulk copies that a loader issues at once; asked for beforehand as well, four layers with the
+// append, 44 tokens on 107 72.5 -> 75.1 us, 2 x (2000 + 203) 183.3 -> 184.6, 6 x (3000 + 400) in a window 422.8 -> 424.7.  Not at d = 128,
+// whose tiles' steps are long beside it: one agent 1377.0 / 1375.6, injection pass 5135 / 5145.
 template <class Par>
 __device__ __forceinline__ void ask_for_blocks(const Par& P, int a, int hk, int it0, int count, uint32_t chunk_bytes) {
   const int l = threadIdx.x & 31;

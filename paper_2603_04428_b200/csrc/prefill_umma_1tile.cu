@@ -151,7 +151,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_1tile_kernel(const _
   __syncthreads();
   fence_after_sync();
   const uint32_t tb = sm.tmem_base;
-  if (warp == kLoadWarp) ask_for_blocks(P, a, hk, it0, min(n_iter, kRawSlots), kChunkBytes);
   if (warp < kSoftmaxWarps / 2 && !bad_len) {
     const int h = (int)threadIdx.x / tile_q, i = i_min + (int)threadIdx.x % tile_q;
     if (i < q_len && h < n_rep) ask_for_row<kD>(P.q + ((size_t)(q0 + i) * y.Hq + (size_t)hk * n_rep + h) * kD);
