@@ -222,7 +222,7 @@ __device__ __noinline__ void find_agent(const Par& P, RangeStart& rs) {
   }
 }
 
-// more_rounds: 0, 1, or 2 for 1 where the pairs are few (see below)
+// more_rounds: -1 for none, 0, 1, or 2 for 1 where the pairs are few (see below)
 template <class Par>
 __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_t nw, int more_rounds) {
   const int lane = threadIdx.x & 31;
@@ -275,14 +275,16 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
 #pragma unroll 4
     for (int a = 0; a < n_agents; ++a) total += parts_of(__shfl_sync(0xffffffffu, nc, a), size, inv);
     const unsigned fits = __ballot_sync(0xffffffffu, total * Hkv <= (int)most && lane <= kWholeSlack);
-    // A pair whole in one CTA needs no records and no ticket (2 us).  That is worth a round of chunks, one per warp (0.9 us at d = 128;
-    // not where a round is two chunks' work: d = 256, and eight heads but for few pairs), and more where there are many.  Measured, us a
-    // launch, cut and whole: 8 KV heads, one agent x 350 tokens 6.4 / 5.6, x 480 6.5 / 5.8, x 600 (two rounds more) 6.4 / 7.2; 32 agents x
-    // 4096 41.3 / 38.3; d = 256, one x 350 9.0 / 9.9, 20 agents in a window of 1024 27.0 / 26.2; eight heads, 16 x 700 15.0 / 15.9.
+    // A pair whole in one CTA needs no records and no ticket (2 us).  That is worth a round of chunks, one per warp, where the pairs are
+    // few, and a seventh of the rounds where there are many.  Measured, us a launch, cut and whole: eight heads, 16 x 700 tokens
+    // 15.0 / 15.9; d = 256, one x 350 9.0 / 9.9, 20 agents in a window of 1024 27.0 / 26.2.  Up to four heads at d = 128 stay cut all
+    // the same: terms of p * s below 2^-24 are cut off against the reference of all the chunks that a warp adds up, and twice the
+    // chunks lose more.  Error against 64 bits (relative, outlier channels), cut and whole, 8 KV heads: one agent x 480 tokens 1.44e-4 /
+    // 1.95e-4 (6.5 / 5.8 us), 32 x 4096 8.5e-4 / 10.6e-4 (39.4 / 35.9 us); d = 256, 20 in a window 3.13e-4 / 3.13e-4.
     const int l = fits ? __ffs(fits) - 1 : 0, pairs = n_agents * Hkv;
     const int rounds = (size0 + l + (int)nw - 1) / (int)nw;
-    const int extra = more_rounds == 1 || 4 * pairs <= (int)most ? min(more_rounds, 1) : 0;
-    const bool uncut = pairs <= (int)most && (nc_max + (int)nw - 1) / (int)nw <= rounds + extra + ((rounds * 37) >> 8);
+    const int extra = more_rounds < 0 ? 0 : (rounds * 37 >> 8) + (more_rounds == 1 || 4 * pairs <= (int)most ? min(more_rounds, 1) : 0);
+    const bool uncut = pairs <= (int)most && (nc_max + (int)nw - 1) / (int)nw <= rounds + extra;
     if (fits || uncut) {
       const int best = uncut ? nc_max : size0 + l;
       rs.n_ctas = uncut ? pairs : __shfl_sync(0xffffffffu, total, l) * Hkv;
@@ -299,8 +301,8 @@ __device__ inline RangeStart find_range(const Par& P, int cta, int grid, uint32_
       rs.splits = __shfl_sync(0xffffffffu, m, a);
       const int at = cta - (__shfl_sync(0xffffffffu, inc, a) - rs.splits * Hkv), n = __shfl_sync(0xffffffffu, nc, a);
       const float per = __fdividef(1.f, (float)rs.splits);
-      auto quotient = [&](int x) {                       // below 2^24 the float quotient is off by one at most
-        if (x >= 1 << 24) return x / rs.splits;
+      auto quotient = [&](int x) {                       // CTAs and a pair's chunks; below 2^20 the float quotient is off by one at most
+        if (x >= 1 << 20) return x / rs.splits;
         int q = (int)((float)x * per);
         q -= q * rs.splits > x;
         return q + ((q + 1) * rs.splits <= x);
@@ -518,13 +520,9 @@ __device__ __forceinline__ void stage_query_row(uint4 (*qfrag)[32], float (*qsum
   }
 }
 
-// The fused append (one new token per agent).  The CTA that holds the chunk of an agent's newest position quantizes that
-// token's K and V rows (Section 3.2 quantizer, the arithmetic of the append kernel) when it stages the segment's query: a
-// warp per 64-element group, two elements per lane, by the warps that have no query row to stage, so that neither waits
-// for the other.  The warp that holds the chunk writes the words into it once it has landed -- in shared memory for this
-// launch, in the pool for the following ones.  Every chunk is held by exactly one warp of the grid, so nobody else reads
-// or writes these words during the launch.  (One warp doing all of it, eight elements per lane, was 3.5 us on the
-// critical path of every launch: 500 instructions that run once per launch and come from far away.)
+// The fused append (one new token per agent).  The warp that holds the chunk of an agent's newest position writes the new row's
+// words into it once it has landed -- in shared memory for this launch, in the pool for the following ones.  Every chunk is held
+// by exactly one warp of the grid, so nobody else reads or writes these words during the launch.
 // The value codes are token-packed: one nibble of each of the row's d_v words is replaced.
 template <int G, int H>
 __device__ __noinline__ void patch_new_row(const Smem<G, H>& sm, uint8_t* keys, uint8_t* values, uint8_t* gchunk, int tau, int lane) {
@@ -1014,7 +1012,7 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
   // ---- this CTA's unit range and its first two segments: one warp, the others set up shared memory (lengths and block
   // tables are inputs that no kernel writes) ----
   if (warp == 0) {
-    const RangeStart rs = find_range(P, cta, gridDim.x, NW, G == 4 ? 0 : H == 8 ? 2 : 1);
+    const RangeStart rs = find_range(P, cta, gridDim.x, NW, G == 4 ? 0 : H == 8 ? 2 : G == 3 ? 1 : -1);
     if (lane == 0) {
       if (rs.any_bad && cta == 0) raise_flag(P.flags, Q4KV_FLAG_BAD_LENGTH);
       sm.range = rs;
@@ -1073,7 +1071,10 @@ __global__ void __launch_bounds__(warps_of(G) * 32, kCtasPerSm) decode_mma_kerne
 
   const int my_chunks = n_chunks > warp ? (n_chunks - warp + NW - 1) / NW : 0;
   const int g = lane >> 2, tid = lane & 3;
-  // this warp's row of a segment's query; the new row's groups are quantized by the warps behind the query's (from 4 on)
+  // This warp's row of a segment's query.  The CTA that holds the newest position's chunk quantizes that token's K and V rows
+  // (Section 3.2 quantizer, the arithmetic of the append kernel) when it stages the query: a warp per 64-element group, two
+  // elements per lane, by the warps behind the query's (from 4 on), so that neither waits for the other.  (One warp doing all of
+  // it, eight elements per lane, was 3.5 us on the critical path of every launch: 500 instructions that come from far away.)
   constexpr int kNewWarps = NW - 4, kNewRounds = (G + Gv + kNewWarps - 1) / kNewWarps;
   auto query_row = [&](const Segment& s) { return P.q + ((size_t)(kSingles ? P.q_offs[s.a] : s.a) * y.Hq + (size_t)s.hk * n_rep + warp) * D + 8 * lane; };
   auto new_pair = [&](const Segment& s, int grp) {
@@ -1379,6 +1380,8 @@ cudaError_t launch_decode_mma(const Layout& y, const void* pool, int n_blocks, i
   // No more CTAs than can be of use: one that finds nothing to do costs the next launch a microsecond, because its CTAs come in as
   // this one's leave.  No fewer than pairs, which one CTA would take in turn: a launch on contexts of 30 tokens took 25.5 us with
   // a CTA per eight chunks, 4.3 with one per pair, on 100 tokens 7.2 and 4.3, at d = 256 13.8 and 6.7.
+  // Every pair is rounded up at the longest length, the only one known here: 16 KV heads of 837, 1088 and 227 tokens take 7.36 us with
+  // 240 CTAs and 7.31 with 204, but three of 1088 7.54 and 8.01, a round more for every pair.
   // Two CTAs per SM for small batches too.  One, so that the next launch's CTAs sit beside this one's: us a launch with one and with two,
   // 8 KV heads: 2 x 4096 9.8 / 9.2, 6 x 1500 9.4 / 8.8, 8 x 1000 9.8 / 8.6, 10 x 1000 12.0 / 9.6, 5 x 1100 9.1 / 7.9, 3 x 4096 11.1 / 10.4;
   // the other way round 16 agents x 300..700, 9.3 / 9.7.  It also doubles the chunks that a warp adds up, and the tensor cores truncate
