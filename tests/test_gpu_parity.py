@@ -520,12 +520,15 @@ def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
     ((1, 8, 2, 128, 128, False), [1], 0),                    # one chunk per pair, a CTA each
     ((1, 8, 2, 128, 128, False), [32, 33, 0, 7], 0),
     ((1, 8, 2, 128, 128, False), [255], 0),                  # eight chunks: a round of one CTA
-    ((1, 8, 2, 128, 128, False), [257, 1], 0),               # nine to sixteen: two rounds, whole
+    ((1, 8, 2, 128, 128, False), [257, 1], 0),               # nine to sixteen: two rounds, cut
     ((1, 8, 2, 128, 128, False), [512, 100], 0),
     ((1, 8, 2, 128, 128, False), [513, 769], 0),             # three rounds: cut
     ((1, 32, 8, 128, 128, False), [3000, 2900], 0),          # two rounds of chunks
-    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(18)], 0),       # 144 pairs: whole, one per SM
-    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(20)], 0),       # 160: two per SM
+    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(18)], 0),       # 144 pairs, whole
+    ((1, 32, 8, 128, 128, False), [200 + 11 * i for i in range(20)], 0),       # 160
+    ((1, 16, 16, 128, 128, False), [60 + 17 * i for i in range(18)], 0),       # 288, below two CTAs per SM
+    ((1, 16, 16, 128, 128, False), [60 + 17 * i for i in range(20)], 0),       # 320, above: equal ranges
+    ((1, 8, 8, 128, 128, False), [20 + 40 * i for i in range(32)], 0),         # 256 of a full warp of agents
     ((1, 4, 2, 128, 128, False), [100 + 7 * i for i in range(34)], 0),         # more agents than lanes: equal ranges
     ((1, 8, 2, 128, 128, False), [900, 300, 64], 200),       # a window
     ((1, 16, 2, 128, 128, False), [256, 257, 480], 0),       # eight heads, few pairs
@@ -536,7 +539,7 @@ def test_decode_query_heads_per_kv_head(H, spec_args, lens, window):
     ((1, 4, 4, 192, 128, False), [1, 255, 257, 520], 0),
 ])
 def test_decode_launch_sizes(H, spec_args, lens, window):
-    """Sizes at which the launch chooses its CTAs: a pair whole in one, cut, one or two CTAs per SM."""
+    """Sizes at which the launch chooses its CTAs: a pair whole in one, cut, more or fewer pairs than CTAs."""
     p = Pair(H, spec_args, lens, seed=43).fill()
     q = p.q(7, len(lens))
     scale = 1.0 / math.sqrt(spec_args[3])
